@@ -16,6 +16,7 @@
 #include <map>
 #include <new>
 #include <string>
+#include <tuple>
 #include <vector>
 
 using namespace gabp;
@@ -140,7 +141,7 @@ struct gabp_svm_s {
         cudaGraphExec_t exec = nullptr;
         std::vector<cudaEvent_t> ev;   // 2 per bracketed round when captured with profiling on
     };
-    std::map<std::pair<int, int>, Graph> graphs;   // by (rounds, profiling stride)
+    std::map<std::tuple<int, int, int>, Graph> graphs;   // by (rounds, profiling stride, message path)
     int profiling = 0;   // 0 off, k >= 1: the pair sweep of every k-th round is bracketed by events
     gabp_svm_profile prof{};
     bool solved = false;
@@ -212,7 +213,7 @@ Plan make_plan(int64_t n, int64_t m, int Nt, long long ntiles, int npad, int q_m
     // the BF16 store keeps an FP32 copy for the refinement residuals
     p.qref = q_mode == GABP_Q_BF16 ? align_up((size_t)dense_tiles * TT * sizeof(float), 256) : 0;
     p.work = (sparse ? 2 : 1) * align_up((size_t)ntiles * sizeof(int4), 256) + align_up((size_t)Nt * sizeof(int4), 256);
-    p.tab = align_up(align_up(sizeof(Inst), 16) + kMaxStages * align_up(sizeof(Sched), 16) + sizeof(StopOp) + 64, 256);
+    p.tab = align_up(align_up(sizeof(Inst), 16) + 2 * kMaxStages * align_up(sizeof(Sched), 16) + sizeof(StopOp) + 64, 256);
     p.nbl = align_up((size_t)((n + 31) / 32) * sizeof(int2), 256);
     p.ctrl = align_up(sizeof(Ctrl), 256);
     p.rhist = align_up((size_t)kRhistCap * sizeof(double), 256);
@@ -259,7 +260,7 @@ gabp_status build_sweep_list(gabp_svm_t h)
     int B[kMaxStages + 1];
     stage_bounds(Nt, h->nstages, B);
     const int nblk = (int)((h->n + 31) / 32);
-    Sched sc[kMaxStages];
+    Sched sc[2 * kMaxStages] = {};   // the same segments for both message paths
     for (int st = 0; st < h->nstages; ++st) {
         const long long off = (long long)wl.size();
         for (int I = 0; I < Nt; ++I)
@@ -270,7 +271,7 @@ gabp_status build_sweep_list(gabp_svm_t h)
                     wl.push_back(make_int4(0, I, J, (int)wl.size()));
                 }
             }
-        sc[st] = Sched{(long long)wl.size() - off, nblk, 1, off, Nt <= kWarpFinNt ? nblk : 0, 0};
+        sc[st] = sc[kMaxStages + st] = Sched{(long long)wl.size() - off, nblk, 1, off, Nt <= kWarpFinNt ? nblk : 0, 0};
     }
     h->nlive = (long long)wl.size();
     h->stats.tiles_kept = h->nlive;
@@ -297,7 +298,7 @@ gabp_status build_sweep_list(gabp_svm_t h)
     CK(cudaMemcpyAsync(h->slab, slab.data(), slab.size() * sizeof(int), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(h->srow, srow.data(), srow.size() * sizeof(int), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(h->tslot, tslot.data(), tslot.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(h->sched, sc, (size_t)h->nstages * sizeof(Sched), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(h->sched, sc, sizeof(sc), cudaMemcpyHostToDevice, s));
     CK(cudaStreamSynchronize(s));   // the host lists go out of scope
     return GABP_OK;
 }
@@ -339,6 +340,8 @@ gabp_status ensure_pair_storage(gabp_svm_t h, long long nslot)
     const size_t st = align_up(tt * (mb ? 4 : 8), 256);
     p.Pst = b;
     p.Hst = b + st;
+    p.nslot = nslot;
+    set_history(p, h->nstages, 2 * st);
     b += 2 * st;
     p.qstore = nullptr;
     p.qref = nullptr;
@@ -352,7 +355,6 @@ gabp_status ensure_pair_storage(gabp_svm_t h, long long nslot)
         b += align_up(tt * 2, 256) + align_up(tt * 4, 256);
     }
     p.part = (float*)b;
-    p.nslot = nslot;
     p.srow = h->srow;
     p.tslot = h->tslot;
     p.rsum = h->rsum;
@@ -444,6 +446,7 @@ gabp_status stage_and_form(gabp_svm_t h, const void* X, const float* y)
         p.tslot = nullptr;
         p.rsum = nullptr;
         p.rfix = reinterpret_cast<unsigned long long*>(h->rsum);
+        p.hist = 0;
         CK(cudaMemsetAsync(h->rsum, 0, (size_t)n * sizeof(double), s));
         CK(cudaMemcpyAsync(h->d_tab, &p, sizeof(Inst), cudaMemcpyHostToDevice, s));
         launch_form_q(h->d_tab, h->work_all, h->ntiles, s);
@@ -467,12 +470,14 @@ gabp_status stage_and_form(gabp_svm_t h, const void* X, const float* y)
             CK(launch_form_q_tc(h->d_tab, h->work, h->nlive, s));
             h->prof.kernel_launches += 1;
         }
+        launch_pair_z(h->d_tab, h->work, h->nlive, h->opts.q_mode, true, s);
     } else if (h->opts.q_mode == GABP_Q_F32) {
         launch_form_q(h->d_tab, h->work_all, h->ntiles, s);
         CK(cudaGetLastError());
         if (gabp_status st = build_sweep_list(h)) return st;
         launch_init(p, h->opts.diag_rule, (float)h->delta, s);
-        h->prof.kernel_launches += 2;
+        launch_pair_z(h->d_tab, h->work_all, h->ntiles, h->opts.q_mode, true, s);
+        h->prof.kernel_launches += 3;
         CK(cudaGetLastError());
     } else {
         // Precision form: the diagonal weighting uses the FP32 Gram's row sums
@@ -486,11 +491,14 @@ gabp_status stage_and_form(gabp_svm_t h, const void* X, const float* y)
         launch_init(p, h->opts.diag_rule, (float)h->delta, s);
         CK(cudaGetLastError());
         h->prof.kernel_launches += 4;
+        launch_pair_z(h->d_tab, h->work_all, h->ntiles, h->opts.q_mode, true, s);
+        h->prof.kernel_launches += 1;
         if (h->opts.q_mode == GABP_Q_BF16) {
             CK(launch_form_q_tc(h->d_tab, h->work_all, h->ntiles, s));
             h->prof.kernel_launches += 1;
         }
     }
+    CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s));
     h->formed = true;
     return GABP_OK;
@@ -516,10 +524,10 @@ static bool bracketed(int stride, int k) { return stride > 0 && k % stride == st
 // A captured chunk of `rounds` synchronous rounds; with profiling on, the
 // pair sweep of every profiling-th round in it is bracketed by two
 // event-record nodes.
-gabp_status get_graph(gabp_svm_t h, int rounds, gabp_svm_s::Graph** out)
+gabp_status get_graph(gabp_svm_t h, int rounds, int path, gabp_svm_s::Graph** out)
 {
     const int stride = h->profiling;
-    const auto key = std::make_pair(rounds, stride);
+    const auto key = std::make_tuple(rounds, stride, path);
     auto it = h->graphs.find(key);
     if (it != h->graphs.end()) { *out = &it->second; return GABP_OK; }
     gabp_svm_s::Graph G;
@@ -531,7 +539,7 @@ gabp_status get_graph(gabp_svm_t h, int rounds, gabp_svm_s::Graph** out)
     CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < rounds; ++k)
         launch_round(h->d_tab, h->work, h->nbl, h->sched, h->nstages, h->grid, h->opts.q_mode, h->opts.msg_bf16,
-                     h->stream, bracketed(stride, k) ? &G.ev[(size_t)2 * (k / stride)] : nullptr);
+                     1 << path, h->stream, bracketed(stride, k) ? &G.ev[(size_t)2 * (k / stride)] : nullptr);
     cudaError_t e = cudaStreamEndCapture(h->stream, &g);
     if (e != cudaSuccess) return fail(GABP_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
     e = cudaGraphInstantiate(&G.exec, g, 0);
@@ -564,7 +572,7 @@ gabp_status run_rounds(gabp_svm_t h, int iters, double tol, Ctrl* out)
     if (iters > 0) {
         const int len = tol > 0 ? std::min<int>(h->opts.chunk, iters) : iters;
         gabp_svm_s::Graph* g = nullptr;
-        if (gabp_status st = get_graph(h, len, &g)) return st;
+        if (gabp_status st = get_graph(h, len, h->hctrl->path, &g)) return st;
         const int max_chunks = (iters + len - 1) / len + 1;
         int t_before = h->hctrl->t;
         for (int c = 0; c < max_chunks; ++c) {
@@ -745,6 +753,8 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
     p.Pst = take(pl.state / 2);
     p.Hst = take(pl.state / 2);
     p.msg_bf16 = o.msg_bf16;
+    if (o.sparse_tau > 0) p.hist = 0;   // (set with the kept tiles' arrays)
+    else set_history(p, h->nstages, pl.state);
     p.qstore = pl.q ? take(pl.q) : nullptr;
     p.qref = pl.qref ? (float*)take(pl.qref) : (o.q_mode == GABP_Q_F32 ? (float*)p.qstore : nullptr);
     h->work_diag = (int4*)take(align_up((size_t)h->Nt * sizeof(int4), 256));
@@ -764,7 +774,7 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
         char* tb = (char*)take(pl.tab);
         h->d_tab = (Inst*)tb;
         h->sched = (Sched*)(tb + align_up(sizeof(Inst), 16));   // one per stage
-        h->d_ops = (StopOp*)(tb + align_up(sizeof(Inst), 16) + kMaxStages * align_up(sizeof(Sched), 16));
+        h->d_ops = (StopOp*)(tb + align_up(sizeof(Inst), 16) + 2 * kMaxStages * align_up(sizeof(Sched), 16));
         h->d_members = (int*)((char*)h->d_ops + align_up(sizeof(StopOp), 16));
     }
     h->nbl = (int2*)take(pl.nbl);
@@ -789,13 +799,14 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
     int B[kMaxStages + 1];
     stage_bounds(h->Nt, h->nstages, B);
     const int nblk = (int)((n + 31) / 32);
-    Sched sc[kMaxStages];
+    Sched sc[2 * kMaxStages] = {};   // the same segments for both message paths
     for (int st = 0; st < h->nstages; ++st) {
         const long long off = (long long)wl.size();
         for (int I = 0; I < h->Nt; ++I)
             for (int J = std::max(I, B[st]); J < B[st + 1]; ++J)
                 wl.push_back(make_int4(0, I, J, (int)((long long)I * h->Nt - (long long)I * (I - 1) / 2 + (J - I))));
-        sc[st] = Sched{(long long)wl.size() - off, nblk, 1, off, h->Nt <= kWarpFinNt ? nblk : 0, 0};
+        sc[st] = sc[kMaxStages + st] =
+            Sched{(long long)wl.size() - off, nblk, 1, off, h->Nt <= kWarpFinNt ? nblk : 0, 0};
     }
     std::vector<int2> nb((size_t)nblk);
     for (int b = 0; b < nblk; ++b) nb[(size_t)b] = make_int2(0, b);
@@ -809,7 +820,7 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h->work_diag, wd.data(), wd.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(h->sched, sc, (size_t)h->nstages * sizeof(Sched), cudaMemcpyHostToDevice, h->stream);
+        e = cudaMemcpyAsync(h->sched, sc, sizeof(sc), cudaMemcpyHostToDevice, h->stream);
     const int zero_slot = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_members, &zero_slot, sizeof(int), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);

@@ -78,6 +78,7 @@ struct Member {
     bool used = false;
     bool formed = false;     // Q formation finished (event)
     bool active = false;     // in the round lists
+    int path = -1;           // its message path, -1 until its control block has been read
     bool finished = false;   // results available
     Inst inst{};
     void* mem = nullptr;
@@ -200,18 +201,20 @@ __global__ void __launch_bounds__(kListThreads)
     __shared__ long long sc[kListThreads];
     __shared__ long long m_off[kListThreads];
     __shared__ int m_k[kListThreads], m_a[kListThreads], m_b[kListThreads], m_c[kListThreads];
-    __shared__ long long s_tiles[kMaxStages];
+    __shared__ long long s_tiles[2 * kMaxStages];
     __shared__ long long s_blocks[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = (int)blockDim.x >> 5;
-    // ---- tiles, stage by stage
+    // ---- tiles, stage by stage: first of the instances that keep a history,
+    // then of those that store their messages
     long long base = 0;
-    for (int s = 0; s < S; ++s) {
+    for (int ps = 0; ps < 2 * S; ++ps) {
+        const int path = ps / S, s = ps % S;
         long long carry = 0;
         for (int c0 = 0; c0 < cap; c0 += (int)blockDim.x) {
             const int k = c0 + tid;
             long long cnt = 0;
             int Nt = 0, Bs = 0, Be = 0;
-            if (k < cap && live[k]) {
+            if (k < cap && live[k] && tab[k].ctrl->path == path) {
                 Nt = tab[k].Nt;
                 int B[kMaxStages + 1];
                 stage_bounds(Nt, S, B);
@@ -243,7 +246,7 @@ __global__ void __launch_bounds__(kListThreads)
             carry += total;
             __syncthreads();
         }
-        if (tid == 0) s_tiles[s] = carry;
+        if (tid == 0) s_tiles[ps] = carry;
         base += carry;
     }
     // ---- node blocks: instances with at most kWarpFinNt tile rows first
@@ -274,7 +277,7 @@ __global__ void __launch_bounds__(kListThreads)
         bbase += carry;
     }
     __syncthreads();
-    if (blockIdx.x == 0 && tid < S) {
+    if (blockIdx.x == 0 && tid < 2 * S) {
         long long off = 0;
         for (int s2 = 0; s2 < tid; ++s2) off += s_tiles[s2];
         Sched q{};
@@ -283,7 +286,7 @@ __global__ void __launch_bounds__(kListThreads)
         q.ninst = cap;
         q.off = off;
         q.nsmall = (int)s_blocks[0];
-        sched[tid] = q;
+        sched[tid / S * kMaxStages + tid % S] = q;
     }
 }
 
@@ -432,7 +435,7 @@ class Engine {
         const size_t b_bl = aup((size_t)cap_members * sizeof(int2), 256);
         const size_t b_bt = aup((size_t)cap_members * sizeof(double), 256);
         char* base = nullptr;
-        const size_t b_sched = aup((size_t)kMaxStages * sizeof(Sched), 256);
+        const size_t b_sched = aup((size_t)2 * kMaxStages * sizeof(Sched), 256);
         const size_t b_live = aup((size_t)cap_members * sizeof(int), 256);
         EK(cudaMalloc((void**)&base,
                       b_tab + b_ctrl + 2 * b_work + 2 * b_nbl + b_ops + b_f3 + b_mem + 2 * b_bl + 2 * b_bt + b_sched + b_live));
@@ -451,7 +454,7 @@ class Engine {
         d_begin_tol = (double*)carve(b_bt);
         d_restart_list = (int2*)carve(b_bl);
         d_restart_tol = (double*)carve(b_bt);
-        d_sched = (Sched*)carve(b_sched);   // one per stage
+        d_sched = (Sched*)carve(b_sched);   // one per message path and stage
         d_live = (int*)carve(b_live);
         EK(cudaMemsetAsync(d_ctrl, 0, b_ctrl, stream));
         EK(cudaMemsetAsync(d_sched, 0, b_sched, stream));
@@ -571,7 +574,7 @@ class Engine {
         set_grid(0);
         std::memset(h_ops, 0, (size_t)cap_members * sizeof(StopOp));
         EK(cudaMemsetAsync(d_ctrl, 0, (size_t)cap_members * sizeof(Ctrl), stream));
-        EK(cudaMemsetAsync(d_sched, 0, (size_t)kMaxStages * sizeof(Sched), stream));
+        EK(cudaMemsetAsync(d_sched, 0, (size_t)2 * kMaxStages * sizeof(Sched), stream));
         return GABP_OK;
     }
 
@@ -654,6 +657,7 @@ class Engine {
         p.Pst = take(pl.state / 2);
         p.Hst = take(pl.state / 2);
         p.msg_bf16 = msg_bf16;
+        set_history(p, nstages, pl.state);
         p.qstore = pl.q ? take(pl.q) : nullptr;
         p.qref = pl.qref ? (float*)take(pl.qref) : (q_mode == 0 ? (float*)p.qstore : nullptr);
         M.final3 = (double*)take(pl.final3);
@@ -795,7 +799,8 @@ class Engine {
         launch_form_q(d_tab, d_tl, (long long)tiles_lead.size(), s);
         launch_init_list(d_tab, d_n, (int)nb.size(), diag_rule, (float)delta, s);
         if (q_mode == 1) EK(launch_form_q_tc(d_tab, d_tl, (long long)tiles_lead.size(), s));
-        launches += q_mode == 0 ? 5 : (q_mode == 1 ? 7 : 6);
+        launch_pair_z(d_tab, d_tl, (long long)tiles_lead.size(), q_mode, false, s);
+        launches += q_mode == 0 ? 6 : (q_mode == 1 ? 8 : 7);
         EK(cudaGetLastError());
         size_t g = 0;
         while (g < evg.size() && evg[g].refs > 0) ++g;
@@ -876,15 +881,33 @@ class Engine {
         return GABP_OK;
     }
 
+    // Message paths among the active instances (launch_round's mask).
+    int paths() const
+    {
+        int mask = 0;
+        for (const auto& M : mem)
+            if (M.used && M.active) mask |= M.path < 0 ? (1 << PATH_HIST) | (1 << PATH_STORED) : 1 << M.path;
+        return mask;
+    }
+    // The control blocks on the host show the paths of the armed instances.
+    void note_paths()
+    {
+        for (int k = 0; k < cap_members; ++k) {
+            Member& M = mem[(size_t)k];
+            if (M.used && M.active) M.path = h_ctrl[k].path;
+        }
+    }
+
     gabp_status graph_for(int rounds, cudaGraphExec_t* out)
     {
-        const int key = rounds * 16 + ctas_per_sm;
+        const int mask = paths();
+        const int key = (rounds * 16 + ctas_per_sm) * 4 + mask;
         auto it = graphs.find(key);
         if (it != graphs.end()) { *out = it->second; return GABP_OK; }
         cudaGraph_t g = nullptr;
         EK(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
         for (int k = 0; k < rounds; ++k)
-            launch_round(d_tab, d_work, d_nbl, d_sched, nstages, grid, q_mode, msg_bf16, stream);
+            launch_round(d_tab, d_work, d_nbl, d_sched, nstages, grid, q_mode, msg_bf16, mask, stream);
         EK(cudaStreamEndCapture(stream, &g));
         cudaGraphExec_t ex = nullptr;
         cudaError_t e = cudaGraphInstantiate(&ex, g, 0);
@@ -915,6 +938,7 @@ class Engine {
     {
         NvtxRange nv("gabp.batch.wait_rounds");
         EK(cudaStreamSynchronize(stream));
+        note_paths();
         return GABP_OK;
     }
 
@@ -1295,8 +1319,11 @@ gabp_status gabp_batch_solve(const gabp_problem* probs, int64_t count, const gab
         std::vector<int> all((size_t)count);
         for (int64_t k = 0; k < count; ++k) all[(size_t)k] = (int)k;
         if (gabp_status st = E.activate_list(all)) return st;
+        if (cudaMemcpyAsync(E.h_ctrl, E.d_ctrl, (size_t)count * sizeof(Ctrl), cudaMemcpyDeviceToHost, E.stream) != cudaSuccess)
+            return E.fail(GABP_ECUDA, "control read failed");
     }
-    cudaStreamSynchronize(E.stream);
+    if (cudaStreamSynchronize(E.stream) != cudaSuccess) return E.fail(GABP_ECUDA, "activation failed");
+    E.note_paths();
     ph.form_ms = ms_since(t0);
     t0 = clk::now();
     if (o.chunk <= 0) {

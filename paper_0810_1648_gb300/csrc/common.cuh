@@ -64,7 +64,38 @@ struct Ctrl {
                                          // ||b - Q mu||_inf * it
     double tol;
     double rinf;              // ||r(kstar)||_inf as seen by the convergence test
+    int path;                 // PATH_HIST or PATH_STORED, set when a solve is armed (choose_path)
+    unsigned int rq_bits;         // formation: the largest 1 / Q_ii (float bits)
+    unsigned int zpair_bits[2];   // formation, instances that it leaves open: the largest z and |q| / d over
+                                  // the pairs at Step 1 (float bits, k_pair_z)
+    // PATH_HIST: bounds on z and |q| / d over the pairs and rounds; the round's
+    // largest change of a mean over two rounds and largest mean (float bits)
+    float z, u;
+    unsigned int dmax_bits, mumax_bits;
+    float change;             // the changes of the last rounds as E weighs them, relative to the largest mean
+    int even;                 // whether the even orders beyond q^2 count
+    int terms;                // odd terms of E in the next round
 };
+
+// How the rounds of an instance hold the messages.
+//
+// With d_i = Ptilde_i - P_ji, the cavity precision, Algorithm 2's update of a
+// pair is P_ij(t + 1) = -q^2 / d_i, H_ij(t + 1) = -q (htilde_i(t) - H_ji(t)) / d_i:
+// the messages of round t + 1 are a function of the node aggregates of round
+// t, of q, and of the messages of round t, which are the same function one
+// round earlier.  Unrolled, a message is an alternating chain of the two
+// nodes' aggregates over the last rounds in which every step back is damped
+// by |q| / d, two steps by z = q^2 / (d_i d_j).  Where that dies out within the
+// rounds kept,
+//   PATH_HIST    keeps the last rounds' aggregates of the nodes (n values a
+//                round) and no messages: a round reads Q alone (4 B a pair in
+//                FP32, 2 B in BF16, none when recomputed) instead of reading
+//                and writing 12 to 32 B of messages beside it (sweep_hist.cu);
+//   PATH_STORED  stores the messages (sweep.cu): matrices with pairs so
+//                strongly coupled that the chains would be longer.
+constexpr int PATH_HIST = 0, PATH_STORED = 1;
+// Rounds of history kept.
+constexpr int kHist = 8;
 
 // One solver instance as the kernels see it.
 struct Inst {
@@ -113,9 +144,31 @@ struct Inst {
                       // cancels in ||x_i||^2 + ||x_j||^2 - 2 x_i . x_j for near pairs)
     int msg_bf16;     // messages stored in BF16 (precision forms)
     int task;         // 0 SVM (labels in Q, alpha clipped to [0, C]), 1 KRR (y = 1 in Q, alpha unclipped)
+    // PATH_HIST: the message arrays Pst / Hst, which that path does not use,
+    // hold instead (set_history)
+    float* hring;     // [stages][kHist][4][npad]: {Ptilde, htilde, mu, D = mu - mu two rounds earlier} of the
+                      // last rounds (round t in slot t % kHist)
+    float* hnow;      // [stages][3][npad]: {1 / Ptilde, D / Ptilde, (D(t-2) - 2 D) / Ptilde^2} of the latest round
+    float* hs46;      // [2][nslot][T]: slot sums of q^4 / Ptilde^2 and q^6 / Ptilde^3 of the last live round
+    int hist;         // the history fits (else only PATH_STORED)
+    int nstages;      // stages of a round (1 = synchronous)
     int form_next;    // formation: 1 + the next instance built from the same features (its Q
                       // tiles come from the same Gram tiles), 0 = none
 };
+
+// Lays the history of PATH_HIST into p's message arrays p.Pst, p.Hst (adjacent,
+// `bytes` together); p.hist = 0 where it does not fit (a single tile with many
+// stages).  p.nslot has to be set.
+inline void set_history(Inst& p, int stages, size_t bytes)
+{
+    const size_t vec = (size_t)p.npad * sizeof(float), slots = (size_t)2 * p.nslot * T * sizeof(float);
+    char* b = static_cast<char*>(p.Pst);
+    p.nstages = stages;
+    p.hs46 = reinterpret_cast<float*>(b);
+    p.hnow = reinterpret_cast<float*>(b + slots);
+    p.hring = reinterpret_cast<float*>(b + slots + 3 * stages * vec);
+    p.hist = slots + (size_t)(3 + 4 * kHist) * stages * vec <= bytes;
+}
 
 // Slot partials.  Every node has one slot per tile it belongs to (a tile
 // whose row block or column block is the node's block), ordered by the
@@ -287,8 +340,23 @@ cudaError_t prepare_sweep_rc();
 // pair sweep and ev[1] after the (last stage's) pair sweep.
 // nstages > 1: the staged schedule, sched[0 .. nstages-1] one per stage, a
 // stage finalize (aggregates only) between the stages.
+// paths: the message paths among the instances (1 << PATH_HIST, 1 <<
+// PATH_STORED or both); sched[kMaxStages + st] is the PATH_STORED segment of
+// stage st, sched[st] the PATH_HIST one.
 void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sched* sched, int nstages,
-                  const RoundGrid& g, int q_mode, int msg_bf16, cudaStream_t s, cudaEvent_t* ev = nullptr);
+                  const RoundGrid& g, int q_mode, int msg_bf16, int paths, cudaStream_t s, cudaEvent_t* ev = nullptr);
+// One pair sweep of PATH_HIST instances over a stage's tile list (sweep_hist.cu).
+void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, int stage_no, int grid, int q_mode,
+                       cudaStream_t s);
+cudaError_t prepare_sweep_hist();
+// Formation, after launch_init over the same instances: Ctrl::zpair_bits over
+// the listed tiles for the instances whose diagonal alone does not show that
+// PATH_HIST is the right path, from the FP32 entries (stored ones, or the
+// FP32 Gram's when Q is recomputed).
+// single: tab holds one instance.
+void launch_pair_z(const Inst* tab, const int4* tiles, long long ntiles, int q_mode, bool single, cudaStream_t s);
+void launch_pair_z_gram(const Inst* tab, const int4* tiles, long long ntiles, int grid, bool single, cudaStream_t s);
+
 // Final FP32-Gram residual r = 1 - Q mu (FP64 sums), dual objective and
 // alpha = clip(mu, 0, C) of the listed instances (their tiles, node blocks
 // and slots), per ops[slot]; results in ops[slot].final3 and f3_all[3 slot].

@@ -14,6 +14,7 @@
 // rounding and is clamped at 0.
 #include "common.cuh"
 #include "gabp_svm.h"
+#include "hist.cuh"
 
 #include <float.h>
 #include <mutex>
@@ -229,7 +230,9 @@ __global__ void k_stage_list(const Inst* __restrict__ tab, const int2* __restric
 
 // ------------------------------------------- final residual and Q alpha
 // For every instance k listed: off-diagonal sums sum_{j != i} Q_ij mu_j
-// (-> part[0]) and sum_{j != i} Q_ij alpha_j (-> part[1]).
+// (-> part[2], the residual slots every round writes anew) and sum_{j != i}
+// Q_ij alpha_j (-> part[3]): the P and H slots keep the sums of the current
+// messages, which a staged round that goes on from here reads.
 //
 // Per listed tile: partial sums of (Q mu)_i and (Q alpha)_i over the tile's
 // pairs (both roles) into the slot partials, with alpha = clip(mu, 0, C) and
@@ -275,7 +278,7 @@ __device__ __forceinline__ void final_tile_sums(const Inst& p, const float* __re
         rs[0][a] = rm;
         rs[1][a] = ra;
     }
-    float* const parts[2] = {p.part, p.part + part_len(p)};
+    float* const parts[2] = {p.part + 2 * part_len(p), p.part + 3 * part_len(p)};
     reduce_and_write<2>(es, rs, cs, parts, n, I, J, tile_slots(p, w));
 }
 
@@ -317,6 +320,54 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_final_tiles_q(const Inst* __res
     final_tile_sums<true>(p, ops[w.x].mu, w, acc, es);
 }
 
+// k_pair_z (sweep_hist.cu) for instances that do not store Q (only those that
+// their margin leaves open get as far as the Gram tile).
+__global__ void __launch_bounds__(NTHREADS) k_pair_z_gram(const Inst* __restrict__ tab, const int4* __restrict__ work,
+                                                          long long ntiles, bool single)
+{
+    __shared__ __align__(16) TileSmem sm;
+    __shared__ int s_go;
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    if (single) {
+        if (tid == 0) s_go = pair_z_open(tab[0]);
+        __syncthreads();
+        if (!s_go) return;
+        __syncthreads();
+    }
+    for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
+        const int4 w = work[L];
+        for (int k = w.x; k >= 0; k = tab[k].form_next - 1) {
+            const Inst& p = tab[k];
+            if (tid == 0) s_go = pair_z_open(p);
+            __syncthreads();
+            const int go = s_go;
+            __syncthreads();   // s_go is read before the next instance writes it
+            if (!go) continue;
+            float acc[8][8];
+            const GramSide S{p.X, p.sq, p.n};
+            gram_tile(S, S, p.m, w.y, w.z, sm.g, acc);
+            float best[2] = {0.f, FLT_MIN};   // the second never 0: the pass has run
+#pragma unroll
+            for (int a = 0; a < 8; ++a) {
+                const int i = w.y * T + ty * 8 + a, ii = min(i, p.n - 1);
+                const float si = p.sq[ii], ri = 1.f / p.qdiag[ii];
+#pragma unroll
+                for (int b = 0; b < 8; ++b) {
+                    const int j = w.z * T + tx * 8 + b;
+                    if (i < j && j < p.n)
+                        note_pair_z(rbf_from_gram(acc[a][b], si, p.sq[j], p.gamma) + p.lam2, ri, 1.f / p.qdiag[j], best);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                best[q] = warp_max_f(best[q]);
+                if ((tid & 31) == 0) atomicMax(&p.ctrl->zpair_bits[q], __float_as_uint(best[q]));
+            }
+            __syncthreads();
+        }
+    }
+}
+
 // Per node of a listed node block: r_i = b0_i - Q_ii mu_i - sum part0,
 // (Q alpha)_i = Q_ii alpha_i + sum part1; writes alpha (and r in FP32 when
 // requested); block partials {max |r_i|, sum b0_i alpha_i - 1/2 alpha_i
@@ -337,7 +388,7 @@ __global__ void __launch_bounds__(256) k_final_nodes(const Inst* __restrict__ ta
     if (x < n) {
         // the node's slots (see slot_begin)
         const int X = x / T, ns = slot_count(p, X);
-        const float* p0 = p.part + (size_t)slot_begin(p, X) * T + (x - X * T);
+        const float* p0 = p.part + 2 * part_len(p) + (size_t)slot_begin(p, X) * T + (x - X * T);
         const float* p1 = p0 + part_len(p);
         for (int k = g; k < ns; k += 8) {
             s0 += (double)p0[(size_t)k * T];
@@ -498,6 +549,12 @@ void launch_stage(const void* X, int x_dtype, int n, int m, float* y, float* Xf,
                   float* b, float* b0, int task, Ctrl* ctrl, cudaStream_t s)
 {
     k_stage<<<(n + 255) / 256, 256, 0, s>>>(X, x_dtype, n, m, y, Xf, sq, b, b0, task, ctrl);
+}
+
+void launch_pair_z_gram(const Inst* tab, const int4* tiles, long long ntiles, int grid, bool single,
+                        cudaStream_t s)
+{
+    k_pair_z_gram<<<grid, NTHREADS, 0, s>>>(tab, tiles, ntiles, single);
 }
 
 void launch_final(const Inst* tab, const StopOp* ops, const int4* tiles, long long ntiles, const int2* nbl,

@@ -116,6 +116,39 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
         : "memory");
 }
 
+// 1/d for the cavity precisions: the hardware approximate reciprocal
+// refined by one Newton-Raphson step r <- r (2 - d r) (error within about one
+// unit in the last place for normal positive d; checked against IEEE division
+// by gabp_selftest_reciprocal).
+__device__ __forceinline__ float rcp_nr(float d)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return fmaf(r, fmaf(-d, r, 1.0f), r);
+}
+
+// Sums the eight values {x0 .. x7} over the warp in a fixed order:
+// afterwards every lane of the group (lane / 4) % 8 = k holds the total of
+// value k (nine shuffles).
+__device__ __forceinline__ float reduce_scatter8x(const float (&x)[8], int lane)
+{
+    const bool hi = (lane & 16) != 0;
+    float y[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        y[k] = (hi ? x[k + 4] : x[k]) + __shfl_xor_sync(0xffffffffu, hi ? x[k] : x[k + 4], 16);
+    const bool b8 = (lane & 8) != 0;
+    float z[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        z[k] = (b8 ? y[k + 2] : y[k]) + __shfl_xor_sync(0xffffffffu, b8 ? y[k] : y[k + 2], 8);
+    const bool b4 = (lane & 4) != 0;
+    float v = (b4 ? z[1] : z[0]) + __shfl_xor_sync(0xffffffffu, b4 ? z[0] : z[1], 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v;
+}
+
 // First error of a kernel -> the instance's control block.
 __device__ __forceinline__ void record_error(Ctrl* c, int code, long long where)
 {

@@ -27,6 +27,7 @@
 // node's per-tile sums go to its own slot (common.cuh), so the reduction order
 // is fixed and the result reproducible.
 #include "common.cuh"
+#include "hist.cuh"
 #include "ptx.cuh"
 #include "qtile_epi.cuh"
 
@@ -75,17 +76,6 @@ constexpr int STAGES = 4;                     // barrier slots of the stage ring
 template <class MSG>
 __host__ __device__ constexpr int stages() { return MSG::NSTAGE; }
 constexpr int SWEEP_THREADS = NTHREADS + 32;  // + one producer warp
-// 1/d for the cavity precisions: the hardware approximate reciprocal
-// refined by one Newton-Raphson step r <- r (2 - d r) (error within about one
-// unit in the last place for normal positive d; checked against IEEE division
-// by gabp_selftest_reciprocal).
-__device__ __forceinline__ float rcp_nr(float d)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-    return fmaf(r, fmaf(-d, r, 1.0f), r);
-}
-
 // Message storage: FP32 pairs (plain and precision forms) or BF16 pairs
 // (precision forms with refinement).  Arithmetic is FP32 either way; sums use
 // the stored (rounded) values so that the aggregates match the messages the
@@ -437,28 +427,6 @@ __device__ __forceinline__ void st4(float* row, int lane, const float (&o)[4])
     }
 }
 
-// Sums the eight values {x0 .. x7} over the warp in a fixed order:
-// afterwards every lane of the group (lane / 4) % 8 = k holds the total of
-// value k (nine shuffles: the three sums of two rows, or the H and residual
-// sums of four rows once P is frozen).
-__device__ __forceinline__ float reduce_scatter8x(const float (&x)[8], int lane)
-{
-    const bool hi = (lane & 16) != 0;
-    float y[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        y[k] = (hi ? x[k + 4] : x[k]) + __shfl_xor_sync(0xffffffffu, hi ? x[k] : x[k + 4], 16);
-    const bool b8 = (lane & 8) != 0;
-    float z[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k)
-        z[k] = (b8 ? y[k + 2] : y[k]) + __shfl_xor_sync(0xffffffffu, b8 ? y[k] : y[k + 2], 8);
-    const bool b4 = (lane & 4) != 0;
-    float v = (b4 ? z[1] : z[0]) + __shfl_xor_sync(0xffffffffu, b4 ? z[0] : z[1], 4);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    return v;
-}
 // The three sums {P, H, R} of two rows: values {a0, a1, a2, 0, b0, b1, b2, 0}.
 __device__ __forceinline__ float reduce_scatter8(float a0, float a1, float a2, float b0, float b1, float b2,
                                                  int lane)
@@ -1161,29 +1129,89 @@ __device__ __forceinline__ void acc2(float& s, float& c, float x)
     s = t;
 }
 
-// Node x's next aggregates {Ptilde, htilde, mutilde} from its slot sums (P,
-// H) and its residual r_x(t) = b_x - Q_xx mutilde_x(t) - R in FP64; returns
-// |r_x| (inf for a non-finite one) and flags a non-positive or non-finite
-// aggregate.
-__device__ __forceinline__ double finalize_node(const Inst& p, Ctrl* ctrl, int x, int t, bool frozen, double P,
-                                                double H, double R)
+// What a node's finalize needs of its instance's round.
+struct RoundState {
+    int t;
+    bool frozen;   // P messages at their fixed point
+    bool hist;     // PATH_HIST
+    // PATH_HIST, synchronous: the H messages into x sum to -R + (sum of the P
+    // messages) mutilde(t - 1) + E (sweep_hist.cu), R being the sum the residual
+    // needs anyway; the H slots hold E when there are terms of it
+    bool from_r, with_e;
+};
+__device__ __forceinline__ RoundState round_state(const Inst& p, const Ctrl* ctrl)
 {
+    RoundState s;
+    s.t = *(volatile const int*)&ctrl->t;
+    s.frozen = *(volatile const int*)&ctrl->p_frozen != 0;
+    s.hist = ctrl->path == PATH_HIST;
+    s.from_r = s.hist && p.nstages == 1;
+    s.with_e = s.t > 0 && round_has_e(ctrl, s.frozen);
+    return s;
+}
+// Whether the round's P and H slots are summed.
+__device__ __forceinline__ bool sum_p(const RoundState& s) { return !s.frozen; }
+__device__ __forceinline__ bool sum_h(const RoundState& s) { return !s.from_r || s.with_e; }
+
+struct NodeOut {
+    double absr;    // |r_x|, inf for a non-finite one
+    float dmu, mu;  // PATH_HIST: |change of the mean over two rounds|, |mean|
+};
+
+// Node x's next aggregates {Ptilde, htilde, mutilde} from its slot sums (P,
+// H) and its residual r_x(t) = b_x - Q_xx mutilde_x(t) - R in FP64; flags a
+// non-positive or non-finite aggregate.
+__device__ __forceinline__ NodeOut finalize_node(const Inst& p, Ctrl* ctrl, int x, const RoundState& s, double P,
+                                                 double H, double R)
+{
+    const int t = s.t;
     const float* cur = p.agg + (size_t)(t & 1) * 3 * p.npad;
     float* nxt = p.agg + (size_t)((t + 1) & 1) * 3 * p.npad;
     const double qd = p.qdiag[x], bx = p.b[x];
-    const float Pn = frozen ? cur[x] : (float)(qd + P);
+    const float Pc = cur[x], Pn = s.frozen ? Pc : (float)(qd + P);
+    const float mu1 = (s.hist && t > 0) ? nxt[2 * p.npad + x] : 0.f;   // the mean of round t - 1
+    if (s.from_r) H += (s.frozen ? (double)Pc - qd : P) * mu1 - R;
     const float hn = (float)(bx + H);
     const float mn = hn / Pn;
     nxt[x] = Pn;
     nxt[p.npad + x] = hn;
     nxt[2 * p.npad + x] = mn;
+    NodeOut o{0.0, 0.f, 0.f};
+    if (s.hist) {
+        hist_push(p, 0, t + 1, x, Pn, hn, mn, mu1);
+        o.dmu = fabsf(mn - mu1);
+        o.mu = fabsf(mn);
+        // P is frozen once no Ptilde changes any more: the P messages are then
+        // functions of constant aggregates
+        if (Pn != Pc) ctrl->p_changed = 1;
+    }
     const double r = bx - qd * (double)cur[2 * p.npad + x] - R;
-    double absr = fabs(r);
-    if (!(absr <= DBL_MAX)) absr = INFINITY;
+    o.absr = fabs(r);
+    if (!(o.absr <= DBL_MAX)) o.absr = INFINITY;
     if (!(Pn > 0.f) || !isfinite(Pn) || !isfinite(mn)) record_error(ctrl, ST_ENUMERIC, x);
-    return absr;
+    return o;
+}
+// One warp's node block -> the instance's maxima (lane 0 writes).
+__device__ __forceinline__ void note_block(Ctrl* ctrl, const RoundState& s, NodeOut o, int lane)
+{
+    const double absr = warp_max_d(o.absr);
+    if (lane == 0) atomicMax(&ctrl->rmax_bits, (unsigned long long)__double_as_longlong(absr));
+    if (s.hist) {
+        const float d = warp_max_f(o.dmu), m = warp_max_f(o.mu);
+        if (lane == 0) {
+            atomicMax(&ctrl->dmax_bits, __float_as_uint(d));
+            atomicMax(&ctrl->mumax_bits, __float_as_uint(m));
+        }
+    }
 }
 
+// Step 1 of the round settings (one thread per instance).
+__device__ __forceinline__ void hist_ctrl_start(Ctrl* c)
+{
+    c->dmax_bits = c->mumax_bits = 0u;
+    c->change = 1.f;
+    c->terms = 0;
+}
 // Run by the last node block of an instance to finish a round: ||r(t)||_inf,
 // the stop test (Step 3: k* = t when it is below tol, the limit otherwise),
 // the exact P-freeze flag, and the round counter.
@@ -1213,6 +1241,14 @@ __device__ __forceinline__ void finalize_decide(const Inst& p, Ctrl* ctrl, int t
         ctrl->p_frozen = 1;
         ctrl->t_frozen = t + 1;
     }
+    if (ctrl->path == PATH_HIST) {
+        const float d = __uint_as_float(atomicAdd(&ctrl->dmax_bits, 0u)), m = __uint_as_float(atomicAdd(&ctrl->mumax_bits, 0u));
+        const float delta = d < m ? d / m : (d > 0.f ? 1.f : 0.f);
+        ctrl->change = next_change(delta, ctrl->change, ctrl->u);
+        ctrl->terms = e_terms(ctrl->z, ctrl->change);
+        ctrl->dmax_bits = 0u;
+        ctrl->mumax_bits = 0u;
+    }
     ctrl->p_changed = 0;
     ctrl->t = t + 1;
     ctrl->zero_h = 0;
@@ -1223,10 +1259,10 @@ __device__ __forceinline__ void finalize_decide(const Inst& p, Ctrl* ctrl, int t
 
 // Compensated sums of node x's slots k = k0, k0 + step, ... (of the
 // slot_count of its block) of NA partial arrays (P, H[, R]), eight loads of
-// each in flight; P reads as 0 when frozen (Ptilde is kept then).
+// each in flight; the P and H slots read as 0 where not wanted.
 template <int NA>
-__device__ __forceinline__ void slot_sums(const Inst& p, int x, int k0, int step, bool frozen, float (&s)[NA],
-                                          float (&c)[NA])
+__device__ __forceinline__ void slot_sums(const Inst& p, int x, int k0, int step, bool with_p, bool with_h,
+                                          float (&s)[NA], float (&c)[NA])
 {
     const int X = x / T, ns = slot_count(p, X);
     const size_t len = part_len(p);
@@ -1241,7 +1277,7 @@ __device__ __forceinline__ void slot_sums(const Inst& p, int x, int k0, int step
 #pragma unroll
             for (int a = 0; a < NA; ++a) {
                 const size_t o = a * len + (size_t)(k + u * step) * T;
-                v[a][u] = (a == 0 && frozen) ? 0.f : part[o];
+                v[a][u] = ((a == 0 && !with_p) || (a == 1 && !with_h)) ? 0.f : part[o];
             }
 #pragma unroll
         for (int u = 0; u < 8; ++u)
@@ -1250,7 +1286,8 @@ __device__ __forceinline__ void slot_sums(const Inst& p, int x, int k0, int step
     }
     for (; k < ns; k += step)
 #pragma unroll
-        for (int a = 0; a < NA; ++a) acc2(s[a], c[a], (a == 0 && frozen) ? 0.f : part[a * len + (size_t)k * T]);
+        for (int a = 0; a < NA; ++a)
+            acc2(s[a], c[a], ((a == 0 && !with_p) || (a == 1 && !with_h)) ? 0.f : part[a * len + (size_t)k * T]);
 }
 
 // Node-block units of a round's finalize.  Blocks [0, nsmall) of the list
@@ -1286,18 +1323,16 @@ __global__ void __launch_bounds__(256, 5)
             const Inst& p = tab[nb.x];
             Ctrl* ctrl = p.ctrl;
             if (*(volatile int*)&ctrl->done) continue;
-            const int t = *(volatile int*)&ctrl->t;
-            const bool frozen = *(volatile int*)&ctrl->p_frozen != 0;
-            const int x = nb.y * 32 + lane, n = p.n;
-            double absr = 0.0;
+            const RoundState rs = round_state(p, ctrl);
+            const int x = nb.y * 32 + lane, n = p.n, t = rs.t;
+            NodeOut o{0.0, 0.f, 0.f};
             if (x < n) {
                 float sv[3], cv[3];
-                slot_sums<3>(p, x, 0, 1, frozen, sv, cv);
-                absr = finalize_node(p, ctrl, x, t, frozen, (double)sv[0] + (double)cv[0],
-                                     (double)sv[1] + (double)cv[1], (double)sv[2] + (double)cv[2]);
+                slot_sums<3>(p, x, 0, 1, sum_p(rs), sum_h(rs), sv, cv);
+                o = finalize_node(p, ctrl, x, rs, (double)sv[0] + (double)cv[0], (double)sv[1] + (double)cv[1],
+                                  (double)sv[2] + (double)cv[2]);
             }
-            absr = warp_max_d(absr);
-            if (lane == 0) atomicMax(&ctrl->rmax_bits, (unsigned long long)__double_as_longlong(absr));
+            note_block(ctrl, rs, o, lane);
             __threadfence();
             __syncwarp();
             if (lane == 0) {
@@ -1311,11 +1346,10 @@ __global__ void __launch_bounds__(256, 5)
         const Inst& p = tab[nb.x];
         Ctrl* ctrl = p.ctrl;
         if (*(volatile int*)&ctrl->done) continue;
-        const int t = *(volatile int*)&ctrl->t;
-        const bool frozen = *(volatile int*)&ctrl->p_frozen != 0;
-        const int x = nb.y * 32 + lane, n = p.n;
+        const RoundState rs = round_state(p, ctrl);
+        const int x = nb.y * 32 + lane, n = p.n, t = rs.t;
         float sv[3] = {0.f, 0.f, 0.f}, cv[3] = {0.f, 0.f, 0.f};
-        if (x < n) slot_sums<3>(p, x, g, 8, frozen, sv, cv);
+        if (x < n) slot_sums<3>(p, x, g, 8, sum_p(rs), sum_h(rs), sv, cv);
         __syncthreads();   // red[] of the previous node block is consumed
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -1324,7 +1358,7 @@ __global__ void __launch_bounds__(256, 5)
         }
         __syncthreads();
         if (g == 0) {
-            double absr = 0.0;
+            NodeOut o{0.0, 0.f, 0.f};
             if (x < n) {
                 float a[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -1333,12 +1367,10 @@ __global__ void __launch_bounds__(256, 5)
                     acc2(a[2], a[3], red[2][w][lane]); a[3] += red[3][w][lane];
                     acc2(a[4], a[5], red[4][w][lane]); a[5] += red[5][w][lane];
                 }
-                absr = finalize_node(p, ctrl, x, t, frozen, (double)a[0] + (double)a[1], (double)a[2] + (double)a[3],
-                                     (double)a[4] + (double)a[5]);
+                o = finalize_node(p, ctrl, x, rs, (double)a[0] + (double)a[1], (double)a[2] + (double)a[3],
+                                  (double)a[4] + (double)a[5]);
             }
-            absr = warp_max_d(absr);
-            if (lane == 0)
-                atomicMax(&ctrl->rmax_bits, (unsigned long long)__double_as_longlong(absr));
+            note_block(ctrl, rs, o, lane);
         }
         __threadfence();
         __syncthreads();
@@ -1388,18 +1420,28 @@ __device__ __forceinline__ double offdiag_abs_sum(const Inst& p, int x)
 // Between the stages of a staged round: Ptilde and htilde of every node from
 // all of its slot partials (slots of tiles not yet swept in this round still
 // hold the sums of their current messages) into aggmid, for the next stage;
-// with frozen P, Ptilde is kept.  No residual and no stop test: those come
+// with frozen P, Ptilde is kept (st: the stage they are for).  No residual and no stop test: those come
 // with the round's last stage (k_finalize).  Same node-block units as
 // k_finalize.
-__device__ __forceinline__ void stage_node(const Inst& p, int x, int t, bool frozen, double P, double H)
+__device__ __forceinline__ NodeOut stage_node(const Inst& p, int st, int x, const RoundState& s, double P, double H)
 {
-    const float* cur = p.agg + (size_t)(t & 1) * 3 * p.npad;
-    p.aggmid[x] = frozen ? cur[x] : (float)((double)p.qdiag[x] + P);
-    p.aggmid[p.npad + x] = (float)((double)p.b[x] + H);
+    const float* cur = p.agg + (size_t)(s.t & 1) * 3 * p.npad;
+    const float Pm = s.frozen ? cur[x] : (float)((double)p.qdiag[x] + P), hm = (float)((double)p.b[x] + H);
+    p.aggmid[x] = Pm;
+    p.aggmid[p.npad + x] = hm;
+    NodeOut o{0.0, 0.f, 0.f};
+    if (s.hist) {
+        const float mu = hm / Pm, mu2 = s.t > 1 ? hist_slot(p, st, s.t - 2)[2 * (size_t)p.npad + x] : 0.f;
+        hist_push(p, st, s.t, x, Pm, hm, mu, mu2);
+        o.dmu = fabsf(mu - mu2);
+        o.mu = fabsf(mu);
+        if (Pm != cur[x]) p.ctrl->p_changed = 1;
+    }
+    return o;
 }
 
 __global__ void __launch_bounds__(256)
-    k_finalize_stage(const Inst* __restrict__ tab, const int2* __restrict__ nbl, const Sched* __restrict__ sched)
+    k_finalize_stage(const Inst* __restrict__ tab, const int2* __restrict__ nbl, const Sched* __restrict__ sched, int st)
 {
     int usmall;
     const int units = fin_units(sched, usmall), nsmall = sched->nsmall;
@@ -1412,37 +1454,41 @@ __global__ void __launch_bounds__(256)
             const int2 nb = nbl[bi];
             const Inst& p = tab[nb.x];
             if (*(volatile int*)&p.ctrl->done) continue;
-            const int t = *(volatile int*)&p.ctrl->t;
-            const bool frozen = *(volatile int*)&p.ctrl->p_frozen != 0;
+            const RoundState rs = round_state(p, p.ctrl);
             const int x = nb.y * 32 + lane;
+            NodeOut o{0.0, 0.f, 0.f};
             if (x < p.n) {
                 float sv[2], cv[2];
-                slot_sums<2>(p, x, 0, 1, frozen, sv, cv);
-                stage_node(p, x, t, frozen, (double)sv[0] + (double)cv[0], (double)sv[1] + (double)cv[1]);
+                slot_sums<2>(p, x, 0, 1, sum_p(rs), sum_h(rs), sv, cv);
+                o = stage_node(p, st, x, rs, (double)sv[0] + (double)cv[0], (double)sv[1] + (double)cv[1]);
             }
+            note_block(p.ctrl, rs, o, lane);
             continue;
         }
         const int2 nb = nbl[nsmall + (u - usmall)];
         const Inst& p = tab[nb.x];
         Ctrl* ctrl = p.ctrl;
         if (*(volatile int*)&ctrl->done) continue;   // the same node block for the whole CTA
-        const int t = *(volatile int*)&ctrl->t;
-        const bool frozen = *(volatile int*)&ctrl->p_frozen != 0;
+        const RoundState rs = round_state(p, ctrl);
         const int x = nb.y * 32 + lane, n = p.n;
         float sv[2] = {0.f, 0.f}, cv[2] = {0.f, 0.f};
-        if (x < n) slot_sums<2>(p, x, g, 8, frozen, sv, cv);
+        if (x < n) slot_sums<2>(p, x, g, 8, sum_p(rs), sum_h(rs), sv, cv);
         __syncthreads();   // red[] of the previous node block is consumed
         red[0][g][lane] = sv[0]; red[1][g][lane] = cv[0];
         red[2][g][lane] = sv[1]; red[3][g][lane] = cv[1];
         __syncthreads();
-        if (g == 0 && x < n) {
-            float a[4] = {0.f, 0.f, 0.f, 0.f};
+        if (g == 0) {
+            NodeOut o{0.0, 0.f, 0.f};
+            if (x < n) {
+                float a[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int w = 0; w < 8; ++w) {
-                acc2(a[0], a[1], red[0][w][lane]); a[1] += red[1][w][lane];
-                acc2(a[2], a[3], red[2][w][lane]); a[3] += red[3][w][lane];
+                for (int w = 0; w < 8; ++w) {
+                    acc2(a[0], a[1], red[0][w][lane]); a[1] += red[1][w][lane];
+                    acc2(a[2], a[3], red[2][w][lane]); a[3] += red[3][w][lane];
+                }
+                o = stage_node(p, st, x, rs, (double)a[0] + (double)a[1], (double)a[2] + (double)a[3]);
             }
-            stage_node(p, x, t, frozen, (double)a[0] + (double)a[1], (double)a[2] + (double)a[3]);
+            note_block(ctrl, rs, o, lane);
         }
     }
 }
@@ -1461,6 +1507,7 @@ __global__ void k_reset(Inst p)
         c->converged = 0;
         c->rmax_bits = 0ull;
         c->blocks_done = 0u;
+        hist_ctrl_start(c);
     }
     if (x >= p.n) return;
     zero_slots(p, x, true);
@@ -1469,6 +1516,7 @@ __global__ void k_reset(Inst p)
     p.agg[x] = qd;
     p.agg[p.npad + x] = bx;
     p.agg[2 * p.npad + x] = bx / qd;
+    hist_start(p, x, qd, bx, bx / qd);
 }
 
 // Correction system Q d = r with the current P messages: b := r, the H
@@ -1482,7 +1530,12 @@ __global__ void k_refine_rhs_list(const Inst* __restrict__ tab, const StopOp* __
     Ctrl* c = p.ctrl;
     const int t = *(volatile int*)&c->t;
     const int x = nb.y * 32 + threadIdx.x;
-    if (nb.y == 0 && threadIdx.x == 0) c->zero_h = 1;
+    if (nb.y == 0 && threadIdx.x == 0) {
+        c->zero_h = 1;
+        c->change = 1.f;
+        if (c->path == PATH_HIST)
+            c->terms = e_terms(c->z, 1.f);
+    }
     if (threadIdx.x >= 32 || x >= p.n) return;
     zero_slots(p, x, false);   // the H messages restart from 0
     float* cur = p.agg + (size_t)(t & 1) * 3 * p.npad;
@@ -1490,6 +1543,7 @@ __global__ void k_refine_rhs_list(const Inst* __restrict__ tab, const StopOp* __
     const_cast<float*>(p.b)[x] = bx;
     cur[p.npad + x] = bx;
     cur[2 * p.npad + x] = bx / cur[x];
+    if (c->path == PATH_HIST) hist_restart(p, t, x, cur[x], bx, bx / cur[x]);
 }
 
 // acc = mutilde(buf) (first pass) or acc += mutilde(buf), over node blocks.
@@ -1529,12 +1583,14 @@ __global__ void k_selftest_rcp(const float* __restrict__ d, float* __restrict__ 
 // max_i 1 / (Q_ii - R_i) (the control block is zeroed before formation):
 // with all margins positive Q is strictly diagonally dominant and Varah's
 // bound ||mu - Q^-1 b||_inf <= ||b - Q mu||_inf / min_i (Q_ii - R_i) holds for
-// any mu; a row without a positive margin records +inf (no bound).
+// any mu; a row without a positive margin records +inf (no bound).  Also the
+// largest 1 / Q_ii.
 __device__ __forceinline__ void note_margin(Ctrl* c, float qd, double R)
 {
     const double mg = (double)qd - R;
     const double inv = mg > 0.0 ? 1.0 / mg : INFINITY;
     atomicMax(&c->inv_margin_bits, (unsigned long long)__double_as_longlong(inv));
+    atomicMax(&c->rq_bits, __float_as_uint(1.f / qd));
 }
 
 // Diagonal rule (Section 3.1) from the |Q| row-sum partials of the Q
@@ -1552,10 +1608,14 @@ __global__ void k_init(Inst p, int diag_rule, float delta)
         c->converged = 0;
         c->rmax_bits = 0ull;
         c->blocks_done = 0u;
+        hist_ctrl_start(c);
         c->tol = 0.0;
         c->rinf = -1.0;
     }
-    if (x >= p.n) return;
+    if (x >= p.n) {
+        if (x < p.npad) hist_pad(p, x);
+        return;
+    }
     const double R = offdiag_abs_sum(p, x);
     zero_slots(p, x, true);   // all messages start at 0
     const double lam2 = p.lam2;
@@ -1570,6 +1630,7 @@ __global__ void k_init(Inst p, int diag_rule, float delta)
     p.agg[x] = qf;
     p.agg[p.npad + x] = bx;
     p.agg[2 * p.npad + x] = bx / qf;
+    hist_start(p, x, qf, bx, bx / qf);
     note_margin(p.ctrl, qf, R);
 }
 
@@ -1596,10 +1657,13 @@ __global__ void k_init_list(const Inst* __restrict__ tab, const int2* __restrict
         c->converged = 0;
         c->rmax_bits = 0ull;
         c->blocks_done = 0u;
+        hist_ctrl_start(c);
         c->tol = 0.0;
         c->rinf = -1.0;
     }
     const int x = nb.y * 32 + threadIdx.x;
+    if (nb.y == (p.n - 1) / 32)
+        for (int xp = p.n + threadIdx.x; xp < p.npad; xp += blockDim.x) hist_pad(p, xp);
     if (threadIdx.x >= 32 || x >= p.n) return;
     const double R = offdiag_abs_sum(p, x);
     zero_slots(p, x, true);   // all messages start at 0
@@ -1615,6 +1679,7 @@ __global__ void k_init_list(const Inst* __restrict__ tab, const int2* __restrict
     p.agg[x] = qf;
     p.agg[p.npad + x] = bx;
     p.agg[2 * p.npad + x] = bx / qf;
+    hist_start(p, x, qf, bx, bx / qf);
     note_margin(p.ctrl, qf, R);
 }
 
@@ -1622,8 +1687,10 @@ __global__ void k_begin_list(Inst* tab, const int2* __restrict__ list, const dou
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= count) return;
-    Ctrl* c = tab[list[k].x].ctrl;
+    const Inst& p = tab[list[k].x];
+    Ctrl* c = p.ctrl;
     const int iters = list[k].y;
+    if (c->t == 0) choose_path(p, c);
     c->limit = c->t + iters;
     c->tol = tols[k];
     c->converged = 0;
@@ -1639,6 +1706,7 @@ __global__ void k_begin(Inst* tab, int ninst, int iters, double tol)
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= ninst) return;
     Ctrl* c = tab[k].ctrl;
+    if (c->t == 0) choose_path(tab[k], c);
     c->limit = c->t + iters;
     c->tol = tol;
     c->converged = 0;
@@ -1647,6 +1715,55 @@ __global__ void k_begin(Inst* tab, int ninst, int iters, double tol)
     c->rmax_bits = 0ull;
     c->blocks_done = 0u;
     c->done = (c->status != 0 || iters <= 0) ? 1 : 0;
+}
+
+// Q_ij as the recomputing sweep forms it, from a plain sum over the features
+// (the tensor-core sum can round to the neighbouring BF16 value).
+__device__ float recomputed_q(const Inst& p, int i, int j)
+{
+    float g = 0.f;
+    for (int k = 0; k < p.m; ++k)
+        g = fmaf(__bfloat162float(__float2bfloat16_rn(p.X[(size_t)i * p.m + k])),
+                 __bfloat162float(__float2bfloat16_rn(p.X[(size_t)j * p.m + k])), g);
+    const float t = p.gamma * kLog2e * (2.f * g - p.sqb[i] - p.sqb[j]);
+    return p.y[i] * p.y[j] * __bfloat162float(__float2bfloat16_rn(ex2_approx(fminf(t, 0.f)) + p.lam2));
+}
+
+// The messages {P_ij, P_ji, H_ij, H_ji} of a PATH_HIST pair after t rounds
+// (t > 0), rebuilt from the history of the pair's stage as the sweep of round
+// t - 1 did, with the whole history as chain.
+__device__ float4 hist_pair(const Inst& p, int t, float q, int i, int j)
+{
+    int st = 0;
+    if (p.nstages > 1) {
+        int B[kMaxStages + 1];
+        stage_bounds(p.Nt, p.nstages, B);
+        while (j / T >= B[st + 1]) ++st;
+    }
+    const int t0 = t - 1, lv = min(kHist, t);
+    float PA = 0.f, HA = 0.f, PB = 0.f, HB = 0.f;
+    if (p.ctrl->p_frozen && t0 >= p.ctrl->t_frozen) {
+        const float* now = hist_slot(p, st, t0);
+        const float ia = 1.f / now[i], ib = 1.f / now[j], z = (q * ia) * (q * ib);
+        const float g = 2.f * q / (1.f + sqrtf(1.f + 4.f * z)), u = g * ia, v = g * ib;
+        for (int k = lv - 1; k >= 0; --k) {
+            const float* mu = hist_slot(p, st, t0 - k) + 2 * (size_t)p.npad;
+            HA = (k & 1) ? fmaf(v, HA, mu[j]) : fmaf(u, HA, mu[i]);
+            HB = (k & 1) ? fmaf(u, HB, mu[i]) : fmaf(v, HB, mu[j]);
+        }
+        return make_float4(-q * u, -q * v, -g * HA, -g * HB);
+    }
+    for (int k = lv - 1; k >= 0; --k) {
+        const float* s = hist_slot(p, st, t0 - k);
+        const float* h = s + p.npad;
+        const int a = (k & 1) ? j : i, b = (k & 1) ? i : j;
+        const float ra = 1.f / (s[a] - PA), rb = 1.f / (s[b] - PB);
+        PA = -(q * q) * ra;
+        PB = -(q * q) * rb;
+        HA = -q * (h[a] - HA) * ra;
+        HB = -q * (h[b] - HB) * rb;
+    }
+    return make_float4(PA, PB, HA, HB);
 }
 
 __global__ void k_get_pairs(Inst p, const long long* __restrict__ ij, long long cnt, float4* __restrict__ out)
@@ -1660,6 +1777,13 @@ __global__ void k_get_pairs(Inst p, const long long* __restrict__ ij, long long 
     const int r = (int)(i - I * T), c = (int)(j - J * T);
     if (p.ctrl->t == 0 || L < 0) {
         out[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else if (p.ctrl->path == PATH_HIST) {
+        const size_t o = (size_t)L * TT + r * T + c;
+        float q;
+        if (!p.qstore) q = recomputed_q(p, (int)i, (int)j);
+        else if (p.qstore != p.qref) q = __bfloat162float(static_cast<const __nv_bfloat16*>(p.qstore)[o]);
+        else q = p.qref[o];
+        out[e] = hist_pair(p, p.ctrl->t, q, (int)i, (int)j);
     } else {
         const size_t o = (size_t)L * TT + r * T + c;
         float2 a, b;
@@ -1757,16 +1881,19 @@ cudaError_t prepare_sweep()
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_sweep<__nv_bfloat16, MsgBF16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sweep_smem_bytes<__nv_bfloat16, MsgBF16>());
-    return e;
+    return e == cudaSuccess ? prepare_sweep_hist() : e;
 }
 
 void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sched* sched, int nstages,
-                  const RoundGrid& g, int q_mode, int msg_bf16, cudaStream_t s, cudaEvent_t* ev)
+                  const RoundGrid& g, int q_mode, int msg_bf16, int paths, cudaStream_t s, cudaEvent_t* ev)
 {
     for (int st = 0; st < nstages; ++st) {
-        const Sched* sc = sched + st;
+        const Sched* sc = sched + kMaxStages + st;
         if (ev && st == 0) cudaEventRecordWithFlags(ev[0], s, cudaEventRecordExternal);
-        if (q_mode == 2 && msg_bf16)
+        if (paths & (1 << PATH_HIST)) launch_sweep_hist(tab, work, sched + st, st, g.sweep, q_mode, s);
+        if (!(paths & (1 << PATH_STORED))) {
+            // no instance stores its messages
+        } else if (q_mode == 2 && msg_bf16)
             k_sweep_rc<MsgBF16><<<g.sweep, RC_THREADS, rc_smem_bytes<MsgBF16>(), s>>>(tab, work, sc, st);
         else if (q_mode == 2)
             k_sweep_rc<MsgF32><<<g.sweep, RC_THREADS, rc_smem_bytes<MsgF32>(), s>>>(tab, work, sc, st);
@@ -1781,7 +1908,7 @@ void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sche
                 <<<g.sweep, SWEEP_THREADS, sweep_smem_bytes<float, MsgF32>(), s>>>(tab, work, sc, st);
         if (ev && st == nstages - 1) cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal);
         if (st < nstages - 1)
-            k_finalize_stage<<<g.finalize, 256, 0, s>>>(tab, nbl, sched);
+            k_finalize_stage<<<g.finalize, 256, 0, s>>>(tab, nbl, sched, st + 1);
         else
             k_finalize<<<g.finalize, 256, 0, s>>>(tab, nbl, sched);
     }

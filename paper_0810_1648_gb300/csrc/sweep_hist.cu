@@ -1,0 +1,905 @@
+// Pair sweep of PATH_HIST instances (common.cuh): Algorithm 2's round without
+// stored messages.
+//
+// With H_ij(t+1) = -q (htilde_i - H_ji) / d_i and P_ij(t+1) = -q^2 / d_i (all of
+// round t; d_i = Ptilde_i - P_ji), putting the same expression one round
+// earlier in for H_ji gives exactly
+//   H_ij(t+1) = -q mu_i(t) + P_ij(t+1) mu_j(t-1) + E_ij(t+1),
+//   E_ij(t+1) = (q / d_i(t)) [(q^2 / d_j(t-1)) D_i(t) + E_ji(t)],
+// D_x(t) = mu_x(t) - mu_x(t-2) (aggregates before round 0, and before a restart
+// of H, are 0).  Summed over i, the first term is the sum that the residual
+// needs anyway and the second is mu_j(t-1) times the sum of the P messages; E is
+// of the order of z = q^2 / (d_i d_j) times what still changes.  What is left
+// are sums over i of powers of q with weights of node i, times values of node
+// j (r = 1 / Ptilde):
+//   sum q mu_i                     residual and H
+//   sum q^2k r_i^k = S2k, k = 1, 2, 3   sum P_ij = -(S2 - r S4 + 2 r^2 S6), and E's
+//                                  even orders, r S4 D_j(t-1) + r^2 S6 (D_j(t-3) - 3 D_j(t-1))
+//   sum q^3 r_i D_i                E, times r
+//   sum q^5 r_i^2 (D_i(t-2) - 2 D_i)   E, times r^2
+// with r = r_j(t-1); the terms of higher orders are below FP32 rounding on this
+// path (choose_path).  Once no Ptilde changes, the P sums are known (Ptilde -
+// Q_jj; S4 and S6 of the last live round), and E needs its sums only while it counts
+// (e_terms): most rounds are one symmetric product Q mu.  Under the staged
+// schedule mu in H is the mean of the stage and the P sums are the tile's own.
+//
+// Bound: Q streamed once a round (4 or 2 B a pair), or the Q epilogue of the
+// recomputing kernel.  Measured, a frozen round's sweep: n = 20000, FP32 Q 823
+// us with stored messages (28 B a pair), 140 us here (118 us for 4 B a pair at the
+// copy bandwidth); n = 100000, BF16 Q and messages 10.6 ms and 1.99 ms.
+#include "common.cuh"
+#include "hist.cuh"
+#include "ptx.cuh"
+#include "qtile_epi.cuh"
+
+#include <float.h>
+
+namespace gabp {
+
+namespace {
+
+constexpr int HCW = 8;                         // consumer warps
+constexpr int H_THREADS = (HCW + 1) * 32;      // and one producer warp
+constexpr size_t H_CHUNK = 16384;              // ring stage: 32 rows of FP32 Q, 64 of BF16 Q
+constexpr int H_STAGES = 4;
+constexpr int H_GROUP = 64;                    // rows per row-sum reduction (four steps of 16)
+
+// What a tile sums beside q mu.  Live P: q^2 (round 0, and where nothing else
+// counts), with q^3, or everything; frozen P: nothing, q^3, or q^3 and q^5.
+enum { K_LIVE0, K_LIVE1, K_LIVE, K_SUM, K_ONE, K_TWO };
+// The sums, as rows of HTail::rs and cs.
+enum { S_R, S_M, S_2, S_4, S_6, S_W3, S_W5, S_COUNT };
+// The node values, as rows of HTail::node: mean of the residual, the stage's
+// mean (staged), and hnow's three.
+enum { N_MU0, N_MU, N_R, N_W3, N_W5, N_COUNT };
+
+struct HInfo {
+    const float* ring;     // the stage's history
+    float* part;
+    float* s46;            // slots of S4, then of S6
+    long long plen;
+    Ctrl* ctrl;
+    long long L;
+    int npad, I, J, sR, sC, rows;
+    int t, kind, even, staged, end;
+};
+
+struct HTail {
+    unsigned long long full[H_STAGES], empty[H_STAGES];
+    unsigned long long tfull[2], tempty[2];
+    int cabort;
+    HInfo info[2];
+    alignas(16) float node[2][2][N_COUNT][T];   // [slot][row, column block]
+    alignas(16) float cs[S_COUNT][HCW][T];      // column sums of each warp
+    float rs[S_COUNT][T];                       // row sums
+};
+
+__device__ __forceinline__ void hbar() { asm volatile("bar.sync 1, %0;" ::"n"(HCW * 32) : "memory"); }
+
+template <typename QT>
+__host__ __device__ constexpr int q_rows() { return (int)(H_CHUNK / (T * sizeof(QT))); }
+template <>
+__host__ __device__ constexpr int q_rows<void>() { return T; }
+
+// Producer (one warp): publishes each tile's parameters with the values of its
+// row and column nodes and, where Q is stored, streams its rows (whole:
+// entries outside the pair set are stored as 0) in 16 KB copies, ahead across
+// tiles.  QT = void: Q is recomputed elsewhere.
+template <typename QT>
+__device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, const int4* __restrict__ work,
+                                              long long ntiles, HTail& sm, unsigned char* ring, volatile int* abort_flag,
+                                              int lane, int st)
+{
+    constexpr bool STREAM = q_rows<QT>() < T;
+    const uint64_t pol = l2_evict_first_policy(), pol_keep = l2_evict_last_policy();
+    int stage = 0, slot = 0;
+    uint32_t phase = 0, tph = 0;
+    auto stopped = [&]() { return abort_flag && __shfl_sync(0xffffffffu, *abort_flag, 0) != 0; };
+    auto give_up = [&](Ctrl* ctrl, long long L) {
+        if (lane == 0) {
+            record_error(ctrl, ST_ETIMEOUT, L);
+            if (abort_flag) *abort_flag = 1;
+        }
+    };
+    // The round's settings of an instance do not change during a sweep: they
+    // are read once per run of tiles of the same instance, and the next tile's
+    // list entry ahead of its turn, so that no chain of loads stands between
+    // the copies of two tiles.
+    int inst = -1, t = 0, kind = 0, even = 0;
+    bool done = true, staged = false;
+    uint32_t use = 0;
+    int4 wn = blockIdx.x < ntiles ? work[blockIdx.x] : make_int4(0, 0, 0, 0);
+    for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
+        const int4 w = wn;
+        if (L + gridDim.x < ntiles) wn = work[L + gridDim.x];
+        const Inst& p = tab[w.x];
+        Ctrl* ctrl = p.ctrl;
+        if (w.x != inst) {
+            inst = w.x;
+            done = *(volatile const int*)&ctrl->done != 0;
+            t = *(volatile const int*)&ctrl->t;
+            const int frozen = *(volatile const int*)&ctrl->p_frozen, terms = ctrl->terms;
+            even = ctrl->even;
+            staged = p.nstages > 1;
+            kind = frozen && t > 0                    ? (terms == 0 ? K_SUM : terms == 1 ? K_ONE : K_TWO)
+                   : staged                           ? K_LIVE   // (fewer sums do not fit the registers of sum_tile)
+                   : t == 0 || (!even && terms == 0) ? K_LIVE0
+                   : !even && terms == 1             ? K_LIVE1
+                                                     : K_LIVE;
+            // node values of its tiles: bit a set where row a is copied
+            use = 1u << N_MU0 | (staged ? 1u << N_MU : 0u) | (kind <= K_LIVE ? 1u << N_R : 0u) |
+                  (kind == K_LIVE0 || kind == K_SUM ? 0u : 1u << N_W3) | (kind == K_LIVE || kind == K_TWO ? 1u << N_W5 : 0u);
+        }
+        if (done) continue;      // instance finished: tile skipped
+        const int I = w.y, J = w.z, rows = min(T, p.n - I * T);
+        if (stopped() || !mbar_wait_warp(&sm.tempty[slot], tph ^ 1u)) {
+            give_up(ctrl, L);
+            return;
+        }
+        if (lane == 0) {
+            HInfo& ti = sm.info[slot];
+            ti.ring = p.hring + hist_offset(p.npad, st, 0);
+            ti.part = p.part;
+            ti.s46 = p.hs46;
+            ti.plen = (long long)part_len(p);
+            ti.ctrl = ctrl;
+            ti.L = L;
+            ti.npad = p.npad; ti.I = I; ti.J = J;
+            const int2 sl = tile_slots(p, w);
+            ti.sR = sl.x; ti.sC = sl.y;
+            ti.rows = rows;
+            ti.t = t;
+            ti.kind = kind;
+            ti.even = even;
+            ti.staged = staged;
+            ti.end = 0;
+            mbar_arrive_expect_tx(&sm.tfull[slot], (uint32_t)__popc(use) * 2 * T * (uint32_t)sizeof(float));
+        }
+        __syncwarp();
+        const int a = lane >> 1;
+        if ((use >> a) & 1u) {
+            const size_t np = p.npad;
+            const float* src = a == N_MU0  ? p.agg + (size_t)(t & 1) * 3 * np + 2 * np
+                               : a == N_MU ? hist_slot(p, st, t) + 2 * np
+                                           : p.hnow + (3 * (size_t)st + (a - N_R)) * np;
+            bulk_load(&sm.node[slot][lane & 1][a][0], src + (size_t)((lane & 1) ? J : I) * T, T * sizeof(float),
+                      &sm.tfull[slot], pol_keep);
+        }
+        if (++slot == 2) { slot = 0; tph ^= 1u; }
+        if constexpr (STREAM) {
+            constexpr int RC = q_rows<QT>();
+            const unsigned char* qt = static_cast<const unsigned char*>(p.qstore) + (size_t)w.w * TT * sizeof(QT);
+            const int nch = (rows + RC - 1) / RC;
+            for (int c = 0; c < nch; ++c) {
+                if (!mbar_wait_warp(&sm.empty[stage], phase ^ 1u)) {
+                    give_up(ctrl, L);
+                    return;
+                }
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(&sm.full[stage], (uint32_t)H_CHUNK);
+                    bulk_load(ring + (size_t)stage * H_CHUNK, qt + (size_t)c * H_CHUNK, (uint32_t)H_CHUNK,
+                              &sm.full[stage], pol);
+                }
+                if (++stage == H_STAGES) { stage = 0; phase ^= 1u; }
+            }
+        }
+    }
+    if (!stopped() && mbar_wait_warp(&sm.tempty[slot], tph ^ 1u) && lane == 0) {
+        sm.info[slot].end = 1;
+        mbar_arrive(&sm.tfull[slot]);
+    }
+}
+
+__device__ __forceinline__ void unpack_bf16(uint2 a, float2 (&q)[2])
+{
+    q[0] = make_float2(__uint_as_float(a.x << 16), __uint_as_float(a.x & 0xffff0000u));
+    q[1] = make_float2(__uint_as_float(a.y << 16), __uint_as_float(a.y & 0xffff0000u));
+}
+// Tiles of few sums (at most q mu, mu of the stage and q^3): a consumer warp
+// takes two rows at a time, one per half-warp: lane (half hf, hl = lane % 16)
+// holds columns 4 hl .. 4 hl + 3 and 64 + 4 hl .. 64 + 4 hl + 3
+// of row 2 cw + hf of each 16 rows, so that a half-warp's loads cover
+// contiguous bytes and eight pairs share the row's values.
+__device__ __forceinline__ void unpack_bf16(uint2 a, uint2 b, float2 (&q)[4])
+{
+    const uint32_t w[4] = {a.x, a.y, b.x, b.y};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) q[k] = make_float2(__uint_as_float(w[k] << 16), __uint_as_float(w[k] & 0xffff0000u));
+}
+
+// Q streamed through the ring by the producer.
+template <typename QT>
+struct StreamedQ {
+    static constexpr int ROWS = q_rows<QT>();
+    unsigned char* ring;
+    int stage;
+    uint32_t phase;
+    bool abort;
+    __device__ __forceinline__ bool acquire(HTail& sm, const HInfo& ti, int lane, bool)
+    {
+        if (!abort && !mbar_wait_warp(&sm.full[stage], phase)) {
+            abort = true;
+            if (lane == 0) record_error(ti.ctrl, ST_ETIMEOUT, ti.L);
+        }
+        return !abort;
+    }
+    __device__ __forceinline__ void release(HTail& sm, int lane, bool)
+    {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.empty[stage]);
+        if (++stage == H_STAGES) { stage = 0; phase ^= 1u; }
+    }
+    __device__ __forceinline__ void load(int lr, int hl, float2 (&q)[4]) const
+    {
+        const QT* row = reinterpret_cast<const QT*>(ring + (size_t)stage * H_CHUNK) + (size_t)(lr & (ROWS - 1)) * T;
+        if constexpr (sizeof(QT) == 4) {
+            const float4 a = *reinterpret_cast<const float4*>(row + 4 * hl), b = *reinterpret_cast<const float4*>(row + 64 + 4 * hl);
+            q[0] = make_float2(a.x, a.y); q[1] = make_float2(a.z, a.w);
+            q[2] = make_float2(b.x, b.y); q[3] = make_float2(b.z, b.w);
+        } else {
+            unpack_bf16(*reinterpret_cast<const uint2*>(row + 4 * hl), *reinterpret_cast<const uint2*>(row + 64 + 4 * hl), q);
+        }
+    }
+    __device__ __forceinline__ void load_row(int lr, int lane, float2 (&q)[2]) const
+    {
+        const QT* row = reinterpret_cast<const QT*>(ring + (size_t)stage * H_CHUNK) + (size_t)(lr & (ROWS - 1)) * T;
+        if constexpr (sizeof(QT) == 4) {
+            const float4 a = *reinterpret_cast<const float4*>(row + 4 * lane);
+            q[0] = make_float2(a.x, a.y); q[1] = make_float2(a.z, a.w);
+        } else {
+            unpack_bf16(*reinterpret_cast<const uint2*>(row + 4 * lane), q);
+        }
+    }
+};
+
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+
+// Sums of four values over the 16 lanes of a half-warp in a fixed order: lane
+// hl holds the total of value hl / 4 (five shuffles).
+__device__ __forceinline__ float half_sums4(const float (&x)[4], int hl)
+{
+    const bool b8 = (hl & 8) != 0, b4 = (hl & 4) != 0;
+    float y[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        y[k] = (b8 ? x[k + 2] : x[k]) + __shfl_xor_sync(0xffffffffu, b8 ? x[k] : x[k + 2], 8);
+    float v = (b4 ? y[1] : y[0]) + __shfl_xor_sync(0xffffffffu, b4 ? y[0] : y[1], 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    return v + __shfl_xor_sync(0xffffffffu, v, 1);
+}
+// The row sums of four steps -> dst[row].
+__device__ __forceinline__ void put_rows(float* dst, float (&x)[4], int r0, int cw, int lane)
+{
+    const int hl = lane & 15;
+    const float v = half_sums4(x, hl);
+    if ((hl & 3) == 0) dst[r0 + 16 * (hl >> 2) + 2 * cw + (lane >> 4)] = v;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = 0.f;
+}
+// The lane's column sums of both half-warps -> d (one row of cs).
+__device__ __forceinline__ void put_cols(float* d, const float2 (&a)[4], int lane)
+{
+    const int hl = lane & 15;
+    float2 m[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        m[k].x = a[k].x + __shfl_xor_sync(0xffffffffu, a[k].x, 16);
+        m[k].y = a[k].y + __shfl_xor_sync(0xffffffffu, a[k].y, 16);
+    }
+    if (lane < 16) *reinterpret_cast<float4*>(d + 4 * hl) = make_float4(m[0].x, m[0].y, m[1].x, m[1].y);
+    else *reinterpret_cast<float4*>(d + 64 + 4 * hl) = make_float4(m[2].x, m[2].y, m[3].x, m[3].y);
+}
+__device__ __forceinline__ void ld_cols(const float* d, int hl, float2 (&v)[4])
+{
+    const float4 a = *reinterpret_cast<const float4*>(d + 4 * hl), b = *reinterpret_cast<const float4*>(d + 64 + 4 * hl);
+    v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w);
+    v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
+}
+
+// Runs `row(q, tile row, step of the group)` over the tile's rows of this
+// lane's half-warp, 64 rows (four steps) at a time, and `group(first row)`
+// after each.
+template <class SRC, class ROW, class GROUP>
+__device__ __forceinline__ void walk_tile(SRC& src, HTail& sm, const HInfo& ti, int cw, int lane, ROW row, GROUP group)
+{
+    constexpr int RC = SRC::ROWS < H_GROUP ? SRC::ROWS : H_GROUP, CPG = H_GROUP / RC, SPC = RC / 16;
+    const int nch = (ti.rows + RC - 1) / RC, hf = lane >> 4, hl = lane & 15;
+#pragma unroll 1
+    for (int c0 = 0; c0 < nch; c0 += CPG) {
+#pragma unroll
+        for (int g = 0; g < CPG; ++g) {
+            if (CPG > 1 && c0 + g >= nch) continue;
+            if (src.acquire(sm, ti, lane, c0 + g == 0)) {
+#pragma unroll
+                for (int s = 0; s < SPC; ++s) {
+                    const int r = (c0 + g) * RC + 16 * s + 2 * cw + hf;
+                    float2 q[4];
+                    src.load(r, hl, q);
+                    row(q, r, g * SPC + s);
+                }
+            }
+            src.release(sm, lane, c0 + g == nch - 1);
+        }
+        group(c0 * RC);
+    }
+}
+
+// q mu, with q^2 (PTWO: live P) and q^3 (ONE) beside it.
+template <bool PTWO, bool ONE, bool STAGED, class SRC>
+__device__ __forceinline__ void sum_tile(SRC& src, HTail& sm, const HInfo& ti, int slot, int cw, int lane)
+{
+    const int hl = lane & 15;
+    const float (*R)[T] = sm.node[slot][0];
+    const float (*C)[T] = sm.node[slot][1];
+    float2 cm[4], cs[4], cr[4], cv[4], aR[4], aM[4], aP[4], aE[4];
+    ld_cols(C[N_MU0], hl, cm);
+    if (STAGED) ld_cols(C[N_MU], hl, cs);
+    if (PTWO) ld_cols(C[N_R], hl, cr);
+    if (ONE) ld_cols(C[N_W3], hl, cv);
+    float xR[4], xM[4], xP[4], xE[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        aR[k] = aM[k] = aP[k] = aE[k] = f2(0.f);
+        xR[k] = xM[k] = xP[k] = xE[k] = 0.f;
+    }
+    auto row = [&](const float2 (&q)[4], int r, int step) {
+        const float2 am = f2(R[N_MU0][r]), as = f2(STAGED ? R[N_MU][r] : 0.f), ar = f2(PTWO ? R[N_R][r] : 0.f),
+                     av = f2(ONE ? R[N_W3][r] : 0.f);
+        float2 sR = f2(0.f), sM = f2(0.f), sP = f2(0.f), sE = f2(0.f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            aR[k] = fma2(q[k], am, aR[k]);
+            sR = fma2(q[k], cm[k], sR);
+            if (STAGED) {
+                aM[k] = fma2(q[k], as, aM[k]);
+                sM = fma2(q[k], cs[k], sM);
+            }
+            const float2 q2 = mul2(q[k], q[k]);
+            if (PTWO) {
+                aP[k] = fma2(q2, ar, aP[k]);
+                sP = fma2(q2, cr[k], sP);
+            }
+            if (ONE) {
+                const float2 q3 = mul2(q2, q[k]);
+                aE[k] = fma2(q3, av, aE[k]);
+                sE = fma2(q3, cv[k], sE);
+            }
+        }
+        xR[step] = sR.x + sR.y;
+        if (STAGED) xM[step] = sM.x + sM.y;
+        if (PTWO) xP[step] = sP.x + sP.y;
+        if (ONE) xE[step] = sE.x + sE.y;
+    };
+    auto group = [&](int r0) {
+        put_rows(sm.rs[S_R], xR, r0, cw, lane);
+        if (STAGED) put_rows(sm.rs[S_M], xM, r0, cw, lane);
+        if (PTWO) put_rows(sm.rs[S_2], xP, r0, cw, lane);
+        if (ONE) put_rows(sm.rs[S_W3], xE, r0, cw, lane);
+    };
+    walk_tile(src, sm, ti, cw, lane, row, group);
+    put_cols(sm.cs[S_R][cw], aR, lane);
+    if (STAGED) put_cols(sm.cs[S_M][cw], aM, lane);
+    if (PTWO) put_cols(sm.cs[S_2][cw], aP, lane);
+    if (ONE) put_cols(sm.cs[S_W3][cw], aE, lane);
+}
+
+__device__ __forceinline__ void ld_cols4(const float* d, int lane, float2 (&v)[2])
+{
+    const float4 a = *reinterpret_cast<const float4*>(d + 4 * lane);
+    v[0] = make_float2(a.x, a.y);
+    v[1] = make_float2(a.z, a.w);
+}
+
+// Tiles of more sums (q^3 and q^5; with live P also q^2, q^4 and q^6): a warp
+// takes one row at a time (row 8 s + cw), each lane four of its columns, which
+// leaves room for all the weights and sums of a lane's columns (eight columns a
+// lane did not fit 96 registers); a row's sums go through one eight-value warp
+// reduction.
+template <bool LIVE, bool STAGED, class SRC>
+__device__ __forceinline__ void wide_tile(SRC& src, HTail& sm, const HInfo& ti, int slot, int cw, int lane)
+{
+    const float (*R)[T] = sm.node[slot][0];
+    const float (*C)[T] = sm.node[slot][1];
+    float2 cm[2], cs[2], cr[2], c3[2], c5[2], a[S_COUNT][2];
+    ld_cols4(C[N_MU0], lane, cm);
+    if (STAGED) ld_cols4(C[N_MU], lane, cs);
+    if (LIVE) ld_cols4(C[N_R], lane, cr);
+    ld_cols4(C[N_W3], lane, c3);
+    ld_cols4(C[N_W5], lane, c5);
+#pragma unroll
+    for (int s = 0; s < S_COUNT; ++s) a[s][0] = a[s][1] = f2(0.f);
+    constexpr int RC = SRC::ROWS < H_GROUP ? SRC::ROWS : H_GROUP;
+    const int nch = (ti.rows + RC - 1) / RC;
+#pragma unroll 1
+    for (int c = 0; c < nch; ++c) {
+        if (src.acquire(sm, ti, lane, c == 0)) {
+#pragma unroll 2
+            for (int s = 0; s < RC / 8; ++s) {
+                const int r = c * RC + 8 * s + cw;
+                float2 q[2], x[S_COUNT];
+                src.load_row(r, lane, q);
+#pragma unroll
+                for (int k = 0; k < S_COUNT; ++k) x[k] = f2(0.f);
+                const float2 rm = f2(R[N_MU0][r]), rs = f2(STAGED ? R[N_MU][r] : 0.f), rr = f2(LIVE ? R[N_R][r] : 0.f),
+                             r3 = f2(R[N_W3][r]), r5 = f2(R[N_W5][r]);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    a[S_R][k] = fma2(q[k], rm, a[S_R][k]);
+                    x[S_R] = fma2(q[k], cm[k], x[S_R]);
+                    if (STAGED) {
+                        a[S_M][k] = fma2(q[k], rs, a[S_M][k]);
+                        x[S_M] = fma2(q[k], cs[k], x[S_M]);
+                    }
+                    const float2 q2 = mul2(q[k], q[k]), q3 = mul2(q2, q[k]), q5 = mul2(q3, q2);
+                    if (LIVE) {
+                        const float2 wi = mul2(q2, rr), wj = mul2(q2, cr[k]), wi2 = mul2(wi, wi), wj2 = mul2(wj, wj);
+                        a[S_2][k] = __fadd2_rn(a[S_2][k], wi);
+                        x[S_2] = __fadd2_rn(x[S_2], wj);
+                        a[S_4][k] = __fadd2_rn(a[S_4][k], wi2);
+                        x[S_4] = __fadd2_rn(x[S_4], wj2);
+                        a[S_6][k] = fma2(wi2, wi, a[S_6][k]);
+                        x[S_6] = fma2(wj2, wj, x[S_6]);
+                    }
+                    a[S_W3][k] = fma2(q3, r3, a[S_W3][k]);
+                    x[S_W3] = fma2(q3, c3[k], x[S_W3]);
+                    a[S_W5][k] = fma2(q5, r5, a[S_W5][k]);
+                    x[S_W5] = fma2(q5, c5[k], x[S_W5]);
+                }
+                float y[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) y[k] = k < S_COUNT ? x[k < S_COUNT ? k : 0].x + x[k < S_COUNT ? k : 0].y : 0.f;
+                const float v = reduce_scatter8x(y, lane);
+                const int k = (lane >> 2) & 7;
+                if ((lane & 3) == 0 && k < S_COUNT) sm.rs[k][r] = v;
+            }
+        }
+        src.release(sm, lane, c == nch - 1);
+    }
+#pragma unroll
+    for (int s = 0; s < S_COUNT; ++s)
+        if (s == S_R || (s == S_M && STAGED) || ((s == S_2 || s == S_4 || s == S_6) && LIVE) || s == S_W3 || s == S_W5)
+            *reinterpret_cast<float4*>(&sm.cs[s][cw][4 * lane]) = make_float4(a[s][0].x, a[s][0].y, a[s][1].x, a[s][1].y);
+}
+
+// The eight consumer warps: tile after tile as the producer publishes them,
+// each tile's sums to its slots in a fixed order.
+template <class SRC>
+__device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* __restrict__ tab,
+                                               const int4* __restrict__ work, long long ntiles, int tid)
+{
+    const int cw = tid >> 5, lane = tid & 31;
+    int slot = 0;
+    uint32_t tph = 0;
+    for (;;) {
+        if (!mbar_wait_warp(&sm.tfull[slot], tph) && lane == 0) {
+            sm.cabort = 1;
+            if (blockIdx.x < ntiles) record_error(tab[work[blockIdx.x].x].ctrl, ST_ETIMEOUT, -1);
+        }
+        hbar();   // also: the previous tile's sums are read out
+        if (*(volatile int*)&sm.cabort) break;
+        if (sm.info[slot].end) break;
+        const HInfo& ti = sm.info[slot];
+        const int kind = ti.kind, rows = ti.rows;
+        const bool diag = ti.I == ti.J, staged = ti.staged, live = kind <= K_LIVE, even = ti.even, first = ti.t == 0;
+        float* part = ti.part;
+        const long long plen = ti.plen;
+        // this thread's node of the tile's sums: row block's for the first 128
+        // threads, column block's for the others; its values of round t - 1
+        const int c = tid & (T - 1);
+        const size_t o = (size_t)(tid < T ? ti.sR : ti.sC) * T + c;
+        float* s46 = ti.s46 + o;
+        float mu1 = 0.f, r1 = 0.f, D1 = 0.f, D3 = 0.f, S4 = 0.f, S6 = 0.f, P = 0.f;
+        if (!first && (staged || kind != K_SUM)) {
+            const size_t np = ti.npad;
+            const float* node = ti.ring + (size_t)(tid < T ? ti.I : ti.J) * T + c;
+            const float* old = node + ((unsigned)(ti.t - 1) % (unsigned)kHist) * 4 * np;
+            mu1 = old[2 * np];
+            if (kind != K_SUM) {
+                r1 = 1.f / old[0];
+                if (even) {
+                    D1 = old[3 * np];
+                    D3 = node[((unsigned)(ti.t + kHist - 3) % (unsigned)kHist) * 4 * np + 3 * np];
+                    if (!live) { S4 = s46[0]; S6 = s46[plen]; }
+                }
+            }
+            if (!live && staged) P = part[o];
+        }
+        if (staged) {
+            if (kind == K_SUM) sum_tile<false, false, true>(src, sm, ti, slot, cw, lane);
+            else if (kind == K_ONE) sum_tile<false, true, true>(src, sm, ti, slot, cw, lane);
+            else if (kind == K_LIVE) wide_tile<true, true>(src, sm, ti, slot, cw, lane);
+            else wide_tile<false, true>(src, sm, ti, slot, cw, lane);
+        } else {
+            if (kind == K_SUM) sum_tile<false, false, false>(src, sm, ti, slot, cw, lane);
+            else if (kind == K_ONE) sum_tile<false, true, false>(src, sm, ti, slot, cw, lane);
+            else if (kind == K_LIVE0) sum_tile<true, false, false>(src, sm, ti, slot, cw, lane);
+            else if (kind == K_LIVE1) sum_tile<true, true, false>(src, sm, ti, slot, cw, lane);
+            else if (kind == K_LIVE) wide_tile<true, false>(src, sm, ti, slot, cw, lane);
+            else wide_tile<false, false>(src, sm, ti, slot, cw, lane);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.tempty[slot]);   // its parameters are not read again
+        if (++slot == 2) { slot = 0; tph ^= 1u; }
+        hbar();
+        // the node's sums; the column sums over the eight warps, both roles on a
+        // diagonal tile.  (Slot entries of nodes beyond n are written, and read
+        // by no one else.)
+        const bool all = kind == K_LIVE, odd = kind != K_SUM && kind != K_LIVE0;
+        const bool has[S_COUNT] = {true, staged, live, all, all, odd, all || kind == K_TWO};
+        float v[S_COUNT];
+#pragma unroll
+        for (int a = 0; a < S_COUNT; ++a) {
+            v[a] = 0.f;
+            if (!has[a]) continue;
+            if (tid < T && c < rows) v[a] = sm.rs[a][c];
+            if (tid >= T || diag) {
+                float s = 0.f;
+#pragma unroll
+                for (int w = 0; w < HCW; ++w) s += sm.cs[a][w][c];
+                v[a] += s;
+            }
+        }
+        if (tid < T || !diag) {
+            if (all && even) { S4 = v[S_4]; S6 = v[S_6]; }
+            if (live) P = fmaf(r1, fmaf(-2.f * r1, S6, S4), -v[S_2]);
+            const float E = r1 * (fmaf(S4, D1, v[S_W3]) + r1 * fmaf(S6, D3 - 3.f * D1, v[S_W5]));
+            float* d = part + o;
+            if (live) d[0] = P;
+            if (all && even) { s46[0] = S4; s46[plen] = S6; }
+            if (staged) d[plen] = fmaf(P, mu1, E - v[S_M]);
+            else if (odd) d[plen] = E;
+            d[2 * plen] = v[S_R];
+        }
+    }
+}
+
+__device__ __forceinline__ void init_htail(HTail& sm)
+{
+    for (int s = 0; s < H_STAGES; ++s) { mbar_init(&sm.full[s], 1); mbar_init(&sm.empty[s], HCW); }
+    for (int s = 0; s < 2; ++s) { mbar_init(&sm.tfull[s], 1); mbar_init(&sm.tempty[s], HCW); }
+    sm.cabort = 0;
+}
+
+// A single instance that has stopped: the rest of a captured chunk of rounds
+// (skipping its tiles one by one took 640 us a round at n = 100000).
+__device__ __forceinline__ bool nothing_to_do(const Inst* tab, const Sched* sched)
+{
+    return sched->ntiles == 0 || (sched->ninst == 1 && *(volatile const int*)&tab[0].ctrl->done != 0);
+}
+
+// Q stored (FP32 or BF16) and streamed.
+template <typename QT>
+__global__ void __launch_bounds__(H_THREADS, 2)
+    k_sweep_hist(const Inst* __restrict__ tab, const int4* __restrict__ work, const Sched* __restrict__ sched, int stage_no)
+{
+    const long long ntiles = sched->ntiles;
+    if (nothing_to_do(tab, sched)) return;
+    work += sched->off;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* ring = align_smem(smem_raw, 128);
+    HTail& sm = *reinterpret_cast<HTail*>(ring + H_STAGES * H_CHUNK);
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        init_htail(sm);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    if (tid >= HCW * 32) {
+        hist_producer<QT>(tab, work, ntiles, sm, ring, nullptr, tid & 31, stage_no);
+        return;
+    }
+    StreamedQ<QT> src{ring, 0, 0u, false};
+    hist_consumers(src, sm, tab, work, ntiles, tid);
+}
+
+constexpr size_t hist_smem_bytes() { return 128 + H_STAGES * H_CHUNK + sizeof(HTail); }
+
+// ---- Q recomputed in every sweep -------------------------------------------
+// As the fused recompute of sweep.cu, without messages to stream: warps 0-7
+// consume, warp 8 publishes the tiles, warp 9 copies the BF16 feature blocks,
+// one thread of warp 10 issues the tcgen05 MMAs into a double-buffered TMEM
+// accumulator, and warps 12-19 (two per TMEM lane quarter, one per column
+// half) turn the Gram rows into BF16 Q values in a double-buffered shared
+// tile, bitwise the values of the BF16 store.
+constexpr int HR_XSTAGES = 2;
+constexpr int HR_EPI = 8;
+constexpr int HR_THREADS = (12 + HR_EPI) * 32;
+constexpr uint32_t HR_TMEM_COLS = 256;
+constexpr size_t HR_QTILE = (size_t)TT * sizeof(__nv_bfloat16);
+
+struct HrExtra {
+    unsigned long long xfull[HR_XSTAGES], xempty[HR_XSTAGES];
+    unsigned long long accfull[2], accempty[2];
+    unsigned long long qfull[2], qempty[2];
+    unsigned long long drain;
+    uint32_t tmem_base;
+    int abort;
+    ColTile cols[HR_EPI];
+};
+constexpr size_t hist_rc_smem_bytes()
+{
+    return 1024 + HR_XSTAGES * 2 * BLK_BYTES + 2 * HR_QTILE + sizeof(HTail) + sizeof(HrExtra);
+}
+
+// Q from the shared tile.  Its rows are stored with their 16-byte chunks
+// permuted: chunk k of row r sits at chunk k ^ (r % 8), so that the epilogue's
+// stores (one row per lane, the same chunk) spread over all banks.
+struct TileQ {
+    static constexpr int ROWS = T;
+    const unsigned char* qtile;   // [2][T][T] BF16
+    HrExtra* ex;
+    int it;
+    bool abort;
+    __device__ __forceinline__ bool acquire(HTail& sm, const HInfo& ti, int lane, bool first)
+    {
+        if (first && !abort && !mbar_wait_warp(&ex->qfull[it & 1], (uint32_t)((it >> 1) & 1))) {
+            abort = true;
+            if (lane == 0) record_error(ti.ctrl, ST_ETIMEOUT, ti.L);
+        }
+        return !abort;
+    }
+    __device__ __forceinline__ void release(HTail&, int lane, bool last)
+    {
+        if (!last) return;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ex->qempty[it & 1]);
+        ++it;
+    }
+    __device__ __forceinline__ void load(int r, int hl, float2 (&q)[4]) const
+    {
+        const unsigned char* row = qtile + (size_t)(it & 1) * HR_QTILE + (size_t)r * T * 2;
+        const int o = (((hl >> 1) ^ (r & 7)) << 4) + ((hl & 1) << 3);
+        unpack_bf16(*reinterpret_cast<const uint2*>(row + o), *reinterpret_cast<const uint2*>(row + 128 + o), q);
+    }
+    __device__ __forceinline__ void load_row(int r, int lane, float2 (&q)[2]) const
+    {
+        const unsigned char* row = qtile + (size_t)(it & 1) * HR_QTILE + (size_t)r * T * 2;
+        unpack_bf16(*reinterpret_cast<const uint2*>(row + (((lane >> 1) ^ (r & 7)) << 4) + ((lane & 1) << 3)), q);
+    }
+};
+
+__global__ void __launch_bounds__(HR_THREADS, 1)
+    k_sweep_hist_rc(const Inst* __restrict__ tab, const int4* __restrict__ work, const Sched* __restrict__ sched,
+                    int stage_no)
+{
+    const long long ntiles = sched->ntiles;
+    if (nothing_to_do(tab, sched)) return;
+    work += sched->off;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* xops = align_smem(smem_raw, 1024);
+    unsigned char* qtile = xops + HR_XSTAGES * 2 * BLK_BYTES;
+    HTail& sm = *reinterpret_cast<HTail*>(qtile + 2 * HR_QTILE);
+    HrExtra& ex = *reinterpret_cast<HrExtra*>(reinterpret_cast<unsigned char*>(&sm) + sizeof(HTail));
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        init_htail(sm);
+        for (int s = 0; s < HR_XSTAGES; ++s) { mbar_init(&ex.xfull[s], 1); mbar_init(&ex.xempty[s], 1); }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&ex.accfull[b], 1);
+            mbar_init(&ex.accempty[b], HR_EPI);
+            mbar_init(&ex.qfull[b], HR_EPI);
+            mbar_init(&ex.qempty[b], HCW);
+        }
+        mbar_init(&ex.drain, 1);
+        ex.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 10) tmem_alloc(&ex.tmem_base, HR_TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = ex.tmem_base;
+    volatile int* abort_flag = &ex.abort;
+
+    if (warp < HCW) {
+        TileQ src{qtile, &ex, 0, false};
+        hist_consumers(src, sm, tab, work, ntiles, tid);
+    } else if (warp == 8) {
+        hist_producer<void>(tab, work, ntiles, sm, nullptr, abort_flag, lane, stage_no);
+    } else if (warp == 9) {
+        if (lane == 0) {
+            const uint64_t pol = l2_evict_last_policy();   // the features are read again by many tiles
+            int xs = 0;
+            uint32_t ph = 0;
+            bool run = true;
+            for (long long L = blockIdx.x; L < ntiles && run; L += gridDim.x) {
+                const int4 w = work[L];
+                const Inst& p = tab[w.x];
+                if (*(volatile const int*)&p.ctrl->done) continue;
+                const unsigned char* Xp = static_cast<const unsigned char*>(p.Xp);
+                const int nkc = p.nkc;
+                for (int kc = 0; kc < nkc; ++kc) {
+                    if (*abort_flag || !mbar_wait(&ex.xempty[xs], ph ^ 1u)) {
+                        *abort_flag = 1;
+                        record_error(p.ctrl, ST_ETIMEOUT, L);
+                        run = false;
+                        break;
+                    }
+                    unsigned char* A = xops + (size_t)xs * 2 * BLK_BYTES;
+                    mbar_arrive_expect_tx(&ex.xfull[xs], 2 * BLK_BYTES);
+                    bulk_load(A, Xp + ((size_t)w.y * nkc + kc) * BLK_BYTES, BLK_BYTES, &ex.xfull[xs], pol);
+                    bulk_load(A + BLK_BYTES, Xp + ((size_t)w.z * nkc + kc) * BLK_BYTES, BLK_BYTES, &ex.xfull[xs], pol);
+                    if (++xs == HR_XSTAGES) { xs = 0; ph ^= 1u; }
+                }
+            }
+        }
+    } else if (warp == 10) {
+        if (lane == 0) {
+            constexpr uint32_t IDESC = idesc_bf16_f32(T, T);
+            int xs = 0, acc = 0;
+            uint32_t ph = 0, aph = 0;
+            for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
+                const Inst& p = tab[work[L].x];
+                if (*(volatile const int*)&p.ctrl->done) continue;
+                const int nkc = p.nkc;
+                bool ok = !*abort_flag && mbar_wait(&ex.accempty[acc], aph ^ 1u);
+                tc_fence_after();
+                const uint32_t d = tbase + (uint32_t)acc * T;
+                for (int kc = 0; kc < nkc && ok; ++kc) {
+                    if (*abort_flag || !mbar_wait(&ex.xfull[xs], ph)) { ok = false; break; }
+                    tc_fence_after();
+                    const unsigned char* A = xops + (size_t)xs * 2 * BLK_BYTES;
+#pragma unroll
+                    for (int s = 0; s < KCH / 16; ++s)
+                        tc_mma_bf16(d, smem_desc(A + s * 256, 128, 1024), smem_desc(A + BLK_BYTES + s * 256, 128, 1024), IDESC,
+                                    (kc | s) != 0);
+                    tc_commit(&ex.xempty[xs]);
+                    if (++xs == HR_XSTAGES) { xs = 0; ph ^= 1u; }
+                }
+                if (!ok) {
+                    *abort_flag = 1;
+                    record_error(p.ctrl, ST_ETIMEOUT, L);
+                    break;
+                }
+                tc_commit(&ex.accfull[acc]);
+                if (++acc == 2) { acc = 0; aph ^= 1u; }
+            }
+            tc_commit(&ex.drain);
+            if (!mbar_wait(&ex.drain, 0u)) *abort_flag = 1;
+        }
+    } else if (warp >= 12) {
+        const int ew = warp - 12, g = warp & 3, half = ew >> 2, r = 32 * g + lane;
+        int it = 0;
+        for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
+            const int4 w = work[L];
+            const Inst& p = tab[w.x];
+            Ctrl* ctrl = p.ctrl;
+            if (*(volatile const int*)&ctrl->done) continue;
+            const int n = p.n, I = w.y, J = w.z, i = I * T + r, acc = it & 1;
+            const uint32_t par = (uint32_t)((it >> 1) & 1);
+            const float* y = p.y;
+            const float* sqb = p.sqb;
+            const float gamma = p.gamma, lam2 = p.lam2;
+            const float yi = i < n ? y[i] : 0.f, si = i < n ? sqb[i] : 0.f;
+            stage_tile_cols(ex.cols[ew], y, sqb, n, J, gamma, lane, 2 * half, 2 * half + 2);
+            const bool stop = __shfl_sync(0xffffffffu, *abort_flag, 0) != 0;
+            if (stop || !mbar_wait_warp(&ex.accfull[acc], par) || !mbar_wait_warp(&ex.qempty[acc], par ^ 1u)) {
+                if (lane == 0) {
+                    *abort_flag = 1;
+                    record_error(ctrl, ST_ETIMEOUT, L);
+                }
+                break;
+            }
+            tc_fence_after();
+            const float ai = -gamma * kLog2e * si, c2 = 2.f * gamma * kLog2e;
+            const uint32_t s1 = __float_as_uint(yi) & 0x80000000u, si2 = s1 | (s1 >> 16);
+            uint4* qrow = reinterpret_cast<uint4*>(qtile + (size_t)acc * HR_QTILE + (size_t)r * T * 2);
+            const int sw = r & 7;
+#pragma unroll 1
+            for (int cc = 2 * half; cc < 2 * half + 2; ++cc) {
+                const uint32_t valid = chunk_valid(n, I, J, r, cc);
+                float v[32];
+                tmem_ld32(tbase + (uint32_t)acc * T + ((uint32_t)(32 * g) << 16) + (uint32_t)(32 * cc), v);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float vh[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) vh[u] = v[16 * h + u];
+                    uint4 out[2];
+                    q_half_bf16(vh, 32 * cc + 16 * h, ai, si2, ex.cols[ew], c2, lam2, (valid >> (16 * h)) & 0xffffu, out);
+                    qrow[(4 * cc + 2 * h) ^ sw] = out[0];
+                    qrow[(4 * cc + 2 * h + 1) ^ sw] = out[1];
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&ex.accempty[acc]);
+                mbar_arrive(&ex.qfull[acc]);
+            }
+            ++it;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 10) {
+        tc_fence_after();
+        tmem_dealloc(tbase, HR_TMEM_COLS);
+    }
+}
+
+// What choose_path() wants to know of the pairs, over listed tiles, for the
+// instances whose margin leaves it open (the others cost a look at their
+// control block).  From the FP32 entries, so that the forms with BF16 entries
+// decide alike.
+__global__ void __launch_bounds__(256) k_pair_z(const Inst* __restrict__ tab, const int4* __restrict__ work, long long ntiles,
+                                               bool single)
+{
+    __shared__ int s_go;
+    const int tid = threadIdx.x;
+    if (single) {
+        if (tid == 0) s_go = pair_z_open(tab[0]);
+        __syncthreads();
+        if (!s_go) return;
+        __syncthreads();
+    }
+    for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
+        const int4 w = work[L];
+        for (int k = w.x; k >= 0; k = tab[k].form_next - 1) {
+            const Inst& p = tab[k];
+            if (tid == 0) s_go = pair_z_open(p);
+            __syncthreads();
+            const int go = s_go;
+            __syncthreads();   // s_go is read before the next instance writes it
+            if (!go) continue;
+            const float* q = p.qref + (size_t)w.w * TT;
+            const int c0 = 4 * (tid & 31);
+            float rj[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) rj[e] = 1.f / p.qdiag[min(w.z * T + c0 + e, p.n - 1)];   // (entries beyond n are 0)
+            float best[2] = {0.f, FLT_MIN};   // the second never 0: the pass has run
+#pragma unroll 4
+            for (int r = tid >> 5; r < T; r += 8) {
+                const float ri = __fdividef(1.f, p.qdiag[min(w.y * T + r, p.n - 1)]);
+                const float4 a = *reinterpret_cast<const float4*>(q + r * T + c0);
+                note_pair_z(a.x, ri, rj[0], best);
+                note_pair_z(a.y, ri, rj[1], best);
+                note_pair_z(a.z, ri, rj[2], best);
+                note_pair_z(a.w, ri, rj[3], best);
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                best[e] = warp_max_f(best[e]);
+                if ((tid & 31) == 0 && __float_as_uint(best[e]) > *(volatile unsigned*)&p.ctrl->zpair_bits[e])
+                    atomicMax(&p.ctrl->zpair_bits[e], __float_as_uint(best[e]));
+            }
+        }
+    }
+}
+
+}  // namespace
+
+cudaError_t prepare_sweep_hist()
+{
+    cudaError_t e = cudaFuncSetAttribute(k_sweep_hist<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)hist_smem_bytes());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_sweep_hist<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)hist_smem_bytes());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_sweep_hist_rc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hist_rc_smem_bytes());
+    return e;
+}
+
+void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, int stage_no, int grid, int q_mode,
+                       cudaStream_t s)
+{
+    if (q_mode == 2)
+        k_sweep_hist_rc<<<grid, HR_THREADS, hist_rc_smem_bytes(), s>>>(tab, work, sched, stage_no);
+    else if (q_mode == 1)
+        k_sweep_hist<__nv_bfloat16><<<grid, H_THREADS, hist_smem_bytes(), s>>>(tab, work, sched, stage_no);
+    else
+        k_sweep_hist<float><<<grid, H_THREADS, hist_smem_bytes(), s>>>(tab, work, sched, stage_no);
+}
+
+void launch_pair_z(const Inst* tab, const int4* tiles, long long ntiles, int q_mode, bool single, cudaStream_t s)
+{
+    if (ntiles <= 0) return;
+    const int grid = (int)(ntiles < 4 * num_sms() ? ntiles : 4 * num_sms());
+    if (q_mode == 2) launch_pair_z_gram(tab, tiles, ntiles, grid, single, s);
+    else k_pair_z<<<grid, 256, 0, s>>>(tab, tiles, ntiles, single);
+}
+
+}  // namespace gabp
