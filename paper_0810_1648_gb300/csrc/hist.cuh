@@ -15,13 +15,14 @@ __host__ __device__ __forceinline__ size_t hist_offset(int npad, int st, int t)
 }
 __device__ __forceinline__ float* hist_slot(const Inst& p, int st, int t) { return p.hring + hist_offset(p.npad, st, t); }
 
-// Appends node x's aggregates of round t to stage st's history; mu2 is the
-// mean two rounds earlier.
-__device__ __forceinline__ void hist_push(const Inst& p, int st, int t, int x, float P, float h, float mu, float mu2)
+// Appends node x's aggregates of round t to stage st's history; mu2 and D2 are
+// its mean and D two rounds earlier.
+__device__ __forceinline__ void hist_push(const Inst& p, int st, int t, int x, float P, float h, float mu, float mu2,
+                                          float D2)
 {
     const size_t np = p.npad;
     float* s = hist_slot(p, st, t);
-    const float D = mu - mu2, D2 = hist_slot(p, st, t + kHist - 2)[3 * np + x], ip = 1.f / P;
+    const float D = mu - mu2, ip = 1.f / P;
     s[x] = P;
     s[np + x] = h;
     s[2 * np + x] = mu;
@@ -46,7 +47,7 @@ __device__ __forceinline__ void hist_start(const Inst& p, int x, float P, float 
 {
     if (!p.hist) return;
     hist_clear(p, x);
-    hist_push(p, 0, 0, x, P, h, mu, 0.f);
+    hist_push(p, 0, 0, x, P, h, mu, 0.f, 0.f);
 }
 // The H messages restart from 0 at round t with right-hand side h and the P
 // messages kept.
@@ -54,7 +55,7 @@ __device__ __forceinline__ void hist_restart(const Inst& p, int t, int x, float 
 {
     hist_clear(p, x);
     p.agg[(size_t)((t + 1) & 1) * 3 * p.npad + 2 * (size_t)p.npad + x] = 0.f;   // mu(t - 1)
-    hist_push(p, 0, t, x, P, h, mu, 0.f);
+    hist_push(p, 0, t, x, P, h, mu, 0.f, 0.f);
 }
 // Nodes x in [n, npad) that fill the last tile: their entries of Q are 0, and
 // with finite values they add 0 to every sum, so that the sweep needs no

@@ -1153,6 +1153,25 @@ __device__ __forceinline__ RoundState round_state(const Inst& p, const Ctrl* ctr
 __device__ __forceinline__ bool sum_p(const RoundState& s) { return !s.frozen; }
 __device__ __forceinline__ bool sum_h(const RoundState& s) { return !s.from_r || s.with_e; }
 
+// A node's values that its finalize reads beside the slots, loaded before the
+// slot sums so that their latency is hidden.
+struct NodeIn {
+    float qd, b, P, mu, mu1, D1;   // Q_xx, b_x, Ptilde, the means of rounds t and t - 1, D of round t - 1
+};
+__device__ __forceinline__ NodeIn node_in(const Inst& p, int x, const RoundState& s)
+{
+    const size_t np = p.npad;
+    const float* cur = p.agg + (size_t)(s.t & 1) * 3 * np;
+    NodeIn v;
+    v.qd = p.qdiag[x];
+    v.b = p.b[x];
+    v.P = cur[x];
+    v.mu = cur[2 * np + x];
+    v.mu1 = (s.hist && s.t > 0) ? p.agg[(size_t)((s.t + 1) & 1) * 3 * np + 2 * np + x] : 0.f;
+    v.D1 = s.hist ? hist_slot(p, 0, s.t + kHist - 1)[3 * np + x] : 0.f;
+    return v;
+}
+
 struct NodeOut {
     double absr;    // |r_x|, inf for a non-finite one
     float dmu, mu;  // PATH_HIST: |change of the mean over two rounds|, |mean|
@@ -1161,16 +1180,14 @@ struct NodeOut {
 // Node x's next aggregates {Ptilde, htilde, mutilde} from its slot sums (P,
 // H) and its residual r_x(t) = b_x - Q_xx mutilde_x(t) - R in FP64; flags a
 // non-positive or non-finite aggregate.
-__device__ __forceinline__ NodeOut finalize_node(const Inst& p, Ctrl* ctrl, int x, const RoundState& s, double P,
-                                                 double H, double R)
+__device__ __forceinline__ NodeOut finalize_node(const Inst& p, Ctrl* ctrl, int x, const RoundState& s, const NodeIn& v,
+                                                 double P, double H, double R)
 {
     const int t = s.t;
-    const float* cur = p.agg + (size_t)(t & 1) * 3 * p.npad;
     float* nxt = p.agg + (size_t)((t + 1) & 1) * 3 * p.npad;
-    const double qd = p.qdiag[x], bx = p.b[x];
-    const float Pc = cur[x], Pn = s.frozen ? Pc : (float)(qd + P);
-    const float mu1 = (s.hist && t > 0) ? nxt[2 * p.npad + x] : 0.f;   // the mean of round t - 1
-    if (s.from_r) H += (s.frozen ? (double)Pc - qd : P) * mu1 - R;
+    const double qd = v.qd, bx = v.b;
+    const float Pn = s.frozen ? v.P : (float)(qd + P);
+    if (s.from_r) H = (s.with_e ? H : 0.0) + (s.frozen ? (double)v.P - qd : P) * v.mu1 - R;
     const float hn = (float)(bx + H);
     const float mn = hn / Pn;
     nxt[x] = Pn;
@@ -1178,29 +1195,42 @@ __device__ __forceinline__ NodeOut finalize_node(const Inst& p, Ctrl* ctrl, int 
     nxt[2 * p.npad + x] = mn;
     NodeOut o{0.0, 0.f, 0.f};
     if (s.hist) {
-        hist_push(p, 0, t + 1, x, Pn, hn, mn, mu1);
-        o.dmu = fabsf(mn - mu1);
+        hist_push(p, 0, t + 1, x, Pn, hn, mn, v.mu1, v.D1);
+        o.dmu = fabsf(mn - v.mu1);
         o.mu = fabsf(mn);
         // P is frozen once no Ptilde changes any more: the P messages are then
         // functions of constant aggregates
-        if (Pn != Pc) ctrl->p_changed = 1;
+        if (Pn != v.P) ctrl->p_changed = 1;
     }
-    const double r = bx - qd * (double)cur[2 * p.npad + x] - R;
+    const double r = bx - qd * (double)v.mu - R;
     o.absr = fabs(r);
     if (!(o.absr <= DBL_MAX)) o.absr = INFINITY;
     if (!(Pn > 0.f) || !isfinite(Pn) || !isfinite(mn)) record_error(ctrl, ST_ENUMERIC, x);
     return o;
 }
+// Largest of a nonnegative value over the warp, by its bits (integer warp
+// reductions; the high word first for a double).
+__device__ __forceinline__ unsigned long long warp_max_bits(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned hi = (unsigned)(b >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)b : 0u);
+    return ((unsigned long long)mh << 32) | ml;
+}
+__device__ __forceinline__ unsigned warp_max_bits(float v)
+{
+    return __reduce_max_sync(0xffffffffu, v == v ? __float_as_uint(v) : 0u);
+}
 // One warp's node block -> the instance's maxima (lane 0 writes).
 __device__ __forceinline__ void note_block(Ctrl* ctrl, const RoundState& s, NodeOut o, int lane)
 {
-    const double absr = warp_max_d(o.absr);
-    if (lane == 0) atomicMax(&ctrl->rmax_bits, (unsigned long long)__double_as_longlong(absr));
+    const unsigned long long r = warp_max_bits(o.absr);
+    if (lane == 0 && r) atomicMax(&ctrl->rmax_bits, r);
     if (s.hist) {
-        const float d = warp_max_f(o.dmu), m = warp_max_f(o.mu);
+        const unsigned d = warp_max_bits(o.dmu), m = warp_max_bits(o.mu);
         if (lane == 0) {
-            atomicMax(&ctrl->dmax_bits, __float_as_uint(d));
-            atomicMax(&ctrl->mumax_bits, __float_as_uint(m));
+            atomicMax(&ctrl->dmax_bits, d);
+            atomicMax(&ctrl->mumax_bits, m);
         }
     }
 }
@@ -1215,37 +1245,42 @@ __device__ __forceinline__ void hist_ctrl_start(Ctrl* c)
 // Run by the last node block of an instance to finish a round: ||r(t)||_inf,
 // the stop test (Step 3: k* = t when it is below tol, the limit otherwise),
 // the exact P-freeze flag, and the round counter.
-__device__ __forceinline__ void finalize_decide(const Inst& p, Ctrl* ctrl, int t)
+// The values that the blocks of the round left are read together, with
+// volatile loads behind the fence (one after another as atomics they took
+// longer than the rest of the kernel at n = 1000).
+__device__ __forceinline__ void finalize_decide(const Inst& p, Ctrl* ctrl, const RoundState& s)
 {
     __threadfence();
-    const double rmax = __longlong_as_double((long long)atomicAdd(&ctrl->rmax_bits, 0ull));
-    const int status = atomicAdd(&ctrl->status, 0);
+    const volatile Ctrl* c = ctrl;
+    const int t = s.t, status = c->status, p_changed = c->p_changed, limit = c->limit, p_frozen = c->p_frozen;
+    const double rmax = __longlong_as_double((long long)c->rmax_bits), tol = c->tol;
+    const float d = __uint_as_float(c->dmax_bits), m = __uint_as_float(c->mumax_bits);
+    const float z = c->z, u = c->u, change = c->change;
     if (p.rhist && t < p.rhist_cap) p.rhist[t] = rmax;
     if (status != 0) {
         ctrl->done = 1;
         ctrl->kstar = t;
         ctrl->rinf = rmax;
-    } else if (rmax < ctrl->tol) {
+    } else if (rmax < tol) {
         ctrl->done = 1;
         ctrl->kstar = t;
         ctrl->converged = 1;
         ctrl->rinf = rmax;
-    } else if (t + 1 >= ctrl->limit) {
+    } else if (t + 1 >= limit) {
         ctrl->done = 1;
         ctrl->kstar = t + 1;
     }
     // No P message changed in this round: P is at its floating-point fixed
     // point (its recursion does not involve b or H), so later rounds would
     // rewrite the same values; they stop writing them.
-    if (!ctrl->p_frozen && t > 0 && atomicAdd(&ctrl->p_changed, 0) == 0) {
+    if (!p_frozen && t > 0 && p_changed == 0) {
         ctrl->p_frozen = 1;
         ctrl->t_frozen = t + 1;
     }
-    if (ctrl->path == PATH_HIST) {
-        const float d = __uint_as_float(atomicAdd(&ctrl->dmax_bits, 0u)), m = __uint_as_float(atomicAdd(&ctrl->mumax_bits, 0u));
-        const float delta = d < m ? d / m : (d > 0.f ? 1.f : 0.f);
-        ctrl->change = next_change(delta, ctrl->change, ctrl->u);
-        ctrl->terms = e_terms(ctrl->z, ctrl->change);
+    if (s.hist) {
+        const float delta = d < m ? d / m : (d > 0.f ? 1.f : 0.f), next = next_change(delta, change, u);
+        ctrl->change = next;
+        ctrl->terms = e_terms(z, next);
         ctrl->dmax_bits = 0u;
         ctrl->mumax_bits = 0u;
     }
@@ -1254,40 +1289,40 @@ __device__ __forceinline__ void finalize_decide(const Inst& p, Ctrl* ctrl, int t
     ctrl->zero_h = 0;
     ctrl->rmax_bits = 0ull;
     ctrl->blocks_done = 0u;
-    __threadfence();
 }
 
 // Compensated sums of node x's slots k = k0, k0 + step, ... (of the
-// slot_count of its block) of NA partial arrays (P, H[, R]), eight loads of
-// each in flight; the P and H slots read as 0 where not wanted.
-template <int NA>
-__device__ __forceinline__ void slot_sums(const Inst& p, int x, int k0, int step, bool with_p, bool with_h,
-                                          float (&s)[NA], float (&c)[NA])
+// slot_count of its block) of the partial arrays FIRST .. FIRST + NA - 1, DEPTH
+// loads of each in flight to the last slot (slots that are not there read as
+// 0, which leaves the sums as they are).
+template <int FIRST, int NA, int DEPTH>
+__device__ __forceinline__ void sum_arrays(const Inst& p, int x, int k0, int step, float* s, float* c)
 {
     const int X = x / T, ns = slot_count(p, X);
     const size_t len = part_len(p);
-    const float* part = p.part + (size_t)slot_begin(p, X) * T + (x - X * T);
+    const float* part = p.part + FIRST * len + (size_t)slot_begin(p, X) * T + (x - X * T);
+    for (int k = k0; k < ns; k += DEPTH * step) {
+        float v[NA][DEPTH];
 #pragma unroll
-    for (int a = 0; a < NA; ++a) s[a] = c[a] = 0.f;
-    int k = k0;
-    for (; k + 7 * step < ns; k += 8 * step) {
-        float v[NA][8];
+        for (int u = 0; u < DEPTH; ++u)
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
+            for (int a = 0; a < NA; ++a) v[a][u] = k + u * step < ns ? part[a * len + (size_t)(k + u * step) * T] : 0.f;
 #pragma unroll
-            for (int a = 0; a < NA; ++a) {
-                const size_t o = a * len + (size_t)(k + u * step) * T;
-                v[a][u] = ((a == 0 && !with_p) || (a == 1 && !with_h)) ? 0.f : part[o];
-            }
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
+        for (int u = 0; u < DEPTH; ++u)
 #pragma unroll
             for (int a = 0; a < NA; ++a) acc2(s[a], c[a], v[a][u]);
     }
-    for (; k < ns; k += step)
+}
+// Of the arrays P, H[, R], those that the round reads.
+template <int NA>
+__device__ __forceinline__ void slot_sums(const Inst& p, int x, int k0, int step, const RoundState& rs, float (&s)[NA],
+                                          float (&c)[NA])
+{
 #pragma unroll
-        for (int a = 0; a < NA; ++a)
-            acc2(s[a], c[a], ((a == 0 && !with_p) || (a == 1 && !with_h)) ? 0.f : part[a * len + (size_t)k * T]);
+    for (int a = 0; a < NA; ++a) s[a] = c[a] = 0.f;
+    if (sum_p(rs)) sum_arrays<0, NA, 8>(p, x, k0, step, s, c);
+    else if (sum_h(rs)) sum_arrays<1, NA - 1, 8>(p, x, k0, step, s + 1, c + 1);
+    else if (NA == 3) sum_arrays<2, 1, 16>(p, x, k0, step, s + 2, c + 2);
 }
 
 // Node-block units of a round's finalize.  Blocks [0, nsmall) of the list
@@ -1324,12 +1359,13 @@ __global__ void __launch_bounds__(256, 5)
             Ctrl* ctrl = p.ctrl;
             if (*(volatile int*)&ctrl->done) continue;
             const RoundState rs = round_state(p, ctrl);
-            const int x = nb.y * 32 + lane, n = p.n, t = rs.t;
+            const int x = nb.y * 32 + lane, n = p.n;
             NodeOut o{0.0, 0.f, 0.f};
             if (x < n) {
+                const NodeIn v = node_in(p, x, rs);
                 float sv[3], cv[3];
-                slot_sums<3>(p, x, 0, 1, sum_p(rs), sum_h(rs), sv, cv);
-                o = finalize_node(p, ctrl, x, rs, (double)sv[0] + (double)cv[0], (double)sv[1] + (double)cv[1],
+                slot_sums<3>(p, x, 0, 1, rs, sv, cv);
+                o = finalize_node(p, ctrl, x, rs, v, (double)sv[0] + (double)cv[0], (double)sv[1] + (double)cv[1],
                                   (double)sv[2] + (double)cv[2]);
             }
             note_block(ctrl, rs, o, lane);
@@ -1337,7 +1373,7 @@ __global__ void __launch_bounds__(256, 5)
             __syncwarp();
             if (lane == 0) {
                 const unsigned prev = atomicAdd(&ctrl->blocks_done, 1u);
-                if (prev == (unsigned)((n + 31) / 32 - 1)) finalize_decide(p, ctrl, t);
+                if (prev == (unsigned)((n + 31) / 32 - 1)) finalize_decide(p, ctrl, rs);
             }
             continue;
         }
@@ -1347,9 +1383,11 @@ __global__ void __launch_bounds__(256, 5)
         Ctrl* ctrl = p.ctrl;
         if (*(volatile int*)&ctrl->done) continue;
         const RoundState rs = round_state(p, ctrl);
-        const int x = nb.y * 32 + lane, n = p.n, t = rs.t;
+        const int x = nb.y * 32 + lane, n = p.n;
+        NodeIn v{};
+        if (g == 0 && x < n) v = node_in(p, x, rs);
         float sv[3] = {0.f, 0.f, 0.f}, cv[3] = {0.f, 0.f, 0.f};
-        if (x < n) slot_sums<3>(p, x, g, 8, sum_p(rs), sum_h(rs), sv, cv);
+        if (x < n) slot_sums<3>(p, x, g, 8, rs, sv, cv);
         __syncthreads();   // red[] of the previous node block is consumed
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -1367,7 +1405,7 @@ __global__ void __launch_bounds__(256, 5)
                     acc2(a[2], a[3], red[2][w][lane]); a[3] += red[3][w][lane];
                     acc2(a[4], a[5], red[4][w][lane]); a[5] += red[5][w][lane];
                 }
-                o = finalize_node(p, ctrl, x, rs, (double)a[0] + (double)a[1], (double)a[2] + (double)a[3],
+                o = finalize_node(p, ctrl, x, rs, v, (double)a[0] + (double)a[1], (double)a[2] + (double)a[3],
                                   (double)a[4] + (double)a[5]);
             }
             note_block(ctrl, rs, o, lane);
@@ -1379,7 +1417,7 @@ __global__ void __launch_bounds__(256, 5)
             s_last = (prev == (unsigned)((n + 31) / 32 - 1));
         }
         __syncthreads();
-        if (s_last && tid == 0) finalize_decide(p, ctrl, t);
+        if (s_last && tid == 0) finalize_decide(p, ctrl, rs);
     }
 }
 
@@ -1431,8 +1469,10 @@ __device__ __forceinline__ NodeOut stage_node(const Inst& p, int st, int x, cons
     p.aggmid[p.npad + x] = hm;
     NodeOut o{0.0, 0.f, 0.f};
     if (s.hist) {
-        const float mu = hm / Pm, mu2 = s.t > 1 ? hist_slot(p, st, s.t - 2)[2 * (size_t)p.npad + x] : 0.f;
-        hist_push(p, st, s.t, x, Pm, hm, mu, mu2);
+        const size_t np = p.npad;
+        const float* old = hist_slot(p, st, s.t + kHist - 2);
+        const float mu = hm / Pm, mu2 = s.t > 1 ? old[2 * np + x] : 0.f;
+        hist_push(p, st, s.t, x, Pm, hm, mu, mu2, old[3 * np + x]);
         o.dmu = fabsf(mu - mu2);
         o.mu = fabsf(mu);
         if (Pm != cur[x]) p.ctrl->p_changed = 1;
@@ -1459,7 +1499,7 @@ __global__ void __launch_bounds__(256)
             NodeOut o{0.0, 0.f, 0.f};
             if (x < p.n) {
                 float sv[2], cv[2];
-                slot_sums<2>(p, x, 0, 1, sum_p(rs), sum_h(rs), sv, cv);
+                slot_sums<2>(p, x, 0, 1, rs, sv, cv);
                 o = stage_node(p, st, x, rs, (double)sv[0] + (double)cv[0], (double)sv[1] + (double)cv[1]);
             }
             note_block(p.ctrl, rs, o, lane);
@@ -1472,7 +1512,7 @@ __global__ void __launch_bounds__(256)
         const RoundState rs = round_state(p, ctrl);
         const int x = nb.y * 32 + lane, n = p.n;
         float sv[2] = {0.f, 0.f}, cv[2] = {0.f, 0.f};
-        if (x < n) slot_sums<2>(p, x, g, 8, sum_p(rs), sum_h(rs), sv, cv);
+        if (x < n) slot_sums<2>(p, x, g, 8, rs, sv, cv);
         __syncthreads();   // red[] of the previous node block is consumed
         red[0][g][lane] = sv[0]; red[1][g][lane] = cv[0];
         red[2][g][lane] = sv[1]; red[3][g][lane] = cv[1];

@@ -25,8 +25,8 @@
 //
 // Bound: Q streamed once a round (4 or 2 B a pair), or the Q epilogue of the
 // recomputing kernel.  Measured, a frozen round's sweep: n = 20000, FP32 Q 823
-// us with stored messages (28 B a pair), 140 us here (118 us for 4 B a pair at the
-// copy bandwidth); n = 100000, BF16 Q and messages 10.6 ms and 1.99 ms.
+// us with stored messages (28 B a pair), 123 us here (118 us for 4 B a pair at the
+// copy bandwidth); n = 100000, BF16 Q and messages 10.6 ms and 1.60 ms (1.47).
 #include "common.cuh"
 #include "hist.cuh"
 #include "ptx.cuh"
@@ -47,8 +47,12 @@ constexpr int H_GROUP = 64;                    // rows per row-sum reduction (fo
 // What a tile sums beside q mu.  Live P: q^2 (round 0, and where nothing else
 // counts), with q^3, or everything; frozen P: nothing, q^3, or q^3 and q^5.
 enum { K_LIVE0, K_LIVE1, K_LIVE, K_SUM, K_ONE, K_TWO };
-// The sums, as rows of HTail::rs and cs.
+// The sums of a wide tile, as rows of HTail::rs and cs; a small tile (sum_tile)
+// has three at most, q mu, then mu of the stage or q^2, then q^3, and takes
+// rows 0-2 and 3-5 in turn.
 enum { S_R, S_M, S_2, S_4, S_6, S_W3, S_W5, S_COUNT };
+constexpr int S_SMALL = 3;
+__device__ __forceinline__ bool is_wide(int kind) { return kind == K_LIVE || kind == K_TWO; }
 // The node values, as rows of HTail::node: mean of the residual, the stage's
 // mean (staged), and hnow's three.
 enum { N_MU0, N_MU, N_R, N_W3, N_W5, N_COUNT };
@@ -328,7 +332,7 @@ __device__ __forceinline__ void walk_tile(SRC& src, HTail& sm, const HInfo& ti, 
 
 // q mu, with q^2 (PTWO: live P) and q^3 (ONE) beside it.
 template <bool PTWO, bool ONE, bool STAGED, class SRC>
-__device__ __forceinline__ void sum_tile(SRC& src, HTail& sm, const HInfo& ti, int slot, int cw, int lane)
+__device__ __forceinline__ void sum_tile(SRC& src, HTail& sm, const HInfo& ti, int slot, int base, int cw, int lane)
 {
     const int hl = lane & 15;
     const float (*R)[T] = sm.node[slot][0];
@@ -373,16 +377,16 @@ __device__ __forceinline__ void sum_tile(SRC& src, HTail& sm, const HInfo& ti, i
         if (ONE) xE[step] = sE.x + sE.y;
     };
     auto group = [&](int r0) {
-        put_rows(sm.rs[S_R], xR, r0, cw, lane);
-        if (STAGED) put_rows(sm.rs[S_M], xM, r0, cw, lane);
-        if (PTWO) put_rows(sm.rs[S_2], xP, r0, cw, lane);
-        if (ONE) put_rows(sm.rs[S_W3], xE, r0, cw, lane);
+        put_rows(sm.rs[base], xR, r0, cw, lane);
+        if (STAGED) put_rows(sm.rs[base + 1], xM, r0, cw, lane);
+        if (PTWO) put_rows(sm.rs[base + 1], xP, r0, cw, lane);
+        if (ONE) put_rows(sm.rs[base + 2], xE, r0, cw, lane);
     };
     walk_tile(src, sm, ti, cw, lane, row, group);
-    put_cols(sm.cs[S_R][cw], aR, lane);
-    if (STAGED) put_cols(sm.cs[S_M][cw], aM, lane);
-    if (PTWO) put_cols(sm.cs[S_2][cw], aP, lane);
-    if (ONE) put_cols(sm.cs[S_W3][cw], aE, lane);
+    put_cols(sm.cs[base][cw], aR, lane);
+    if (STAGED) put_cols(sm.cs[base + 1][cw], aM, lane);
+    if (PTWO) put_cols(sm.cs[base + 1][cw], aP, lane);
+    if (ONE) put_cols(sm.cs[base + 2][cw], aE, lane);
 }
 
 __device__ __forceinline__ void ld_cols4(const float* d, int lane, float2 (&v)[2])
@@ -463,35 +467,58 @@ __device__ __forceinline__ void wide_tile(SRC& src, HTail& sm, const HInfo& ti, 
             *reinterpret_cast<float4*>(&sm.cs[s][cw][4 * lane]) = make_float4(a[s][0].x, a[s][0].y, a[s][1].x, a[s][1].y);
 }
 
+// Sum k of the thread's node: its row's (threads 0-127) and / or the eight
+// warps' column sums (threads 128-255, and on a diagonal tile both).
+__device__ __forceinline__ float node_sum(const HTail& sm, int k, int tid, int rows, bool diag)
+{
+    const int c = tid & (T - 1);
+    float v = (tid < T && c < rows) ? sm.rs[k][c] : 0.f;
+    if (tid >= T || diag) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < HCW; ++w) s += sm.cs[k][w][c];
+        v += s;
+    }
+    return v;
+}
+
 // The eight consumer warps: tile after tile as the producer publishes them,
-// each tile's sums to its slots in a fixed order.
+// each tile's sums to its slots in a fixed order.  One barrier a tile: a warp
+// that has put its sums away waits for the next tile to be published, and the
+// barrier then both completes the sums and makes the outcome of that wait (go
+// on, end, give up) common.  Small tiles alternate between two sets of sums; a
+// wide tile takes more.  (With two barriers a tile and every sum's code passed
+// through by every tile: 144 us against 123 us a round at n = 20000.)
 template <class SRC>
 __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* __restrict__ tab,
                                                const int4* __restrict__ work, long long ntiles, int tid)
 {
     const int cw = tid >> 5, lane = tid & 31;
-    int slot = 0;
+    int slot = 0, base = 0;
     uint32_t tph = 0;
-    for (;;) {
+    auto await_tile = [&]() {
         if (!mbar_wait_warp(&sm.tfull[slot], tph) && lane == 0) {
             sm.cabort = 1;
             if (blockIdx.x < ntiles) record_error(tab[work[blockIdx.x].x].ctrl, ST_ETIMEOUT, -1);
         }
-        hbar();   // also: the previous tile's sums are read out
+    };
+    await_tile();
+    hbar();
+    for (;;) {
         if (*(volatile int*)&sm.cabort) break;
         if (sm.info[slot].end) break;
         const HInfo& ti = sm.info[slot];
         const int kind = ti.kind, rows = ti.rows;
-        const bool diag = ti.I == ti.J, staged = ti.staged, live = kind <= K_LIVE, even = ti.even, first = ti.t == 0;
+        const bool diag = ti.I == ti.J, staged = ti.staged, wide = is_wide(kind), live = kind <= K_LIVE, even = ti.even;
         float* part = ti.part;
         const long long plen = ti.plen;
         // this thread's node of the tile's sums: row block's for the first 128
         // threads, column block's for the others; its values of round t - 1
         const int c = tid & (T - 1);
         const size_t o = (size_t)(tid < T ? ti.sR : ti.sC) * T + c;
-        float* s46 = ti.s46 + o;
+        float* s46 = nullptr;
         float mu1 = 0.f, r1 = 0.f, D1 = 0.f, D3 = 0.f, S4 = 0.f, S6 = 0.f, P = 0.f;
-        if (!first && (staged || kind != K_SUM)) {
+        if (ti.t > 0 && (staged || kind != K_SUM)) {
             const size_t np = ti.npad;
             const float* node = ti.ring + (size_t)(tid < T ? ti.I : ti.J) * T + c;
             const float* old = node + ((unsigned)(ti.t - 1) % (unsigned)kHist) * 4 * np;
@@ -499,6 +526,7 @@ __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* 
             if (kind != K_SUM) {
                 r1 = 1.f / old[0];
                 if (even) {
+                    s46 = ti.s46 + o;
                     D1 = old[3 * np];
                     D3 = node[((unsigned)(ti.t + kHist - 3) % (unsigned)kHist) * 4 * np + 3 * np];
                     if (!live) { S4 = s46[0]; S6 = s46[plen]; }
@@ -506,52 +534,67 @@ __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* 
             }
             if (!live && staged) P = part[o];
         }
-        if (staged) {
-            if (kind == K_SUM) sum_tile<false, false, true>(src, sm, ti, slot, cw, lane);
-            else if (kind == K_ONE) sum_tile<false, true, true>(src, sm, ti, slot, cw, lane);
-            else if (kind == K_LIVE) wide_tile<true, true>(src, sm, ti, slot, cw, lane);
-            else wide_tile<false, true>(src, sm, ti, slot, cw, lane);
+        if (kind == K_SUM) {
+            if (staged) sum_tile<false, false, true>(src, sm, ti, slot, base, cw, lane);
+            else sum_tile<false, false, false>(src, sm, ti, slot, base, cw, lane);
+        } else if (kind == K_ONE) {
+            if (staged) sum_tile<false, true, true>(src, sm, ti, slot, base, cw, lane);
+            else sum_tile<false, true, false>(src, sm, ti, slot, base, cw, lane);
+        } else if (kind == K_LIVE0) {
+            sum_tile<true, false, false>(src, sm, ti, slot, base, cw, lane);
+        } else if (kind == K_LIVE1) {
+            sum_tile<true, true, false>(src, sm, ti, slot, base, cw, lane);
         } else {
-            if (kind == K_SUM) sum_tile<false, false, false>(src, sm, ti, slot, cw, lane);
-            else if (kind == K_ONE) sum_tile<false, true, false>(src, sm, ti, slot, cw, lane);
-            else if (kind == K_LIVE0) sum_tile<true, false, false>(src, sm, ti, slot, cw, lane);
-            else if (kind == K_LIVE1) sum_tile<true, true, false>(src, sm, ti, slot, cw, lane);
+            hbar();   // the previous tile's sums are read out
+            if (kind == K_LIVE && staged) wide_tile<true, true>(src, sm, ti, slot, cw, lane);
             else if (kind == K_LIVE) wide_tile<true, false>(src, sm, ti, slot, cw, lane);
+            else if (staged) wide_tile<false, true>(src, sm, ti, slot, cw, lane);
             else wide_tile<false, false>(src, sm, ti, slot, cw, lane);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.tempty[slot]);   // its parameters are not read again
         if (++slot == 2) { slot = 0; tph ^= 1u; }
+        await_tile();
         hbar();
-        // the node's sums; the column sums over the eight warps, both roles on a
-        // diagonal tile.  (Slot entries of nodes beyond n are written, and read
-        // by no one else.)
-        const bool all = kind == K_LIVE, odd = kind != K_SUM && kind != K_LIVE0;
-        const bool has[S_COUNT] = {true, staged, live, all, all, odd, all || kind == K_TWO};
-        float v[S_COUNT];
-#pragma unroll
-        for (int a = 0; a < S_COUNT; ++a) {
-            v[a] = 0.f;
-            if (!has[a]) continue;
-            if (tid < T && c < rows) v[a] = sm.rs[a][c];
-            if (tid >= T || diag) {
-                float s = 0.f;
-#pragma unroll
-                for (int w = 0; w < HCW; ++w) s += sm.cs[a][w][c];
-                v[a] += s;
+        // (slot entries of nodes beyond n are written, and read by no one else)
+        const bool mine = tid < T || !diag;
+        float* d = part + o;
+        if (!wide) {
+            const float R = node_sum(sm, base, tid, rows, diag);
+            if (mine) d[2 * plen] = R;
+            if (kind != K_SUM || staged) {
+                // q mu of the stage or q^2; q^3
+                const float v1 = (staged || live) ? node_sum(sm, base + 1, tid, rows, diag) : 0.f;
+                const float v2 = (kind == K_ONE || kind == K_LIVE1) ? node_sum(sm, base + 2, tid, rows, diag) : 0.f;
+                const float E = r1 * (fmaf(S4, D1, v2) + r1 * S6 * (D3 - 3.f * D1));
+                if (mine) {
+                    if (live) d[0] = -v1;
+                    if (staged) d[plen] = fmaf(P, mu1, E - v1);
+                    else if (kind != K_LIVE0) d[plen] = E;
+                }
             }
+        } else {
+            const float R = node_sum(sm, S_R, tid, rows, diag);
+            const float M = staged ? node_sum(sm, S_M, tid, rows, diag) : 0.f;
+            if (live) {
+                const float S2 = node_sum(sm, S_2, tid, rows, diag);
+                if (even && s46) {
+                    S4 = node_sum(sm, S_4, tid, rows, diag);
+                    S6 = node_sum(sm, S_6, tid, rows, diag);
+                }
+                P = fmaf(r1, fmaf(-2.f * r1, S6, S4), -S2);
+            }
+            const float W3 = node_sum(sm, S_W3, tid, rows, diag), W5 = node_sum(sm, S_W5, tid, rows, diag);
+            const float E = r1 * (fmaf(S4, D1, W3) + r1 * fmaf(S6, D3 - 3.f * D1, W5));
+            if (mine) {
+                d[2 * plen] = R;
+                if (live) d[0] = P;
+                if (live && s46) { s46[0] = S4; s46[plen] = S6; }
+                d[plen] = staged ? fmaf(P, mu1, E - M) : E;
+            }
+            hbar();   // before the next tile writes its sums
         }
-        if (tid < T || !diag) {
-            if (all && even) { S4 = v[S_4]; S6 = v[S_6]; }
-            if (live) P = fmaf(r1, fmaf(-2.f * r1, S6, S4), -v[S_2]);
-            const float E = r1 * (fmaf(S4, D1, v[S_W3]) + r1 * fmaf(S6, D3 - 3.f * D1, v[S_W5]));
-            float* d = part + o;
-            if (live) d[0] = P;
-            if (all && even) { s46[0] = S4; s46[plen] = S6; }
-            if (staged) d[plen] = fmaf(P, mu1, E - v[S_M]);
-            else if (odd) d[plen] = E;
-            d[2 * plen] = v[S_R];
-        }
+        base = S_SMALL - base;
     }
 }
 
