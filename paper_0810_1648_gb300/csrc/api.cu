@@ -46,6 +46,9 @@ gabp_status fail(gabp_status st, const char* fmt, ...)
     } while (0)
 
 constexpr int kRhistCap = 1 << 16;
+// A handle keeps its decision workspace for the next call up to this size
+// (allocating it on each call took longer than a small decision).
+constexpr size_t kDecisionKeep = (size_t)64 << 20;
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -135,6 +138,8 @@ struct gabp_svm_s {
     float* alpha = nullptr;
     double* final3 = nullptr;
     double* blockbuf = nullptr;
+    void* dws = nullptr;            // workspace of decisions, kept up to kDecisionKeep bytes
+    size_t dws_bytes = 0;
     Ctrl* hctrl = nullptr;          // pinned mirror of the control block
     double* hfinal = nullptr;       // pinned {rinf, objective, nsv}
     struct Graph {
@@ -511,6 +516,7 @@ void destroy_all(gabp_svm_t h)
     clear_graphs(h);
     if (h->pool) cudaFree(h->pool);
     if (h->spool) cudaFree(h->spool);
+    if (h->dws) cudaFree(h->dws);
     if (h->hctrl) cudaFreeHost(h->hctrl);
     if (h->hfinal) cudaFreeHost(h->hfinal);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -1017,59 +1023,70 @@ gabp_status gabp_svm_decision(gabp_svm_t h, const void* Xtest, int64_t t, float*
     const bool dev = h->opts.ptr_mode == 1;
     const int xd = h->opts.x_dtype;
     const int64_t m = h->m;
-    const int Ntt = (int)((t + T - 1) / T);
-    const long long ntl = (long long)Ntt * h->Nt;
-    const size_t bx = align_up((size_t)t * m * sizeof(float), 256), bsq = align_up((size_t)t * 4, 256);
-    const size_t bin = (!dev && xd != 0) ? align_up((size_t)t * m * x_elem_bytes(xd), 256) : 0;
-    const size_t bpart = align_up((size_t)h->Nt * t * sizeof(float), 256);
-    const size_t bw = align_up((size_t)ntl * sizeof(int2), 256), bout = align_up((size_t)t * 4, 256);
-    char* tmp = nullptr;
-    CK(cudaMallocAsync((void**)&tmp, bx + bsq + bin + bpart + bw + bout, s));
-    float* Xt = (float*)tmp;
-    float* sqt = (float*)(tmp + bx);
-    void* in = tmp + bx + bsq;
-    float* part = (float*)(tmp + bx + bsq + bin);
-    int2* w = (int2*)(tmp + bx + bsq + bin + bpart);
-    float* dout = (float*)(tmp + bx + bsq + bin + bpart + bw);
-    std::vector<int2> wl((size_t)ntl);
-    size_t k = 0;
-    for (int I = 0; I < Ntt; ++I)
-        for (int J = 0; J < h->Nt; ++J) wl[k++] = make_int2(I, J);
-    gabp_status st = GABP_OK;
+    // The test rows go through in slabs (so that the workspace stays bounded),
+    // their planes packed and checked in one pass over the caller's rows.
+    const int64_t slab = std::min<int64_t>(t, (int64_t)1 << 17);
+    const int Ntt = (int)((slab + T - 1) / T);
+    const int per = decision_splits(1, INT_MAX) + Ntt;   // entries of a slab: at most 2 * SMs + its tiles
+    const size_t bxp = align_up(pack3_bytes(Ntt, (int)m), 1024), bsq = align_up((size_t)Ntt * T * 4, 256);
+    const size_t bin = dev ? 0 : align_up((size_t)slab * m * x_elem_bytes(xd), 256);
+    const size_t bpart = align_up((size_t)per * T * sizeof(float), 256), bw = align_up((size_t)per * sizeof(int4), 256);
+    const size_t bdiag = align_up((size_t)Ntt * sizeof(int4), 256), bout = dev ? 0 : align_up((size_t)slab * 4, 256);
+    const size_t btab = align_up(2 * sizeof(Inst), 256), bctrl = align_up(sizeof(Ctrl), 256);
+    const size_t need = bxp + bsq + bin + bpart + bw + bdiag + bout + btab + bctrl;
+    if (need > h->dws_bytes) {
+        if (h->dws) CK(cudaFreeAsync(h->dws, s));
+        h->dws = nullptr;
+        h->dws_bytes = 0;
+        CK(cudaMallocAsync(&h->dws, need, s));
+        h->dws_bytes = need;
+    }
+    char* b = static_cast<char*>(h->dws);
+    auto take = [&](size_t bytes) { char* r = b; b += bytes; return r; };
+    Inst two[2] = {Inst{}, h->inst};
+    Inst& te = two[0];
+    te.m = (int)m;
+    te.nkc = h->inst.nkc;
+    te.Xp3 = take(bxp);
+    te.sq3 = (float*)take(bsq);
+    void* in = take(bin);
+    float* part = (float*)take(bpart);
+    int4* w = (int4*)take(bw);
+    int4* diag = (int4*)take(bdiag);
+    float* dout = (float*)take(bout);
+    Inst* tab = (Inst*)take(btab);
+    te.ctrl = (Ctrl*)take(bctrl);
     auto run = [&]() -> gabp_status {
-        CK(cudaMemcpyAsync(w, wl.data(), wl.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
-        const void* src = Xtest;
-        if (!dev) {
-            if (xd != 0) {
-                CK(cudaMemcpyAsync(in, Xtest, (size_t)t * m * x_elem_bytes(xd), cudaMemcpyHostToDevice, s));
-                src = in;
-            } else {
-                CK(cudaMemcpyAsync(Xt, Xtest, (size_t)t * m * sizeof(float), cudaMemcpyHostToDevice, s));
-                src = Xt;
+        CK(cudaMemsetAsync(te.ctrl, 0, sizeof(Ctrl), s));
+        for (int64_t r0 = 0; r0 < t; r0 += slab) {
+            const int tc = (int)std::min<int64_t>(slab, t - r0);
+            te.n = tc;
+            te.Nt = (tc + T - 1) / T;
+            CK(cudaMemcpyAsync(tab, two, sizeof two, cudaMemcpyHostToDevice, s));
+            const char* src = (const char*)Xtest + (size_t)r0 * m * x_elem_bytes(xd);
+            if (!dev) {
+                CK(cudaMemcpyAsync(in, src, (size_t)tc * m * x_elem_bytes(xd), cudaMemcpyHostToDevice, s));
+                src = (const char*)in;
             }
+            CK(launch_pack3_rows(src, xd, tc, (int)m, te.Nt, (void*)te.Xp3, r0, te.ctrl, diag, s));
+            CK(launch_decision_tc(tab, diag, w, tc, h->Nt, h->alpha, part, te.ctrl, dev ? out + r0 : dout, s));
+            h->prof.kernel_launches += 5;
+            if (!dev) CK(cudaMemcpyAsync(out + r0, dout, (size_t)tc * sizeof(float), cudaMemcpyDeviceToHost, s));
         }
-        CK(cudaMemcpyAsync(h->hctrl, h->inst.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(h->hctrl, te.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        const int saved_status = h->hctrl->status;
-        launch_stage(src, xd, (int)t, (int)m, nullptr, Xt, sqt, nullptr, nullptr, 0, h->inst.ctrl, s);
-        h->prof.kernel_launches += 1;
-        CK(cudaMemcpyAsync(h->hctrl, h->inst.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        if (h->hctrl->status != saved_status) {
-            CK(cudaMemsetAsync(&h->inst.ctrl->status, 0, sizeof(int), s));
-            CK(cudaStreamSynchronize(s));
+        if (h->hctrl->status == ST_EINVAL)
             return fail(GABP_EINVAL, "test row %lld: non-finite feature", h->hctrl->bad_index);
-        }
-        launch_decision(h->inst, Xt, sqt, (int)t, h->alpha, w, ntl, part, dev ? out : dout, s);
-        h->prof.kernel_launches += 2;
-        CK(cudaGetLastError());
-        if (!dev) CK(cudaMemcpyAsync(out, dout, (size_t)t * sizeof(float), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
+        if (h->hctrl->status != 0) return fail(GABP_ETIMEOUT, "a bounded device wait ran out in the decision");
         return GABP_OK;
     };
-    st = run();
-    cudaFreeAsync(tmp, s);
-    cudaStreamSynchronize(s);
+    gabp_status st = run();
+    if (h->dws_bytes > kDecisionKeep) {
+        cudaFreeAsync(h->dws, s);
+        h->dws = nullptr;
+        h->dws_bytes = 0;
+        cudaStreamSynchronize(s);
+    }
     return st;
 }
 
@@ -1105,7 +1122,7 @@ gabp_status gabp_svm_get_stats(gabp_svm_t h, gabp_svm_stats* st)
     h->stats.gamma = h->gamma;
     h->stats.C = h->C;
     h->stats.diag_delta = h->delta;
-    h->stats.device_bytes = (int64_t)(h->pool_bytes + h->spool_bytes);
+    h->stats.device_bytes = (int64_t)(h->pool_bytes + h->spool_bytes + h->dws_bytes);
     h->stats.q_mode = h->opts.q_mode;
     h->stats.diag_rule = h->opts.diag_rule;
     *st = h->stats;

@@ -311,6 +311,9 @@ inline void launch_form_norms(const Inst* tab, const int4* diag_work, long long 
 // The three BF16 planes of FP32 rows (zero padding to whole tiles and chunks).
 cudaError_t launch_pack3(const float* Xf, int n, int m, int Nt, void* Xp3, cudaStream_t s);
 cudaError_t launch_pack3_list(const Inst* tab, const int2* nbl, int nblocks, cudaStream_t s);
+// The planes of a caller's rows, checked, and their diagonal tile list (k_pack3_rows).
+cudaError_t launch_pack3_rows(const void* X, int x_dtype, int n, int m, int Nt, void* Xp3, long long row0, Ctrl* check,
+                              int4* diag, cudaStream_t s);
 size_t pack3_bytes(int Nt, int m);
 // Precision form: BF16 operand packing + norms, and the tensor-core Q formation (BF16 store).
 cudaError_t launch_pack_bf16(const float* Xf, int n, int m, int nkc, int Nt, void* Xp, float* sqb, cudaStream_t s);
@@ -375,9 +378,17 @@ cudaError_t launch_pack_list(const Inst* tab, const int2* nbl, int nblocks, cuda
 void launch_init_list(const Inst* tab, const int2* nbl, int nblocks, int diag_rule, float delta, cudaStream_t s);
 // Arms listed instances: list entries {slot, iters} with their tolerances.
 void launch_begin_list(Inst* tab, const int2* list, const double* tols, int count, cudaStream_t s);
-// Decision values for t test rows (Xt FP32, sqt norms) using alpha.
-void launch_decision(const Inst& p, const float* Xt, const float* sqt, int t, const float* alpha,
-                     const int2* work, long long ntiles, float* part, float* out, cudaStream_t s);
+// q mu and q alpha slot sums (part[2], part[3]) of the listed tiles, Q from the
+// FP32-accurate Gram (forms that do not store it).
+cudaError_t launch_final_tiles_gram(const Inst* tab, const StopOp* ops, const int4* tiles, long long ntiles, cudaStream_t s);
+// Decision values of t test rows using alpha: tab = {the test rows as an
+// instance (n = t, Xp3 packed, sq3 to fill), the training instance}, diag = {0,
+// I, I, I} for its tiles; every test tile is summed in decision_splits(Ntt, Nt)
+// ranges of the training tiles, work and part hold so many entries (x T) per
+// test tile.  out is written unless check->status is set.
+int decision_splits(int Ntt, int Nt);
+cudaError_t launch_decision_tc(const Inst* tab, const int4* diag, int4* work, int t, int Nt, const float* alpha, float* part,
+                               const Ctrl* check, float* out, cudaStream_t s);
 // Gather helpers for inspection.
 void launch_get_q(const Inst& p, const int4* work, long long ntiles, int q_bf16, float* Qdense,
                   cudaStream_t s);

@@ -1,10 +1,8 @@
-// SIMT FP32 Gram tiles fused with the RBF kernel, and everything built on them:
-//   - input staging (FP64 -> FP32, row norms, label/finiteness checks),
-//   - the final residual r = 1 - Q mu and Q alpha for the dual objective
-//     (Q read back from the FP32 tiles, or recomputed here when not stored),
-//   - the decision values f(x) = sum_i alpha_i y_i (K(x_i, x) + lambda^2)
-//     (Section 1.1).
-// (The stored Q tiles themselves are formed on the tensor cores: gram_tc32.cu.)
+// Input staging (FP64 -> FP32, label / finiteness checks), the final residual r
+// = 1 - Q mu and Q alpha for the dual objective from stored FP32 tiles, and SIMT
+// FP32 Gram tiles fused with the RBF kernel for the decision values of callers
+// without a handle (gabp_decision_noalloc).  (Q tiles, decisions of a handle and
+// final passes without stored tiles run on the tensor cores: gram_tc32.cu.)
 //
 // One CTA computes one 128 x 128 Gram tile G = X_I X_J^T by SIMT FP32 FMAs
 // (8 x 8 outputs per thread, K-chunks of 16 double-buffered in shared memory),
@@ -236,21 +234,17 @@ __global__ void k_stage_list(const Inst* __restrict__ tab, const int2* __restric
 //
 // Per listed tile: partial sums of (Q mu)_i and (Q alpha)_i over the tile's
 // pairs (both roles) into the slot partials, with alpha = clip(mu, 0, C) and
-// mu = ops[k].mu.  acc holds the tile's stored FP32 Q values (STORED) or its
-// FP32 Gram values, from which Q is formed exactly as at formation, so both
-// give the same values.
-template <bool STORED>
+// mu = ops[k].mu, from the tile's stored FP32 Q values in acc (instances that do
+// not store Q: gram_tc32.cu).
 __device__ __forceinline__ void final_tile_sums(const Inst& p, const float* __restrict__ mu, int4 w,
                                                 float (&acc)[8][8], EpiSmem& es)
 {
     const int n = p.n, I = w.y, J = w.z;
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    float yj[8], sj[8], mj[8], aj[8];
+    float mj[8], aj[8];
 #pragma unroll
     for (int b = 0; b < 8; ++b) {
         const int j = J * T + tx * 8 + b;
-        yj[b] = j < n ? p.y[j] : 0.f;
-        sj[b] = j < n ? p.sq[j] : 0.f;
         mj[b] = j < n ? mu[j] : 0.f;
         aj[b] = p.task ? mj[b] : fminf(fmaxf(mj[b], 0.f), p.C);
     }
@@ -260,16 +254,13 @@ __device__ __forceinline__ void final_tile_sums(const Inst& p, const float* __re
 #pragma unroll
     for (int a = 0; a < 8; ++a) {
         const int r = ty * 8 + a, i = I * T + r;
-        const float yi = i < n ? p.y[i] : 0.f, si = i < n ? p.sq[i] : 0.f;
         const float mi = i < n ? mu[i] : 0.f, ai = p.task ? mi : fminf(fmaxf(mi, 0.f), p.C);
         float rm = 0.f, ra = 0.f;
 #pragma unroll
         for (int b = 0; b < 8; ++b) {
             const int c = tx * 8 + b, j = J * T + c;
             const bool v = i < n && j < n && (I != J || c > r);
-            const float q0 =
-                STORED ? acc[a][b] : yi * yj[b] * (rbf_from_gram(acc[a][b], si, sj[b], p.gamma) + p.lam2);
-            const float q = v ? q0 : 0.f;
+            const float q = v ? acc[a][b] : 0.f;
             rm = fmaf(q, mj[b], rm);
             ra = fmaf(q, aj[b], ra);
             cs[0][b] = fmaf(q, mi, cs[0][b]);
@@ -280,22 +271,6 @@ __device__ __forceinline__ void final_tile_sums(const Inst& p, const float* __re
     }
     float* const parts[2] = {p.part + 2 * part_len(p), p.part + 3 * part_len(p)};
     reduce_and_write<2>(es, rs, cs, parts, n, I, J, tile_slots(p, w));
-}
-
-// Q recomputed by the FP32 Gram (forms without an FP32 store).  One CTA per
-// listed tile.
-__global__ void __launch_bounds__(NTHREADS) k_final_tiles(const Inst* __restrict__ tab,
-                                                          const StopOp* __restrict__ ops,
-                                                          const int4* __restrict__ work)
-{
-    __shared__ __align__(16) TileSmem sm;
-    const int4 w = work[blockIdx.x];
-    const Inst& p = tab[w.x];
-    float acc[8][8];
-    const GramSide S{p.X, p.sq, p.n};
-    gram_tile(S, S, p.m, w.y, w.z, sm.g, acc);
-    __syncthreads();   // Gram smem is reused by the epilogue
-    final_tile_sums<false>(p, ops[w.x].mu, w, acc, sm.e);
 }
 
 // Q read back from the FP32 tiles (Inst::qref): no Gram, small footprint, so
@@ -317,7 +292,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_final_tiles_q(const Inst* __res
         acc[a][0] = u0.x; acc[a][1] = u0.y; acc[a][2] = u0.z; acc[a][3] = u0.w;
         acc[a][4] = u1.x; acc[a][5] = u1.y; acc[a][6] = u1.z; acc[a][7] = u1.w;
     }
-    final_tile_sums<true>(p, ops[w.x].mu, w, acc, es);
+    final_tile_sums(p, ops[w.x].mu, w, acc, es);
 }
 
 // k_pair_z (sweep_hist.cu) for instances that do not store Q (only those that
@@ -465,49 +440,6 @@ __global__ void k_final_reduce(const Inst* __restrict__ tab, const StopOp* __res
 }
 
 // ----------------------------------------------------------------- decision
-// Rectangle of tiles (test tile I, training tile J): part[J][s] =
-// sum_{j in J} alpha_j y_j (K(x_j, xt_s) + lambda^2).
-__global__ void __launch_bounds__(NTHREADS) k_decision_tiles(Inst p, const float* __restrict__ Xt,
-                                                             const float* __restrict__ sqt, int t,
-                                                             const float* __restrict__ alpha,
-                                                             const int2* __restrict__ work,
-                                                             float* __restrict__ part)
-{
-    __shared__ __align__(16) TileSmem sm;
-    const long long L = blockIdx.x;
-    const int I = work[L].x, J = work[L].y, n = p.n;
-    const GramSide A{Xt, sqt, t}, B{p.X, p.sq, n};
-    float acc[8][8];
-    gram_tile(A, B, p.m, I, J, sm.g, acc);
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    float wj[8], sj[8];
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const int j = J * T + tx * 8 + b;
-        wj[b] = j < n ? alpha[j] * p.y[j] : 0.f;
-        sj[b] = j < n ? p.sq[j] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-        const int r = ty * 8 + a, s = I * T + r;
-        const float si = s < t ? sqt[s] : 0.f;
-        float f = 0.f;
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            const float kv = rbf_from_gram(acc[a][b], si, sj[b], p.gamma) + p.lam2;
-            f = fmaf(wj[b], kv, f);
-        }
-        f = sum16(f);
-        if (tx == 0) sm.e.rowv[0][r] = f;
-    }
-    __syncthreads();
-    if (tid < T) {
-        const int s = I * T + tid;
-        if (s < t) part[(size_t)J * t + s] = sm.e.rowv[0][tid];
-    }
-}
-
 __global__ void k_decision_sum(const float* __restrict__ part, int t, int Ntrain_tiles, float* __restrict__ out)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -564,17 +496,10 @@ void launch_final(const Inst* tab, const StopOp* ops, const int4* tiles, long lo
         if (q_stored)
             k_final_tiles_q<<<(unsigned)ntiles, NTHREADS, 0, s>>>(tab, ops, tiles);
         else
-            k_final_tiles<<<(unsigned)ntiles, NTHREADS, 0, s>>>(tab, ops, tiles);
+            (void)launch_final_tiles_gram(tab, ops, tiles, ntiles, s);   // errors surface at the caller's cudaGetLastError
     }
     if (nblocks > 0) k_final_nodes<<<nblocks, 256, 0, s>>>(tab, ops, nbl);
     if (nmembers > 0) k_final_reduce<<<nmembers, 256, 0, s>>>(tab, ops, members, f3_all);
-}
-
-void launch_decision(const Inst& p, const float* Xt, const float* sqt, int t, const float* alpha,
-                     const int2* work, long long ntiles, float* part, float* out, cudaStream_t s)
-{
-    k_decision_tiles<<<(unsigned)ntiles, NTHREADS, 0, s>>>(p, Xt, sqt, t, alpha, work, part);
-    k_decision_sum<<<(t + 255) / 256, 256, 0, s>>>(part, t, p.Nt, out);
 }
 
 void launch_get_q(const Inst& p, const int4* work, long long ntiles, int q_bf16, float* Qdense,

@@ -19,18 +19,26 @@
 // large, the norms and the Gram value then carry the same truncation, which
 // cancels in d^2 instead of shrinking every K by ~2 gamma ||x||^2 x 1e-8.
 //
-// k_form_q_tc32 is persistent with warp roles: warp 0 streams the six 16 KB
-// operand blocks of each (tile, chunk) into a two-stage shared-memory ring;
-// warp 1 allocates 512 TMEM columns (four 128 x 128 FP32 accumulators, one per
-// K-step) and one thread issues the 24 MMAs of a chunk (6 products x K = 64
-// in steps of 16); warps 2-9 (two per TMEM lane quarter, one per column half)
-// add each chunk's accumulators into registers, then form the Q entries
-// (norm expansion, clamp, expf, bias, labels), store them, and reduce |Q| over
-// rows (four interleaved partial sums), over columns
-// (a warp transpose-sum, then the four lane quarters in shared memory) and to
-// the tile maximum.  Instances chained behind the listed one (the points of a
-// parameter grid over the same features) take their Q tiles from the same
-// Gram sums.
+// k_gram_tc32 is persistent with warp roles: warp 0 streams the operand blocks
+// of each (tile, chunk), two copies of three planes, into a two-stage
+// shared-memory ring; warp 1 allocates 512 TMEM columns (four 128 x 128 FP32
+// accumulators, one per K-step) and one thread issues the 24 MMAs of a chunk (6
+// products x K = 64 in steps of 16); warps 2-17 (four per TMEM lane quarter, one
+// per 32 columns) add each chunk's accumulators into registers and run the
+// epilogue of the mode:
+//   formation   Q entries (norm expansion, clamp, expf, bias, labels), stored in
+//               32-byte pieces, and |Q| over rows (four interleaved partial
+//               sums), over columns (a warp transpose-sum, then the four lane
+//               quarters in shared memory) and the tile maximum.  Instances
+//               chained behind the listed one (the points of a parameter grid
+//               over the same features) take their Q tiles from the same Gram
+//               sums;
+//   final pass  the same entries, not stored, times the means and the weights
+//               (instances that recompute Q);
+//   decision    entries of test rows against training rows, times the weights,
+//               summed over a range of training tiles in registers.
+// Bound by the epilogue: with eight epilogue warps (64 columns each, all four
+// accumulators handed over at once) two warps a scheduler left it waiting.
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -41,7 +49,7 @@ namespace gabp {
 namespace {
 
 constexpr int NPLANE = 3;
-constexpr int T3_EPI_WARPS = 8;
+constexpr int T3_EPI_WARPS = 16;                     // four per TMEM lane quarter, one per 32 columns
 constexpr int T3_THREADS = (2 + T3_EPI_WARPS) * 32;
 constexpr int T3_STAGES = 2;
 constexpr size_t T3_STAGE_BYTES = (size_t)2 * NPLANE * BLK_BYTES;   // A planes, then B planes: 96 KB
@@ -52,12 +60,12 @@ constexpr size_t T3_STAGE_BYTES = (size_t)2 * NPLANE * BLK_BYTES;   // A planes,
 // nearest).  Measured against the FP64 oracle (n = 2048, with the norms from
 // the same products): mean relative error of K -2e-8 with four accumulators
 // against +1.2e-6 with one (clustered data, gamma ||x||^2 ~ 24), +1.2e-7
-// against +2.6e-7 (m = 128); formation 1.01 against 0.83 ms at n = 20000,
-// m = 128.  With four, TMEM holds one chunk at a time.
-constexpr int T3_NACC = 4;
-static_assert(T3_NACC == 1 || T3_NACC == 2 || T3_NACC == 4, "1, 2 or 4 accumulators per chunk");
-constexpr int T3_NBUF = T3_NACC == 4 ? 1 : 2;
-constexpr uint32_t T3_TMEM_COLS = (uint32_t)(T3_NACC * T3_NBUF * T <= 256 ? 256 : 512);
+// against +2.6e-7 (m = 128).  Each accumulator is handed over by itself, so the
+// MMAs of the next chunk's first K-step run while the epilogue still reads the
+// last ones.
+constexpr int T3_NACC = KCH / 16;
+constexpr uint32_t T3_TMEM_COLS = T3_NACC * T;
+static_assert(T3_TMEM_COLS == 512, "all of TMEM");
 constexpr uint32_t T3_IDESC = idesc_bf16_f32(T, T);
 constexpr int T3_PRODUCTS = 6;
 
@@ -111,6 +119,39 @@ __global__ void k_pack3(const float* __restrict__ Xf, int n, int m, int nkc, int
     pack3_group(Xf, n, m, nkc, (int)(e / groups), (int)(e % groups), Xp3);
 }
 
+// The planes of a caller's rows (FP32, FP64 or BF16: x_dtype), every feature
+// checked to be finite (check->status, bad_index = the first found row + row0),
+// and the diagonal tile list of the rows.
+template <class XT>
+__global__ void k_pack3_rows(const XT* __restrict__ X, int n, int m, int nkc, int Nt, uint4* __restrict__ Xp3,
+                             long long row0, Ctrl* __restrict__ check, int4* __restrict__ diag)
+{
+    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long groups = (long long)nkc * (KCH / 8);
+    if (e < Nt) diag[e] = make_int4(0, (int)e, (int)e, (int)e);
+    if (e >= (long long)Nt * T * groups) return;
+    const int r = (int)(e / groups), gk = (int)(e % groups);
+    const int kc = gk / (KCH / 8), kg = gk % (KCH / 8);
+    __align__(16) __nv_bfloat16 v[NPLANE][8];
+    bool ok = true;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int k = kc * KCH + kg * 8 + u;
+        float x = 0.f;
+        if (r < n && k < m) {
+            x = (float)X[(size_t)r * m + k];
+            ok &= isfinite(x);
+        }
+        split3(x, v[0][u], v[1][u], v[2][u]);
+    }
+    if (!ok && atomicCAS(&check->status, 0, (int)ST_EINVAL) == 0) check->bad_index = row0 + r;
+#pragma unroll
+    for (int pl = 0; pl < NPLANE; ++pl) {
+        const size_t blk = ((size_t)(r / T) * nkc + kc) * NPLANE + pl;
+        Xp3[blk * (BLK_BYTES / 16) + core_off16(r % T, kg)] = *reinterpret_cast<const uint4*>(v[pl]);
+    }
+}
+
 // Listed node blocks (32 rows, 8 threads a row); the last block of an
 // instance also writes the zero rows that pad its last tile.
 __global__ void k_pack3_list(const Inst* __restrict__ tab, const int2* __restrict__ nbl)
@@ -128,17 +169,26 @@ __global__ void k_pack3_list(const Inst* __restrict__ tab, const int2* __restric
     }
 }
 
+// What the epilogue makes of the Gram tiles.
+enum T3Mode {
+    T3_FORM,     // Q tiles, |Q| sums (and, norms_only, the squared norms)
+    T3_FINAL,    // sums q mu and q alpha of a tile's pairs, Q not stored
+    T3_DECIDE    // decision values: rows = test rows, sums over the training columns
+};
+
 struct T3Smem {
     unsigned long long xfull[T3_STAGES], xempty[T3_STAGES];
-    unsigned long long accfull[T3_NBUF], accempty[T3_NBUF];
+    unsigned long long accfull[T3_NACC], accempty[T3_NACC];
     unsigned long long drain;
     uint32_t tmem_base;
     int abort;
-    float colsum[4][T];                 // per lane quarter: column sums over its 32 rows
-    float rowsum[2][T];                 // per column half: row sums
+    float colsum[2][4][T];              // per lane quarter: column sums over its 32 rows
+    float rowsum[2][4][T];              // per 32-column group: row sums
     float tmx[T3_EPI_WARPS];
-    alignas(16) uint32_t cy[T3_EPI_WARPS][64];   // a warp's 64 columns: sign bits of the labels
-    alignas(16) float cs[T3_EPI_WARPS][64];   // and FP32 norms
+    alignas(16) uint32_t cy[T3_EPI_WARPS][32];   // a warp's 32 columns: sign bits of the labels (decision: weights)
+    alignas(16) float cs[T3_EPI_WARPS][32];      // FP32 norms
+    alignas(16) float cm[T3_EPI_WARPS][32];      // final pass: means
+    alignas(16) float ca[T3_EPI_WARPS][32];      // and weights alpha
 };
 
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(T3_EPI_WARPS * 32) : "memory"); }
@@ -193,17 +243,37 @@ __device__ __forceinline__ void q_chunk32(const float* g, const uint32_t* sy, co
     }
 }
 
+// 32 consecutive floats of a row, eight per store (a whole 32-byte sector).
+__device__ __forceinline__ void store_row32(float* d, const float (&q)[32])
+{
+#pragma unroll
+    for (int c = 0; c < 32; c += 8)
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d + c), "f"(q[c]), "f"(q[c + 1]),
+                     "f"(q[c + 2]), "f"(q[c + 3]), "f"(q[c + 4]), "f"(q[c + 5]), "f"(q[c + 6]), "f"(q[c + 7])
+                     : "memory");
+}
+
+// The decision's operands: tab[0] describes the test rows as an instance (n,
+// Nt, nkc, Xp3, sq3), tab[1] is the training set; a work entry {0, I, J0, J1}
+// sums test tile I over the training tiles [J0, J1).
+struct DecideArgs {
+    const float* alpha;
+    float* part;      // [entries][T]
+};
+
+template <int MODE>
 __global__ void __launch_bounds__(T3_THREADS, 1)
-    k_form_q_tc32(const Inst* __restrict__ tab, const int4* __restrict__ work, long long ntiles, int norms_only)
+    k_gram_tc32(const Inst* __restrict__ tab, const int4* __restrict__ work, long long ntiles, int norms_only,
+                const StopOp* __restrict__ ops, DecideArgs dec)
 {
     extern __shared__ unsigned char smem_raw[];
-    unsigned char* ops = align_smem(smem_raw, 1024);
-    T3Smem& sm = *reinterpret_cast<T3Smem*>(ops + T3_STAGES * T3_STAGE_BYTES);
+    unsigned char* oper = align_smem(smem_raw, 1024);
+    T3Smem& sm = *reinterpret_cast<T3Smem*>(oper + T3_STAGES * T3_STAGE_BYTES);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
         for (int s = 0; s < T3_STAGES; ++s) { mbar_init(&sm.xfull[s], 1); mbar_init(&sm.xempty[s], 1); }
-        for (int b = 0; b < T3_NBUF; ++b) { mbar_init(&sm.accfull[b], 1); mbar_init(&sm.accempty[b], T3_EPI_WARPS); }
+        for (int a = 0; a < T3_NACC; ++a) { mbar_init(&sm.accfull[a], 1); mbar_init(&sm.accempty[a], T3_EPI_WARPS); }
         mbar_init(&sm.drain, 1);
         sm.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -213,79 +283,76 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = sm.tmem_base;
+    // (a decision's work entry covers several tiles)
+    auto first_j = [&](int4 w) { return w.z; };
+    auto last_j = [&](int4 w) { return MODE == T3_DECIDE ? w.w : w.z + 1; };
 
     if (warp == 0) {
         // ------------------------------------------------ operand producer
         if (lane == 0) {
-            const uint64_t pol = l2_evict_first_policy();
+            const uint64_t pol = l2_evict_last_policy();   // the planes are read again by many tiles
             int stage = 0;
             uint32_t ph = 0;
             bool run = true;
             for (long long L = blockIdx.x; L < ntiles && run; L += gridDim.x) {
                 const int4 w = work[L];
                 const Inst& p = tab[w.x];
-                const unsigned char* Xp3 = static_cast<const unsigned char*>(p.Xp3);
-                const int I = w.y, J = w.z, nkc = p.nkc;
-                for (int kc = 0; kc < nkc; ++kc) {
-                    if (*(volatile int*)&sm.abort || !mbar_wait(&sm.xempty[stage], ph ^ 1u)) {
-                        sm.abort = 1;
-                        record_error(p.ctrl, ST_ETIMEOUT, L);
-                        run = false;
-                        break;
+                const unsigned char* A3 = static_cast<const unsigned char*>(p.Xp3);
+                const unsigned char* B3 = MODE == T3_DECIDE ? static_cast<const unsigned char*>(tab[1].Xp3) : A3;
+                const int I = w.y, nkc = p.nkc;
+                for (int J = first_j(w); J < last_j(w) && run; ++J)
+                    for (int kc = 0; kc < nkc; ++kc) {
+                        if (*(volatile int*)&sm.abort || !mbar_wait(&sm.xempty[stage], ph ^ 1u)) {
+                            sm.abort = 1;
+                            record_error(p.ctrl, ST_ETIMEOUT, L);
+                            run = false;
+                            break;
+                        }
+                        unsigned char* S = oper + (size_t)stage * T3_STAGE_BYTES;
+                        mbar_arrive_expect_tx(&sm.xfull[stage], (uint32_t)T3_STAGE_BYTES);
+                        // a block's three planes lie behind one another
+                        bulk_load(S, A3 + ((size_t)I * nkc + kc) * NPLANE * BLK_BYTES, NPLANE * BLK_BYTES, &sm.xfull[stage], pol);
+                        bulk_load(S + (size_t)NPLANE * BLK_BYTES, B3 + ((size_t)J * nkc + kc) * NPLANE * BLK_BYTES,
+                                  NPLANE * BLK_BYTES, &sm.xfull[stage], pol);
+                        if (++stage == T3_STAGES) { stage = 0; ph ^= 1u; }
                     }
-                    unsigned char* S = ops + (size_t)stage * T3_STAGE_BYTES;
-                    mbar_arrive_expect_tx(&sm.xfull[stage], (uint32_t)T3_STAGE_BYTES);
-#pragma unroll
-                    for (int pl = 0; pl < NPLANE; ++pl) {
-                        bulk_load(S + (size_t)pl * BLK_BYTES, Xp3 + (((size_t)I * nkc + kc) * NPLANE + pl) * BLK_BYTES,
-                                  BLK_BYTES, &sm.xfull[stage], pol);
-                        bulk_load(S + (size_t)(NPLANE + pl) * BLK_BYTES,
-                                  Xp3 + (((size_t)J * nkc + kc) * NPLANE + pl) * BLK_BYTES, BLK_BYTES, &sm.xfull[stage],
-                                  pol);
-                    }
-                    if (++stage == T3_STAGES) { stage = 0; ph ^= 1u; }
-                }
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            int stage = 0, acc = 0;
+            int stage = 0;
             uint32_t ph = 0, aph = 0;
             bool run = true;
             for (long long L = blockIdx.x; L < ntiles && run; L += gridDim.x) {
-                const Inst& p = tab[work[L].x];
+                const int4 w = work[L];
+                const Inst& p = tab[w.x];
                 Ctrl* ctrl = p.ctrl;
-                const int nkc = p.nkc;
-                for (int kc = 0; kc < nkc; ++kc) {
-                    if (*(volatile int*)&sm.abort || !mbar_wait(&sm.accempty[acc], aph ^ 1u) ||
-                        !mbar_wait(&sm.xfull[stage], ph)) {
-                        sm.abort = 1;
-                        record_error(ctrl, ST_ETIMEOUT, L);
-                        run = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const unsigned char* S = ops + (size_t)stage * T3_STAGE_BYTES;
-                    constexpr int SPA = (KCH / 16) / T3_NACC;   // K-steps per accumulator
+                const int chunks = p.nkc * (last_j(w) - first_j(w));
+                for (int kc = 0; kc < chunks && run; ++kc) {
+                    if (*(volatile int*)&sm.abort || !mbar_wait(&sm.xfull[stage], ph)) run = false;
+                    const unsigned char* S = oper + (size_t)stage * T3_STAGE_BYTES;
 #pragma unroll
                     for (int a = 0; a < T3_NACC; ++a) {
-                        const uint32_t d = tbase + (uint32_t)(acc * T3_NACC + a) * T;
+                        if (run && !mbar_wait(&sm.accempty[a], aph ^ 1u)) run = false;
+                        if (!run) break;
+                        tc_fence_after();
+                        const uint32_t d = tbase + (uint32_t)a * T;
 #pragma unroll
-                        for (int q = 0; q < T3_PRODUCTS; ++q) {
-#pragma unroll
-                            for (int s = a * SPA; s < (a + 1) * SPA; ++s) {
-                                const uint64_t ad = smem_desc(S + (size_t)prod_a(q) * BLK_BYTES + s * 256, 128, 1024);
-                                const uint64_t bd =
-                                    smem_desc(S + (size_t)(NPLANE + prod_b(q)) * BLK_BYTES + s * 256, 128, 1024);
-                                tc_mma_bf16(d, ad, bd, T3_IDESC, (q != 0 || s != a * SPA) ? 1u : 0u);
-                            }
-                        }
+                        for (int q = 0; q < T3_PRODUCTS; ++q)
+                            tc_mma_bf16(d, smem_desc(S + (size_t)prod_a(q) * BLK_BYTES + a * 256, 128, 1024),
+                                        smem_desc(S + (size_t)(NPLANE + prod_b(q)) * BLK_BYTES + a * 256, 128, 1024), T3_IDESC,
+                                        q != 0 ? 1u : 0u);
+                        tc_commit(&sm.accfull[a]);
+                    }
+                    if (!run) {
+                        sm.abort = 1;
+                        record_error(ctrl, ST_ETIMEOUT, L);
+                        break;
                     }
                     tc_commit(&sm.xempty[stage]);
-                    tc_commit(&sm.accfull[acc]);
                     if (++stage == T3_STAGES) { stage = 0; ph ^= 1u; }
-                    if (++acc == T3_NBUF) { acc = 0; aph ^= 1u; }
+                    aph ^= 1u;
                 }
             }
             // every MMA issued above must finish before the columns are freed
@@ -295,158 +362,207 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
     } else {
         // --------------------------------------------------------- epilogue
         // warp w reads TMEM lanes 32 (w % 4) ..: rows 32 g + lane, columns
-        // [64 half, 64 half + 64)
-        const int ew = warp - 2, g = warp & 3, half = ew >> 2;
-        const int r = 32 * g + lane, c0 = 64 * half;
+        // [32 cg, 32 cg + 32)
+        const int ew = warp - 2, g = warp & 3, cg = ew >> 2;
+        const int r = 32 * g + lane, c0 = 32 * cg;
         const int etid = tid - 64;
-        int acc = 0;
         uint32_t aph = 0;
         for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
             const int4 w = work[L];
-            const int nkc = tab[w.x].nkc;
-            float ga[64];
-#pragma unroll
-            for (int c = 0; c < 64; ++c) ga[c] = 0.f;
+            const int nkc = tab[w.x].nkc, I = w.y, i = I * T + r;
+            float fs = 0.f, fc = 0.f;   // decision: the row's compensated sum over its training tiles
             bool ok = true;
-            for (int kc = 0; kc < nkc; ++kc) {
-                const bool stop = __shfl_sync(0xffffffffu, *(volatile int*)&sm.abort, 0) != 0;
-                if (stop || !mbar_wait_warp(&sm.accfull[acc], aph)) {
-                    ok = false;
-                    break;
+            for (int J = first_j(w); J < last_j(w) && ok; ++J) {
+                if (MODE == T3_DECIDE) {
+                    const Inst& tr = tab[1];
+                    const int j = J * T + c0 + lane;
+                    __syncwarp();   // the previous tile's values are read
+                    sm.cy[ew][lane] = j < tr.n ? __float_as_uint(dec.alpha[j] * tr.y[j]) : 0u;
+                    sm.cs[ew][lane] = j < tr.n ? tr.sq3[j] : 0.f;
+                    __syncwarp();
                 }
-                tc_fence_after();
-                // the chunk's accumulators added to the running sums in order,
-                // 16 columns at a time
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                float ga[32];
+                for (int kc = 0; kc < nkc; ++kc) {
+                    const bool stop = __shfl_sync(0xffffffffu, *(volatile int*)&sm.abort, 0) != 0;
+                    // the chunk's accumulators added to the running sums in order
 #pragma unroll
                     for (int a = 0; a < T3_NACC; ++a) {
-                        float v[16];
-                        tmem_ld16(tbase + (uint32_t)(acc * T3_NACC + a) * T + ((uint32_t)(32 * g) << 16) +
-                                      (uint32_t)(c0 + 16 * j),
-                                  v);
+                        if (stop || !ok || !mbar_wait_warp(&sm.accfull[a], aph)) { ok = false; break; }
+                        tc_fence_after();
+                        float v[32];
+                        tmem_ld32(tbase + (uint32_t)a * T + ((uint32_t)(32 * g) << 16) + (uint32_t)c0, v);
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&sm.accempty[a]);
                         if (kc == 0 && a == 0) {
 #pragma unroll
-                            for (int c = 0; c < 16; ++c) ga[16 * j + c] = v[c];
+                            for (int c = 0; c < 32; ++c) ga[c] = v[c];
                         } else {
                             // two columns per instruction, each rounded as a scalar add
 #pragma unroll
-                            for (int c = 0; c < 16; c += 2) {
-                                const float2 t2 = __fadd2_rn(make_float2(ga[16 * j + c], ga[16 * j + c + 1]),
-                                                             make_float2(v[c], v[c + 1]));
-                                ga[16 * j + c] = t2.x;
-                                ga[16 * j + c + 1] = t2.y;
+                            for (int c = 0; c < 32; c += 2) {
+                                const float2 t2 = __fadd2_rn(make_float2(ga[c], ga[c + 1]), make_float2(v[c], v[c + 1]));
+                                ga[c] = t2.x;
+                                ga[c + 1] = t2.y;
                             }
                         }
                     }
+                    if (!ok) break;
+                    aph ^= 1u;
                 }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm.accempty[acc]);
-                if (++acc == T3_NBUF) { acc = 0; aph ^= 1u; }
-            }
-            if (!ok && lane == 0) {
-                sm.abort = 1;
-                record_error(tab[w.x].ctrl, ST_ETIMEOUT, L);
-            }
-            epi_bar();   // every epilogue warp takes the stop decision together
-            if (*(volatile int*)&sm.abort) break;
-            const int I = w.y, J = w.z;
-            const int i = I * T + r;
-            if (norms_only) {
-                // diagonal tile: x_i . x_i is the Gram value at (r, r), held by the
-                // warp of r's lane quarter whose column half contains r
-                if (half == (g >> 1)) {
-                    float d = 0.f;
+                if (MODE == T3_DECIDE) {
+                    if (!ok) break;
+                    const Inst& tr = tab[1];
+                    const float si = i < tab[0].n ? tab[0].sq3[i] : 0.f, ngam = -tr.gamma, lam2 = tr.lam2;
+                    float f[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                    for (int c = 0; c < 64; ++c) d = (c0 + c == r) ? ga[c] : d;
-                    for (int k = w.x; k >= 0; k = tab[k].form_next - 1)
-                        if (i < tab[k].n) tab[k].sq3[i] = d;
+                    for (int c4 = 0; c4 < 32; c4 += 4) {
+                        const float4 w4 = *reinterpret_cast<const float4*>(&sm.cy[ew][c4]);
+                        const float4 s4 = *reinterpret_cast<const float4*>(&sm.cs[ew][c4]);
+                        const float wj[4] = {w4.x, w4.y, w4.z, w4.w}, sj[4] = {s4.x, s4.y, s4.z, s4.w};
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) {
+                            const float d2 = fmaxf(0.f, si + sj[t] - 2.f * ga[c4 + t]);
+                            f[t] = fmaf(wj[t], expf(ngam * d2) + lam2, f[t]);
+                        }
+                    }
+                    // TwoSum, as the finalize's slot sums
+                    const float x = (f[0] + f[1]) + (f[2] + f[3]), t = fs + x, bp = t - fs;
+                    fc += (fs - (t - bp)) + (x - bp);
+                    fs = t;
+                    continue;
                 }
-                continue;
-            }
-            for (int k = w.x; k >= 0;) {
-                const Inst& p = tab[k];
-                const int n = p.n;
-                // this warp's 64 column labels and norms
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int j = J * T + c0 + 32 * u + lane;
-                    sm.cy[ew][32 * u + lane] = j < n ? (__float_as_uint(p.y[j]) & 0x80000000u) : 0u;
-                    sm.cs[ew][32 * u + lane] = j < n ? p.sq3[j] : 0.f;
+                if (!ok && lane == 0) {
+                    sm.abort = 1;
+                    record_error(tab[w.x].ctrl, ST_ETIMEOUT, L);
                 }
-                __syncwarp();
-                const float si = i < n ? p.sq3[i] : 0.f, ngam = -p.gamma, lam2 = p.lam2;
-                const uint32_t syi = i < n ? (__float_as_uint(p.y[i]) & 0x80000000u) : 0u;
-                // interior tile: every pair valid
-                const bool full = I != J && (I + 1) * T <= n && (J + 1) * T <= n;
-                float* qt = p.qref ? p.qref + (size_t)w.w * TT + (size_t)r * T + c0 : nullptr;
-                float rs4[4] = {0.f, 0.f, 0.f, 0.f}, tmx = 0.f;   // row sum in four interleaved parts
+                epi_bar();   // every epilogue warp takes the stop decision together
+                if (*(volatile int*)&sm.abort) { ok = false; break; }
+                if (MODE == T3_FORM && norms_only) {
+                    // diagonal tile: x_i . x_i is the Gram value at (r, r), held by the
+                    // warp of r's lane quarter whose columns contain r
+                    if (cg == g) {
+                        float d = 0.f;
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
+                        for (int c = 0; c < 32; ++c) d = c == lane ? ga[c] : d;
+                        for (int k = w.x; k >= 0; k = tab[k].form_next - 1)
+                            if (i < tab[k].n) tab[k].sq3[i] = d;
+                    }
+                    continue;
+                }
+                for (int k = w.x; k >= 0;) {
+                    const Inst& p = tab[k];
+                    const int n = p.n, j = J * T + c0 + lane;
+                    // this warp's 32 column labels and norms
+                    sm.cy[ew][lane] = j < n ? (__float_as_uint(p.y[j]) & 0x80000000u) : 0u;
+                    sm.cs[ew][lane] = j < n ? p.sq3[j] : 0.f;
+                    float mi = 0.f, ai = 0.f;
+                    if (MODE == T3_FINAL) {
+                        const float* mu = ops[k].mu;
+                        const float mj = j < n ? mu[j] : 0.f;
+                        sm.cm[ew][lane] = mj;
+                        sm.ca[ew][lane] = p.task ? mj : fminf(fmaxf(mj, 0.f), p.C);
+                        mi = i < n ? mu[i] : 0.f;
+                        ai = p.task ? mi : fminf(fmaxf(mi, 0.f), p.C);
+                    }
+                    __syncwarp();
+                    const float si = i < n ? p.sq3[i] : 0.f, ngam = -p.gamma, lam2 = p.lam2;
+                    const uint32_t syi = i < n ? (__float_as_uint(p.y[i]) & 0x80000000u) : 0u;
+                    // interior tile: every pair valid
+                    const bool full = I != J && (I + 1) * T <= n && (J + 1) * T <= n;
+                    float rs4[4] = {0.f, 0.f, 0.f, 0.f};   // row sum in four interleaved parts
                     float q[32];
                     if (full)
-                        q_chunk32<true>(ga + 32 * u, sm.cy[ew] + 32 * u, sm.cs[ew] + 32 * u, si, syi, ngam, lam2,
-                                        0, 0, 0, 0, 0, q, rs4);
+                        q_chunk32<true>(ga, sm.cy[ew], sm.cs[ew], si, syi, ngam, lam2, 0, 0, 0, 0, 0, q, rs4);
                     else
-                        q_chunk32<false>(ga + 32 * u, sm.cy[ew] + 32 * u, sm.cs[ew] + 32 * u, si, syi, ngam, lam2,
-                                         i, n, c0 + 32 * u, J * T, I == J ? r : -1, q, rs4);
-                    if (p.tilemax) {
+                        q_chunk32<false>(ga, sm.cy[ew], sm.cs[ew], si, syi, ngam, lam2, i, n, c0, J * T, I == J ? r : -1, q, rs4);
+                    constexpr int NSUM = MODE == T3_FINAL ? 2 : 1;
+                    if (MODE == T3_FORM) {
+                        if (p.tilemax) {
+                            float tmx = 0.f;
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) tmx = fmaxf(tmx, fabsf(q[c]));
-                    }
-                    if (qt) {
+                            for (int c = 0; c < 32; ++c) tmx = fmaxf(tmx, fabsf(q[c]));
+                            tmx = warp_max_f(tmx);
+                            if (lane == 0) sm.tmx[ew] = tmx;
+                        }
+                        if (p.qref) store_row32(p.qref + (size_t)w.w * TT + (size_t)r * T + c0, q);
 #pragma unroll
-                        for (int c4 = 0; c4 < 32; c4 += 4)
-                            *reinterpret_cast<float4*>(qt + 32 * u + c4) = make_float4(q[c4], q[c4 + 1], q[c4 + 2], q[c4 + 3]);
-                    }
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) q[c] = fabsf(q[c]);
-                    sm.colsum[g][c0 + 32 * u + lane] = transpose_sum32(q, lane);
-                }
-                sm.rowsum[half][r] = (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
-                tmx = warp_max_f(tmx);
-                if (lane == 0) sm.tmx[ew] = tmx;
-                epi_bar();
-                // per-node slot partials (fixed order): row sums of the tile's rows,
-                // column sums of its columns; both roles on a diagonal tile
-                // (slot sl.x of the row block, sl.y of the column block).  Where
-                // rfix is set they are added to the nodes' fixed-point sums instead.
-                int x = -1, off = 0, role = 0;
-                float v = 0.f;
-                if (I == J) {
-                    if (etid < T) {
-                        x = I * T + etid;
-                        off = etid;
-                        v = (sm.rowsum[0][etid] + sm.rowsum[1][etid]) +
-                            (((sm.colsum[0][etid] + sm.colsum[1][etid]) + sm.colsum[2][etid]) + sm.colsum[3][etid]);
-                    }
-                } else if (etid < T) {
-                    x = I * T + etid;
-                    off = etid;
-                    v = sm.rowsum[0][etid] + sm.rowsum[1][etid];
-                } else if (etid < 2 * T) {
-                    off = etid - T;
-                    x = J * T + off;
-                    role = 1;
-                    v = ((sm.colsum[0][off] + sm.colsum[1][off]) + sm.colsum[2][off]) + sm.colsum[3][off];
-                }
-                if (x >= 0 && x < n) {
-                    if (p.rfix) {
-                        atomicAdd(p.rfix + x, (unsigned long long)rsum_fix(v, pow2i(rsum_shift(n, lam2))));
+                        for (int c = 0; c < 32; ++c) q[c] = fabsf(q[c]);
+                        sm.colsum[0][g][c0 + lane] = transpose_sum32(q, lane);
+                        sm.rowsum[0][cg][r] = (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
                     } else {
-                        const int2 sl = tile_slots(p, w);
-                        p.part[(size_t)(role ? sl.y : sl.x) * T + off] = v;
+                        // sums of q mu and q alpha: the row's over the columns, the columns' over the rows
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) {
+                            const float xi = s ? ai : mi;
+                            float f[4] = {0.f, 0.f, 0.f, 0.f}, v[32];
+#pragma unroll
+                            for (int c4 = 0; c4 < 32; c4 += 4) {
+                                const float4 x4 = *reinterpret_cast<const float4*>(s ? &sm.ca[ew][c4] : &sm.cm[ew][c4]);
+                                const float xj[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+                                for (int t = 0; t < 4; ++t) {
+                                    f[t] = fmaf(q[c4 + t], xj[t], f[t]);
+                                    v[c4 + t] = q[c4 + t] * xi;
+                                }
+                            }
+                            sm.rowsum[s][cg][r] = (f[0] + f[1]) + (f[2] + f[3]);
+                            sm.colsum[s][g][c0 + lane] = transpose_sum32(v, lane);
+                        }
                     }
+                    epi_bar();
+                    // per-node slot partials (fixed order): row sums of the tile's rows,
+                    // column sums of its columns; both roles on a diagonal tile
+                    // (slot sl.x of the row block, sl.y of the column block).  Where
+                    // rfix is set they are added to the nodes' fixed-point sums instead.
+                    if (etid < 2 * T) {
+                        const int off = etid & (T - 1), role = etid / T;
+                        const int x = (role ? J : I) * T + off;
+                        if (x < n && !(I == J && role)) {
+#pragma unroll
+                            for (int s = 0; s < NSUM; ++s) {
+                                const float (*rw)[T] = sm.rowsum[s];
+                                const float (*cl)[T] = sm.colsum[s];
+                                const float vr = (rw[0][off] + rw[1][off]) + (rw[2][off] + rw[3][off]);
+                                const float vc = ((cl[0][off] + cl[1][off]) + cl[2][off]) + cl[3][off];
+                                const float v = I == J ? vr + vc : role ? vc : vr;
+                                if (MODE == T3_FORM && p.rfix) {
+                                    atomicAdd(p.rfix + x, (unsigned long long)rsum_fix(v, pow2i(rsum_shift(n, lam2))));
+                                } else {
+                                    const int2 sl = tile_slots(p, w);
+                                    // final pass: the residual slots and the spare ones
+                                    float* dst = p.part + (MODE == T3_FINAL ? (2 + s) * part_len(p) : 0);
+                                    dst[(size_t)(role ? sl.y : sl.x) * T + off] = v;
+                                }
+                            }
+                        }
+                    }
+                    if (MODE == T3_FORM && etid == 0 && p.tilemax) {
+                        float m2 = 0.f;
+                        for (int e = 0; e < T3_EPI_WARPS; ++e) m2 = fmaxf(m2, sm.tmx[e]);
+                        p.tilemax[w.w] = m2;
+                    }
+                    epi_bar();   // shared sums read before the next instance or tile writes them
+                    k = MODE == T3_FORM ? p.form_next - 1 : -1;
                 }
-                if (etid == 0 && p.tilemax) {
-                    float m2 = 0.f;
-                    for (int e = 0; e < T3_EPI_WARPS; ++e) m2 = fmaxf(m2, sm.tmx[e]);
-                    p.tilemax[w.w] = m2;
-                }
-                epi_bar();   // shared sums read before the next instance or tile writes them
-                k = p.form_next - 1;
             }
+            if (MODE == T3_DECIDE) {
+                if (!ok && lane == 0) {
+                    sm.abort = 1;
+                    record_error(tab[w.x].ctrl, ST_ETIMEOUT, L);
+                }
+                sm.rowsum[0][cg][r] = fs;
+                sm.rowsum[1][cg][r] = fc;
+                epi_bar();
+                if (etid < T) {
+                    double v = 0.0;
+                    for (int c = 0; c < 4; ++c) v += (double)sm.rowsum[0][c][etid] + (double)sm.rowsum[1][c][etid];
+                    dec.part[L * T + etid] = (float)v;
+                }
+                epi_bar();
+                if (*(volatile int*)&sm.abort) break;
+            }
+            if (!ok) break;
         }
     }
     tc_fence_before();
@@ -458,6 +574,42 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
 }
 
 constexpr size_t t3_smem_bytes() { return 1024 + T3_STAGES * T3_STAGE_BYTES + sizeof(T3Smem); }
+
+// The opted-in shared memory, once per kernel and device.
+template <int MODE>
+cudaError_t launch_gram(const Inst* tab, const int4* work, long long ntiles, int norms_only, const StopOp* ops,
+                        const DecideArgs& dec, cudaStream_t s)
+{
+    if (ntiles <= 0) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(k_gram_tc32<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t3_smem_bytes());
+    if (e != cudaSuccess) return e;
+    const int sms = num_sms();
+    k_gram_tc32<MODE><<<(int)(ntiles < sms ? ntiles : sms), T3_THREADS, t3_smem_bytes(), s>>>(tab, work, ntiles, norms_only,
+                                                                                           ops, dec);
+    return cudaGetLastError();
+}
+
+// out[s] of test row s of tile I: its entries' sums in order (FP64), unless a
+// test row was refused.
+__global__ void k_decision_out(const float* __restrict__ part, int t, int per, const Ctrl* __restrict__ check,
+                               float* __restrict__ out)
+{
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= t || check->status != 0) return;
+    const float* p = part + (size_t)(s / T) * per * T + s % T;
+    double f = 0.0;
+    for (int k = 0; k < per; ++k) f += (double)p[(size_t)k * T];
+    out[s] = (float)f;
+}
+// Work entry e = I per + k of a decision: test tile I, the k-th of `per` even
+// ranges of the Nt training tiles.
+__global__ void k_decision_work(int4* __restrict__ work, int Ntt, int Nt, int per)
+{
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= Ntt * per) return;
+    const int k = e % per;
+    work[e] = make_int4(0, e / per, (int)((long long)k * Nt / per), (int)((long long)(k + 1) * Nt / per));
+}
 
 }  // namespace
 
@@ -471,6 +623,21 @@ cudaError_t launch_pack3(const float* Xf, int n, int m, int Nt, void* Xp3, cudaS
     return cudaGetLastError();
 }
 
+cudaError_t launch_pack3_rows(const void* X, int x_dtype, int n, int m, int Nt, void* Xp3, long long row0, Ctrl* check,
+                              int4* diag, cudaStream_t s)
+{
+    const int nkc = bf16_chunks(m);
+    const unsigned grid = (unsigned)(((long long)Nt * T * nkc * (KCH / 8) + 255) / 256);
+    uint4* out = static_cast<uint4*>(Xp3);
+    if (x_dtype == 1)
+        k_pack3_rows<<<grid, 256, 0, s>>>(static_cast<const double*>(X), n, m, nkc, Nt, out, row0, check, diag);
+    else if (x_dtype == 2)
+        k_pack3_rows<<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(X), n, m, nkc, Nt, out, row0, check, diag);
+    else
+        k_pack3_rows<<<grid, 256, 0, s>>>(static_cast<const float*>(X), n, m, nkc, Nt, out, row0, check, diag);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_pack3_list(const Inst* tab, const int2* nbl, int nblocks, cudaStream_t s)
 {
     if (nblocks > 0) k_pack3_list<<<nblocks, 256, 0, s>>>(tab, nbl);
@@ -479,17 +646,30 @@ cudaError_t launch_pack3_list(const Inst* tab, const int2* nbl, int nblocks, cud
 
 cudaError_t launch_form_q_tc32(const Inst* tab, const int4* work, long long ntiles, int norms_only, cudaStream_t s)
 {
-    if (ntiles <= 0) return cudaSuccess;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_form_q_tc32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)t3_smem_bytes());
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    const int sms = num_sms();
-    const int grid = (int)(ntiles < sms ? ntiles : sms);
-    k_form_q_tc32<<<grid, T3_THREADS, t3_smem_bytes(), s>>>(tab, work, ntiles, norms_only);
+    return launch_gram<T3_FORM>(tab, work, ntiles, norms_only, nullptr, DecideArgs{}, s);
+}
+
+cudaError_t launch_final_tiles_gram(const Inst* tab, const StopOp* ops, const int4* tiles, long long ntiles, cudaStream_t s)
+{
+    return launch_gram<T3_FINAL>(tab, tiles, ntiles, 0, ops, DecideArgs{}, s);
+}
+
+int decision_splits(int Ntt, int Nt)
+{
+    const int per = (2 * num_sms() + Ntt - 1) / Ntt;
+    return per < Nt ? per : Nt;
+}
+
+cudaError_t launch_decision_tc(const Inst* tab, const int4* diag, int4* work, int t, int Nt, const float* alpha, float* part,
+                               const Ctrl* check, float* out, cudaStream_t s)
+{
+    const int Ntt = (t + T - 1) / T, per = decision_splits(Ntt, Nt);
+    k_decision_work<<<(Ntt * per + 255) / 256, 256, 0, s>>>(work, Ntt, Nt, per);
+    cudaError_t e = launch_gram<T3_FORM>(tab, diag, Ntt, 1, nullptr, DecideArgs{}, s);   // the test rows' norms
+    if (e != cudaSuccess) return e;
+    e = launch_gram<T3_DECIDE>(tab, work, (long long)Ntt * per, 0, nullptr, DecideArgs{alpha, part}, s);
+    if (e != cudaSuccess) return e;
+    k_decision_out<<<(t + 255) / 256, 256, 0, s>>>(part, t, per, check, out);
     return cudaGetLastError();
 }
 
