@@ -1423,10 +1423,11 @@ __global__ void __launch_bounds__(256, 5)
 
 // Node x's P and residual (when `with_p`) and H slot partials := 0, the sums
 // of all-zero messages: the staged schedule's stage finalize reads the slots
-// of tiles not yet swept in a round, and under the tile-sparse option the
-// slots of dropped tiles are never written by a sweep.
+// of tiles not yet swept in a round.  (A synchronous round writes every slot
+// before it reads one.)
 __device__ __forceinline__ void zero_slots(const Inst& p, int x, bool with_p)
 {
+    if (p.nstages == 1) return;
     const int X = x / T, ns = slot_count(p, X);
     const size_t len = part_len(p);
     float* partP = p.part + (size_t)slot_begin(p, X) * T + (x - X * T);
@@ -1441,17 +1442,26 @@ __device__ __forceinline__ void zero_slots(const Inst& p, int x, bool with_p)
     }
 }
 
-// The whole matrix's sum_{j != i} |Q_ij| of node x: the formation's slot sums
-// (array 0) added in fixed point (rsum_fix), or the first pass's sums of the
-// tile-sparse option (the same value).
-__device__ __forceinline__ double offdiag_abs_sum(const Inst& p, int x)
+// The whole matrix's sum_{j != i} |Q_ij| of the nodes x = 32 block + lane of a
+// CTA of eight warps: the formation's slot sums (array 0) added in fixed point
+// (rsum_fix; each warp every eighth slot, integers, so in any order), or the
+// first pass's sums of the tile-sparse option (the same value).  Warp 0 has the
+// result.
+__device__ __forceinline__ double offdiag_abs_sum(const Inst& p, int x, long long (&red)[8][32])
 {
-    if (p.rsum) return p.rsum[x];
-    const int X = x / T, ns = slot_count(p, X), sh = rsum_shift(p.n, p.lam2);
-    const double scale = pow2i(sh);
-    const float* s0 = p.part + (size_t)slot_begin(p, X) * T + (x - X * T);
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, sh = rsum_shift(p.n, p.lam2);
     long long a = 0;
-    for (int k = 0; k < ns; ++k) a += rsum_fix(s0[(size_t)k * T], scale);
+    if (!p.rsum && x < p.n) {
+        const int X = x / T, ns = slot_count(p, X);
+        const double scale = pow2i(sh);
+        const float* s0 = p.part + (size_t)slot_begin(p, X) * T + (x - X * T);
+#pragma unroll 8
+        for (int k = g; k < ns; k += 8) a += rsum_fix(s0[(size_t)k * T], scale);
+    }
+    red[g][lane] = a;
+    __syncthreads();
+    if (p.rsum) return x < p.n ? p.rsum[x] : 0.0;
+    for (int w = 1; w < 8; ++w) a += g == 0 ? red[w][lane] : 0;
     return rsum_unfix(a, sh);
 }
 
@@ -1619,27 +1629,28 @@ __global__ void k_selftest_rcp(const float* __restrict__ d, float* __restrict__ 
     if (i < cnt) out[i] = rcp_nr(d[i]);
 }
 
-// Row x's diagonal margin Q_xx - R_x into the instance's running
-// max_i 1 / (Q_ii - R_i) (the control block is zeroed before formation):
-// with all margins positive Q is strictly diagonally dominant and Varah's
-// bound ||mu - Q^-1 b||_inf <= ||b - Q mu||_inf / min_i (Q_ii - R_i) holds for
-// any mu; a row without a positive margin records +inf (no bound).  Also the
-// largest 1 / Q_ii.
-__device__ __forceinline__ void note_margin(Ctrl* c, float qd, double R)
+// 1 / (Q_xx - R_x), whose maximum over the rows goes to the control block
+// (zeroed before formation): with all margins positive Q is strictly diagonally
+// dominant and Varah's bound ||mu - Q^-1 b||_inf <= ||b - Q mu||_inf / min_i (Q_ii
+// - R_i) holds for any mu; a row without a positive margin gives +inf (no
+// bound).
+__device__ __forceinline__ double inv_margin(float qd, double R)
 {
     const double mg = (double)qd - R;
-    const double inv = mg > 0.0 ? 1.0 / mg : INFINITY;
-    atomicMax(&c->inv_margin_bits, (unsigned long long)__double_as_longlong(inv));
-    atomicMax(&c->rq_bits, __float_as_uint(1.f / qd));
+    return mg > 0.0 ? 1.0 / mg : INFINITY;
 }
 
 // Diagonal rule (Section 3.1) from the |Q| row-sum partials of the Q
 // formation, then Algorithm 2 Step 1: messages 0, so Ptilde = Q_ii,
-// htilde = b_i, mutilde = b_i / Q_ii.  CTA 0 resets the control block.
-__global__ void k_init(Inst p, int diag_rule, float delta)
+// htilde = b_i, mutilde = b_i / Q_ii.  One CTA of eight warps per 32 nodes
+// (block nb of the instance; one thread a node read its slots one by one, 0.6
+// ms at n = 100000); block 0 resets the control block.
+__device__ __forceinline__ void init_block(const Inst& p, int nb, int diag_rule, float delta)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    __shared__ long long red[8][32];
+    const int tid = threadIdx.x, x = nb * 32 + (tid & 31);
+    const double R = offdiag_abs_sum(p, x, red);
+    if (nb == 0 && tid == 0) {
         Ctrl* c = p.ctrl;
         c->t = 0;
         c->done = 1;
@@ -1652,26 +1663,40 @@ __global__ void k_init(Inst p, int diag_rule, float delta)
         c->tol = 0.0;
         c->rinf = -1.0;
     }
-    if (x >= p.n) {
-        if (x < p.npad) hist_pad(p, x);
-        return;
+    if (tid >= 32) return;
+    if (nb == (p.n - 1) / 32)
+        for (int xp = p.n + tid; xp < p.npad; xp += 32) hist_pad(p, xp);
+    double inv = 0.0;
+    float rq = 0.f;
+    if (x < p.n) {
+        zero_slots(p, x, true);   // all messages start at 0
+        const double lam2 = p.lam2;
+        const double base = 1.0 + lam2 + 1.0 / (double)p.C;
+        double qd = base;
+        if (diag_rule == 0) {
+            const double dom = (1.0 + (double)delta) * R;
+            qd = dom > base ? dom : base;
+        }
+        const float qf = (float)qd, bx = p.b[x];
+        p.qdiag[x] = qf;
+        p.agg[x] = qf;
+        p.agg[p.npad + x] = bx;
+        p.agg[2 * p.npad + x] = bx / qf;
+        hist_start(p, x, qf, bx, bx / qf);
+        inv = inv_margin(qf, R);
+        rq = 1.f / qf;
     }
-    const double R = offdiag_abs_sum(p, x);
-    zero_slots(p, x, true);   // all messages start at 0
-    const double lam2 = p.lam2;
-    const double base = 1.0 + lam2 + 1.0 / (double)p.C;
-    double qd = base;
-    if (diag_rule == 0) {
-        const double dom = (1.0 + (double)delta) * R;
-        qd = dom > base ? dom : base;
+    const unsigned long long ib = warp_max_bits(inv);
+    const unsigned rb = warp_max_bits(rq);
+    if (tid == 0) {
+        atomicMax(&p.ctrl->inv_margin_bits, ib);
+        atomicMax(&p.ctrl->rq_bits, rb);
     }
-    const float qf = (float)qd, bx = p.b[x];
-    p.qdiag[x] = qf;
-    p.agg[x] = qf;
-    p.agg[p.npad + x] = bx;
-    p.agg[2 * p.npad + x] = bx / qf;
-    hist_start(p, x, qf, bx, bx / qf);
-    note_margin(p.ctrl, qf, R);
+}
+
+__global__ void __launch_bounds__(256) k_init(Inst p, int diag_rule, float delta)
+{
+    init_block(p, blockIdx.x, diag_rule, delta);
 }
 
 __global__ void k_row_abs_sums(Inst p, double* __restrict__ rsum)
@@ -1683,44 +1708,12 @@ __global__ void k_row_abs_sums(Inst p, double* __restrict__ rsum)
     }
 }
 
-// k_init over listed node blocks (block 0 of an instance resets its control block).
-__global__ void k_init_list(const Inst* __restrict__ tab, const int2* __restrict__ nbl, int diag_rule, float delta)
+// k_init over listed node blocks.
+__global__ void __launch_bounds__(256) k_init_list(const Inst* __restrict__ tab, const int2* __restrict__ nbl, int diag_rule,
+                                                   float delta)
 {
     const int2 nb = nbl[blockIdx.x];
-    const Inst& p = tab[nb.x];
-    if (nb.y == 0 && threadIdx.x == 0) {
-        Ctrl* c = p.ctrl;
-        c->t = 0;
-        c->done = 1;
-        c->limit = 0;
-        c->kstar = 0;
-        c->converged = 0;
-        c->rmax_bits = 0ull;
-        c->blocks_done = 0u;
-        hist_ctrl_start(c);
-        c->tol = 0.0;
-        c->rinf = -1.0;
-    }
-    const int x = nb.y * 32 + threadIdx.x;
-    if (nb.y == (p.n - 1) / 32)
-        for (int xp = p.n + threadIdx.x; xp < p.npad; xp += blockDim.x) hist_pad(p, xp);
-    if (threadIdx.x >= 32 || x >= p.n) return;
-    const double R = offdiag_abs_sum(p, x);
-    zero_slots(p, x, true);   // all messages start at 0
-    const double lam2 = p.lam2;
-    const double base = 1.0 + lam2 + 1.0 / (double)p.C;
-    double qd = base;
-    if (diag_rule == 0) {
-        const double dom = (1.0 + (double)delta) * R;
-        qd = dom > base ? dom : base;
-    }
-    const float qf = (float)qd, bx = p.b[x];
-    p.qdiag[x] = qf;
-    p.agg[x] = qf;
-    p.agg[p.npad + x] = bx;
-    p.agg[2 * p.npad + x] = bx / qf;
-    hist_start(p, x, qf, bx, bx / qf);
-    note_margin(p.ctrl, qf, R);
+    init_block(tab[nb.x], nb.y, diag_rule, delta);
 }
 
 __global__ void k_begin_list(Inst* tab, const int2* __restrict__ list, const double* __restrict__ tols, int count)
@@ -1842,7 +1835,7 @@ __global__ void k_get_pairs(Inst p, const long long* __restrict__ ij, long long 
 
 void launch_init(const Inst& p, int diag_rule, float delta, cudaStream_t s)
 {
-    k_init<<<(p.n + 255) / 256, 256, 0, s>>>(p, diag_rule, delta);
+    k_init<<<(p.n + 31) / 32, 256, 0, s>>>(p, diag_rule, delta);
 }
 
 void launch_row_abs_sums(const Inst& p, double* rsum, cudaStream_t s)
@@ -1864,7 +1857,7 @@ void launch_axpy_list(const Inst* tab, const StopOp* ops, const int2* nbl, int n
 
 void launch_init_list(const Inst* tab, const int2* nbl, int nblocks, int diag_rule, float delta, cudaStream_t s)
 {
-    if (nblocks > 0) k_init_list<<<nblocks, 32, 0, s>>>(tab, nbl, diag_rule, delta);
+    if (nblocks > 0) k_init_list<<<nblocks, 256, 0, s>>>(tab, nbl, diag_rule, delta);
 }
 
 void launch_begin_list(Inst* tab, const int2* list, const double* tols, int count, cudaStream_t s)
