@@ -176,19 +176,38 @@ enum T3Mode {
     T3_DECIDE    // decision values: rows = test rows, sums over the training columns
 };
 
+// The sums of a tile's epilogue (two in turn).
+struct T3Sums {
+    float col[2][4][T];     // per lane quarter: column sums over its 32 rows
+    float row[2][4][T];     // per 32-column group: row sums
+    float tmx[T3_EPI_WARPS];
+};
+
+// The columns' ([0]) and rows' ([1]) constants of an item (two in turn): label
+// sign, norm and, in the final pass, mean and alpha; in a decision mu[0] holds
+// the columns' weights y alpha.
+struct T3Const {
+    alignas(16) float y[2][T];
+    float sq[2][T];
+    float mu[2][T];
+    float al[2][T];
+};
+
+// 4 bytes to shared memory, asynchronously; zero where !ok (src is then not read).
+__device__ __forceinline__ void copy_word(float* dst, const float* src, int ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                 :: "r"(smem_u32(dst)), "l"(src), "r"(ok ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void copy_words_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 struct T3Smem {
     unsigned long long xfull[T3_STAGES], xempty[T3_STAGES];
     unsigned long long accfull[T3_NACC], accempty[T3_NACC];
     unsigned long long drain;
     uint32_t tmem_base;
     int abort;
-    float colsum[2][4][T];              // per lane quarter: column sums over its 32 rows
-    float rowsum[2][4][T];              // per 32-column group: row sums
-    float tmx[T3_EPI_WARPS];
-    alignas(16) uint32_t cy[T3_EPI_WARPS][32];   // a warp's 32 columns: sign bits of the labels (decision: weights)
-    alignas(16) float cs[T3_EPI_WARPS][32];      // FP32 norms
-    alignas(16) float cm[T3_EPI_WARPS][32];      // final pass: means
-    alignas(16) float ca[T3_EPI_WARPS][32];      // and weights alpha
+    T3Sums sums[2];
+    T3Const cst[2];
 };
 
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(T3_EPI_WARPS * 32) : "memory"); }
@@ -309,8 +328,8 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                             break;
                         }
                         unsigned char* S = oper + (size_t)stage * T3_STAGE_BYTES;
-                        mbar_arrive_expect_tx(&sm.xfull[stage], (uint32_t)T3_STAGE_BYTES);
                         // a block's three planes lie behind one another
+                        mbar_arrive_expect_tx(&sm.xfull[stage], (uint32_t)T3_STAGE_BYTES);
                         bulk_load(S, A3 + ((size_t)I * nkc + kc) * NPLANE * BLK_BYTES, NPLANE * BLK_BYTES, &sm.xfull[stage], pol);
                         bulk_load(S + (size_t)NPLANE * BLK_BYTES, B3 + ((size_t)J * nkc + kc) * NPLANE * BLK_BYTES,
                                   NPLANE * BLK_BYTES, &sm.xfull[stage], pol);
@@ -367,27 +386,65 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
         const int r = 32 * g + lane, c0 = 32 * cg;
         const int etid = tid - 64;
         uint32_t aph = 0;
+        int buf = 0;
+        // The constants of an item (a tile, or one of the instances that share
+        // it) are copied to shared memory while the item before it is computed,
+        // so that neither their latency nor registers for them are in the way:
+        // threads 0..127 take the tile's columns, 128..255 its rows.  fetch()
+        // starts the copies; settle(), before the barrier that ends the current
+        // item, waits for the thread's own and puts them in the form that is used.
+        const int cx = etid & (T - 1), crole = etid / T;
+        const auto fetch = [&](int b, int k, int I, int J) {
+            if (crole >= 2 || (MODE == T3_FORM && norms_only)) return;
+            const Inst& p = MODE == T3_DECIDE && crole == 0 ? tab[1] : tab[k];
+            T3Const& c = sm.cst[b];
+            const int x = (crole ? I : J) * T + cx, ok = x < p.n, xs = ok ? x : 0;
+            if (MODE != T3_DECIDE || crole == 0) copy_word(&c.y[crole][cx], p.y + xs, ok);
+            copy_word(&c.sq[crole][cx], p.sq3 + xs, ok);
+            if (MODE == T3_FINAL) copy_word(&c.mu[crole][cx], ops[k].mu + xs, ok);
+            if (MODE == T3_DECIDE && crole == 0) copy_word(&c.mu[0][cx], dec.alpha + xs, ok);
+        };
+        const auto settle = [&](int b, int k) {
+            if (crole >= 2 || (MODE == T3_FORM && norms_only)) return;
+            copy_words_wait();
+            T3Const& c = sm.cst[b];
+            if (MODE == T3_DECIDE) {
+                if (crole == 0) c.mu[0][cx] *= c.y[0][cx];
+                return;
+            }
+            c.y[crole][cx] = __uint_as_float(__float_as_uint(c.y[crole][cx]) & 0x80000000u);
+            if (MODE == T3_FINAL) {
+                const float m = c.mu[crole][cx];
+                c.al[crole][cx] = tab[k].task ? m : fminf(fmaxf(m, 0.f), tab[k].C);
+            }
+        };
+        int4 wn = blockIdx.x < ntiles ? work[blockIdx.x] : make_int4(0, 0, 0, 0);
+        if (blockIdx.x < ntiles) {
+            fetch(0, wn.x, wn.y, first_j(wn));
+            settle(0, wn.x);
+        }
+        epi_bar();
         for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
-            const int4 w = work[L];
+            const int4 w = wn;
             const int nkc = tab[w.x].nkc, I = w.y, i = I * T + r;
+            const bool more = L + gridDim.x < ntiles;
+            if (more) wn = work[L + gridDim.x];
             float fs = 0.f, fc = 0.f;   // decision: the row's compensated sum over its training tiles
             bool ok = true;
             for (int J = first_j(w); J < last_j(w) && ok; ++J) {
-                if (MODE == T3_DECIDE) {
-                    const Inst& tr = tab[1];
-                    const int j = J * T + c0 + lane;
-                    __syncwarp();   // the previous tile's values are read
-                    sm.cy[ew][lane] = j < tr.n ? __float_as_uint(dec.alpha[j] * tr.y[j]) : 0u;
-                    sm.cs[ew][lane] = j < tr.n ? tr.sq3[j] : 0.f;
-                    __syncwarp();
-                }
+                // the item that follows: an instance sharing the tile, the row's next
+                // training tile, or the next entry
+                int kn = MODE == T3_FORM ? tab[w.x].form_next - 1 : -1, In = I, Jn = J;
+                if (MODE == T3_DECIDE && J + 1 < last_j(w)) { kn = w.x; Jn = J + 1; }
+                if (kn < 0 && more) { kn = wn.x; In = wn.y; Jn = first_j(wn); }
+                if (kn >= 0) fetch(buf ^ 1, kn, In, Jn);
                 float ga[32];
-                for (int kc = 0; kc < nkc; ++kc) {
+                for (int kc = 0; kc < nkc && ok; ++kc) {
                     const bool stop = __shfl_sync(0xffffffffu, *(volatile int*)&sm.abort, 0) != 0;
                     // the chunk's accumulators added to the running sums in order
 #pragma unroll
                     for (int a = 0; a < T3_NACC; ++a) {
-                        if (stop || !ok || !mbar_wait_warp(&sm.accfull[a], aph)) { ok = false; break; }
+                        if (stop || !mbar_wait_warp(&sm.accfull[a], aph)) { ok = false; break; }
                         tc_fence_after();
                         float v[32];
                         tmem_ld32(tbase + (uint32_t)a * T + ((uint32_t)(32 * g) << 16) + (uint32_t)c0, v);
@@ -407,18 +464,20 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                             }
                         }
                     }
-                    if (!ok) break;
                     aph ^= 1u;
                 }
+                if (!ok && lane == 0) {
+                    sm.abort = 1;
+                    record_error(tab[w.x].ctrl, ST_ETIMEOUT, L);
+                }
                 if (MODE == T3_DECIDE) {
-                    if (!ok) break;
-                    const Inst& tr = tab[1];
-                    const float si = i < tab[0].n ? tab[0].sq3[i] : 0.f, ngam = -tr.gamma, lam2 = tr.lam2;
+                    const T3Const& cc = sm.cst[buf];
+                    const float si = cc.sq[1][r], ngam = -tab[1].gamma, lam2 = tab[1].lam2;
                     float f[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                     for (int c4 = 0; c4 < 32; c4 += 4) {
-                        const float4 w4 = *reinterpret_cast<const float4*>(&sm.cy[ew][c4]);
-                        const float4 s4 = *reinterpret_cast<const float4*>(&sm.cs[ew][c4]);
+                        const float4 w4 = *reinterpret_cast<const float4*>(&cc.mu[0][c0 + c4]);
+                        const float4 s4 = *reinterpret_cast<const float4*>(&cc.sq[0][c0 + c4]);
                         const float wj[4] = {w4.x, w4.y, w4.z, w4.w}, sj[4] = {s4.x, s4.y, s4.z, s4.w};
 #pragma unroll
                         for (int t = 0; t < 4; ++t) {
@@ -430,15 +489,16 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                     const float x = (f[0] + f[1]) + (f[2] + f[3]), t = fs + x, bp = t - fs;
                     fc += (fs - (t - bp)) + (x - bp);
                     fs = t;
+                    if (J + 1 < last_j(w)) {
+                        settle(buf ^ 1, kn);
+                        epi_bar();
+                        if (*(volatile int*)&sm.abort) { ok = false; break; }
+                        buf ^= 1;
+                    }
                     continue;
                 }
-                if (!ok && lane == 0) {
-                    sm.abort = 1;
-                    record_error(tab[w.x].ctrl, ST_ETIMEOUT, L);
-                }
-                epi_bar();   // every epilogue warp takes the stop decision together
-                if (*(volatile int*)&sm.abort) { ok = false; break; }
                 if (MODE == T3_FORM && norms_only) {
+                    if (!ok) break;
                     // diagonal tile: x_i . x_i is the Gram value at (r, r), held by the
                     // warp of r's lane quarter whose columns contain r
                     if (cg == g) {
@@ -452,44 +512,39 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                 }
                 for (int k = w.x; k >= 0;) {
                     const Inst& p = tab[k];
-                    const int n = p.n, j = J * T + c0 + lane;
-                    // this warp's 32 column labels and norms
-                    sm.cy[ew][lane] = j < n ? (__float_as_uint(p.y[j]) & 0x80000000u) : 0u;
-                    sm.cs[ew][lane] = j < n ? p.sq3[j] : 0.f;
-                    float mi = 0.f, ai = 0.f;
-                    if (MODE == T3_FINAL) {
-                        const float* mu = ops[k].mu;
-                        const float mj = j < n ? mu[j] : 0.f;
-                        sm.cm[ew][lane] = mj;
-                        sm.ca[ew][lane] = p.task ? mj : fminf(fmaxf(mj, 0.f), p.C);
-                        mi = i < n ? mu[i] : 0.f;
-                        ai = p.task ? mi : fminf(fmaxf(mi, 0.f), p.C);
+                    const int n = p.n, next = MODE == T3_FORM ? p.form_next - 1 : -1;
+                    const T3Const& cc = sm.cst[buf];
+                    const float si = cc.sq[1][r], mi = cc.mu[1][r], ai = cc.al[1][r], ngam = -p.gamma, lam2 = p.lam2;
+                    const uint32_t syi = __float_as_uint(cc.y[1][r]);
+                    const uint32_t* cy = reinterpret_cast<const uint32_t*>(&cc.y[0][c0]);
+                    if (k != w.x) {   // (a tile's first item started the copies for the second above)
+                        kn = next;
+                        if (kn < 0 && more) { kn = wn.x; In = wn.y; Jn = first_j(wn); }
+                        if (kn >= 0) fetch(buf ^ 1, kn, In, Jn);
                     }
-                    __syncwarp();
-                    const float si = i < n ? p.sq3[i] : 0.f, ngam = -p.gamma, lam2 = p.lam2;
-                    const uint32_t syi = i < n ? (__float_as_uint(p.y[i]) & 0x80000000u) : 0u;
                     // interior tile: every pair valid
                     const bool full = I != J && (I + 1) * T <= n && (J + 1) * T <= n;
                     float rs4[4] = {0.f, 0.f, 0.f, 0.f};   // row sum in four interleaved parts
                     float q[32];
                     if (full)
-                        q_chunk32<true>(ga, sm.cy[ew], sm.cs[ew], si, syi, ngam, lam2, 0, 0, 0, 0, 0, q, rs4);
+                        q_chunk32<true>(ga, cy, &cc.sq[0][c0], si, syi, ngam, lam2, 0, 0, 0, 0, 0, q, rs4);
                     else
-                        q_chunk32<false>(ga, sm.cy[ew], sm.cs[ew], si, syi, ngam, lam2, i, n, c0, J * T, I == J ? r : -1, q, rs4);
+                        q_chunk32<false>(ga, cy, &cc.sq[0][c0], si, syi, ngam, lam2, i, n, c0, J * T, I == J ? r : -1, q, rs4);
                     constexpr int NSUM = MODE == T3_FINAL ? 2 : 1;
+                    T3Sums& su = sm.sums[buf];
                     if (MODE == T3_FORM) {
                         if (p.tilemax) {
                             float tmx = 0.f;
 #pragma unroll
                             for (int c = 0; c < 32; ++c) tmx = fmaxf(tmx, fabsf(q[c]));
                             tmx = warp_max_f(tmx);
-                            if (lane == 0) sm.tmx[ew] = tmx;
+                            if (lane == 0) su.tmx[ew] = tmx;
                         }
                         if (p.qref) store_row32(p.qref + (size_t)w.w * TT + (size_t)r * T + c0, q);
 #pragma unroll
                         for (int c = 0; c < 32; ++c) q[c] = fabsf(q[c]);
-                        sm.colsum[0][g][c0 + lane] = transpose_sum32(q, lane);
-                        sm.rowsum[0][cg][r] = (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
+                        su.col[0][g][c0 + lane] = transpose_sum32(q, lane);
+                        su.row[0][cg][r] = (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
                     } else {
                         // sums of q mu and q alpha: the row's over the columns, the columns' over the rows
 #pragma unroll
@@ -498,7 +553,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                             float f[4] = {0.f, 0.f, 0.f, 0.f}, v[32];
 #pragma unroll
                             for (int c4 = 0; c4 < 32; c4 += 4) {
-                                const float4 x4 = *reinterpret_cast<const float4*>(s ? &sm.ca[ew][c4] : &sm.cm[ew][c4]);
+                                const float4 x4 = *reinterpret_cast<const float4*>(s ? &cc.al[0][c0 + c4] : &cc.mu[0][c0 + c4]);
                                 const float xj[4] = {x4.x, x4.y, x4.z, x4.w};
 #pragma unroll
                                 for (int t = 0; t < 4; ++t) {
@@ -506,11 +561,16 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                                     v[c4 + t] = q[c4 + t] * xi;
                                 }
                             }
-                            sm.rowsum[s][cg][r] = (f[0] + f[1]) + (f[2] + f[3]);
-                            sm.colsum[s][g][c0 + lane] = transpose_sum32(v, lane);
+                            su.row[s][cg][r] = (f[0] + f[1]) + (f[2] + f[3]);
+                            su.col[s][g][c0 + lane] = transpose_sum32(v, lane);
                         }
                     }
+                    // One barrier a tile: the sums are complete, and every epilogue
+                    // warp takes a stop together; the next tile's sums go to the
+                    // other buffer.
+                    if (kn >= 0) settle(buf ^ 1, kn);
                     epi_bar();
+                    if (*(volatile int*)&sm.abort) { ok = false; break; }
                     // per-node slot partials (fixed order): row sums of the tile's rows,
                     // column sums of its columns; both roles on a diagonal tile
                     // (slot sl.x of the row block, sl.y of the column block).  Where
@@ -521,8 +581,8 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                         if (x < n && !(I == J && role)) {
 #pragma unroll
                             for (int s = 0; s < NSUM; ++s) {
-                                const float (*rw)[T] = sm.rowsum[s];
-                                const float (*cl)[T] = sm.colsum[s];
+                                const float (*rw)[T] = su.row[s];
+                                const float (*cl)[T] = su.col[s];
                                 const float vr = (rw[0][off] + rw[1][off]) + (rw[2][off] + rw[3][off]);
                                 const float vc = ((cl[0][off] + cl[1][off]) + cl[2][off]) + cl[3][off];
                                 const float v = I == J ? vr + vc : role ? vc : vr;
@@ -539,28 +599,26 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                     }
                     if (MODE == T3_FORM && etid == 0 && p.tilemax) {
                         float m2 = 0.f;
-                        for (int e = 0; e < T3_EPI_WARPS; ++e) m2 = fmaxf(m2, sm.tmx[e]);
+                        for (int e = 0; e < T3_EPI_WARPS; ++e) m2 = fmaxf(m2, su.tmx[e]);
                         p.tilemax[w.w] = m2;
                     }
-                    epi_bar();   // shared sums read before the next instance or tile writes them
-                    k = MODE == T3_FORM ? p.form_next - 1 : -1;
+                    buf ^= 1;
+                    k = next;
                 }
             }
             if (MODE == T3_DECIDE) {
-                if (!ok && lane == 0) {
-                    sm.abort = 1;
-                    record_error(tab[w.x].ctrl, ST_ETIMEOUT, L);
-                }
-                sm.rowsum[0][cg][r] = fs;
-                sm.rowsum[1][cg][r] = fc;
-                epi_bar();
-                if (etid < T) {
-                    double v = 0.0;
-                    for (int c = 0; c < 4; ++c) v += (double)sm.rowsum[0][c][etid] + (double)sm.rowsum[1][c][etid];
-                    dec.part[L * T + etid] = (float)v;
-                }
+                T3Sums& su = sm.sums[buf];
+                su.row[0][cg][r] = fs;
+                su.row[1][cg][r] = fc;
+                if (more) settle(buf ^ 1, wn.x);
                 epi_bar();
                 if (*(volatile int*)&sm.abort) break;
+                if (etid < T) {
+                    double v = 0.0;
+                    for (int c = 0; c < 4; ++c) v += (double)su.row[0][c][etid] + (double)su.row[1][c][etid];
+                    dec.part[L * T + etid] = (float)v;
+                }
+                buf ^= 1;
             }
             if (!ok) break;
         }
