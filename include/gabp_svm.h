@@ -303,7 +303,10 @@ GABP_API gabp_status gabp_batch_last_phases(double* out7);
  * compatible sizes and options; instance memory is returned to the CUDA
  * stream-ordered pool at the end of every call.  This frees the calling
  * thread's kept engine (a thread that exits without calling it leaves it
- * allocated until the process ends).  Always GABP_OK. */
+ * allocated until the process ends).  It also returns what the library keeps
+ * for the next handle or server: at most 512 MiB of unused device memory per
+ * device (given back by itself when a larger request needs it) and 4 MiB of
+ * pinned host memory.  Always GABP_OK. */
 GABP_API gabp_status gabp_batch_release(void);
 
 /*

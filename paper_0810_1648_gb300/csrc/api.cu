@@ -56,31 +56,6 @@ size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 void gabp::set_last_error(const char* msg) { g_err = msg; }
 
-cudaError_t gabp::device_available(size_t* avail, bool trim)
-{
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    cudaMemPool_t pool;
-    e = cudaDeviceGetDefaultMemPool(&pool, dev);
-    if (e != cudaSuccess) return e;
-    if (trim) {
-        e = cudaMemPoolTrimTo(pool, 0);
-        if (e != cudaSuccess) return e;
-    }
-    size_t free_b = 0, total_b = 0;
-    e = cudaMemGetInfo(&free_b, &total_b);
-    if (e != cudaSuccess) return e;
-    uint64_t reserved = 0, used = 0;
-    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
-        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
-        cudaGetLastError();
-        reserved = used = 0;
-    }
-    *avail = free_b + (reserved > used ? (size_t)(reserved - used) : 0);
-    return cudaSuccess;
-}
-
 int gabp::fault_mask()
 {
     const char* v = std::getenv("GABP_FAULT");
@@ -111,7 +86,7 @@ struct gabp_svm_s {
     int Nt = 0, npad = 0;
     long long ntiles = 0;
     double gamma = 0, C = 0, lambda = 0, delta = 0;
-    void* pool = nullptr;
+    DevBlock pool;
     size_t pool_bytes = 0;
     // tile-sparse option: the message state and Q of the kept tiles live in a
     // second allocation sized after the tile-maxima pass (grown on refit)
@@ -138,13 +113,15 @@ struct gabp_svm_s {
     float* alpha = nullptr;
     double* final3 = nullptr;
     double* blockbuf = nullptr;
-    void* dws = nullptr;            // workspace of decisions, kept up to kDecisionKeep bytes
+    DevBlock dws;                   // workspace of decisions, kept up to kDecisionKeep bytes
     size_t dws_bytes = 0;
-    Ctrl* hctrl = nullptr;          // pinned mirror of the control block
+    Ctrl* hctrl = nullptr;          // pinned mirror of the control block, as of the last wait for the stream
+    Ctrl* hdec = nullptr;           // and of a decision's
     double* hfinal = nullptr;       // pinned {rinf, objective, nsv}
     struct Graph {
         cudaGraphExec_t exec = nullptr;
         std::vector<cudaEvent_t> ev;   // 2 per bracketed round when captured with profiling on
+        int uses = 0;                  // chunks run with this key
     };
     std::map<std::tuple<int, int, int>, Graph> graphs;   // by (rounds, profiling stride, message path)
     int profiling = 0;   // 0 off, k >= 1: the pair sweep of every k-th round is bracketed by events
@@ -174,6 +151,9 @@ gabp_status check_formed(gabp_svm_t h)
     if (!h->formed) return fail(GABP_ESTATE, "the last refit failed; refit again before using the handle");
     return GABP_OK;
 }
+
+// The pinned mirrors: two control blocks and {rinf, objective, nsv}.
+constexpr size_t kMirrorBytes = 2 * sizeof(Ctrl) + 4 * sizeof(double);
 
 // Device memory plan of one handle (bytes, 256-aligned sub-buffers).
 struct Plan {
@@ -320,10 +300,11 @@ gabp_status ensure_spool(gabp_svm_t h, size_t need, const char* what)
     h->spool = nullptr;
     h->spool_bytes = 0;
     size_t free_b = 0;
-    CK(device_available(&free_b, true));   // cudaMalloc below: the pool's unused memory back first
+    CK(device_available(&free_b, false));
     const size_t margin = (size_t)256 << 20;
     if (need + margin > free_b)
         return fail(GABP_ENOMEM, "%s need %.2f GB of device memory, %.2f GB free", what, need / 1e9, free_b / 1e9);
+    CK(device_available(&free_b, true));   // cudaMalloc: the pools' unused memory back first
     cudaError_t e = cudaMalloc(&h->spool, need);
     if (e != cudaSuccess) return fail(GABP_ENOMEM, "cudaMalloc(%zu): %s", need, cudaGetErrorString(e));
     h->spool_bytes = need;
@@ -380,7 +361,6 @@ gabp_status stage_and_form(gabp_svm_t h, const void* X, const float* y)
     // 1 + lambda^2 + 1/C as the SVM's 2-norm soft margin does
     p.C = (float)(h->opts.task == GABP_TASK_KRR ? 1.0 / h->C : h->C);
     p.task = h->opts.task;
-    clear_graphs(h);
     h->solved = false;
     h->formed = false;
     h->kstar = 0;
@@ -407,7 +387,7 @@ gabp_status stage_and_form(gabp_svm_t h, const void* X, const float* y)
     const void* src = X;
     if (!dev) {
         if (xd != 0) {   // FP64 / BF16 rows: widened to FP32 by the staging kernel
-            CK(cudaMallocAsync(&tmp, (size_t)n * m * x_elem_bytes(xd), s));
+            CK(pool_alloc(&tmp, (size_t)n * m * x_elem_bytes(xd), s));
             CK(cudaMemcpyAsync(tmp, X, (size_t)n * m * x_elem_bytes(xd), cudaMemcpyHostToDevice, s));
             src = tmp;
         } else {
@@ -503,7 +483,12 @@ gabp_status stage_and_form(gabp_svm_t h, const void* X, const float* y)
             h->prof.kernel_launches += 1;
         }
     }
+    // the message path is known from here on; the mirror of the control block
+    // then holds until the first rounds
+    launch_begin(h->d_tab, 1, 0, 0.0, s);
+    h->prof.kernel_launches += 1;
     CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     h->formed = true;
     return GABP_OK;
@@ -514,11 +499,10 @@ void destroy_all(gabp_svm_t h)
     if (!h) return;
     if (h->stream) cudaStreamSynchronize(h->stream);
     clear_graphs(h);
-    if (h->pool) cudaFree(h->pool);
+    scratch_free(&h->pool, h->stream);
+    scratch_free(&h->dws, h->stream);
     if (h->spool) cudaFree(h->spool);
-    if (h->dws) cudaFree(h->dws);
-    if (h->hctrl) cudaFreeHost(h->hctrl);
-    if (h->hfinal) cudaFreeHost(h->hfinal);
+    pinned_free(h->hctrl, kMirrorBytes);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete h;
 }
@@ -527,37 +511,52 @@ void destroy_all(gabp_svm_t h)
 // (every `stride`-th round: k = stride - 1, 2 stride - 1, ...), and its pair.
 static bool bracketed(int stride, int k) { return stride > 0 && k % stride == stride - 1; }
 
-// A captured chunk of `rounds` synchronous rounds; with profiling on, the
+// `rounds` synchronous rounds on the handle's stream.
+static void launch_rounds(gabp_svm_t h, int rounds, int path, gabp_svm_s::Graph* G)
+{
+    const int stride = G ? h->profiling : 0;
+    for (int k = 0; k < rounds; ++k)
+        launch_round(h->d_tab, h->work, h->nbl, h->sched, h->nstages, h->grid, h->opts.q_mode, h->opts.msg_bf16,
+                     1 << path, h->stream, bracketed(stride, k) ? &G->ev[(size_t)2 * (k / stride)] : nullptr);
+}
+
+// A handle's chunk becomes a graph at its kGraphAfter-th use: capturing and
+// instantiating 16 rounds costs the host 95 us, while launching them one by
+// one (70 us) goes on beside the device.  What a chunk launches depends only
+// on what is fixed at create, so its graph serves later refits too; the few
+// kept ones are dropped when calls with ever new round counts come.
+constexpr int kGraphAfter = 4;
+constexpr size_t kGraphsKept = 8;
+
+// A chunk of `rounds` synchronous rounds, *out->exec null where it is launched
+// directly; with profiling on it is always captured, and the
 // pair sweep of every profiling-th round in it is bracketed by two
 // event-record nodes.
 gabp_status get_graph(gabp_svm_t h, int rounds, int path, gabp_svm_s::Graph** out)
 {
     const int stride = h->profiling;
     const auto key = std::make_tuple(rounds, stride, path);
-    auto it = h->graphs.find(key);
-    if (it != h->graphs.end()) { *out = &it->second; return GABP_OK; }
-    gabp_svm_s::Graph G;
+    if (h->graphs.size() >= kGraphsKept && h->graphs.find(key) == h->graphs.end()) clear_graphs(h);
+    gabp_svm_s::Graph& G = h->graphs[key];
+    *out = &G;
+    if (G.exec || (stride == 0 && G.uses < kGraphAfter)) return GABP_OK;
     if (stride > 0) {
         G.ev.resize((size_t)2 * (rounds / stride));
         for (auto& e : G.ev) CK(cudaEventCreate(&e));
     }
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    for (int k = 0; k < rounds; ++k)
-        launch_round(h->d_tab, h->work, h->nbl, h->sched, h->nstages, h->grid, h->opts.q_mode, h->opts.msg_bf16,
-                     1 << path, h->stream, bracketed(stride, k) ? &G.ev[(size_t)2 * (k / stride)] : nullptr);
+    launch_rounds(h, rounds, path, &G);
     cudaError_t e = cudaStreamEndCapture(h->stream, &g);
     if (e != cudaSuccess) return fail(GABP_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
     e = cudaGraphInstantiate(&G.exec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return fail(GABP_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
-    auto res = h->graphs.emplace(key, std::move(G));
-    *out = &res.first->second;
     return GABP_OK;
 }
 
 // Runs up to `iters` synchronous rounds from the current state with the
-// residual test `tol`, as captured graphs of `chunk` rounds, reading the
+// residual test `tol`, in chunks of `chunk` rounds (get_graph), reading the
 // control block after each replay.  *out = the final control block.
 gabp_status run_rounds(gabp_svm_t h, int iters, double tol, Ctrl* out)
 {
@@ -573,16 +572,21 @@ gabp_status run_rounds(gabp_svm_t h, int iters, double tol, Ctrl* out)
         static const int kTimeout = ST_ETIMEOUT;
         CK(cudaMemcpyAsync(&p.ctrl->status, &kTimeout, sizeof(int), cudaMemcpyHostToDevice, s));
     }
-    CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
     if (iters > 0) {
         const int len = tol > 0 ? std::min<int>(h->opts.chunk, iters) : iters;
-        gabp_svm_s::Graph* g = nullptr;
-        if (gabp_status st = get_graph(h, len, h->hctrl->path, &g)) return st;
+        const int path = h->hctrl->path;
         const int max_chunks = (iters + len - 1) / len + 1;
         int t_before = h->hctrl->t;
         for (int c = 0; c < max_chunks; ++c) {
-            CK(cudaGraphLaunch(g->exec, s));
+            gabp_svm_s::Graph* g = nullptr;
+            if (gabp_status st = get_graph(h, len, path, &g)) return st;
+            ++g->uses;
+            if (g->exec) {
+                CK(cudaGraphLaunch(g->exec, s));
+            } else {
+                launch_rounds(h, len, path, nullptr);
+                CK(cudaGetLastError());
+            }
             h->prof.kernel_launches += 2 * len;
             CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
@@ -602,6 +606,10 @@ gabp_status run_rounds(gabp_svm_t h, int iters, double tol, Ctrl* out)
             t_before = h->hctrl->t;
             if (h->hctrl->done) break;
         }
+    }
+    else {
+        CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
     }
     const Ctrl c = *h->hctrl;
     *out = c;
@@ -701,7 +709,7 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
 
     const Plan pl = make_plan(n, m, h->Nt, h->ntiles, h->npad, o.q_mode, o.msg_bf16, o.sparse_tau > 0);
     size_t free_b = 0;
-    e = device_available(&free_b, true);   // cudaMalloc below: the pool's unused memory back first
+    e = device_available(&free_b, false);
     if (e != cudaSuccess) { destroy_all(h); return fail(GABP_ECUDA, "cudaMemGetInfo: %s", cudaGetErrorString(e)); }
     const size_t margin = (size_t)256 << 20;
     if (pl.total + margin > free_b) {
@@ -722,15 +730,18 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
         destroy_all(h);
         return fail(GABP_ENOMEM, "injected device allocation failure (GABP_FAULT=alloc)");
     }
-    e = cudaMalloc(&h->pool, pl.total);
+    e = scratch_alloc(&h->pool, pl.total, h->stream);
     if (e != cudaSuccess) { destroy_all(h); return fail(GABP_ENOMEM, "cudaMalloc(%zu): %s", pl.total, cudaGetErrorString(e)); }
     h->pool_bytes = pl.total;
-    if (cudaMallocHost(&h->hctrl, sizeof(Ctrl)) != cudaSuccess ||
-        cudaMallocHost(&h->hfinal, 4 * sizeof(double)) != cudaSuccess) {
+    void* mirror = nullptr;
+    if (pinned_alloc(&mirror, kMirrorBytes) != cudaSuccess) {
         destroy_all(h);
         return fail(GABP_ENOMEM, "pinned host allocation failed");
     }
-    char* base = static_cast<char*>(h->pool);
+    h->hctrl = static_cast<Ctrl*>(mirror);
+    h->hdec = h->hctrl + 1;
+    h->hfinal = reinterpret_cast<double*>(h->hctrl + 2);
+    char* base = static_cast<char*>(h->pool.p);
     size_t off = 0;
     auto take = [&](size_t bytes) { void* r = base + off; off += bytes; return r; };
     Inst& p = h->inst;
@@ -829,7 +840,6 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
         e = cudaMemcpyAsync(h->sched, sc, sizeof(sc), cudaMemcpyHostToDevice, h->stream);
     const int zero_slot = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_members, &zero_slot, sizeof(int), cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) { destroy_all(h); return fail(GABP_ECUDA, "work list copy: %s", cudaGetErrorString(e)); }
 
     gabp_status st = stage_and_form(h, X, y);
@@ -859,8 +869,6 @@ gabp_status gabp_svm_solve(gabp_svm_t h, int32_t iters, double tol, float* alpha
     if (std::isnan(tol)) return fail(GABP_EINVAL, "tol is NaN");
     cudaStream_t s = h->stream;
     Inst& p = h->inst;
-    CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
     if (h->hctrl->status != 0) return fail(GABP_ESTATE, "state is invalid after an earlier failure; refit first");
     const bool refine = h->opts.q_mode != GABP_Q_F32 && h->opts.refine > 0;
     const bool same_matrix = h->opts.q_mode == GABP_Q_F32;   // the sweeps and the final pass see one Q
@@ -868,9 +876,8 @@ gabp_status gabp_svm_solve(gabp_svm_t h, int32_t iters, double tol, float* alpha
         // The refined solve always starts from Step 1 (b = 1, messages 0).
         launch_reset(p, s);
         h->prof.kernel_launches += 1;
+        h->hctrl->t = 0;
     }
-    CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
     const int t0 = h->hctrl->t;
     if ((long long)t0 + (long long)iters * (1 + h->opts.refine) >= (long long)INT_MAX)
         return fail(GABP_EINVAL, "too many rounds");
@@ -1034,14 +1041,19 @@ gabp_status gabp_svm_decision(gabp_svm_t h, const void* Xtest, int64_t t, float*
     const size_t bdiag = align_up((size_t)Ntt * sizeof(int4), 256), bout = dev ? 0 : align_up((size_t)slab * 4, 256);
     const size_t btab = align_up(2 * sizeof(Inst), 256), bctrl = align_up(sizeof(Ctrl), 256);
     const size_t need = bxp + bsq + bin + bpart + bw + bdiag + bout + btab + bctrl;
+    void* big = nullptr;
     if (need > h->dws_bytes) {
-        if (h->dws) CK(cudaFreeAsync(h->dws, s));
-        h->dws = nullptr;
+        if (h->dws.p) CK(cudaStreamSynchronize(s));
+        scratch_free(&h->dws, s);
         h->dws_bytes = 0;
-        CK(cudaMallocAsync(&h->dws, need, s));
-        h->dws_bytes = need;
+        if (need > kDecisionKeep) {
+            CK(pool_alloc(&big, need, s));
+        } else {
+            CK(scratch_alloc(&h->dws, need, s));
+            h->dws_bytes = need;
+        }
     }
-    char* b = static_cast<char*>(h->dws);
+    char* b = static_cast<char*>(big ? big : h->dws.p);
     auto take = [&](size_t bytes) { char* r = b; b += bytes; return r; };
     Inst two[2] = {Inst{}, h->inst};
     Inst& te = two[0];
@@ -1073,18 +1085,16 @@ gabp_status gabp_svm_decision(gabp_svm_t h, const void* Xtest, int64_t t, float*
             h->prof.kernel_launches += 5;
             if (!dev) CK(cudaMemcpyAsync(out + r0, dout, (size_t)tc * sizeof(float), cudaMemcpyDeviceToHost, s));
         }
-        CK(cudaMemcpyAsync(h->hctrl, te.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(h->hdec, te.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        if (h->hctrl->status == ST_EINVAL)
-            return fail(GABP_EINVAL, "test row %lld: non-finite feature", h->hctrl->bad_index);
-        if (h->hctrl->status != 0) return fail(GABP_ETIMEOUT, "a bounded device wait ran out in the decision");
+        if (h->hdec->status == ST_EINVAL)
+            return fail(GABP_EINVAL, "test row %lld: non-finite feature", h->hdec->bad_index);
+        if (h->hdec->status != 0) return fail(GABP_ETIMEOUT, "a bounded device wait ran out in the decision");
         return GABP_OK;
     };
     gabp_status st = run();
-    if (h->dws_bytes > kDecisionKeep) {
-        cudaFreeAsync(h->dws, s);
-        h->dws = nullptr;
-        h->dws_bytes = 0;
+    if (big) {
+        cudaFreeAsync(big, s);
         cudaStreamSynchronize(s);
     }
     return st;
@@ -1138,7 +1148,7 @@ gabp_status gabp_svm_get_q(gabp_svm_t h, float* Q)
     if (h->n > 46340) return fail(GABP_EINVAL, "n too large for a dense copy");
     const size_t bytes = (size_t)h->n * h->n * sizeof(float);
     float* d = nullptr;
-    CK(cudaMallocAsync((void**)&d, bytes, h->stream));
+    CK(pool_alloc((void**)&d, bytes, h->stream));
     CK(cudaMemsetAsync(d, 0, bytes, h->stream));
     launch_get_q(h->inst, h->work, h->nlive, h->opts.q_mode == GABP_Q_BF16, d, h->stream);
     cudaError_t e = cudaGetLastError();

@@ -347,6 +347,8 @@ class Engine {
     int chunk = 16;
     std::map<int, cudaGraphExec_t> graphs;
     std::vector<int> pending;     // added, Q not formed yet
+    DevBlock lists;               // the instance table, control blocks and lists
+    size_t pinned_bytes = 0;      // their pinned mirrors (from h_ctrl on)
     char* arena = nullptr;        // one allocation for a known set of instances (gabp_batch_solve)
     size_t arena_size = 0, arena_off = 0;
     struct EvGroup {
@@ -368,13 +370,9 @@ class Engine {
         for (auto& m : mem) release(m);
         if (arena) cudaFreeAsync(arena, stream);
         if (stream) cudaStreamSynchronize(stream);
-        if (d_tab) cudaFree(d_tab);
+        scratch_free(&lists, stream);
         for (auto& g : evg) cudaEventDestroy(g.ev);
-        if (h_tab) cudaFreeHost(h_tab);
-        if (h_live) cudaFreeHost(h_live);
-        if (h_ctrl) cudaFreeHost(h_ctrl);
-        if (h_f3) cudaFreeHost(h_f3);
-        if (h_ops) cudaFreeHost(h_ops);
+        pinned_free(h_ctrl, pinned_bytes);
         if (side) cudaStreamDestroy(side);
         if (sstream) cudaStreamDestroy(sstream);
         if (rejoin_ev) cudaEventDestroy(rejoin_ev);
@@ -434,11 +432,11 @@ class Engine {
         const size_t b_mem = aup((size_t)cap_members * sizeof(int), 256);
         const size_t b_bl = aup((size_t)cap_members * sizeof(int2), 256);
         const size_t b_bt = aup((size_t)cap_members * sizeof(double), 256);
-        char* base = nullptr;
         const size_t b_sched = aup((size_t)2 * kMaxStages * sizeof(Sched), 256);
         const size_t b_live = aup((size_t)cap_members * sizeof(int), 256);
-        EK(cudaMalloc((void**)&base,
-                      b_tab + b_ctrl + 2 * b_work + 2 * b_nbl + b_ops + b_f3 + b_mem + 2 * b_bl + 2 * b_bt + b_sched + b_live));
+        EK(scratch_alloc(&lists, b_tab + b_ctrl + 2 * b_work + 2 * b_nbl + b_ops + b_f3 + b_mem + 2 * b_bl + 2 * b_bt +
+                                     b_sched + b_live, stream));
+        char* base = static_cast<char*>(lists.p);
         size_t off = 0;
         auto carve = [&](size_t bytes) { char* r = base + off; off += bytes; return r; };
         d_tab = (Inst*)carve(b_tab);
@@ -458,12 +456,18 @@ class Engine {
         d_live = (int*)carve(b_live);
         EK(cudaMemsetAsync(d_ctrl, 0, b_ctrl, stream));
         EK(cudaMemsetAsync(d_sched, 0, b_sched, stream));
-        EK(cudaMallocHost((void**)&h_ctrl, (size_t)cap_members * sizeof(Ctrl)));
-        EK(cudaMallocHost((void**)&h_tab, (size_t)cap_members * sizeof(Inst)));
-        EK(cudaMallocHost((void**)&h_live, (size_t)cap_members * sizeof(int)));
-        EK(cudaMallocHost((void**)&h_f3, (size_t)cap_members * 3 * sizeof(double)));
-        EK(cudaMallocHost((void**)&h_ops, (size_t)cap_members * sizeof(StopOp)));
-        std::memset(h_ops, 0, (size_t)cap_members * sizeof(StopOp));
+        // the pinned mirrors in one block
+        pinned_bytes = b_ctrl + b_tab + b_live + b_f3 + b_ops;
+        void* mirror = nullptr;
+        EK(pinned_alloc(&mirror, pinned_bytes));
+        std::memset(mirror, 0, pinned_bytes);
+        base = static_cast<char*>(mirror);
+        off = 0;
+        h_ctrl = (Ctrl*)carve(b_ctrl);
+        h_tab = (Inst*)carve(b_tab);
+        h_live = (int*)carve(b_live);
+        h_f3 = (double*)carve(b_f3);
+        h_ops = (StopOp*)carve(b_ops);
         mem.resize((size_t)cap_members);
         set_grid(0);
         EK(cudaStreamSynchronize(stream));
@@ -534,7 +538,7 @@ class Engine {
     {
         if (fault_mask() > 0 && (fault_mask() & FAULT_ALLOC))
             return fail(GABP_ENOMEM, "injected device allocation failure (GABP_FAULT=alloc)");
-        EK(cudaMallocAsync((void**)&arena, bytes, side));
+        EK(pool_alloc((void**)&arena, bytes, side));
         arena_size = bytes;
         arena_off = 0;
         return GABP_OK;
@@ -626,7 +630,7 @@ class Engine {
                 bytes_in_use -= pl.total;
                 return fail(GABP_ENOMEM, "injected device allocation failure (GABP_FAULT=alloc)");
             }
-            EK(cudaMallocAsync(&M.mem, pl.total, s));
+            EK(pool_alloc(&M.mem, pl.total, s));
             b = static_cast<char*>(M.mem);
         }
         size_t off = 0;
@@ -704,7 +708,7 @@ class Engine {
             const void* src = pr.X;
             void* tmp = nullptr;
             if (!ptr_mode) {
-                EK(cudaMallocAsync(&tmp, (size_t)n * m * x_elem_bytes(x_dtype), s));
+                EK(pool_alloc(&tmp, (size_t)n * m * x_elem_bytes(x_dtype), s));
                 if (gabp_status st = fetch(tmp, pr.X, (size_t)n * m * x_elem_bytes(x_dtype), s)) return st;
                 src = tmp;
             }
@@ -1378,6 +1382,8 @@ gabp_status gabp_batch_release(void)
     gabp::set_last_error("");
     delete gabp::g_batch_engine;
     gabp::g_batch_engine = nullptr;
+    gabp::scratch_trim();
+    gabp::pinned_trim();
     return GABP_OK;
 }
 

@@ -402,11 +402,27 @@ cudaError_t launch_selftest_wait(unsigned long long limit_ns, int* status_dev, c
 // Sets the thread-local message returned by gabp_last_error().
 void set_last_error(const char* msg);
 // Device memory available to the library: cudaMemGetInfo's free bytes plus
-// what the device's default stream-ordered pool holds reserved but unused
-// (instance memory of the batched and served forms goes back to that pool and
-// stays reserved for reuse).  trim = true first returns the pool's unused
-// memory to the device (for plain cudaMalloc callers).
+// what the device's default stream-ordered pool and the scratch pool hold
+// reserved but unused (instance memory of the batched and served forms goes
+// back to the default pool and stays reserved for reuse).  trim = true first
+// returns that to the device (for plain cudaMalloc callers).
 cudaError_t device_available(size_t* avail, bool trim);
+
+// Memory kept for the next taker (scratch.cu).  Blocks are given back only
+// once the work that used them has been waited for.
+struct DevBlock {
+    void* p = nullptr;
+    bool pooled = false;   // from the scratch pool, else from cudaMalloc
+};
+bool scratch_fits(size_t bytes);   // small enough for the scratch pool
+cudaError_t scratch_alloc(DevBlock* b, size_t bytes, cudaStream_t s);
+void scratch_free(DevBlock* b, cudaStream_t s);
+void scratch_trim();               // the scratch pool's unused memory back to the device
+// cudaMallocAsync, tried again with the scratch pool's unused memory given back.
+cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s);
+cudaError_t pinned_alloc(void** p, size_t bytes);
+void pinned_free(void* p, size_t bytes);
+void pinned_trim();                // the kept pinned blocks back to the system
 // Host-side fault injection for tests of the failure paths: the environment
 // variable GABP_FAULT holds comma-separated tokens, read at each public call:
 //   alloc    the call's device allocation fails (create, batch, server admission)
