@@ -146,12 +146,13 @@ __device__ __forceinline__ ZU zu_pairs(const Ctrl* c)
 // admit it, or show a z so much smaller that its rounds take fewer terms
 // (z from the diagonal above 2^-20: most instances of up to about 10000 points;
 // the pass costs about as much as one round).
-__device__ __forceinline__ bool pair_z_open(const Inst& p)
+__device__ __forceinline__ bool pair_z_asks(const Inst& p)
 {
     const Ctrl* c = p.ctrl;
     const double inv = __longlong_as_double((long long)c->inv_margin_bits);
-    return p.hist && inv > 0.0 && inv < 1e30 && zu_diagonal(p, c).z > 9.5e-7f && orders_suffice(zu_pairs(c));
+    return p.hist && inv > 0.0 && inv < 1e30 && zu_diagonal(p, c).z > 9.5e-7f;
 }
+__device__ __forceinline__ bool pair_z_open(const Inst& p) { return pair_z_asks(p) && orders_suffice(zu_pairs(p.ctrl)); }
 // At Step 1: the message path of an instance and the bounds its rounds go by.
 __device__ __forceinline__ void choose_path(const Inst& p, Ctrl* c)
 {

@@ -867,45 +867,45 @@ __global__ void __launch_bounds__(HR_THREADS, 1)
 // instances whose margin leaves it open (the others cost a look at their
 // control block).  From the FP32 entries, so that the forms with BF16 entries
 // decide alike.
-__global__ void __launch_bounds__(256) k_pair_z(const Inst* __restrict__ tab, const int4* __restrict__ work, long long ntiles,
-                                               bool single)
+//
+// What bounds it: one read of the entries, 4 bytes a pair.  A warp has its 16
+// rows of a tile in flight at once and meets no barrier (whether an instance is
+// open is read by every thread, from lines that stay in L1).  With four rows in
+// flight and the check shared through a barrier: 38 us at n = 6238 (1225
+// tiles); now 27; a batch of 18 instances: 167 -> 73 us.
+__global__ void __launch_bounds__(256, 2) k_pair_z(const Inst* __restrict__ tab, const int4* __restrict__ work,
+                                                  long long ntiles, bool single)
 {
-    __shared__ int s_go;
-    const int tid = threadIdx.x;
-    if (single) {
-        if (tid == 0) s_go = pair_z_open(tab[0]);
-        __syncthreads();
-        if (!s_go) return;
-        __syncthreads();
-    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (single && !pair_z_open(tab[0])) return;
     for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
         const int4 w = work[L];
         for (int k = w.x; k >= 0; k = tab[k].form_next - 1) {
             const Inst& p = tab[k];
-            if (tid == 0) s_go = pair_z_open(p);
-            __syncthreads();
-            const int go = s_go;
-            __syncthreads();   // s_go is read before the next instance writes it
-            if (!go) continue;
-            const float* q = p.qref + (size_t)w.w * TT;
-            const int c0 = 4 * (tid & 31);
-            float rj[4];
+            if (!pair_z_asks(p)) continue;
+            const float* q = p.qref + (size_t)w.w * TT + warp * T + 4 * lane;
+            float4 a[T / 8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) rj[e] = 1.f / p.qdiag[min(w.z * T + c0 + e, p.n - 1)];   // (entries beyond n are 0)
+            for (int r = 0; r < T / 8; ++r) a[r] = *reinterpret_cast<const float4*>(q + (size_t)r * 8 * T);
+            if (!orders_suffice(zu_pairs(p.ctrl))) continue;   // settled by other tiles
+            float rj[4], ri = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                rj[e] = __fdividef(1.f, p.qdiag[min(w.z * T + 4 * lane + e, p.n - 1)]);   // (entries beyond n are 0)
+            if (lane < T / 8) ri = __fdividef(1.f, p.qdiag[min(w.y * T + 8 * lane + warp, p.n - 1)]);
             float best[2] = {0.f, FLT_MIN};   // the second never 0: the pass has run
-#pragma unroll 4
-            for (int r = tid >> 5; r < T; r += 8) {
-                const float ri = __fdividef(1.f, p.qdiag[min(w.y * T + r, p.n - 1)]);
-                const float4 a = *reinterpret_cast<const float4*>(q + r * T + c0);
-                note_pair_z(a.x, ri, rj[0], best);
-                note_pair_z(a.y, ri, rj[1], best);
-                note_pair_z(a.z, ri, rj[2], best);
-                note_pair_z(a.w, ri, rj[3], best);
+#pragma unroll
+            for (int r = 0; r < T / 8; ++r) {
+                const float rr = __shfl_sync(0xffffffffu, ri, r);
+                note_pair_z(a[r].x, rr, rj[0], best);
+                note_pair_z(a[r].y, rr, rj[1], best);
+                note_pair_z(a[r].z, rr, rj[2], best);
+                note_pair_z(a[r].w, rr, rj[3], best);
             }
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 best[e] = warp_max_f(best[e]);
-                if ((tid & 31) == 0 && __float_as_uint(best[e]) > *(volatile unsigned*)&p.ctrl->zpair_bits[e])
+                if (lane == 0 && __float_as_uint(best[e]) > *(volatile unsigned*)&p.ctrl->zpair_bits[e])
                     atomicMax(&p.ctrl->zpair_bits[e], __float_as_uint(best[e]));
             }
         }
@@ -940,7 +940,8 @@ void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, in
 void launch_pair_z(const Inst* tab, const int4* tiles, long long ntiles, int q_mode, bool single, cudaStream_t s)
 {
     if (ntiles <= 0) return;
-    const int grid = (int)(ntiles < 4 * num_sms() ? ntiles : 4 * num_sms());
+    const long long most = (q_mode == 2 ? 4 : 2) * num_sms();
+    const int grid = (int)(ntiles < most ? ntiles : most);
     if (q_mode == 2) launch_pair_z_gram(tab, tiles, ntiles, grid, single, s);
     else k_pair_z<<<grid, 256, 0, s>>>(tab, tiles, ntiles, single);
 }
