@@ -204,7 +204,7 @@ Plan make_plan(int64_t n, int64_t m, int Nt, long long ntiles, int npad, int q_m
     p.rhist = align_up((size_t)kRhistCap * sizeof(double), 256);
     p.final3 = 256;
     p.blockbuf = align_up((size_t)3 * ((n + 31) / 32) * sizeof(double), 256);
-    p.total = p.X + 10 * p.vec + p.agg + p.part + p.state + p.q + p.qref + p.work + p.tilemax + p.sparse + p.ctrl + p.rhist +
+    p.total = p.X + 9 * p.vec + p.agg + p.part + p.state + p.q + p.qref + p.work + p.tilemax + p.sparse + p.ctrl + p.rhist +
               p.final3 + p.blockbuf + p.xp + p.xp3 + p.tab + p.nbl + 2048;
     return p;
 }
@@ -395,10 +395,10 @@ gabp_status stage_and_form(gabp_svm_t h, const void* X, const float* y)
             src = p.X;
         }
     }
-    launch_stage(src, xd, (int)n, (int)m, const_cast<float*>(p.y), (float*)p.X, (float*)p.sq, (float*)p.b,
-                 const_cast<float*>(p.b0), p.task, p.ctrl, s);
+    // (with the rows' three BF16 planes for the tensor-core FP32 Gram)
+    CK(launch_stage(src, xd, (int)n, (int)m, h->Nt, (float*)p.X, const_cast<float*>(p.y), (float*)p.b,
+                    const_cast<float*>(p.b0), p.task, (void*)p.Xp3, 0, p.ctrl, nullptr, s));
     h->prof.kernel_launches += 1;
-    CK(cudaGetLastError());
     if (tmp) CK(cudaFreeAsync(tmp, s));
     CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -406,12 +406,10 @@ gabp_status stage_and_form(gabp_svm_t h, const void* X, const float* y)
         return fail(GABP_EINVAL, h->opts.task == GABP_TASK_KRR ? "row %lld: non-finite feature or target"
                                                                 : "row %lld: non-finite feature or label not +-1",
                     (long long)h->hctrl->bad_index);
-    // the FP32 rows as three BF16 planes for the tensor-core FP32 Gram, and
-    // the norms from the same products (diagonal tiles)
-    CK(launch_pack3(p.X, (int)n, (int)m, h->Nt, (void*)p.Xp3, s));
+    // the norms from the same products as the Gram (diagonal tiles)
     launch_form_norms(h->d_tab, h->work_diag, h->Nt, s);
     CK(cudaGetLastError());
-    h->prof.kernel_launches += 2;
+    h->prof.kernel_launches += 1;
     if (h->opts.sparse_tau > 0) {
         // Tile-sparse option.  Pass 1 over every tile: tile maxima and |Q|
         // row sums (the whole matrix's, for the diagonal rule), Q not
@@ -750,7 +748,6 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
     p.m = (int)m;
     p.npad = h->npad;
     p.X = (const float*)take(pl.X);
-    p.sq = (const float*)take(pl.vec);
     p.y = (const float*)take(pl.vec);
     p.b = (const float*)take(pl.vec);
     p.b0 = (const float*)take(pl.vec);
@@ -1080,7 +1077,8 @@ gabp_status gabp_svm_decision(gabp_svm_t h, const void* Xtest, int64_t t, float*
                 CK(cudaMemcpyAsync(in, src, (size_t)tc * m * x_elem_bytes(xd), cudaMemcpyHostToDevice, s));
                 src = (const char*)in;
             }
-            CK(launch_pack3_rows(src, xd, tc, (int)m, te.Nt, (void*)te.Xp3, r0, te.ctrl, diag, s));
+            CK(launch_stage(src, xd, tc, (int)m, te.Nt, nullptr, nullptr, nullptr, nullptr, 0, (void*)te.Xp3, r0,
+                            te.ctrl, diag, s));
             CK(launch_decision_tc(tab, diag, w, tc, h->Nt, h->alpha, part, te.ctrl, dev ? out + r0 : dout, s));
             h->prof.kernel_launches += 5;
             if (!dev) CK(cudaMemcpyAsync(out + r0, dout, (size_t)tc * sizeof(float), cudaMemcpyDeviceToHost, s));

@@ -69,7 +69,7 @@ MemberPlan member_plan(int64_t n, int64_t m, int q_mode, int msg_bf16, bool alia
     p.blockbuf = aup((size_t)3 * ((n + 31) / 32) * 8, 256);
     p.xp = q_mode != 0 ? aup(bf16_pack_bytes(Nt, (int)m), 1024) : 0;
     p.xp3 = aup(pack3_bytes(Nt, (int)m), 1024);   // the FP32 Gram's three BF16 planes
-    p.total = aup(p.X + 10 * p.vec + p.agg + p.part + p.state + p.q + p.qref + p.final3 + p.blockbuf + p.xp + p.xp3 +
+    p.total = aup(p.X + 9 * p.vec + p.agg + p.part + p.state + p.q + p.qref + p.final3 + p.blockbuf + p.xp + p.xp3 +
                   3072, 1024);
     return p;
 }
@@ -641,7 +641,6 @@ class Engine {
         p.m = (int)m;
         p.npad = (int)aup((size_t)n, 128);
         p.X = alias_x() ? static_cast<const float*>(pr.X) : (const float*)take(pl.X);
-        p.sq = (const float*)take(pl.vec);
         p.y = alias_y() ? pr.y : (const float*)take(pl.vec);
         p.b = (const float*)take(pl.vec);
         p.b0 = (const float*)take(pl.vec);
@@ -712,8 +711,8 @@ class Engine {
                 if (gabp_status st = fetch(tmp, pr.X, (size_t)n * m * x_elem_bytes(x_dtype), s)) return st;
                 src = tmp;
             }
-            launch_stage(src, x_dtype, (int)n, (int)m, const_cast<float*>(p.y), (float*)p.X, (float*)p.sq,
-                         (float*)p.b, const_cast<float*>(p.b0), p.task, p.ctrl, s);
+            EK(launch_stage(src, x_dtype, (int)n, (int)m, p.Nt, (float*)p.X, const_cast<float*>(p.y), (float*)p.b,
+                            const_cast<float*>(p.b0), p.task, (void*)p.Xp3, 0, p.ctrl, nullptr, s));
             ++launches;
             if (tmp) EK(cudaFreeAsync(tmp, s));
             M.staged = true;
@@ -796,15 +795,14 @@ class Engine {
         EK(cudaMemcpyAsync(d_n, nb.data(), nb.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
         if (!nb_stage.empty())
             EK(cudaMemcpyAsync(d_ns, nb_stage.data(), nb_stage.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
-        launch_stage_list(d_tab, d_ns, (int)nb_stage.size(), s);
+        EK(launch_stage_list(d_tab, d_ns, (int)nb_stage.size(), s));
         if (q_mode != 0) EK(launch_pack_list(d_tab, d_n, (int)nb.size(), s));
-        EK(launch_pack3_list(d_tab, d_n, (int)nb.size(), s));
         launch_form_norms(d_tab, d_dl, (long long)diag_lead.size(), s);
         launch_form_q(d_tab, d_tl, (long long)tiles_lead.size(), s);
         launch_init_list(d_tab, d_n, (int)nb.size(), diag_rule, (float)delta, s);
         if (q_mode == 1) EK(launch_form_q_tc(d_tab, d_tl, (long long)tiles_lead.size(), s));
         launch_pair_z(d_tab, d_tl, (long long)tiles_lead.size(), q_mode, false, s);
-        launches += q_mode == 0 ? 6 : (q_mode == 1 ? 8 : 7);
+        launches += q_mode == 0 ? 5 : (q_mode == 1 ? 7 : 6);
         EK(cudaGetLastError());
         size_t g = 0;
         while (g < evg.size() && evg[g].refs > 0) ++g;

@@ -104,7 +104,6 @@ struct Inst {
     int m;            // features
     int npad;         // stride of the per-node arrays inside agg
     const float* X;   // n x m FP32, row-major
-    const float* sq;  // ||x_i||^2 of the FP32 rows
     const float* y;   // labels +-1
     const float* b;   // working right-hand side (b0, or a refinement residual)
     const float* b0;  // the problem's right-hand side: ones (SVM), the targets (KRR)
@@ -277,12 +276,12 @@ struct GramSide {
 };
 
 // ---- launchers (defined in the .cu files) --------------------------------
-// Inputs: convert/validate X and y, row norms, right-hand sides.  SVM (task 0):
-// y must be +-1, b = b0 = 1.  KRR (task 1): y holds finite targets, which move
-// to b and b0, and y becomes 1 (no labels in Q).  y, b, b0 may be null (test
-// points).  Returns nothing; errors go to ctrl->status.
-void launch_stage(const void* X, int x_dtype, int n, int m, float* y, float* Xf, float* sq,
-                  float* b, float* b0, int task, Ctrl* ctrl, cudaStream_t s);
+// Inputs: convert/validate X and y, right-hand sides, and the three BF16 planes
+// of the rows (gram_tc32.cu).  SVM (task 0): y must be +-1, b = b0 = 1.  KRR (task
+// 1): y holds finite targets, which move to b and b0, and y becomes 1 (no labels
+// in Q).  y, b and b0 are null for test points.  Errors go to check->status.
+cudaError_t launch_stage(const void* X, int x_dtype, int n, int m, int Nt, float* Xf, float* y, float* b, float* b0,
+                         int task, void* Xp3, long long row0, Ctrl* check, int4* diag, cudaStream_t s);
 // Bytes of one feature of the input layout x_dtype (0 FP32, 1 FP64, 2 BF16).
 inline size_t x_elem_bytes(int x_dtype) { return x_dtype == 1 ? 8 : x_dtype == 2 ? 2 : 4; }
 // Refinement schedule of the precision forms (0 selects the default): the
@@ -309,11 +308,7 @@ inline void launch_form_norms(const Inst* tab, const int4* diag_work, long long 
     (void)launch_form_q_tc32(tab, diag_work, ntiles, 1, s);
 }
 // The three BF16 planes of FP32 rows (zero padding to whole tiles and chunks).
-cudaError_t launch_pack3(const float* Xf, int n, int m, int Nt, void* Xp3, cudaStream_t s);
-cudaError_t launch_pack3_list(const Inst* tab, const int2* nbl, int nblocks, cudaStream_t s);
 // The planes of a caller's rows, checked, and their diagonal tile list (k_pack3_rows).
-cudaError_t launch_pack3_rows(const void* X, int x_dtype, int n, int m, int Nt, void* Xp3, long long row0, Ctrl* check,
-                              int4* diag, cudaStream_t s);
 size_t pack3_bytes(int Nt, int m);
 // Precision form: BF16 operand packing + norms, and the tensor-core Q formation (BF16 store).
 cudaError_t launch_pack_bf16(const float* Xf, int n, int m, int nkc, int Nt, void* Xp, float* sqb, cudaStream_t s);
@@ -373,7 +368,7 @@ void launch_axpy_list(const Inst* tab, const StopOp* ops, const int2* nbl, int n
 void launch_refine_rhs_list(const Inst* tab, const StopOp* ops, const int2* nbl, int nblocks, cudaStream_t s);
 // Formation over listed node blocks of several instances (FP32 rows already in X):
 // staging checks / norms / b = 1; BF16 packing + norms; diagonal rule + Step 1.
-void launch_stage_list(const Inst* tab, const int2* nbl, int nblocks, cudaStream_t s);
+cudaError_t launch_stage_list(const Inst* tab, const int2* nbl, int nblocks, cudaStream_t s);
 cudaError_t launch_pack_list(const Inst* tab, const int2* nbl, int nblocks, cudaStream_t s);
 void launch_init_list(const Inst* tab, const int2* nbl, int nblocks, int diag_rule, float delta, cudaStream_t s);
 // Arms listed instances: list entries {slot, iters} with their tolerances.

@@ -170,62 +170,6 @@ __device__ __forceinline__ void reduce_and_write(EpiSmem& es, float (&rs)[NQ][8]
     }
 }
 
-// ---------------------------------------------------------------- staging
-// One row: FP32 copy (from FP32, FP64 or BF16 input; BF16 widens exactly),
-// squared norm, finiteness and label checks, b_i = 1 (the SVM right-hand
-// side: the linear term 1'h of the dual).
-__device__ __forceinline__ void stage_row(const void* __restrict__ X, int x_dtype, int i, int m,
-                                          float* __restrict__ y, float* __restrict__ Xf,
-                                          float* __restrict__ sq, float* __restrict__ b,
-                                          float* __restrict__ b0, int task, Ctrl* ctrl)
-{
-    float s = 0.f;
-    bool ok = true;
-    for (int k = 0; k < m; ++k) {
-        const size_t e = (size_t)i * m + k;
-        const float v = x_dtype == 1   ? (float)static_cast<const double*>(X)[e]
-                        : x_dtype == 2 ? __bfloat162float(static_cast<const __nv_bfloat16*>(X)[e])
-                                       : static_cast<const float*>(X)[e];
-        ok &= isfinite(v);
-        if (Xf != X) Xf[e] = v;
-        s = fmaf(v, v, s);
-    }
-    sq[i] = s;
-    float rhs = 1.f;   // SVM: Q alpha = 1 (Section 3)
-    if (y) {
-        const float yi = y[i];
-        if (task) {    // KRR: (K + lambda_r I) c = y (Section 1.2)
-            ok &= isfinite(yi);
-            rhs = yi;
-            y[i] = 1.f;
-        } else {
-            ok &= (yi == 1.f || yi == -1.f);
-        }
-    }
-    if (b) b[i] = rhs;
-    if (b0) b0[i] = rhs;
-    if (!ok && atomicCAS(&ctrl->status, 0, (int)ST_EINVAL) == 0) ctrl->bad_index = i;
-}
-
-__global__ void k_stage(const void* __restrict__ X, int x_dtype, int n, int m, float* __restrict__ y,
-                        float* __restrict__ Xf, float* __restrict__ sq, float* __restrict__ b,
-                        float* __restrict__ b0, int task, Ctrl* ctrl)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) stage_row(X, x_dtype, i, m, y, Xf, sq, b, b0, task, ctrl);
-}
-
-// Listed node blocks of instances whose FP32 rows already sit in their X.
-__global__ void k_stage_list(const Inst* __restrict__ tab, const int2* __restrict__ nbl)
-{
-    const int2 nb = nbl[blockIdx.x];
-    const Inst& p = tab[nb.x];
-    const int i = nb.y * 32 + threadIdx.x;
-    if (threadIdx.x < 32 && i < p.n)
-        stage_row(p.X, 0, i, p.m, const_cast<float*>(p.y), const_cast<float*>(p.X), const_cast<float*>(p.sq),
-                  const_cast<float*>(p.b), const_cast<float*>(p.b0), p.task, p.ctrl);
-}
-
 // ------------------------------------------- final residual and Q alpha
 // For every instance k listed: off-diagonal sums sum_{j != i} Q_ij mu_j
 // (-> part[2], the residual slots every round writes anew) and sum_{j != i}
@@ -319,18 +263,18 @@ __global__ void __launch_bounds__(NTHREADS) k_pair_z_gram(const Inst* __restrict
             __syncthreads();   // s_go is read before the next instance writes it
             if (!go) continue;
             float acc[8][8];
-            const GramSide S{p.X, p.sq, p.n};
+            const GramSide S{p.X, p.sq3, p.n};
             gram_tile(S, S, p.m, w.y, w.z, sm.g, acc);
             float best[2] = {0.f, FLT_MIN};   // the second never 0: the pass has run
 #pragma unroll
             for (int a = 0; a < 8; ++a) {
                 const int i = w.y * T + ty * 8 + a, ii = min(i, p.n - 1);
-                const float si = p.sq[ii], ri = 1.f / p.qdiag[ii];
+                const float si = p.sq3[ii], ri = 1.f / p.qdiag[ii];
 #pragma unroll
                 for (int b = 0; b < 8; ++b) {
                     const int j = w.z * T + tx * 8 + b;
                     if (i < j && j < p.n)
-                        note_pair_z(rbf_from_gram(acc[a][b], si, p.sq[j], p.gamma) + p.lam2, ri, 1.f / p.qdiag[j], best);
+                        note_pair_z(rbf_from_gram(acc[a][b], si, p.sq3[j], p.gamma) + p.lam2, ri, 1.f / p.qdiag[j], best);
                 }
             }
 #pragma unroll
@@ -471,17 +415,6 @@ __global__ void k_get_q(Inst p, const int4* __restrict__ work, int q_bf16, float
 }
 
 }  // namespace
-
-void launch_stage_list(const Inst* tab, const int2* nbl, int nblocks, cudaStream_t s)
-{
-    if (nblocks > 0) k_stage_list<<<nblocks, 32, 0, s>>>(tab, nbl);
-}
-
-void launch_stage(const void* X, int x_dtype, int n, int m, float* y, float* Xf, float* sq,
-                  float* b, float* b0, int task, Ctrl* ctrl, cudaStream_t s)
-{
-    k_stage<<<(n + 255) / 256, 256, 0, s>>>(X, x_dtype, n, m, y, Xf, sq, b, b0, task, ctrl);
-}
 
 void launch_pair_z_gram(const Inst* tab, const int4* tiles, long long ntiles, int grid, bool single,
                         cudaStream_t s)

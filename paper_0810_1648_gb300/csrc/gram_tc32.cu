@@ -91,81 +91,142 @@ __device__ __forceinline__ size_t core_off16(int rr, int kg)
     return (size_t)((rr / 8) * (KCH / 8) + kg) * 8 + (rr % 8);
 }
 
-// Row r (of Nt*T, zero beyond n) and 8-feature group gk of chunk kc -> the
-// three planes' blocks ((I nkc + kc) 3 + plane).
-__device__ __forceinline__ void pack3_group(const float* __restrict__ Xf, int n, int m, int nkc, int r, int gk,
-                                            uint4* __restrict__ Xp3)
+// ---------------------------------------------------------------- staging
+// Inputs to what the kernels read, in one pass: the FP32 rows (FP64 rounds,
+// BF16 widens exactly) where a copy is kept, their three BF16 planes, the
+// finiteness and label checks, the right-hand sides.
+//
+// What bounds it: 4 bytes read and 6 to 10 written per feature.  A thread takes 8
+// features of a row (32 bytes of FP32, one 16-byte unit of each plane); 8
+// consecutive threads take 8 rows of the same group, so that they write whole
+// 128-byte core matrices, and a warp reads 128 consecutive bytes of each row.
+// With one thread a row for the checks and norms and a second pass for the
+// planes: 107 + 14 us at n = 6238, m = 617; 40 + 10 us at n = 20000, m = 128;
+// now 22 and 10 us.
+
+// 8 consecutive features, in 16-byte loads where the rows are aligned to them.
+template <class XT>
+__device__ __forceinline__ void load8(const XT* __restrict__ x, float (&v)[8])
 {
-    const int kc = gk / (KCH / 8), kg = gk % (KCH / 8);
+    constexpr int W = 16 / sizeof(XT);
+#pragma unroll
+    for (int u = 0; u < 8; u += W) {
+        const uint4 q = __ldg(reinterpret_cast<const uint4*>(x + u));
+        XT e[W];
+        memcpy(e, &q, 16);
+#pragma unroll
+        for (int t = 0; t < W; ++t) v[u + t] = (float)e[t];
+    }
+}
+
+__device__ __forceinline__ bool rows_aligned(const void* X, size_t row_bytes)
+{
+    return ((reinterpret_cast<uintptr_t>(X) | row_bytes) & 15) == 0;
+}
+
+// Row r (of Nt*T, zero beyond n) and 8-feature group gk -> Xf where it is kept
+// and the three planes' blocks ((I nkc + kc) 3 + plane); false where a feature is
+// not finite.
+template <class XT>
+__device__ __forceinline__ bool stage_group(const XT* __restrict__ X, bool vec, int n, int m, int nkc, int r, int gk,
+                                            float* __restrict__ Xf, bool vecf, uint4* __restrict__ Xp3)
+{
+    const int kc = gk / (KCH / 8), kg = gk % (KCH / 8), k0 = gk * 8;
     const int I = r / T, rr = r % T;
+    float x[8];
+    bool ok = true;
+    if (r < n && vec && k0 + 8 <= m) {
+        load8(X + (size_t)r * m + k0, x);
+    } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = r < n && k0 + u < m ? (float)X[(size_t)r * m + k0 + u] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) ok &= isfinite(x[u]);
+    if (Xf && r < n) {
+        float* d = Xf + (size_t)r * m + k0;
+        if (vecf && k0 + 8 <= m) {
+            reinterpret_cast<float4*>(d)[0] = make_float4(x[0], x[1], x[2], x[3]);
+            reinterpret_cast<float4*>(d)[1] = make_float4(x[4], x[5], x[6], x[7]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (k0 + u < m) d[u] = x[u];
+        }
+    }
     __align__(16) __nv_bfloat16 v[NPLANE][8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        const int k = kc * KCH + kg * 8 + u;
-        split3((r < n && k < m) ? Xf[(size_t)r * m + k] : 0.f, v[0][u], v[1][u], v[2][u]);
-    }
+    for (int u = 0; u < 8; ++u) split3(x[u], v[0][u], v[1][u], v[2][u]);
 #pragma unroll
     for (int pl = 0; pl < NPLANE; ++pl) {
         const size_t blk = ((size_t)I * nkc + kc) * NPLANE + pl;
         Xp3[blk * (BLK_BYTES / 16) + core_off16(rr, kg)] = *reinterpret_cast<const uint4*>(v[pl]);
     }
+    return ok;
 }
 
-__global__ void k_pack3(const float* __restrict__ Xf, int n, int m, int nkc, int Nt, uint4* __restrict__ Xp3)
+// Row i's label (SVM: +-1, b = b0 = 1: the linear term 1'h of the dual) or
+// target (KRR: (K + lambda_r I) c = y; the target moves to b and b0, the label
+// becomes 1); false where it is not valid.
+__device__ __forceinline__ bool stage_label(float* __restrict__ y, float* __restrict__ b, float* __restrict__ b0, int i,
+                                            int task)
 {
-    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long groups = (long long)nkc * (KCH / 8);
-    if (e >= (long long)Nt * T * groups) return;
-    pack3_group(Xf, n, m, nkc, (int)(e / groups), (int)(e % groups), Xp3);
+    const float yi = y[i];
+    const float rhs = task ? yi : 1.f;
+    if (task) y[i] = 1.f;
+    b[i] = rhs;
+    b0[i] = rhs;
+    return task ? isfinite(yi) : yi == 1.f || yi == -1.f;
 }
 
-// The planes of a caller's rows (FP32, FP64 or BF16: x_dtype), every feature
-// checked to be finite (check->status, bad_index = the first found row + row0),
-// and the diagonal tile list of the rows.
+// Row (of 8 consecutive ones) and group of thread e of a pass over whole rows.
+__device__ __forceinline__ void stage_item(long long e, int groups, int& r, int& gk)
+{
+    const long long q = e >> 3;
+    gk = (int)(q % groups);
+    r = (int)(q / groups) * 8 + (int)(e & 7);
+}
+
+// A caller's rows (FP32, FP64 or BF16).  Xf: where the FP32 rows are kept (null:
+// nowhere, or X itself); y, b, b0: labels, null for test rows; diag: where the
+// diagonal tile list goes, or null.  Errors go to check->status, bad_index =
+// the first found row + row0.
 template <class XT>
-__global__ void k_pack3_rows(const XT* __restrict__ X, int n, int m, int nkc, int Nt, uint4* __restrict__ Xp3,
-                             long long row0, Ctrl* __restrict__ check, int4* __restrict__ diag)
+__global__ void k_stage_rows(const XT* __restrict__ X, int n, int m, int nkc, int Nt, float* __restrict__ Xf,
+                             float* __restrict__ y, float* __restrict__ b, float* __restrict__ b0, int task,
+                             uint4* __restrict__ Xp3, long long row0, Ctrl* __restrict__ check, int4* __restrict__ diag)
 {
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long groups = (long long)nkc * (KCH / 8);
-    if (e < Nt) diag[e] = make_int4(0, (int)e, (int)e, (int)e);
+    const int groups = nkc * (KCH / 8);
+    if (diag && e < Nt) diag[e] = make_int4(0, (int)e, (int)e, (int)e);
     if (e >= (long long)Nt * T * groups) return;
-    const int r = (int)(e / groups), gk = (int)(e % groups);
-    const int kc = gk / (KCH / 8), kg = gk % (KCH / 8);
-    __align__(16) __nv_bfloat16 v[NPLANE][8];
-    bool ok = true;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        const int k = kc * KCH + kg * 8 + u;
-        float x = 0.f;
-        if (r < n && k < m) {
-            x = (float)X[(size_t)r * m + k];
-            ok &= isfinite(x);
-        }
-        split3(x, v[0][u], v[1][u], v[2][u]);
-    }
+    int r, gk;
+    stage_item(e, groups, r, gk);
+    bool ok = stage_group(X, rows_aligned(X, (size_t)m * sizeof(XT)), n, m, nkc, r, gk, Xf,
+                          rows_aligned(Xf, (size_t)m * sizeof(float)), Xp3);
+    if (y && gk == 0 && r < n) ok &= stage_label(y, b, b0, r, task);
     if (!ok && atomicCAS(&check->status, 0, (int)ST_EINVAL) == 0) check->bad_index = row0 + r;
-#pragma unroll
-    for (int pl = 0; pl < NPLANE; ++pl) {
-        const size_t blk = ((size_t)(r / T) * nkc + kc) * NPLANE + pl;
-        Xp3[blk * (BLK_BYTES / 16) + core_off16(r % T, kg)] = *reinterpret_cast<const uint4*>(v[pl]);
-    }
 }
 
-// Listed node blocks (32 rows, 8 threads a row); the last block of an
-// instance also writes the zero rows that pad its last tile.
-__global__ void k_pack3_list(const Inst* __restrict__ tab, const int2* __restrict__ nbl)
+// Listed node blocks (32 rows) of instances whose FP32 rows already sit in
+// their X; the last block of an instance also writes the zero rows that pad its
+// last tile.
+__global__ void __launch_bounds__(256) k_stage_list(const Inst* __restrict__ tab, const int2* __restrict__ nbl)
 {
     const int2 nb = nbl[blockIdx.x];
     const Inst& p = tab[nb.x];
-    const int rl = threadIdx.x >> 3, gsub = threadIdx.x & 7;
-    const int r = nb.y * 32 + rl, n = p.n;
-    const bool last = nb.y == (n - 1) / 32;
+    const int n = p.n, m = p.m, nkc = p.nkc, groups = nkc * (KCH / 8);
+    const int rows = nb.y == (n - 1) / 32 ? p.Nt * T - nb.y * 32 : 32;
+    const bool vec = rows_aligned(p.X, (size_t)m * sizeof(float));
     uint4* Xp3 = static_cast<uint4*>(const_cast<void*>(p.Xp3));
-    const int groups = p.nkc * (KCH / 8);
-    for (int rw = r; rw < p.Nt * T; rw += 32) {
-        for (int gk = gsub; gk < groups; gk += 8) pack3_group(p.X, n, p.m, p.nkc, rw, gk, Xp3);
-        if (!last) break;
+    for (int e = threadIdx.x; e < rows * groups; e += blockDim.x) {
+        int r, gk;
+        stage_item(e, groups, r, gk);
+        r += nb.y * 32;
+        bool ok = stage_group(p.X, vec, n, m, nkc, r, gk, nullptr, false, Xp3);
+        if (gk == 0 && r < n)
+            ok &= stage_label(const_cast<float*>(p.y), const_cast<float*>(p.b), const_cast<float*>(p.b0), r, p.task);
+        if (!ok && atomicCAS(&p.ctrl->status, 0, (int)ST_EINVAL) == 0) p.ctrl->bad_index = r;
     }
 }
 
@@ -673,32 +734,28 @@ __global__ void k_decision_work(int4* __restrict__ work, int Ntt, int Nt, int pe
 
 size_t pack3_bytes(int Nt, int m) { return (size_t)NPLANE * Nt * bf16_chunks(m) * BLK_BYTES; }
 
-cudaError_t launch_pack3(const float* Xf, int n, int m, int Nt, void* Xp3, cudaStream_t s)
-{
-    const int nkc = bf16_chunks(m);
-    const long long total = (long long)Nt * T * nkc * (KCH / 8);
-    k_pack3<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(Xf, n, m, nkc, Nt, static_cast<uint4*>(Xp3));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pack3_rows(const void* X, int x_dtype, int n, int m, int Nt, void* Xp3, long long row0, Ctrl* check,
-                              int4* diag, cudaStream_t s)
+cudaError_t launch_stage(const void* X, int x_dtype, int n, int m, int Nt, float* Xf, float* y, float* b, float* b0,
+                         int task, void* Xp3, long long row0, Ctrl* check, int4* diag, cudaStream_t s)
 {
     const int nkc = bf16_chunks(m);
     const unsigned grid = (unsigned)(((long long)Nt * T * nkc * (KCH / 8) + 255) / 256);
     uint4* out = static_cast<uint4*>(Xp3);
+    if (Xf == X) Xf = nullptr;
     if (x_dtype == 1)
-        k_pack3_rows<<<grid, 256, 0, s>>>(static_cast<const double*>(X), n, m, nkc, Nt, out, row0, check, diag);
+        k_stage_rows<<<grid, 256, 0, s>>>(static_cast<const double*>(X), n, m, nkc, Nt, Xf, y, b, b0, task, out, row0,
+                                          check, diag);
     else if (x_dtype == 2)
-        k_pack3_rows<<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(X), n, m, nkc, Nt, out, row0, check, diag);
+        k_stage_rows<<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(X), n, m, nkc, Nt, Xf, y, b, b0, task, out,
+                                          row0, check, diag);
     else
-        k_pack3_rows<<<grid, 256, 0, s>>>(static_cast<const float*>(X), n, m, nkc, Nt, out, row0, check, diag);
+        k_stage_rows<<<grid, 256, 0, s>>>(static_cast<const float*>(X), n, m, nkc, Nt, Xf, y, b, b0, task, out, row0,
+                                          check, diag);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack3_list(const Inst* tab, const int2* nbl, int nblocks, cudaStream_t s)
+cudaError_t launch_stage_list(const Inst* tab, const int2* nbl, int nblocks, cudaStream_t s)
 {
-    if (nblocks > 0) k_pack3_list<<<nblocks, 256, 0, s>>>(tab, nbl);
+    if (nblocks > 0) k_stage_list<<<nblocks, 256, 0, s>>>(tab, nbl);
     return cudaGetLastError();
 }
 
