@@ -515,12 +515,14 @@ static void launch_rounds(gabp_svm_t h, int rounds, int path, gabp_svm_s::Graph*
     const int stride = G ? h->profiling : 0;
     for (int k = 0; k < rounds; ++k)
         launch_round(h->d_tab, h->work, h->nbl, h->sched, h->nstages, h->grid, h->opts.q_mode, h->opts.msg_bf16,
-                     1 << path, h->stream, bracketed(stride, k) ? &G->ev[(size_t)2 * (k / stride)] : nullptr);
+                     1 << path, G ? CHAIN_NONE : k == 0 ? CHAIN_AFTER_FIRST : CHAIN_ALL, h->stream, bracketed(stride, k) ? &G->ev[(size_t)2 * (k / stride)] : nullptr);
 }
 
 // A handle's chunk becomes a graph at its kGraphAfter-th use: capturing and
 // instantiating 16 rounds costs the host 95 us, while launching them one by
-// one (70 us) goes on beside the device.  What a chunk launches depends only
+// one (70 us) goes on beside the device, one round of two kernels 1 us slower
+// than in the graph (a staged round of eight, n = 12960: 15 us, so those are
+// captured at once).  What a chunk launches depends only
 // on what is fixed at create, so its graph serves later refits too; the few
 // kept ones are dropped when calls with ever new round counts come.
 constexpr int kGraphAfter = 4;
@@ -537,7 +539,7 @@ gabp_status get_graph(gabp_svm_t h, int rounds, int path, gabp_svm_s::Graph** ou
     if (h->graphs.size() >= kGraphsKept && h->graphs.find(key) == h->graphs.end()) clear_graphs(h);
     gabp_svm_s::Graph& G = h->graphs[key];
     *out = &G;
-    if (G.exec || (stride == 0 && G.uses < kGraphAfter)) return GABP_OK;
+    if (G.exec || (stride == 0 && h->nstages == 1 && G.uses < kGraphAfter)) return GABP_OK;
     if (stride > 0) {
         G.ev.resize((size_t)2 * (rounds / stride));
         for (auto& e : G.ev) CK(cudaEventCreate(&e));

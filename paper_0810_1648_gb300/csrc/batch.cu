@@ -909,7 +909,7 @@ class Engine {
         cudaGraph_t g = nullptr;
         EK(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
         for (int k = 0; k < rounds; ++k)
-            launch_round(d_tab, d_work, d_nbl, d_sched, nstages, grid, q_mode, msg_bf16, mask, stream);
+            launch_round(d_tab, d_work, d_nbl, d_sched, nstages, grid, q_mode, msg_bf16, mask, CHAIN_NONE, stream);
         EK(cudaStreamEndCapture(stream, &g));
         cudaGraphExec_t ex = nullptr;
         cudaError_t e = cudaGraphInstantiate(&ex, g, 0);

@@ -333,6 +333,28 @@ RoundGrid round_grid(long long max_tiles, int max_nblocks, int q_mode, int ctas_
 cudaError_t prepare_sweep();
 // Fused-recompute form: also raises the shared-memory limit of its sweep kernel.
 cudaError_t prepare_sweep_rc();
+// Launches a kernel of a round.  chained: it may start while the stream's last
+// kernel, of the same chain, still runs (it passes chain_wait() before it reads
+// what that one writes), which takes the launch and the kernel's start off a
+// round's path: n = 1000, 19.4 -> 16.4 us a round; n = 6238, 29.7 -> 27.1.  The
+// kernels of a captured graph are not chained: they start as early (15.2 and
+// 26.2 us), and chained ones later (staged, n = 12960: 133 -> 146 us).
+enum Chain { CHAIN_NONE, CHAIN_AFTER_FIRST, CHAIN_ALL };   // which kernels of a round
+template <class... P, class... A>
+void launch_chained(bool chained, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 // One round over every live instance of tab: pair sweep then per-node
 // finalize.  When ev is not null, ev[0] is recorded before the (first stage's)
 // pair sweep and ev[1] after the (last stage's) pair sweep.
@@ -342,10 +364,11 @@ cudaError_t prepare_sweep_rc();
 // PATH_STORED or both); sched[kMaxStages + st] is the PATH_STORED segment of
 // stage st, sched[st] the PATH_HIST one.
 void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sched* sched, int nstages,
-                  const RoundGrid& g, int q_mode, int msg_bf16, int paths, cudaStream_t s, cudaEvent_t* ev = nullptr);
+                  const RoundGrid& g, int q_mode, int msg_bf16, int paths, Chain chain, cudaStream_t s,
+                  cudaEvent_t* ev = nullptr);
 // One pair sweep of PATH_HIST instances over a stage's tile list (sweep_hist.cu).
 void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, int stage_no, int grid, int q_mode,
-                       cudaStream_t s);
+                       bool chained, cudaStream_t s);
 cudaError_t prepare_sweep_hist();
 // Formation, after launch_init over the same instances: Ctrl::zpair_bits over
 // the listed tiles for the instances whose diagonal alone does not show that

@@ -13,6 +13,14 @@ namespace gabp {
 
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // bounded waits: 2 s
 
+// Kernels of a round are launched so that each may start while the one before
+// it still runs (launch_chained): the next kernel may start from here on ...
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// ... and waits here until the one before it has ended and its writes are seen.
+// Every thread of a chained kernel passes it before it reads what a kernel of
+// the round writes, and before it leaves.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void* ptr)
 {
     return (uint32_t)__cvta_generic_to_shared(ptr);

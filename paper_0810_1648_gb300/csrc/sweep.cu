@@ -854,6 +854,7 @@ template <typename QT, class MSG>
 __global__ void __launch_bounds__(SWEEP_THREADS, sweep_ctas<MSG>())
     k_sweep(const Inst* __restrict__ tab, const int4* __restrict__ work, const Sched* __restrict__ sched, int stage_no)
 {
+    chain_next();
     const long long ntiles = sched->ntiles;
     work += sched->off;
     constexpr size_t SB = stage_bytes<QT, MSG>();
@@ -868,6 +869,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS, sweep_ctas<MSG>())
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    chain_wait();
     if (warp == NWARPS) {
         sweep_producer<QT, MSG, SB>(tab, work, ntiles, sm, ring, nullptr, lane, stage_no);
         return;
@@ -945,6 +947,7 @@ __global__ void __launch_bounds__(RC_THREADS, 1)
     k_sweep_rc(const Inst* __restrict__ tab, const int4* __restrict__ work, const Sched* __restrict__ sched,
                int stage_no)
 {
+    chain_next();
     const long long ntiles = sched->ntiles;
     work += sched->off;
 
@@ -969,6 +972,7 @@ __global__ void __launch_bounds__(RC_THREADS, 1)
         ex.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    chain_wait();
     if (warp == 2) tmem_alloc(&ex.tmem_base, RC_TMEM_COLS);
     tc_fence_before();
     __syncthreads();
@@ -1348,6 +1352,8 @@ __global__ void __launch_bounds__(256, 5)
     const int units = fin_units(sched, usmall), nsmall = sched->nsmall;
     __shared__ float red[6][8][32];
     __shared__ int s_last;
+    chain_next();
+    chain_wait();
     const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
     for (int u = blockIdx.x; u < units; u += gridDim.x) {
         if (u < usmall) {
@@ -1496,6 +1502,8 @@ __global__ void __launch_bounds__(256)
     int usmall;
     const int units = fin_units(sched, usmall), nsmall = sched->nsmall;
     __shared__ float red[4][8][32];
+    chain_next();
+    chain_wait();
     const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
     for (int u = blockIdx.x; u < units; u += gridDim.x) {
         if (u < usmall) {
@@ -1918,32 +1926,37 @@ cudaError_t prepare_sweep()
 }
 
 void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sched* sched, int nstages,
-                  const RoundGrid& g, int q_mode, int msg_bf16, int paths, cudaStream_t s, cudaEvent_t* ev)
+                  const RoundGrid& g, int q_mode, int msg_bf16, int paths, Chain mode, cudaStream_t s, cudaEvent_t* ev)
 {
+    bool chain = mode == CHAIN_ALL;
     for (int st = 0; st < nstages; ++st) {
         const Sched* sc = sched + kMaxStages + st;
         if (ev && st == 0) cudaEventRecordWithFlags(ev[0], s, cudaEventRecordExternal);
-        if (paths & (1 << PATH_HIST)) launch_sweep_hist(tab, work, sched + st, st, g.sweep, q_mode, s);
-        if (!(paths & (1 << PATH_STORED))) {
-            // no instance stores its messages
-        } else if (q_mode == 2 && msg_bf16)
-            k_sweep_rc<MsgBF16><<<g.sweep, RC_THREADS, rc_smem_bytes<MsgBF16>(), s>>>(tab, work, sc, st);
-        else if (q_mode == 2)
-            k_sweep_rc<MsgF32><<<g.sweep, RC_THREADS, rc_smem_bytes<MsgF32>(), s>>>(tab, work, sc, st);
-        else if (q_mode == 1 && msg_bf16)
-            k_sweep<__nv_bfloat16, MsgBF16>
-                <<<g.sweep, SWEEP_THREADS, sweep_smem_bytes<__nv_bfloat16, MsgBF16>(), s>>>(tab, work, sc, st);
-        else if (q_mode == 1)
-            k_sweep<__nv_bfloat16, MsgF32>
-                <<<g.sweep, SWEEP_THREADS, sweep_smem_bytes<__nv_bfloat16, MsgF32>(), s>>>(tab, work, sc, st);
-        else
-            k_sweep<float, MsgF32>
-                <<<g.sweep, SWEEP_THREADS, sweep_smem_bytes<float, MsgF32>(), s>>>(tab, work, sc, st);
+        if (paths & (1 << PATH_HIST)) {
+            launch_sweep_hist(tab, work, sched + st, st, g.sweep, q_mode, chain, s);
+            chain = mode != CHAIN_NONE;
+        }
+        if (paths & (1 << PATH_STORED)) {
+            if (q_mode == 2 && msg_bf16)
+                launch_chained(chain, k_sweep_rc<MsgBF16>, g.sweep, RC_THREADS, rc_smem_bytes<MsgBF16>(), s, tab, work, sc, st);
+            else if (q_mode == 2)
+                launch_chained(chain, k_sweep_rc<MsgF32>, g.sweep, RC_THREADS, rc_smem_bytes<MsgF32>(), s, tab, work, sc, st);
+            else if (q_mode == 1 && msg_bf16)
+                launch_chained(chain, k_sweep<__nv_bfloat16, MsgBF16>, g.sweep, SWEEP_THREADS,
+                               sweep_smem_bytes<__nv_bfloat16, MsgBF16>(), s, tab, work, sc, st);
+            else if (q_mode == 1)
+                launch_chained(chain, k_sweep<__nv_bfloat16, MsgF32>, g.sweep, SWEEP_THREADS,
+                               sweep_smem_bytes<__nv_bfloat16, MsgF32>(), s, tab, work, sc, st);
+            else
+                launch_chained(chain, k_sweep<float, MsgF32>, g.sweep, SWEEP_THREADS, sweep_smem_bytes<float, MsgF32>(), s,
+                               tab, work, sc, st);
+            chain = mode != CHAIN_NONE;
+        }
         if (ev && st == nstages - 1) cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal);
         if (st < nstages - 1)
-            k_finalize_stage<<<g.finalize, 256, 0, s>>>(tab, nbl, sched, st + 1);
+            launch_chained(chain, k_finalize_stage, g.finalize, 256, 0, s, tab, nbl, sched, st + 1);
         else
-            k_finalize<<<g.finalize, 256, 0, s>>>(tab, nbl, sched);
+            launch_chained(chain, k_finalize, g.finalize, 256, 0, s, tab, nbl, sched);
     }
 }
 

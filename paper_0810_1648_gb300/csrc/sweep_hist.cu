@@ -617,8 +617,8 @@ template <typename QT>
 __global__ void __launch_bounds__(H_THREADS, 2)
     k_sweep_hist(const Inst* __restrict__ tab, const int4* __restrict__ work, const Sched* __restrict__ sched, int stage_no)
 {
+    chain_next();
     const long long ntiles = sched->ntiles;
-    if (nothing_to_do(tab, sched)) return;
     work += sched->off;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* ring = align_smem(smem_raw, 128);
@@ -629,6 +629,8 @@ __global__ void __launch_bounds__(H_THREADS, 2)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    chain_wait();
+    if (nothing_to_do(tab, sched)) return;
     if (tid >= HCW * 32) {
         hist_producer<QT>(tab, work, ntiles, sm, ring, nullptr, tid & 31, stage_no);
         return;
@@ -707,7 +709,9 @@ __global__ void __launch_bounds__(HR_THREADS, 1)
     k_sweep_hist_rc(const Inst* __restrict__ tab, const int4* __restrict__ work, const Sched* __restrict__ sched,
                     int stage_no)
 {
+    chain_next();
     const long long ntiles = sched->ntiles;
+    chain_wait();
     if (nothing_to_do(tab, sched)) return;
     work += sched->off;
     extern __shared__ unsigned char smem_raw[];
@@ -927,14 +931,15 @@ cudaError_t prepare_sweep_hist()
 }
 
 void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, int stage_no, int grid, int q_mode,
-                       cudaStream_t s)
+                       bool chained, cudaStream_t s)
 {
     if (q_mode == 2)
-        k_sweep_hist_rc<<<grid, HR_THREADS, hist_rc_smem_bytes(), s>>>(tab, work, sched, stage_no);
+        launch_chained(chained, k_sweep_hist_rc, grid, HR_THREADS, hist_rc_smem_bytes(), s, tab, work, sched, stage_no);
     else if (q_mode == 1)
-        k_sweep_hist<__nv_bfloat16><<<grid, H_THREADS, hist_smem_bytes(), s>>>(tab, work, sched, stage_no);
+        launch_chained(chained, k_sweep_hist<__nv_bfloat16>, grid, H_THREADS, hist_smem_bytes(), s, tab, work, sched,
+                       stage_no);
     else
-        k_sweep_hist<float><<<grid, H_THREADS, hist_smem_bytes(), s>>>(tab, work, sched, stage_no);
+        launch_chained(chained, k_sweep_hist<float>, grid, H_THREADS, hist_smem_bytes(), s, tab, work, sched, stage_no);
 }
 
 void launch_pair_z(const Inst* tab, const int4* tiles, long long ntiles, int q_mode, bool single, cudaStream_t s)
