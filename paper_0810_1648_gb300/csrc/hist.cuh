@@ -89,7 +89,12 @@ __device__ __forceinline__ int e_terms(float z, float change)
 }
 // Whether the even orders q^4, q^6 count: without them the P messages into a
 // node are off by at most z u of Ptilde, E by z u change.
-__device__ __forceinline__ bool even_orders(float z, float u) { return 2.f * z * u > kLeftOut; }
+// (2: q^4 and q^6; 1: q^4 alone, where what q^6 adds is at most 2 z^2 u of Ptilde
+// and 4 z^2 u change of a mean)
+__device__ __forceinline__ int even_orders(float z, float u)
+{
+    return 4.f * z * z * u > kLeftOut ? 2 : 2.f * z * u > kLeftOut ? 1 : 0;
+}
 // Whether the tiles of a round after the first write E (live rounds with even
 // orders always do).
 __device__ __forceinline__ bool round_has_e(const Ctrl* c, bool frozen) { return c->terms > 0 || (!frozen && c->even); }

@@ -45,14 +45,18 @@ constexpr int H_STAGES = 4;
 constexpr int H_GROUP = 64;                    // rows per row-sum reduction (four steps of 16)
 
 // What a tile sums beside q mu.  Live P: q^2 (round 0, and where nothing else
-// counts), with q^3, or everything; frozen P: nothing, q^3, or q^3 and q^5.
-enum { K_LIVE0, K_LIVE1, K_LIVE, K_SUM, K_ONE, K_TWO };
+// counts), with q^3, with q^3 and q^4, or everything; frozen P: nothing, q^3, or
+// q^3 and q^5.
+enum { K_LIVE0, K_LIVE1, K_LIVE4, K_LIVE, K_SUM, K_ONE, K_TWO };
 // The sums of a wide tile, as rows of HTail::rs and cs; a small tile (sum_tile)
-// has three at most, q mu, then mu of the stage or q^2, then q^3, and takes
-// rows 0-2 and 3-5 in turn.
+// has three at most, of q mu, mu of the stage, q^2 and q^3 in this order, and
+// takes rows 0-2 and 3-5 in turn.
 enum { S_R, S_M, S_2, S_4, S_6, S_W3, S_W5, S_COUNT };
 constexpr int S_SMALL = 3;
-__device__ __forceinline__ bool is_wide(int kind) { return kind == K_LIVE || kind == K_TWO; }
+__device__ __forceinline__ bool is_wide(int kind, bool staged)
+{
+    return kind == K_LIVE4 || kind == K_LIVE || kind == K_TWO || (kind == K_LIVE1 && staged);
+}
 // The node values, as rows of HTail::node: mean of the residual, the stage's
 // mean (staged), and hnow's three.
 enum { N_MU0, N_MU, N_R, N_W3, N_W5, N_COUNT };
@@ -126,10 +130,10 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
             even = ctrl->even;
             staged = p.nstages > 1;
             kind = frozen && t > 0                    ? (terms == 0 ? K_SUM : terms == 1 ? K_ONE : K_TWO)
-                   : staged                           ? K_LIVE   // (fewer sums do not fit the registers of sum_tile)
-                   : t == 0 || (!even && terms == 0) ? K_LIVE0
-                   : !even && terms == 1             ? K_LIVE1
-                                                     : K_LIVE;
+                   : t == 0 || (!even && terms == 0)  ? K_LIVE0
+                   : !even && terms == 1              ? K_LIVE1
+                   : even <= 1 && terms <= 1          ? K_LIVE4
+                                                      : K_LIVE;
             // node values of its tiles: bit a set where row a is copied
             use = 1u << N_MU0 | (staged ? 1u << N_MU : 0u) | (kind <= K_LIVE ? 1u << N_R : 0u) |
                   (kind == K_LIVE0 || kind == K_SUM ? 0u : 1u << N_W3) | (kind == K_LIVE || kind == K_TWO ? 1u << N_W5 : 0u);
@@ -379,13 +383,13 @@ __device__ __forceinline__ void sum_tile(SRC& src, HTail& sm, const HInfo& ti, i
     auto group = [&](int r0) {
         put_rows(sm.rs[base], xR, r0, cw, lane);
         if (STAGED) put_rows(sm.rs[base + 1], xM, r0, cw, lane);
-        if (PTWO) put_rows(sm.rs[base + 1], xP, r0, cw, lane);
+        if (PTWO) put_rows(sm.rs[base + 1 + STAGED], xP, r0, cw, lane);
         if (ONE) put_rows(sm.rs[base + 2], xE, r0, cw, lane);
     };
     walk_tile(src, sm, ti, cw, lane, row, group);
     put_cols(sm.cs[base][cw], aR, lane);
     if (STAGED) put_cols(sm.cs[base + 1][cw], aM, lane);
-    if (PTWO) put_cols(sm.cs[base + 1][cw], aP, lane);
+    if (PTWO) put_cols(sm.cs[base + 1 + STAGED][cw], aP, lane);
     if (ONE) put_cols(sm.cs[base + 2][cw], aE, lane);
 }
 
@@ -396,75 +400,127 @@ __device__ __forceinline__ void ld_cols4(const float* d, int lane, float2 (&v)[2
     v[1] = make_float2(a.z, a.w);
 }
 
-// Tiles of more sums (q^3 and q^5; with live P also q^2, q^4 and q^6): a warp
-// takes one row at a time (row 8 s + cw), each lane four of its columns, which
-// leaves room for all the weights and sums of a lane's columns (eight columns a
-// lane did not fit 96 registers); a row's sums go through one eight-value warp
-// reduction.
-template <bool LIVE, bool STAGED, class SRC>
+// Tiles of more sums: a warp takes two rows at a time (rows 16 s + cw and 8
+// more), each lane four of their columns, which leaves room for all the weights
+// and sums of a lane's columns (eight columns a lane did not fit 96 registers).
+// A row's sums go through a warp reduction of eight values, of two rows where
+// there are four at most.  What bounds it is arithmetic (10 to 21 paired
+// instructions for two pairs, and the reductions), so a tile sums only what its
+// instance's round needs: summing everything in every staged round with live P,
+// 450 us a stage over 512 instances of 200 to 4000 points; now 190 (round 0)
+// to 310.
+template <bool LIVE, bool Q4, bool Q6, bool Q5, bool STAGED>
+struct WideSums {
+    static constexpr bool has(int s)
+    {
+        return s == S_R || s == S_W3 || (s == S_M && STAGED) || (s == S_2 && LIVE) || (s == S_4 && Q4) || (s == S_6 && Q6) ||
+               (s == S_W5 && Q5);
+    }
+    static constexpr int index(int s)   // its place among the sums there are
+    {
+        int k = 0;
+        for (int i = 0; i < s; ++i) k += has(i);
+        return k;
+    }
+    static constexpr int count = index(S_COUNT);
+    static constexpr int nth(int k)
+    {
+        for (int i = 0; i < S_COUNT; ++i)
+            if (has(i) && index(i) == k) return i;
+        return S_COUNT;
+    }
+};
+
+template <bool LIVE, bool Q4, bool Q6, bool Q5, bool STAGED, class SRC>
 __device__ __forceinline__ void wide_tile(SRC& src, HTail& sm, const HInfo& ti, int slot, int cw, int lane)
 {
+    using W = WideSums<LIVE, Q4, Q6, Q5, STAGED>;
+    constexpr int NS = W::count, ROWS = NS <= 4 ? 2 : 1;   // rows per reduction
     const float (*R)[T] = sm.node[slot][0];
     const float (*C)[T] = sm.node[slot][1];
-    float2 cm[2], cs[2], cr[2], c3[2], c5[2], a[S_COUNT][2];
+    float2 cm[2], cs[2], cr[2], c3[2], c5[2], a[NS][2];
     ld_cols4(C[N_MU0], lane, cm);
     if (STAGED) ld_cols4(C[N_MU], lane, cs);
     if (LIVE) ld_cols4(C[N_R], lane, cr);
     ld_cols4(C[N_W3], lane, c3);
-    ld_cols4(C[N_W5], lane, c5);
+    if (Q5) ld_cols4(C[N_W5], lane, c5);
 #pragma unroll
-    for (int s = 0; s < S_COUNT; ++s) a[s][0] = a[s][1] = f2(0.f);
+    for (int s = 0; s < NS; ++s) a[s][0] = a[s][1] = f2(0.f);
     constexpr int RC = SRC::ROWS < H_GROUP ? SRC::ROWS : H_GROUP;
     const int nch = (ti.rows + RC - 1) / RC;
+    // the row's sums -> x (in the order of W), the columns' -> a
+    auto row = [&](int r, float2 (&x)[NS]) {
+        constexpr int iR = W::index(S_R), iM = W::index(S_M), i2 = W::index(S_2), i4 = W::index(S_4), i6 = W::index(S_6),
+                      i3 = W::index(S_W3), i5 = W::index(S_W5);
+        float2 q[2];
+        src.load_row(r, lane, q);
+#pragma unroll
+        for (int k = 0; k < NS; ++k) x[k] = f2(0.f);
+        const float2 rm = f2(R[N_MU0][r]), rs = f2(STAGED ? R[N_MU][r] : 0.f), rr = f2(LIVE ? R[N_R][r] : 0.f),
+                     r3 = f2(R[N_W3][r]), r5 = f2(Q5 ? R[N_W5][r] : 0.f);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            a[iR][k] = fma2(q[k], rm, a[iR][k]);
+            x[iR] = fma2(q[k], cm[k], x[iR]);
+            if constexpr (STAGED) {
+                a[iM][k] = fma2(q[k], rs, a[iM][k]);
+                x[iM] = fma2(q[k], cs[k], x[iM]);
+            }
+            const float2 q2 = mul2(q[k], q[k]), q3 = mul2(q2, q[k]);
+            if constexpr (LIVE && !Q4) {
+                a[i2][k] = fma2(q2, rr, a[i2][k]);
+                x[i2] = fma2(q2, cr[k], x[i2]);
+            }
+            if constexpr (Q4) {
+                const float2 wi = mul2(q2, rr), wj = mul2(q2, cr[k]);
+                a[i2][k] = __fadd2_rn(a[i2][k], wi);
+                x[i2] = __fadd2_rn(x[i2], wj);
+                if constexpr (Q6) {
+                    const float2 wi2 = mul2(wi, wi), wj2 = mul2(wj, wj);
+                    a[i4][k] = __fadd2_rn(a[i4][k], wi2);
+                    x[i4] = __fadd2_rn(x[i4], wj2);
+                    a[i6][k] = fma2(wi2, wi, a[i6][k]);
+                    x[i6] = fma2(wj2, wj, x[i6]);
+                } else {
+                    a[i4][k] = fma2(wi, wi, a[i4][k]);
+                    x[i4] = fma2(wj, wj, x[i4]);
+                }
+            }
+            a[i3][k] = fma2(q3, r3, a[i3][k]);
+            x[i3] = fma2(q3, c3[k], x[i3]);
+            if constexpr (Q5) {
+                const float2 q5 = mul2(q3, q2);
+                a[i5][k] = fma2(q5, r5, a[i5][k]);
+                x[i5] = fma2(q5, c5[k], x[i5]);
+            }
+        }
+    };
+    const int k8 = (lane >> 2) & 7;   // the value that this lane has after a reduction
+    float* put = sm.rs[W::nth(ROWS == 2 ? k8 & 3 : k8) % S_COUNT];
+    const bool puts = (lane & 3) == 0 && (ROWS == 2 ? k8 & 3 : k8) < NS;
 #pragma unroll 1
     for (int c = 0; c < nch; ++c) {
         if (src.acquire(sm, ti, lane, c == 0)) {
-#pragma unroll 2
-            for (int s = 0; s < RC / 8; ++s) {
+#pragma unroll(ROWS == 2 ? 1 : 2)
+            for (int s = 0; s < RC / 8; s += ROWS) {
                 const int r = c * RC + 8 * s + cw;
-                float2 q[2], x[S_COUNT];
-                src.load_row(r, lane, q);
-#pragma unroll
-                for (int k = 0; k < S_COUNT; ++k) x[k] = f2(0.f);
-                const float2 rm = f2(R[N_MU0][r]), rs = f2(STAGED ? R[N_MU][r] : 0.f), rr = f2(LIVE ? R[N_R][r] : 0.f),
-                             r3 = f2(R[N_W3][r]), r5 = f2(R[N_W5][r]);
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    a[S_R][k] = fma2(q[k], rm, a[S_R][k]);
-                    x[S_R] = fma2(q[k], cm[k], x[S_R]);
-                    if (STAGED) {
-                        a[S_M][k] = fma2(q[k], rs, a[S_M][k]);
-                        x[S_M] = fma2(q[k], cs[k], x[S_M]);
-                    }
-                    const float2 q2 = mul2(q[k], q[k]), q3 = mul2(q2, q[k]), q5 = mul2(q3, q2);
-                    if (LIVE) {
-                        const float2 wi = mul2(q2, rr), wj = mul2(q2, cr[k]), wi2 = mul2(wi, wi), wj2 = mul2(wj, wj);
-                        a[S_2][k] = __fadd2_rn(a[S_2][k], wi);
-                        x[S_2] = __fadd2_rn(x[S_2], wj);
-                        a[S_4][k] = __fadd2_rn(a[S_4][k], wi2);
-                        x[S_4] = __fadd2_rn(x[S_4], wj2);
-                        a[S_6][k] = fma2(wi2, wi, a[S_6][k]);
-                        x[S_6] = fma2(wj2, wj, x[S_6]);
-                    }
-                    a[S_W3][k] = fma2(q3, r3, a[S_W3][k]);
-                    x[S_W3] = fma2(q3, c3[k], x[S_W3]);
-                    a[S_W5][k] = fma2(q5, r5, a[S_W5][k]);
-                    x[S_W5] = fma2(q5, c5[k], x[S_W5]);
-                }
                 float y[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) y[k] = k < S_COUNT ? x[k < S_COUNT ? k : 0].x + x[k < S_COUNT ? k : 0].y : 0.f;
+                for (int u = 0; u < ROWS; ++u) {
+                    float2 x[NS];
+                    row(r + 8 * u, x);
+#pragma unroll
+                    for (int k = 0; k < 8 / ROWS; ++k) y[8 / ROWS * u + k] = k < NS ? x[k < NS ? k : 0].x + x[k < NS ? k : 0].y : 0.f;
+                }
                 const float v = reduce_scatter8x(y, lane);
-                const int k = (lane >> 2) & 7;
-                if ((lane & 3) == 0 && k < S_COUNT) sm.rs[k][r] = v;
+                if (puts) put[r + (ROWS == 2 ? 8 * (k8 >> 2) : 0)] = v;
             }
         }
         src.release(sm, lane, c == nch - 1);
     }
 #pragma unroll
-    for (int s = 0; s < S_COUNT; ++s)
-        if (s == S_R || (s == S_M && STAGED) || ((s == S_2 || s == S_4 || s == S_6) && LIVE) || s == S_W3 || s == S_W5)
-            *reinterpret_cast<float4*>(&sm.cs[s][cw][4 * lane]) = make_float4(a[s][0].x, a[s][0].y, a[s][1].x, a[s][1].y);
+    for (int s = 0; s < NS; ++s)
+        *reinterpret_cast<float4*>(&sm.cs[W::nth(s)][cw][4 * lane]) = make_float4(a[s][0].x, a[s][0].y, a[s][1].x, a[s][1].y);
 }
 
 // Sum k of the thread's node: its row's (threads 0-127) and / or the eight
@@ -509,7 +565,7 @@ __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* 
         if (sm.info[slot].end) break;
         const HInfo& ti = sm.info[slot];
         const int kind = ti.kind, rows = ti.rows;
-        const bool diag = ti.I == ti.J, staged = ti.staged, wide = is_wide(kind), live = kind <= K_LIVE, even = ti.even;
+        const bool diag = ti.I == ti.J, staged = ti.staged, wide = is_wide(kind, staged), live = kind <= K_LIVE, even = ti.even;
         float* part = ti.part;
         const long long plen = ti.plen;
         // this thread's node of the tile's sums: row block's for the first 128
@@ -541,15 +597,22 @@ __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* 
             if (staged) sum_tile<false, true, true>(src, sm, ti, slot, base, cw, lane);
             else sum_tile<false, true, false>(src, sm, ti, slot, base, cw, lane);
         } else if (kind == K_LIVE0) {
-            sum_tile<true, false, false>(src, sm, ti, slot, base, cw, lane);
-        } else if (kind == K_LIVE1) {
+            if (staged) sum_tile<true, false, true>(src, sm, ti, slot, base, cw, lane);
+            else sum_tile<true, false, false>(src, sm, ti, slot, base, cw, lane);
+        } else if (!wide) {
             sum_tile<true, true, false>(src, sm, ti, slot, base, cw, lane);
         } else {
             hbar();   // the previous tile's sums are read out
-            if (kind == K_LIVE && staged) wide_tile<true, true>(src, sm, ti, slot, cw, lane);
-            else if (kind == K_LIVE) wide_tile<true, false>(src, sm, ti, slot, cw, lane);
-            else if (staged) wide_tile<false, true>(src, sm, ti, slot, cw, lane);
-            else wide_tile<false, false>(src, sm, ti, slot, cw, lane);
+            if (staged) {
+                if (kind == K_LIVE1) wide_tile<true, false, false, false, true>(src, sm, ti, slot, cw, lane);
+                else if (kind == K_LIVE4) wide_tile<true, true, false, false, true>(src, sm, ti, slot, cw, lane);
+                else if (kind == K_LIVE) wide_tile<true, true, true, true, true>(src, sm, ti, slot, cw, lane);
+                else wide_tile<false, false, false, true, true>(src, sm, ti, slot, cw, lane);
+            } else {
+                if (kind == K_LIVE4) wide_tile<true, true, false, false, false>(src, sm, ti, slot, cw, lane);
+                else if (kind == K_LIVE) wide_tile<true, true, true, true, false>(src, sm, ti, slot, cw, lane);
+                else wide_tile<false, false, false, true, false>(src, sm, ti, slot, cw, lane);
+            }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.tempty[slot]);   // its parameters are not read again
@@ -563,13 +626,14 @@ __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* 
             const float R = node_sum(sm, base, tid, rows, diag);
             if (mine) d[2 * plen] = R;
             if (kind != K_SUM || staged) {
-                // q mu of the stage or q^2; q^3
-                const float v1 = (staged || live) ? node_sum(sm, base + 1, tid, rows, diag) : 0.f;
-                const float v2 = (kind == K_ONE || kind == K_LIVE1) ? node_sum(sm, base + 2, tid, rows, diag) : 0.f;
-                const float E = r1 * (fmaf(S4, D1, v2) + r1 * S6 * (D3 - 3.f * D1));
+                const float M = staged ? node_sum(sm, base + 1, tid, rows, diag) : 0.f;
+                const float S2 = live ? node_sum(sm, base + 1 + staged, tid, rows, diag) : 0.f;
+                const float W3 = (kind == K_ONE || kind == K_LIVE1) ? node_sum(sm, base + 2, tid, rows, diag) : 0.f;
+                const float E = r1 * (fmaf(S4, D1, W3) + r1 * S6 * (D3 - 3.f * D1));
+                if (live) P = -S2;
                 if (mine) {
-                    if (live) d[0] = -v1;
-                    if (staged) d[plen] = fmaf(P, mu1, E - v1);
+                    if (live) d[0] = P;
+                    if (staged) d[plen] = fmaf(P, mu1, E - M);
                     else if (kind != K_LIVE0) d[plen] = E;
                 }
             }
@@ -580,11 +644,12 @@ __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* 
                 const float S2 = node_sum(sm, S_2, tid, rows, diag);
                 if (even && s46) {
                     S4 = node_sum(sm, S_4, tid, rows, diag);
-                    S6 = node_sum(sm, S_6, tid, rows, diag);
+                    S6 = kind == K_LIVE ? node_sum(sm, S_6, tid, rows, diag) : 0.f;
                 }
                 P = fmaf(r1, fmaf(-2.f * r1, S6, S4), -S2);
             }
-            const float W3 = node_sum(sm, S_W3, tid, rows, diag), W5 = node_sum(sm, S_W5, tid, rows, diag);
+            const float W3 = node_sum(sm, S_W3, tid, rows, diag);
+            const float W5 = kind == K_LIVE || kind == K_TWO ? node_sum(sm, S_W5, tid, rows, diag) : 0.f;
             const float E = r1 * (fmaf(S4, D1, W3) + r1 * fmaf(S6, D3 - 3.f * D1, W5));
             if (mine) {
                 d[2 * plen] = R;

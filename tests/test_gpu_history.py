@@ -96,3 +96,19 @@ def test_forms_reach_the_solve(kw, n, m, g):
     assert s.stats()["converged"] == 1
     ref = np.linalg.solve(Q, b)
     assert np.max(np.abs(s.mean() - ref)) <= REL * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("n,g", [(900, 2.0), (1410, 0.5), (1665, 0.1)])
+@pytest.mark.parametrize("stages", [1, 3])
+def test_rounds_of_fewer_orders_match_oracle(n, g, stages):
+    """Larger sets, whose live rounds sum fewer and fewer orders (q^2 to q^4 with
+    q^3, q^2 and q^3, q^2 alone), on both schedules."""
+    p = _problem(n, 8, g, 0)
+    Q = oracle.build_q(p.X.astype(np.float64), p.y.astype(np.float64), p.gamma, p.C)
+    s = gabp.GabpSVM(p.X, p.y, p.gamma, p.C, stages=stages)
+    for iters in (1, 2, 3, 5, 12):
+        s.refit(p.X, p.y, p.gamma, p.C)
+        s.solve(iters, 0.0)
+        r = (oracle.gabp(Q, np.ones(n), iters=iters) if stages == 1
+             else oracle.gabp_staged(Q, np.ones(n), iters=iters, stages=stages, block=128))
+        assert np.max(np.abs(s.mean() - r.mu)) <= REL * np.max(np.abs(r.mu)), iters
