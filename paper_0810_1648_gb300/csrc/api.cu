@@ -963,6 +963,7 @@ gabp_status gabp_svm_solve(gabp_svm_t h, int32_t iters, double tol, float* alpha
                            h->opts.ptr_mode == 1 ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    if (h->hctrl->status == ST_ETIMEOUT) return fail(GABP_ETIMEOUT, "a bounded device wait ran out in the final pass");
     h->solved = true;
     h->mean_src = mu;
     gabp_svm_stats& S = h->stats;

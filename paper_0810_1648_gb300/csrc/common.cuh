@@ -396,8 +396,10 @@ cudaError_t launch_pack_list(const Inst* tab, const int2* nbl, int nblocks, cuda
 void launch_init_list(const Inst* tab, const int2* nbl, int nblocks, int diag_rule, float delta, cudaStream_t s);
 // Arms listed instances: list entries {slot, iters} with their tolerances.
 void launch_begin_list(Inst* tab, const int2* list, const double* tols, int count, cudaStream_t s);
-// q mu and q alpha slot sums (part[2], part[3]) of the listed tiles, Q from the
-// FP32-accurate Gram (forms that do not store it).
+// q mu and q alpha slot sums (part[2], part[3]) of the listed tiles: Q from the
+// stored FP32 entries (sweep_hist.cu), or from the FP32-accurate Gram (forms that
+// do not store it, gram_tc32.cu).
+void launch_final_tiles_q(const Inst* tab, const StopOp* ops, const int4* tiles, long long ntiles, cudaStream_t s);
 cudaError_t launch_final_tiles_gram(const Inst* tab, const StopOp* ops, const int4* tiles, long long ntiles, cudaStream_t s);
 // Decision values of t test rows using alpha: tab = {the test rows as an
 // instance (n = t, Xp3 packed, sq3 to fill), the training instance}, diag = {0,

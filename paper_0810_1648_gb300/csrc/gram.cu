@@ -29,17 +29,6 @@ struct GramSmem {
     float B[2][KC][T + 4];
 };
 
-struct EpiSmem {
-    float rowv[2][T];
-    float colw[NWARPS][2][T];
-    float colv[2][T];
-};
-
-union TileSmem {
-    GramSmem g;
-    EpiSmem e;
-};
-
 // acc[a][b] = <x_{I*T + ty*8 + a}, x_{J*T + tx*8 + b}>.  K-chunks of KC
 // features go through two shared-memory buffers: the next chunk's global
 // loads are in flight (in registers) while the current chunk's FMAs run, and
@@ -114,137 +103,12 @@ __device__ __forceinline__ float sum16(float v)
     return v;
 }
 
-// Row sums (rs, per thread's 8 rows) and column sums (cs, per thread's 8
-// columns) of up to two quantities -> per-node slot partials part_q[k][x].
-template <int NQ>
-__device__ __forceinline__ void reduce_and_write(EpiSmem& es, float (&rs)[NQ][8], float (&cs)[NQ][8],
-                                                 float* const (&part)[NQ], int n, int I, int J, int2 sl)
-{
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, warp = tid >> 5, lane = tid & 31;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q)
-#pragma unroll
-        for (int a = 0; a < 8; ++a) {
-            const float v = sum16(rs[q][a]);
-            if (tx == 0) es.rowv[q][ty * 8 + a] = v;
-        }
-#pragma unroll
-    for (int q = 0; q < NQ; ++q)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            const float v = cs[q][b] + __shfl_xor_sync(0xffffffffu, cs[q][b], 16);
-            if (lane < 16) es.colw[warp][q][tx * 8 + b] = v;
-        }
-    __syncthreads();
-    if (tid < T) {
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            float s = 0.f;
-#pragma unroll
-            for (int w = 0; w < NWARPS; ++w) s += es.colw[w][q][tid];
-            es.colv[q][tid] = s;
-        }
-    }
-    __syncthreads();
-    // slot sl.x of the row block (its nodes I T + r), sl.y of the column block
-    const size_t oR = (size_t)sl.x * T, oC = (size_t)sl.y * T;
-    if (I == J) {
-        if (tid < T) {
-            const int x = I * T + tid;
-            if (x < n)
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) part[q][oR + tid] = es.rowv[q][tid] + es.colv[q][tid];
-        }
-    } else {
-        if (tid < T) {
-            const int x = I * T + tid;
-            if (x < n)
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) part[q][oR + tid] = es.rowv[q][tid];
-        } else {
-            const int c = tid - T, x = J * T + c;
-            if (x < n)
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) part[q][oC + c] = es.colv[q][c];
-        }
-    }
-}
-
-// ------------------------------------------- final residual and Q alpha
-// For every instance k listed: off-diagonal sums sum_{j != i} Q_ij mu_j
-// (-> part[2], the residual slots every round writes anew) and sum_{j != i}
-// Q_ij alpha_j (-> part[3]): the P and H slots keep the sums of the current
-// messages, which a staged round that goes on from here reads.
-//
-// Per listed tile: partial sums of (Q mu)_i and (Q alpha)_i over the tile's
-// pairs (both roles) into the slot partials, with alpha = clip(mu, 0, C) and
-// mu = ops[k].mu, from the tile's stored FP32 Q values in acc (instances that do
-// not store Q: gram_tc32.cu).
-__device__ __forceinline__ void final_tile_sums(const Inst& p, const float* __restrict__ mu, int4 w,
-                                                float (&acc)[8][8], EpiSmem& es)
-{
-    const int n = p.n, I = w.y, J = w.z;
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    float mj[8], aj[8];
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const int j = J * T + tx * 8 + b;
-        mj[b] = j < n ? mu[j] : 0.f;
-        aj[b] = p.task ? mj[b] : fminf(fmaxf(mj[b], 0.f), p.C);
-    }
-    float rs[2][8], cs[2][8];
-#pragma unroll
-    for (int b = 0; b < 8; ++b) cs[0][b] = cs[1][b] = 0.f;
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-        const int r = ty * 8 + a, i = I * T + r;
-        const float mi = i < n ? mu[i] : 0.f, ai = p.task ? mi : fminf(fmaxf(mi, 0.f), p.C);
-        float rm = 0.f, ra = 0.f;
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            const int c = tx * 8 + b, j = J * T + c;
-            const bool v = i < n && j < n && (I != J || c > r);
-            const float q = v ? acc[a][b] : 0.f;
-            rm = fmaf(q, mj[b], rm);
-            ra = fmaf(q, aj[b], ra);
-            cs[0][b] = fmaf(q, mi, cs[0][b]);
-            cs[1][b] = fmaf(q, ai, cs[1][b]);
-        }
-        rs[0][a] = rm;
-        rs[1][a] = ra;
-    }
-    float* const parts[2] = {p.part + 2 * part_len(p), p.part + 3 * part_len(p)};
-    reduce_and_write<2>(es, rs, cs, parts, n, I, J, tile_slots(p, w));
-}
-
-// Q read back from the FP32 tiles (Inst::qref): no Gram, small footprint, so
-// several CTAs share an SM and the pass runs at memory speed.
-__global__ void __launch_bounds__(NTHREADS, 2) k_final_tiles_q(const Inst* __restrict__ tab,
-                                                               const StopOp* __restrict__ ops,
-                                                               const int4* __restrict__ work)
-{
-    __shared__ __align__(16) EpiSmem es;
-    const int4 w = work[blockIdx.x];
-    const Inst& p = tab[w.x];
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    const float* qt = p.qref + (size_t)w.w * TT;
-    float acc[8][8];
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-        const float4 u0 = *reinterpret_cast<const float4*>(qt + (ty * 8 + a) * T + tx * 8);
-        const float4 u1 = *reinterpret_cast<const float4*>(qt + (ty * 8 + a) * T + tx * 8 + 4);
-        acc[a][0] = u0.x; acc[a][1] = u0.y; acc[a][2] = u0.z; acc[a][3] = u0.w;
-        acc[a][4] = u1.x; acc[a][5] = u1.y; acc[a][6] = u1.z; acc[a][7] = u1.w;
-    }
-    final_tile_sums(p, ops[w.x].mu, w, acc, es);
-}
-
 // k_pair_z (sweep_hist.cu) for instances that do not store Q (only those that
 // their margin leaves open get as far as the Gram tile).
 __global__ void __launch_bounds__(NTHREADS) k_pair_z_gram(const Inst* __restrict__ tab, const int4* __restrict__ work,
                                                           long long ntiles, bool single)
 {
-    __shared__ __align__(16) TileSmem sm;
+    __shared__ __align__(16) GramSmem sm;
     __shared__ int s_go;
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
     if (single) {
@@ -264,7 +128,7 @@ __global__ void __launch_bounds__(NTHREADS) k_pair_z_gram(const Inst* __restrict
             if (!go) continue;
             float acc[8][8];
             const GramSide S{p.X, p.sq3, p.n};
-            gram_tile(S, S, p.m, w.y, w.z, sm.g, acc);
+            gram_tile(S, S, p.m, w.y, w.z, sm, acc);
             float best[2] = {0.f, FLT_MIN};   // the second never 0: the pass has run
 #pragma unroll
             for (int a = 0; a < 8; ++a) {
@@ -287,6 +151,23 @@ __global__ void __launch_bounds__(NTHREADS) k_pair_z_gram(const Inst* __restrict
     }
 }
 
+// Sum of FP32 values to more than FP64's bits without the FP64 pipe, which on
+// this chip adds about two values a clock and SM: two error-free additions
+// (Knuth) leave the rounding of a rounding error to the third word.  n = 100000
+// (782 slots a node): 0.60 ms in FP64 additions, now 0.12.
+struct Sum3 {
+    float s = 0.f, e = 0.f, d = 0.f;
+    __device__ __forceinline__ static float two_sum(float& a, float x)
+    {
+        const float t = a + x, b = t - a;
+        const float err = (a - (t - b)) + (x - b);
+        a = t;
+        return err;
+    }
+    __device__ __forceinline__ void add(float x) { d += two_sum(e, two_sum(s, x)); }
+    __device__ __forceinline__ double value() const { return isfinite(s) ? (double)s + ((double)e + (double)d) : (double)s; }
+};
+
 // Per node of a listed node block: r_i = b0_i - Q_ii mu_i - sum part0,
 // (Q alpha)_i = Q_ii alpha_i + sum part1; writes alpha (and r in FP32 when
 // requested); block partials {max |r_i|, sum b0_i alpha_i - 1/2 alpha_i
@@ -303,20 +184,21 @@ __global__ void __launch_bounds__(256) k_final_nodes(const Inst* __restrict__ ta
     const float* __restrict__ mu = op.mu;
     const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
     const int x = nb.y * 32 + lane, n = p.n;
-    double s0 = 0.0, s1 = 0.0;
+    Sum3 s0, s1;
     if (x < n) {
         // the node's slots (see slot_begin)
         const int X = x / T, ns = slot_count(p, X);
         const float* p0 = p.part + 2 * part_len(p) + (size_t)slot_begin(p, X) * T + (x - X * T);
         const float* p1 = p0 + part_len(p);
+#pragma unroll 4
         for (int k = g; k < ns; k += 8) {
-            s0 += (double)p0[(size_t)k * T];
-            s1 += (double)p1[(size_t)k * T];
+            s0.add(p0[(size_t)k * T]);
+            s1.add(p1[(size_t)k * T]);
         }
     }
     __shared__ double red[2][8][32];
-    red[0][g][lane] = s0;
-    red[1][g][lane] = s1;
+    red[0][g][lane] = s0.value();
+    red[1][g][lane] = s1.value();
     __syncthreads();
     if (g == 0) {
         double absr = 0.0, obj = 0.0, nsv = 0.0;
@@ -376,6 +258,8 @@ __global__ void k_final_reduce(const Inst* __restrict__ tab, const StopOp* __res
         __syncthreads();
     }
     if (tid == 0) {
+        // tile sums that a bounded wait left out: no residual to go by
+        if (tab[slot].ctrl->status == ST_ETIMEOUT) s[0][0] = INFINITY;
         for (int q = 0; q < 3; ++q) {
             op.final3[q] = s[q][0];
             if (f3_all) f3_all[3 * slot + q] = s[q][0];
@@ -418,7 +302,7 @@ void launch_final(const Inst* tab, const StopOp* ops, const int4* tiles, long lo
 {
     if (ntiles > 0) {
         if (q_stored)
-            k_final_tiles_q<<<(unsigned)ntiles, NTHREADS, 0, s>>>(tab, ops, tiles);
+            launch_final_tiles_q(tab, ops, tiles, ntiles, s);
         else
             (void)launch_final_tiles_gram(tab, ops, tiles, ntiles, s);   // errors surface at the caller's cudaGetLastError
     }

@@ -68,8 +68,10 @@ struct HInfo {
     long long plen;
     Ctrl* ctrl;
     long long L;
-    int npad, I, J, sR, sC, rows;
+    int npad, I, J, sR, sC, rows;   // (npad: n in the final pass)
     int t, kind, even, staged, end;
+    float C;               // final pass: the box, and whether there is none (task)
+    int task;
 };
 
 struct HTail {
@@ -92,11 +94,13 @@ __host__ __device__ constexpr int q_rows<void>() { return T; }
 // Producer (one warp): publishes each tile's parameters with the values of its
 // row and column nodes and, where Q is stored, streams its rows (whole:
 // entries outside the pair set are stored as 0) in 16 KB copies, ahead across
-// tiles.  QT = void: Q is recomputed elsewhere.
-template <typename QT>
+// tiles.  QT = void: Q is recomputed elsewhere.  FINAL: for the final pass, the
+// FP32 entries and the means ops[k].mu of every listed tile, whatever the
+// instance's state.
+template <typename QT, bool FINAL = false>
 __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, const int4* __restrict__ work,
                                               long long ntiles, HTail& sm, unsigned char* ring, volatile int* abort_flag,
-                                              int lane, int st)
+                                              int lane, int st, const StopOp* __restrict__ ops = nullptr)
 {
     constexpr bool STREAM = q_rows<QT>() < T;
     const uint64_t pol = l2_evict_first_policy(), pol_keep = l2_evict_last_policy();
@@ -122,7 +126,10 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
         if (L + gridDim.x < ntiles) wn = work[L + gridDim.x];
         const Inst& p = tab[w.x];
         Ctrl* ctrl = p.ctrl;
-        if (w.x != inst) {
+        if (FINAL) {
+            done = false;
+            use = 1u << N_MU0;
+        } else if (w.x != inst) {
             inst = w.x;
             done = *(volatile const int*)&ctrl->done != 0;
             t = *(volatile const int*)&ctrl->t;
@@ -146,13 +153,18 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
         }
         if (lane == 0) {
             HInfo& ti = sm.info[slot];
-            ti.ring = p.hring + hist_offset(p.npad, st, 0);
+            if (FINAL) {
+                ti.C = p.C;
+                ti.task = p.task;
+            } else {
+                ti.ring = p.hring + hist_offset(p.npad, st, 0);
+                ti.s46 = p.hs46;
+            }
             ti.part = p.part;
-            ti.s46 = p.hs46;
             ti.plen = (long long)part_len(p);
             ti.ctrl = ctrl;
             ti.L = L;
-            ti.npad = p.npad; ti.I = I; ti.J = J;
+            ti.npad = FINAL ? p.n : p.npad; ti.I = I; ti.J = J;
             const int2 sl = tile_slots(p, w);
             ti.sR = sl.x; ti.sC = sl.y;
             ti.rows = rows;
@@ -167,7 +179,8 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
         const int a = lane >> 1;
         if ((use >> a) & 1u) {
             const size_t np = p.npad;
-            const float* src = a == N_MU0  ? p.agg + (size_t)(t & 1) * 3 * np + 2 * np
+            const float* src = FINAL       ? ops[w.x].mu
+                               : a == N_MU0 ? p.agg + (size_t)(t & 1) * 3 * np + 2 * np
                                : a == N_MU ? hist_slot(p, st, t) + 2 * np
                                            : p.hnow + (3 * (size_t)st + (a - N_R)) * np;
             bulk_load(&sm.node[slot][lane & 1][a][0], src + (size_t)((lane & 1) ? J : I) * T, T * sizeof(float),
@@ -176,7 +189,8 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
         if (++slot == 2) { slot = 0; tph ^= 1u; }
         if constexpr (STREAM) {
             constexpr int RC = q_rows<QT>();
-            const unsigned char* qt = static_cast<const unsigned char*>(p.qstore) + (size_t)w.w * TT * sizeof(QT);
+            const void* store = FINAL ? p.qref : p.qstore;
+            const unsigned char* qt = static_cast<const unsigned char*>(store) + (size_t)w.w * TT * sizeof(QT);
             const int nch = (rows + RC - 1) / RC;
             for (int c = 0; c < nch; ++c) {
                 if (!mbar_wait_warp(&sm.empty[stage], phase ^ 1u)) {
@@ -538,6 +552,51 @@ __device__ __forceinline__ float node_sum(const HTail& sm, int k, int tid, int r
     return v;
 }
 
+// ---- final pass
+// Sums q mu and q alpha, alpha = clip(mu, 0, C) (regression: mu), of a tile of
+// stored FP32 entries, as sum_tile does it.  Means of nodes beyond n are not
+// read as they are (nobody writes them): they count as 0.
+template <class SRC>
+__device__ __forceinline__ void final_tile(SRC& src, HTail& sm, const HInfo& ti, int slot, int base, int cw, int lane)
+{
+    const int hl = lane & 15, rows = ti.rows, cols = ti.npad - ti.J * T;
+    const float* R = sm.node[slot][0][N_MU0];
+    const float C = ti.C;
+    const bool box = ti.task == 0;
+    auto clip = [&](float v) { return box ? fminf(fmaxf(v, 0.f), C) : v; };
+    float2 cm[4], ca[4], aR[4], aA[4];
+    ld_cols(sm.node[slot][1][N_MU0], hl, cm);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int c = (k >= 2 ? 64 : 0) + 4 * hl + 2 * (k & 1);
+        cm[k] = make_float2(c < cols ? cm[k].x : 0.f, c + 1 < cols ? cm[k].y : 0.f);
+        ca[k] = make_float2(clip(cm[k].x), clip(cm[k].y));
+        aR[k] = aA[k] = f2(0.f);
+    }
+    float xR[4] = {0.f, 0.f, 0.f, 0.f}, xA[4] = {0.f, 0.f, 0.f, 0.f};
+    auto row = [&](const float2 (&q)[4], int r, int step) {
+        const float m = r < rows ? R[r] : 0.f;
+        const float2 am = f2(m), aa = f2(clip(m));
+        float2 sR = f2(0.f), sA = f2(0.f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            aR[k] = fma2(q[k], am, aR[k]);
+            sR = fma2(q[k], cm[k], sR);
+            aA[k] = fma2(q[k], aa, aA[k]);
+            sA = fma2(q[k], ca[k], sA);
+        }
+        xR[step] = sR.x + sR.y;
+        xA[step] = sA.x + sA.y;
+    };
+    auto group = [&](int r0) {
+        put_rows(sm.rs[base], xR, r0, cw, lane);
+        put_rows(sm.rs[base + 1], xA, r0, cw, lane);
+    };
+    walk_tile(src, sm, ti, cw, lane, row, group);
+    put_cols(sm.cs[base][cw], aR, lane);
+    put_cols(sm.cs[base + 1][cw], aA, lane);
+}
+
 // The eight consumer warps: tile after tile as the producer publishes them,
 // each tile's sums to its slots in a fixed order.  One barrier a tile: a warp
 // that has put its sums away waits for the next tile to be published, and the
@@ -658,6 +717,43 @@ __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* 
                 d[plen] = staged ? fmaf(P, mu1, E - M) : E;
             }
             hbar();   // before the next tile writes its sums
+        }
+        base = S_SMALL - base;
+    }
+}
+
+// The consumers of the final pass: as hist_consumers, sums to the slots 2 and 3.
+template <class SRC>
+__device__ __forceinline__ void final_consumers(SRC& src, HTail& sm, const Inst* __restrict__ tab,
+                                                const int4* __restrict__ work, long long ntiles, int tid)
+{
+    const int cw = tid >> 5, lane = tid & 31;
+    int slot = 0, base = 0;
+    uint32_t tph = 0;
+    auto await_tile = [&]() {
+        if (!mbar_wait_warp(&sm.tfull[slot], tph) && lane == 0) {
+            sm.cabort = 1;
+            if (blockIdx.x < ntiles) record_error(tab[work[blockIdx.x].x].ctrl, ST_ETIMEOUT, -1);
+        }
+    };
+    await_tile();
+    hbar();
+    while (!*(volatile int*)&sm.cabort && !sm.info[slot].end) {
+        const HInfo& ti = sm.info[slot];
+        const bool diag = ti.I == ti.J;
+        const int rows = ti.rows;
+        const long long plen = ti.plen;
+        float* d = ti.part + (size_t)(tid < T ? ti.sR : ti.sC) * T + (tid & (T - 1));
+        final_tile(src, sm, ti, slot, base, cw, lane);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.tempty[slot]);
+        if (++slot == 2) { slot = 0; tph ^= 1u; }
+        await_tile();
+        hbar();
+        const float R = node_sum(sm, base, tid, rows, diag), A = node_sum(sm, base + 1, tid, rows, diag);
+        if (tid < T || !diag) {
+            d[2 * plen] = R;
+            d[3 * plen] = A;
         }
         base = S_SMALL - base;
     }
@@ -932,6 +1028,34 @@ __global__ void __launch_bounds__(HR_THREADS, 1)
     }
 }
 
+// Final pass over listed tiles of stored FP32 entries: off-diagonal sums
+// sum_{j != i} Q_ij mu_j (the residual slots, which every round writes anew) and
+// sum_{j != i} Q_ij alpha_j (slots 3): the P and H slots keep the sums of the
+// current messages, which a staged round that goes on from here reads.
+//
+// What bounds it: one read of the entries, 4 bytes a pair, so it streams them as
+// a round does.  With a CTA a tile that loaded its 64 KB at once: 178 us at n =
+// 20000, 4.2 ms at n = 100000; now 121 us and 3.0 ms.
+__global__ void __launch_bounds__(H_THREADS, 2)
+    k_final_tiles_q(const Inst* __restrict__ tab, const StopOp* __restrict__ ops, const int4* __restrict__ work, long long ntiles)
+{
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* ring = align_smem(smem_raw, 128);
+    HTail& sm = *reinterpret_cast<HTail*>(ring + H_STAGES * H_CHUNK);
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        init_htail(sm);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    if (tid >= HCW * 32) {
+        hist_producer<float, true>(tab, work, ntiles, sm, ring, nullptr, tid & 31, 0, ops);
+        return;
+    }
+    StreamedQ<float> src{ring, 0, 0u, false};
+    final_consumers(src, sm, tab, work, ntiles, tid);
+}
+
 // What choose_path() wants to know of the pairs, over listed tiles, for the
 // instances whose margin leaves it open (the others cost a look at their
 // control block).  From the FP32 entries, so that the forms with BF16 entries
@@ -991,6 +1115,8 @@ cudaError_t prepare_sweep_hist()
         e = cudaFuncSetAttribute(k_sweep_hist<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)hist_smem_bytes());
     if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_final_tiles_q, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hist_smem_bytes());
+    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_sweep_hist_rc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hist_rc_smem_bytes());
     return e;
 }
@@ -1005,6 +1131,12 @@ void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, in
                        stage_no);
     else
         launch_chained(chained, k_sweep_hist<float>, grid, H_THREADS, hist_smem_bytes(), s, tab, work, sched, stage_no);
+}
+
+void launch_final_tiles_q(const Inst* tab, const StopOp* ops, const int4* tiles, long long ntiles, cudaStream_t s)
+{
+    const long long most = 2 * num_sms();
+    k_final_tiles_q<<<(int)(ntiles < most ? ntiles : most), H_THREADS, hist_smem_bytes(), s>>>(tab, ops, tiles, ntiles);
 }
 
 void launch_pair_z(const Inst* tab, const int4* tiles, long long ntiles, int q_mode, bool single, cudaStream_t s)
