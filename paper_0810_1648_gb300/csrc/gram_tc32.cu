@@ -41,6 +41,7 @@
 // accumulators handed over at once) two warps a scheduler left it waiting.
 #include "common.cuh"
 #include "ptx.cuh"
+#include "qtile_epi.cuh"
 
 #include <float.h>
 
@@ -273,65 +274,93 @@ struct T3Smem {
 
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(T3_EPI_WARPS * 32) : "memory"); }
 
-// After it, lane l of the warp holds the sum over the 32 lanes of v[l]
-// (a fixed butterfly: 31 shuffles for 32 values).
-__device__ __forceinline__ float transpose_sum32(float (&v)[32], int lane)
+// ---- epilogue
+// A warp has 32 rows (its lane quarter of TMEM) x 32 columns of the tile, in
+// the layout of 16 x 256-bit loads: lane (lr = lane / 4, lq = lane % 4) holds
+// rows 8 k + lr, k = 0..3, and columns 8 j + 2 lq and the next, j = 0..3, as
+// pairs.  Four rows and eight columns a lane leave little to reduce across lanes
+// (ten shuffles for the tile's row and column sums, where one row of 32 columns
+// a lane took 31), and the pairs go through two-wide arithmetic.
+struct Frag {
+    float2 v[4][4];   // [k][j]
+};
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, Frag& f)
 {
 #pragma unroll
-    for (int w = 16; w >= 1; w >>= 1) {
-        const bool hi = (lane & w) != 0;
+    for (int h = 0; h < 2; ++h) {
+        uint32_t r[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+            "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(taddr + ((uint32_t)(16 * h) << 16))
+            : "memory");
 #pragma unroll
-        for (int k = 0; k < w; ++k) {
-            const float send = hi ? v[k] : v[k + w];
-            const float keep = hi ? v[k + w] : v[k];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, w);
-        }
-    }
-    return v[0];
-}
-
-// FP32 Q entries of 32 columns of one tile row from the Gram values g,
-// the staged column sign bits sy and norms sn: q = y_i y_j (exp(-gamma d2) +
-// lambda^2), d2 = max(0, ||x_i||^2 + ||x_j||^2 - 2 g); the label product is a
-// flip of the sign bit (y = +-1).  Not FULL: entries outside the pair set
-// (i >= n, column j0 + cb + c >= n, or c + cb <= rdiag on a diagonal tile)
-// are 0.  Adds |q| to the row sums rs4[c % 4].
-template <bool FULL>
-__device__ __forceinline__ void q_chunk32(const float* g, const uint32_t* sy, const float* sn, float si, uint32_t syi,
-                                          float ngam, float lam2, int i, int n, int cb, int j0, int rdiag,
-                                          float (&q)[32], float (&rs4)[4])
-{
+        for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int c4 = 0; c4 < 32; c4 += 4) {
-        const uint4 y4 = *reinterpret_cast<const uint4*>(sy + c4);
-        const float4 s4 = *reinterpret_cast<const float4*>(sn + c4);
-        const uint32_t yj[4] = {y4.x, y4.y, y4.z, y4.w};
-        const float sj[4] = {s4.x, s4.y, s4.z, s4.w};
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const float d2 = fmaxf(0.f, si + sj[t] - 2.f * g[c4 + t]);
-            const float e = expf(ngam * d2) + lam2;
-            float qv = __uint_as_float(__float_as_uint(e) ^ syi ^ yj[t]);
-            if (!FULL) {
-                const int c = cb + c4 + t;
-                const bool valid = i < n && j0 + c < n && c > rdiag;
-                qv = valid ? qv : 0.f;
-            }
-            q[c4 + t] = qv;
-            rs4[t] += fabsf(qv);
-        }
+            for (int k = 0; k < 2; ++k)
+                f.v[2 * h + k][j] = make_float2(__uint_as_float(r[4 * j + 2 * k]), __uint_as_float(r[4 * j + 2 * k + 1]));
     }
 }
 
-// 32 consecutive floats of a row, eight per store (a whole 32-byte sector).
-__device__ __forceinline__ void store_row32(float* d, const float (&q)[32])
+// exp(-gamma d2) + lam2 of two entries, d2 = max(0, si + sj - 2 g).
+struct Rbf {
+    float ngam, lam2;
+};
+__device__ __forceinline__ Rbf rbf_of(float gamma, float lam2) { return Rbf{-gamma, lam2}; }
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 rbf2(const Rbf& b, float2 g, float si, float2 sj)
 {
-#pragma unroll
-    for (int c = 0; c < 32; c += 8)
-        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d + c), "f"(q[c]), "f"(q[c + 1]),
-                     "f"(q[c + 2]), "f"(q[c + 3]), "f"(q[c + 4]), "f"(q[c + 5]), "f"(q[c + 6]), "f"(q[c + 7])
-                     : "memory");
+    const float2 d = __ffma2_rn(f2(-2.f), g, __fadd2_rn(f2(si), sj));
+    const float2 t = __fmul2_rn(f2(b.ngam), make_float2(fmaxf(0.f, d.x), fmaxf(0.f, d.y)));
+    return __fadd2_rn(make_float2(expf(t.x), expf(t.y)), f2(b.lam2));
 }
+__device__ __forceinline__ float2 flip(float2 v, uint32_t sx, uint32_t sy)
+{
+    return make_float2(__uint_as_float(__float_as_uint(v.x) ^ sx), __uint_as_float(__float_as_uint(v.y) ^ sy));
+}
+__device__ __forceinline__ float2 ld2(const float* x) { return *reinterpret_cast<const float2*>(x); }
+
+// Sums over the four lanes of a row group: lane lq has that of value lq (rows 8 lq + lr).
+__device__ __forceinline__ float row_sums4(const float2 (&x)[4], int lane)
+{
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = x[k].x + x[k].y;
+    const bool b2 = (lane & 2) != 0, b1 = (lane & 1) != 0;
+    float y[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        y[k] = (b2 ? v[k + 2] : v[k]) + __shfl_xor_sync(0xffffffffu, b2 ? v[k] : v[k + 2], 2);
+    return (b1 ? y[1] : y[0]) + __shfl_xor_sync(0xffffffffu, b1 ? y[0] : y[1], 1);
+}
+// Sums over the eight lanes that share columns: lane lr has that of value lr of
+// {x[0].x, x[0].y, x[1].x, ...}, column 8 (lr / 2) + 2 lq + lr % 2.
+__device__ __forceinline__ float col_sums8(const float2 (&x)[4], int lane)
+{
+    const bool b16 = (lane & 16) != 0, b8 = (lane & 8) != 0, b4 = (lane & 4) != 0;
+    float2 y[2], z;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const float2 keep = b16 ? x[k + 2] : x[k], send = b16 ? x[k] : x[k + 2];
+        y[k].x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, 16);
+        y[k].y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, 16);
+    }
+    const float2 keep = b8 ? y[1] : y[0], send = b8 ? y[0] : y[1];
+    z.x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, 8);
+    z.y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, 8);
+    return (b4 ? z.y : z.x) + __shfl_xor_sync(0xffffffffu, b4 ? z.x : z.y, 4);
+}
+
+// Running compensated sum s + c (+ e) += x + xc.
+__device__ __forceinline__ void add_pair(float& s, float& c, float x, float xc)
+{
+    const float t = s + x, bp = t - s;
+    c += (s - (t - bp)) + (x - bp) + xc;
+    s = t;
+}
+
 
 // The decision's operands: tab[0] describes the test rows as an instance (n,
 // Nt, nkc, Xp3, sq3), tab[1] is the training set; a work entry {0, I, J0, J1}
@@ -444,7 +473,8 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
         // warp w reads TMEM lanes 32 (w % 4) ..: rows 32 g + lane, columns
         // [32 cg, 32 cg + 32)
         const int ew = warp - 2, g = warp & 3, cg = ew >> 2;
-        const int r = 32 * g + lane, c0 = 32 * cg;
+        const int lr = lane >> 2, lq = lane & 3, c0 = 32 * cg;
+        const int r0 = 32 * g + lr, cq = c0 + 2 * lq;   // the lane's first row and column
         const int etid = tid - 64;
         uint32_t aph = 0;
         int buf = 0;
@@ -487,10 +517,11 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
         epi_bar();
         for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
             const int4 w = wn;
-            const int nkc = tab[w.x].nkc, I = w.y, i = I * T + r;
+            const int nkc = tab[w.x].nkc, I = w.y;
             const bool more = L + gridDim.x < ntiles;
             if (more) wn = work[L + gridDim.x];
-            float fs = 0.f, fc = 0.f;   // decision: the row's compensated sum over its training tiles
+            // decision: the rows' compensated sums over the training tiles
+            float fs[4] = {0.f, 0.f, 0.f, 0.f}, fc[4] = {0.f, 0.f, 0.f, 0.f};
             bool ok = true;
             for (int J = first_j(w); J < last_j(w) && ok; ++J) {
                 // the item that follows: an instance sharing the tile, the row's next
@@ -499,7 +530,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                 if (MODE == T3_DECIDE && J + 1 < last_j(w)) { kn = w.x; Jn = J + 1; }
                 if (kn < 0 && more) { kn = wn.x; In = wn.y; Jn = first_j(wn); }
                 if (kn >= 0) fetch(buf ^ 1, kn, In, Jn);
-                float ga[32];
+                Frag G;
                 for (int kc = 0; kc < nkc && ok; ++kc) {
                     const bool stop = __shfl_sync(0xffffffffu, *(volatile int*)&sm.abort, 0) != 0;
                     // the chunk's accumulators added to the running sums in order
@@ -507,22 +538,19 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                     for (int a = 0; a < T3_NACC; ++a) {
                         if (stop || !mbar_wait_warp(&sm.accfull[a], aph)) { ok = false; break; }
                         tc_fence_after();
-                        float v[32];
-                        tmem_ld32(tbase + (uint32_t)a * T + ((uint32_t)(32 * g) << 16) + (uint32_t)c0, v);
+                        Frag V;
+                        tmem_ld_frag(tbase + (uint32_t)a * T + ((uint32_t)(32 * g) << 16) + (uint32_t)c0, V);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&sm.accempty[a]);
                         if (kc == 0 && a == 0) {
-#pragma unroll
-                            for (int c = 0; c < 32; ++c) ga[c] = v[c];
+                            G = V;
                         } else {
-                            // two columns per instruction, each rounded as a scalar add
 #pragma unroll
-                            for (int c = 0; c < 32; c += 2) {
-                                const float2 t2 = __fadd2_rn(make_float2(ga[c], ga[c + 1]), make_float2(v[c], v[c + 1]));
-                                ga[c] = t2.x;
-                                ga[c + 1] = t2.y;
-                            }
+                            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) G.v[k][j] = __fadd2_rn(G.v[k][j], V.v[k][j]);
                         }
                     }
                     aph ^= 1u;
@@ -533,23 +561,16 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                 }
                 if (MODE == T3_DECIDE) {
                     const T3Const& cc = sm.cst[buf];
-                    const float si = cc.sq[1][r], ngam = -tab[1].gamma, lam2 = tab[1].lam2;
-                    float f[4] = {0.f, 0.f, 0.f, 0.f};
+                    const Rbf rb = rbf_of(tab[1].gamma, tab[1].lam2);
+                    float2 f[4] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f)};
 #pragma unroll
-                    for (int c4 = 0; c4 < 32; c4 += 4) {
-                        const float4 w4 = *reinterpret_cast<const float4*>(&cc.mu[0][c0 + c4]);
-                        const float4 s4 = *reinterpret_cast<const float4*>(&cc.sq[0][c0 + c4]);
-                        const float wj[4] = {w4.x, w4.y, w4.z, w4.w}, sj[4] = {s4.x, s4.y, s4.z, s4.w};
+                    for (int j = 0; j < 4; ++j) {
+                        const float2 sj = ld2(&cc.sq[0][cq + 8 * j]), wj = ld2(&cc.mu[0][cq + 8 * j]);
 #pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            const float d2 = fmaxf(0.f, si + sj[t] - 2.f * ga[c4 + t]);
-                            f[t] = fmaf(wj[t], expf(ngam * d2) + lam2, f[t]);
-                        }
+                        for (int k = 0; k < 4; ++k) f[k] = __ffma2_rn(wj, rbf2(rb, G.v[k][j], cc.sq[1][r0 + 8 * k], sj), f[k]);
                     }
-                    // TwoSum, as the finalize's slot sums
-                    const float x = (f[0] + f[1]) + (f[2] + f[3]), t = fs + x, bp = t - fs;
-                    fc += (fs - (t - bp)) + (x - bp);
-                    fs = t;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) add_pair(fs[k], fc[k], f[k].x + f[k].y, 0.f);
                     if (J + 1 < last_j(w)) {
                         settle(buf ^ 1, kn);
                         epi_bar();
@@ -560,14 +581,15 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                 }
                 if (MODE == T3_FORM && norms_only) {
                     if (!ok) break;
-                    // diagonal tile: x_i . x_i is the Gram value at (r, r), held by the
-                    // warp of r's lane quarter whose columns contain r
-                    if (cg == g) {
-                        float d = 0.f;
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) d = c == lane ? ga[c] : d;
+                    // diagonal tile: x_i . x_i is the Gram value at (r, r), of the
+                    // lanes whose columns 2 lq, 2 lq + 1 contain row lr
+                    if (cg == g && (lr >> 1) == lq) {
                         for (int k = w.x; k >= 0; k = tab[k].form_next - 1)
-                            if (i < tab[k].n) tab[k].sq3[i] = d;
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const int x = I * T + r0 + 8 * u;
+                                if (x < tab[k].n) tab[k].sq3[x] = lr & 1 ? G.v[u][u].y : G.v[u][u].x;
+                            }
                     }
                     continue;
                 }
@@ -575,9 +597,8 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                     const Inst& p = tab[k];
                     const int n = p.n, next = MODE == T3_FORM ? p.form_next - 1 : -1;
                     const T3Const& cc = sm.cst[buf];
-                    const float si = cc.sq[1][r], mi = cc.mu[1][r], ai = cc.al[1][r], ngam = -p.gamma, lam2 = p.lam2;
-                    const uint32_t syi = __float_as_uint(cc.y[1][r]);
-                    const uint32_t* cy = reinterpret_cast<const uint32_t*>(&cc.y[0][c0]);
+                    const float lam2 = p.lam2;
+                    const Rbf rb = rbf_of(p.gamma, lam2);
                     if (k != w.x) {   // (a tile's first item started the copies for the second above)
                         kn = next;
                         if (kn < 0 && more) { kn = wn.x; In = wn.y; Jn = first_j(wn); }
@@ -585,46 +606,59 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                     }
                     // interior tile: every pair valid
                     const bool full = I != J && (I + 1) * T <= n && (J + 1) * T <= n;
-                    float rs4[4] = {0.f, 0.f, 0.f, 0.f};   // row sum in four interleaved parts
-                    float q[32];
-                    if (full)
-                        q_chunk32<true>(ga, cy, &cc.sq[0][c0], si, syi, ngam, lam2, 0, 0, 0, 0, 0, q, rs4);
-                    else
-                        q_chunk32<false>(ga, cy, &cc.sq[0][c0], si, syi, ngam, lam2, i, n, c0, J * T, I == J ? r : -1, q, rs4);
                     constexpr int NSUM = MODE == T3_FINAL ? 2 : 1;
                     T3Sums& su = sm.sums[buf];
-                    if (MODE == T3_FORM) {
-                        if (p.tilemax) {
-                            float tmx = 0.f;
+                    // FORM: |Q|; FINAL: q mu and q alpha, the row's over the columns and the columns' over the rows
+                    float2 rsum[NSUM][4], csum[NSUM][4];
 #pragma unroll
-                            for (int c = 0; c < 32; ++c) tmx = fmaxf(tmx, fabsf(q[c]));
-                            tmx = warp_max_f(tmx);
-                            if (lane == 0) su.tmx[ew] = tmx;
+                    for (int s = 0; s < NSUM; ++s)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) rsum[s][k] = csum[s][k] = f2(0.f);
+                    float tmx = 0.f;
+                    float* store = MODE == T3_FORM && p.qref ? p.qref + (size_t)w.w * TT + (size_t)r0 * T + cq : nullptr;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int c = cq + 8 * j;
+                        const float2 sj = ld2(&cc.sq[0][c]), yj = ld2(&cc.y[0][c]);
+                        const uint32_t sx = __float_as_uint(yj.x), sy = __float_as_uint(yj.y);
+                        float2 muj, alj;
+                        if (MODE == T3_FINAL) {
+                            muj = ld2(&cc.mu[0][c]);
+                            alj = ld2(&cc.al[0][c]);
                         }
-                        if (p.qref) store_row32(p.qref + (size_t)w.w * TT + (size_t)r * T + c0, q);
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) q[c] = fabsf(q[c]);
-                        su.col[0][g][c0 + lane] = transpose_sum32(q, lane);
-                        su.row[0][cg][r] = (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
-                    } else {
-                        // sums of q mu and q alpha: the row's over the columns, the columns' over the rows
-#pragma unroll
-                        for (int s = 0; s < 2; ++s) {
-                            const float xi = s ? ai : mi;
-                            float f[4] = {0.f, 0.f, 0.f, 0.f}, v[32];
-#pragma unroll
-                            for (int c4 = 0; c4 < 32; c4 += 4) {
-                                const float4 x4 = *reinterpret_cast<const float4*>(s ? &cc.al[0][c0 + c4] : &cc.mu[0][c0 + c4]);
-                                const float xj[4] = {x4.x, x4.y, x4.z, x4.w};
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) {
-                                    f[t] = fmaf(q[c4 + t], xj[t], f[t]);
-                                    v[c4 + t] = q[c4 + t] * xi;
-                                }
+                        for (int k = 0; k < 4; ++k) {
+                            const int rk = r0 + 8 * k;
+                            float2 e = rbf2(rb, G.v[k][j], cc.sq[1][rk], sj);
+                            if (!full) {
+                                const bool row = I * T + rk < n;
+                                const int least = I == J ? rk : -1;
+                                if (!(row && J * T + c < n && c > least)) e.x = 0.f;
+                                if (!(row && J * T + c + 1 < n && c + 1 > least)) e.y = 0.f;
                             }
-                            su.row[s][cg][r] = (f[0] + f[1]) + (f[2] + f[3]);
-                            su.col[s][g][c0 + lane] = transpose_sum32(v, lane);
+                            const uint32_t si = __float_as_uint(cc.y[1][rk]);
+                            const float2 q = flip(e, si ^ sx, si ^ sy);
+                            if (MODE == T3_FORM) {
+                                rsum[0][k] = __fadd2_rn(rsum[0][k], e);
+                                csum[0][j] = __fadd2_rn(csum[0][j], e);
+                                tmx = fmaxf(tmx, fmaxf(e.x, e.y));
+                                if (store) *reinterpret_cast<float2*>(store + (size_t)(8 * k) * T + 8 * j) = q;
+                            } else {
+                                rsum[0][k] = __ffma2_rn(q, muj, rsum[0][k]);
+                                rsum[NSUM - 1][k] = __ffma2_rn(q, alj, rsum[NSUM - 1][k]);
+                                csum[0][j] = __ffma2_rn(q, f2(cc.mu[1][rk]), csum[0][j]);
+                                csum[NSUM - 1][j] = __ffma2_rn(q, f2(cc.al[1][rk]), csum[NSUM - 1][j]);
+                            }
                         }
+                    }
+#pragma unroll
+                    for (int s = 0; s < NSUM; ++s) {
+                        su.row[s][cg][32 * g + 8 * lq + lr] = row_sums4(rsum[s], lane);
+                        su.col[s][g][c0 + 8 * (lr >> 1) + 2 * lq + (lr & 1)] = col_sums8(csum[s], lane);
+                    }
+                    if (MODE == T3_FORM && p.tilemax) {
+                        tmx = warp_max_f(tmx);
+                        if (lane == 0) su.tmx[ew] = tmx;
                     }
                     // One barrier a tile: the sums are complete, and every epilogue
                     // warp takes a stop together; the next tile's sums go to the
@@ -669,8 +703,20 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
             }
             if (MODE == T3_DECIDE) {
                 T3Sums& su = sm.sums[buf];
-                su.row[0][cg][r] = fs;
-                su.row[1][cg][r] = fc;
+                // a row's four lanes: lane lq has rows 8 lq + lr
+#pragma unroll
+                for (int o = 2; o > 0; o >>= 1) {
+                    const bool up = (lane & o) != 0;
+#pragma unroll
+                    for (int k = 0; k < o; ++k) {
+                        const float xs = __shfl_xor_sync(0xffffffffu, up ? fs[k] : fs[k + o], o);
+                        const float xc = __shfl_xor_sync(0xffffffffu, up ? fc[k] : fc[k + o], o);
+                        if (up) { fs[k] = fs[k + o]; fc[k] = fc[k + o]; }
+                        add_pair(fs[k], fc[k], xs, xc);
+                    }
+                }
+                su.row[0][cg][32 * g + 8 * lq + lr] = fs[0];
+                su.row[1][cg][32 * g + 8 * lq + lr] = fc[0];
                 if (more) settle(buf ^ 1, wn.x);
                 epi_bar();
                 if (*(volatile int*)&sm.abort) break;
