@@ -23,13 +23,13 @@
 // of each (tile, chunk), two copies of three planes, into a two-stage
 // shared-memory ring; warp 1 allocates 512 TMEM columns (four 128 x 128 FP32
 // accumulators, one per K-step) and one thread issues the 24 MMAs of a chunk (6
-// products x K = 64 in steps of 16); warps 2-17 (four per TMEM lane quarter, one
-// per 32 columns) add each chunk's accumulators into registers and run the
-// epilogue of the mode:
-//   formation   Q entries (norm expansion, clamp, expf, bias, labels), stored in
-//               32-byte pieces, and |Q| over rows (four interleaved partial
-//               sums), over columns (a warp transpose-sum, then the four lane
-//               quarters in shared memory) and the tile maximum.  Instances
+// products x K = 64 in steps of 16); warp 2 prepares what the epilogue does next
+// (T3Item and the labels, norms and means); warps 3-18 (four per TMEM lane
+// quarter, one per 32 columns) add each chunk's accumulators into registers and
+// run the epilogue of the mode:
+//   formation   Q entries (norm expansion, clamp, expf, bias, labels), stored,
+//               and |Q| over rows, over columns (in registers, then in shared
+//               memory) and the tile maximum.  Instances
 //               chained behind the listed one (the points of a parameter grid
 //               over the same features) take their Q tiles from the same Gram
 //               sums;
@@ -37,8 +37,11 @@
 //               (instances that recompute Q);
 //   decision    entries of test rows against training rows, times the weights,
 //               summed over a range of training tiles in registers.
-// Bound by the epilogue: with eight epilogue warps (64 columns each, all four
-// accumulators handed over at once) two warps a scheduler left it waiting.
+// Bound by the epilogue's latencies (the FMA pipe is 21 % busy, the stores'
+// path 60 %): with eight epilogue warps (64 columns each, all four accumulators
+// handed over at once) two warps a scheduler left it waiting; with the epilogue
+// looking up lists, tables and slots itself, formation took 522 us (n = 20000, m =
+// 128) and 162 us (n = 12000, m = 64), now 424 and 129.
 #include "common.cuh"
 #include "ptx.cuh"
 #include "qtile_epi.cuh"
@@ -51,7 +54,8 @@ namespace {
 
 constexpr int NPLANE = 3;
 constexpr int T3_EPI_WARPS = 16;                     // four per TMEM lane quarter, one per 32 columns
-constexpr int T3_THREADS = (2 + T3_EPI_WARPS) * 32;
+constexpr int T3_CTL_WARPS = 3;                       // operand producer, MMA issuer, item preparer
+constexpr int T3_THREADS = (T3_CTL_WARPS + T3_EPI_WARPS) * 32;
 constexpr int T3_STAGES = 2;
 constexpr size_t T3_STAGE_BYTES = (size_t)2 * NPLANE * BLK_BYTES;   // A planes, then B planes: 96 KB
 // Accumulators per 64-feature chunk: one per K-step of 16 features, each
@@ -255,12 +259,24 @@ struct T3Const {
     float al[2][T];
 };
 
-// 4 bytes to shared memory, asynchronously; zero where !ok (src is then not read).
-__device__ __forceinline__ void copy_word(float* dst, const float* src, int ok) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
-                 :: "r"(smem_u32(dst)), "l"(src), "r"(ok ? 4 : 0) : "memory");
-}
-__device__ __forceinline__ void copy_words_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// What the epilogue does next: a tile, or one of the instances that share its
+// Gram.  One warp prepares it, with the constants, while the epilogue computes
+// the item before (two in turn): looked up by the epilogue itself, work lists,
+// instance tables and slots were a third of its time.
+struct T3Item {
+    int nkc;                 // chunks of accumulators to take in first; 0: the Gram at hand
+    int end, diag, last;     // no item; a diagonal tile; decision: the entry's last tile
+    int rows, cols;          // rows and columns that there are (may exceed T)
+    float gamma, lam2;
+    float* store;            // where the entries go, or null
+    float* tilemax;          // where the largest |q| goes, or null
+    float* dst[2];           // the row's and the column's slot sums (FINAL: of q mu; those of q alpha plen behind)
+    unsigned long long* fix[2];   // where set, fixed-point sums instead of slots
+    double scale;
+    long long plen;
+    int4 w;                  // norms_only: the work entry
+    Ctrl* ctrl;
+};
 
 struct T3Smem {
     unsigned long long xfull[T3_STAGES], xempty[T3_STAGES];
@@ -270,9 +286,10 @@ struct T3Smem {
     int abort;
     T3Sums sums[2];
     T3Const cst[2];
+    T3Item item[2];
+    unsigned long long ifull[2], iempty[2], sync;
 };
 
-__device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(T3_EPI_WARPS * 32) : "memory"); }
 
 // ---- epilogue
 // A warp has 32 rows (its lane quarter of TMEM) x 32 columns of the tile, in
@@ -383,6 +400,8 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
     if (tid == 0) {
         for (int s = 0; s < T3_STAGES; ++s) { mbar_init(&sm.xfull[s], 1); mbar_init(&sm.xempty[s], 1); }
         for (int a = 0; a < T3_NACC; ++a) { mbar_init(&sm.accfull[a], 1); mbar_init(&sm.accempty[a], T3_EPI_WARPS); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&sm.ifull[b], 1); mbar_init(&sm.iempty[b], T3_EPI_WARPS); }
+        mbar_init(&sm.sync, T3_EPI_WARPS);
         mbar_init(&sm.drain, 1);
         sm.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -468,266 +487,297 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
             tc_commit(&sm.drain);
             if (!mbar_wait(&sm.drain, 0u)) sm.abort = 1;
         }
-    } else {
-        // --------------------------------------------------------- epilogue
-        // warp w reads TMEM lanes 32 (w % 4) ..: rows 32 g + lane, columns
-        // [32 cg, 32 cg + 32)
-        const int ew = warp - 2, g = warp & 3, cg = ew >> 2;
-        const int lr = lane >> 2, lq = lane & 3, c0 = 32 * cg;
-        const int r0 = 32 * g + lr, cq = c0 + 2 * lq;   // the lane's first row and column
-        const int etid = tid - 64;
-        uint32_t aph = 0;
-        int buf = 0;
-        // The constants of an item (a tile, or one of the instances that share
-        // it) are copied to shared memory while the item before it is computed,
-        // so that neither their latency nor registers for them are in the way:
-        // threads 0..127 take the tile's columns, 128..255 its rows.  fetch()
-        // starts the copies; settle(), before the barrier that ends the current
-        // item, waits for the thread's own and puts them in the form that is used.
-        const int cx = etid & (T - 1), crole = etid / T;
-        const auto fetch = [&](int b, int k, int I, int J) {
-            if (crole >= 2 || (MODE == T3_FORM && norms_only)) return;
-            const Inst& p = MODE == T3_DECIDE && crole == 0 ? tab[1] : tab[k];
-            T3Const& c = sm.cst[b];
-            const int x = (crole ? I : J) * T + cx, ok = x < p.n, xs = ok ? x : 0;
-            if (MODE != T3_DECIDE || crole == 0) copy_word(&c.y[crole][cx], p.y + xs, ok);
-            copy_word(&c.sq[crole][cx], p.sq3 + xs, ok);
-            if (MODE == T3_FINAL) copy_word(&c.mu[crole][cx], ops[k].mu + xs, ok);
-            if (MODE == T3_DECIDE && crole == 0) copy_word(&c.mu[0][cx], dec.alpha + xs, ok);
-        };
-        const auto settle = [&](int b, int k) {
-            if (crole >= 2 || (MODE == T3_FORM && norms_only)) return;
-            copy_words_wait();
-            T3Const& c = sm.cst[b];
-            if (MODE == T3_DECIDE) {
-                if (crole == 0) c.mu[0][cx] *= c.y[0][cx];
-                return;
-            }
-            c.y[crole][cx] = __uint_as_float(__float_as_uint(c.y[crole][cx]) & 0x80000000u);
-            if (MODE == T3_FINAL) {
-                const float m = c.mu[crole][cx];
-                c.al[crole][cx] = tab[k].task ? m : fminf(fmaxf(m, 0.f), tab[k].C);
-            }
-        };
+    } else if (warp == 2) {
+        // ----------------------------------------------- items and constants
+        const bool consts = MODE != T3_FORM || !norms_only;
+        int b = 0;
+        uint32_t ph = 0;
+        bool run = true;
         int4 wn = blockIdx.x < ntiles ? work[blockIdx.x] : make_int4(0, 0, 0, 0);
-        if (blockIdx.x < ntiles) {
-            fetch(0, wn.x, wn.y, first_j(wn));
-            settle(0, wn.x);
-        }
-        epi_bar();
-        for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
+        for (long long L = blockIdx.x; L < ntiles && run; L += gridDim.x) {
             const int4 w = wn;
-            const int nkc = tab[w.x].nkc, I = w.y;
-            const bool more = L + gridDim.x < ntiles;
-            if (more) wn = work[L + gridDim.x];
-            // decision: the rows' compensated sums over the training tiles
-            float fs[4] = {0.f, 0.f, 0.f, 0.f}, fc[4] = {0.f, 0.f, 0.f, 0.f};
-            bool ok = true;
-            for (int J = first_j(w); J < last_j(w) && ok; ++J) {
-                // the item that follows: an instance sharing the tile, the row's next
-                // training tile, or the next entry
-                int kn = MODE == T3_FORM ? tab[w.x].form_next - 1 : -1, In = I, Jn = J;
-                if (MODE == T3_DECIDE && J + 1 < last_j(w)) { kn = w.x; Jn = J + 1; }
-                if (kn < 0 && more) { kn = wn.x; In = wn.y; Jn = first_j(wn); }
-                if (kn >= 0) fetch(buf ^ 1, kn, In, Jn);
-                Frag G;
-                for (int kc = 0; kc < nkc && ok; ++kc) {
-                    const bool stop = __shfl_sync(0xffffffffu, *(volatile int*)&sm.abort, 0) != 0;
-                    // the chunk's accumulators added to the running sums in order
+            if (L + gridDim.x < ntiles) wn = work[L + gridDim.x];
+            const int I = w.y;
+            for (int J = first_j(w); J < last_j(w) && run; ++J) {
+                for (int k = w.x; k >= 0 && run;) {
+                    const Inst& p = tab[k];                              // rows
+                    const Inst& cp = MODE == T3_DECIDE ? tab[1] : p;     // columns
+                    const int n = p.n, rows = n - I * T, cols = cp.n - J * T;
+                    const int next = MODE == T3_FORM && consts ? p.form_next - 1 : -1;
+                    // lane + 32 u of the tile's columns ([0]) and rows ([1])
+                    float y[2][4], q[2][4], m[2][4];
+                    if (consts) {
 #pragma unroll
-                    for (int a = 0; a < T3_NACC; ++a) {
-                        if (stop || !mbar_wait_warp(&sm.accfull[a], aph)) { ok = false; break; }
-                        tc_fence_after();
-                        Frag V;
-                        tmem_ld_frag(tbase + (uint32_t)a * T + ((uint32_t)(32 * g) << 16) + (uint32_t)c0, V);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&sm.accempty[a]);
-                        if (kc == 0 && a == 0) {
-                            G = V;
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                                for (int j = 0; j < 4; ++j) G.v[k][j] = __fadd2_rn(G.v[k][j], V.v[k][j]);
-                        }
-                    }
-                    aph ^= 1u;
-                }
-                if (!ok && lane == 0) {
-                    sm.abort = 1;
-                    record_error(tab[w.x].ctrl, ST_ETIMEOUT, L);
-                }
-                if (MODE == T3_DECIDE) {
-                    const T3Const& cc = sm.cst[buf];
-                    const Rbf rb = rbf_of(tab[1].gamma, tab[1].lam2);
-                    float2 f[4] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f)};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float2 sj = ld2(&cc.sq[0][cq + 8 * j]), wj = ld2(&cc.mu[0][cq + 8 * j]);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) f[k] = __ffma2_rn(wj, rbf2(rb, G.v[k][j], cc.sq[1][r0 + 8 * k], sj), f[k]);
-                    }
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) add_pair(fs[k], fc[k], f[k].x + f[k].y, 0.f);
-                    if (J + 1 < last_j(w)) {
-                        settle(buf ^ 1, kn);
-                        epi_bar();
-                        if (*(volatile int*)&sm.abort) { ok = false; break; }
-                        buf ^= 1;
-                    }
-                    continue;
-                }
-                if (MODE == T3_FORM && norms_only) {
-                    if (!ok) break;
-                    // diagonal tile: x_i . x_i is the Gram value at (r, r), of the
-                    // lanes whose columns 2 lq, 2 lq + 1 contain row lr
-                    if (cg == g && (lr >> 1) == lq) {
-                        for (int k = w.x; k >= 0; k = tab[k].form_next - 1)
+                        for (int r = 0; r < 2; ++r) {
+                            const Inst& o = r ? p : cp;
+                            const float* mu = MODE == T3_FINAL ? ops[k].mu : MODE == T3_DECIDE && r == 0 ? dec.alpha : nullptr;
 #pragma unroll
                             for (int u = 0; u < 4; ++u) {
-                                const int x = I * T + r0 + 8 * u;
-                                if (x < tab[k].n) tab[k].sq3[x] = lr & 1 ? G.v[u][u].y : G.v[u][u].x;
-                            }
-                    }
-                    continue;
-                }
-                for (int k = w.x; k >= 0;) {
-                    const Inst& p = tab[k];
-                    const int n = p.n, next = MODE == T3_FORM ? p.form_next - 1 : -1;
-                    const T3Const& cc = sm.cst[buf];
-                    const float lam2 = p.lam2;
-                    const Rbf rb = rbf_of(p.gamma, lam2);
-                    if (k != w.x) {   // (a tile's first item started the copies for the second above)
-                        kn = next;
-                        if (kn < 0 && more) { kn = wn.x; In = wn.y; Jn = first_j(wn); }
-                        if (kn >= 0) fetch(buf ^ 1, kn, In, Jn);
-                    }
-                    // interior tile: every pair valid
-                    const bool full = I != J && (I + 1) * T <= n && (J + 1) * T <= n;
-                    constexpr int NSUM = MODE == T3_FINAL ? 2 : 1;
-                    T3Sums& su = sm.sums[buf];
-                    // FORM: |Q|; FINAL: q mu and q alpha, the row's over the columns and the columns' over the rows
-                    float2 rsum[NSUM][4], csum[NSUM][4];
-#pragma unroll
-                    for (int s = 0; s < NSUM; ++s)
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) rsum[s][k] = csum[s][k] = f2(0.f);
-                    float tmx = 0.f;
-                    float* store = MODE == T3_FORM && p.qref ? p.qref + (size_t)w.w * TT + (size_t)r0 * T + cq : nullptr;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int c = cq + 8 * j;
-                        const float2 sj = ld2(&cc.sq[0][c]), yj = ld2(&cc.y[0][c]);
-                        const uint32_t sx = __float_as_uint(yj.x), sy = __float_as_uint(yj.y);
-                        float2 muj, alj;
-                        if (MODE == T3_FINAL) {
-                            muj = ld2(&cc.mu[0][c]);
-                            alj = ld2(&cc.al[0][c]);
-                        }
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int rk = r0 + 8 * k;
-                            float2 e = rbf2(rb, G.v[k][j], cc.sq[1][rk], sj);
-                            if (!full) {
-                                const bool row = I * T + rk < n;
-                                const int least = I == J ? rk : -1;
-                                if (!(row && J * T + c < n && c > least)) e.x = 0.f;
-                                if (!(row && J * T + c + 1 < n && c + 1 > least)) e.y = 0.f;
-                            }
-                            const uint32_t si = __float_as_uint(cc.y[1][rk]);
-                            const float2 q = flip(e, si ^ sx, si ^ sy);
-                            if (MODE == T3_FORM) {
-                                rsum[0][k] = __fadd2_rn(rsum[0][k], e);
-                                csum[0][j] = __fadd2_rn(csum[0][j], e);
-                                tmx = fmaxf(tmx, fmaxf(e.x, e.y));
-                                if (store) *reinterpret_cast<float2*>(store + (size_t)(8 * k) * T + 8 * j) = q;
-                            } else {
-                                rsum[0][k] = __ffma2_rn(q, muj, rsum[0][k]);
-                                rsum[NSUM - 1][k] = __ffma2_rn(q, alj, rsum[NSUM - 1][k]);
-                                csum[0][j] = __ffma2_rn(q, f2(cc.mu[1][rk]), csum[0][j]);
-                                csum[NSUM - 1][j] = __ffma2_rn(q, f2(cc.al[1][rk]), csum[NSUM - 1][j]);
+                                const int x = (r ? I : J) * T + lane + 32 * u;
+                                const bool in = x < o.n;
+                                y[r][u] = in && (MODE != T3_DECIDE || r == 0) ? o.y[x] : 0.f;
+                                q[r][u] = in ? o.sq3[x] : 0.f;
+                                m[r][u] = in && mu ? mu[x] : 0.f;
                             }
                         }
                     }
-#pragma unroll
-                    for (int s = 0; s < NSUM; ++s) {
-                        su.row[s][cg][32 * g + 8 * lq + lr] = row_sums4(rsum[s], lane);
-                        su.col[s][g][c0 + 8 * (lr >> 1) + 2 * lq + (lr & 1)] = col_sums8(csum[s], lane);
+                    if (*(volatile int*)&sm.abort || !mbar_wait_warp(&sm.iempty[b], ph ^ 1u)) {
+                        if (lane == 0) {
+                            sm.abort = 1;
+                            record_error(p.ctrl, ST_ETIMEOUT, L);
+                        }
+                        run = false;
                     }
-                    if (MODE == T3_FORM && p.tilemax) {
-                        tmx = warp_max_f(tmx);
-                        if (lane == 0) su.tmx[ew] = tmx;
-                    }
-                    // One barrier a tile: the sums are complete, and every epilogue
-                    // warp takes a stop together; the next tile's sums go to the
-                    // other buffer.
-                    if (kn >= 0) settle(buf ^ 1, kn);
-                    epi_bar();
-                    if (*(volatile int*)&sm.abort) { ok = false; break; }
-                    // per-node slot partials (fixed order): row sums of the tile's rows,
-                    // column sums of its columns; both roles on a diagonal tile
-                    // (slot sl.x of the row block, sl.y of the column block).  Where
-                    // rfix is set they are added to the nodes' fixed-point sums instead.
-                    if (etid < 2 * T) {
-                        const int off = etid & (T - 1), role = etid / T;
-                        const int x = (role ? J : I) * T + off;
-                        if (x < n && !(I == J && role)) {
+                    run = __all_sync(0xffffffffu, run);
+                    if (!run) break;
+                    if (consts) {
+                        T3Const& c = sm.cst[b];
 #pragma unroll
-                            for (int s = 0; s < NSUM; ++s) {
-                                const float (*rw)[T] = su.row[s];
-                                const float (*cl)[T] = su.col[s];
-                                const float vr = (rw[0][off] + rw[1][off]) + (rw[2][off] + rw[3][off]);
-                                const float vc = ((cl[0][off] + cl[1][off]) + cl[2][off]) + cl[3][off];
-                                const float v = I == J ? vr + vc : role ? vc : vr;
-                                if (MODE == T3_FORM && p.rfix) {
-                                    atomicAdd(p.rfix + x, (unsigned long long)rsum_fix(v, pow2i(rsum_shift(n, lam2))));
-                                } else {
-                                    const int2 sl = tile_slots(p, w);
-                                    // final pass: the residual slots and the spare ones
-                                    float* dst = p.part + (MODE == T3_FINAL ? (2 + s) * part_len(p) : 0);
-                                    dst[(size_t)(role ? sl.y : sl.x) * T + off] = v;
+                        for (int r = 0; r < 2; ++r)
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const int x = lane + 32 * u;
+                                c.sq[r][x] = q[r][u];
+                                if (MODE == T3_DECIDE) {
+                                    if (r == 0) c.mu[0][x] = m[0][u] * y[0][u];
+                                    continue;
+                                }
+                                c.y[r][x] = __uint_as_float(__float_as_uint(y[r][u]) & 0x80000000u);
+                                if (MODE == T3_FINAL) {
+                                    c.mu[r][x] = m[r][u];
+                                    c.al[r][x] = p.task ? m[r][u] : fminf(fmaxf(m[r][u], 0.f), p.C);
                                 }
                             }
+                    }
+                    if (lane == 0) {
+                        T3Item& t = sm.item[b];
+                        t.nkc = k == w.x ? p.nkc : 0;
+                        t.end = 0;
+                        t.diag = MODE != T3_DECIDE && I == J;
+                        t.last = J + 1 == last_j(w);
+                        t.rows = rows;
+                        t.cols = cols;
+                        t.gamma = cp.gamma;
+                        t.lam2 = cp.lam2;
+                        t.ctrl = p.ctrl;
+                        t.w = w;
+                        if (MODE == T3_DECIDE) {
+                            t.dst[0] = dec.part + L * T;
+                        } else if (consts) {
+                            const int2 sl = p.rfix ? make_int2(0, 0) : tile_slots(p, w);
+                            t.plen = (long long)part_len(p);
+                            float* part = p.part + (MODE == T3_FINAL ? 2 * t.plen : 0);
+                            t.dst[0] = part + (size_t)sl.x * T;
+                            t.dst[1] = part + (size_t)sl.y * T;
+                            t.store = MODE == T3_FORM && p.qref ? p.qref + (size_t)w.w * TT : nullptr;
+                            t.tilemax = MODE == T3_FORM && p.tilemax ? p.tilemax + w.w : nullptr;
+                            t.fix[0] = MODE == T3_FORM && p.rfix ? p.rfix + (size_t)I * T : nullptr;
+                            t.fix[1] = MODE == T3_FORM && p.rfix ? p.rfix + (size_t)J * T : nullptr;
+                            if (MODE == T3_FORM && p.rfix) t.scale = pow2i(rsum_shift(n, p.lam2));
                         }
                     }
-                    if (MODE == T3_FORM && etid == 0 && p.tilemax) {
-                        float m2 = 0.f;
-                        for (int e = 0; e < T3_EPI_WARPS; ++e) m2 = fmaxf(m2, su.tmx[e]);
-                        p.tilemax[w.w] = m2;
-                    }
-                    buf ^= 1;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sm.ifull[b]);
+                    if ((b ^= 1) == 0) ph ^= 1u;
                     k = next;
                 }
             }
-            if (MODE == T3_DECIDE) {
-                T3Sums& su = sm.sums[buf];
-                // a row's four lanes: lane lq has rows 8 lq + lr
+        }
+        if (run && mbar_wait_warp(&sm.iempty[b], ph ^ 1u) && lane == 0) {
+            sm.item[b].end = 1;
+            mbar_arrive(&sm.ifull[b]);
+        }
+    } else {
+        // --------------------------------------------------------- epilogue
+        // warp w reads TMEM lanes 32 (w % 4) ..: rows 32 g ..., columns [32 cg, 32 cg + 32)
+        const int ew = warp - T3_CTL_WARPS, g = warp & 3, cg = ew >> 2;
+        const int lr = lane >> 2, lq = lane & 3, c0 = 32 * cg;
+        const int r0 = 32 * g + lr, cq = c0 + 2 * lq;   // the lane's first row and column
+        const int etid = tid - T3_CTL_WARPS * 32;
+        uint32_t aph = 0, iph = 0, sph = 0;
+        int b = 0, sb = 0;
+        Frag G;
+        // decision: the rows' compensated sums over the entry's training tiles
+        float fs[4] = {0.f, 0.f, 0.f, 0.f}, fc[4] = {0.f, 0.f, 0.f, 0.f};
+        // The epilogue's warps meet (bounded, like every wait): the item's sums are complete.
+        auto meet = [&]() {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.sync);
+            const bool ok = mbar_wait_warp(&sm.sync, sph);
+            sph ^= 1u;
+            return ok;
+        };
+        bool ok = true;
+        for (;;) {
+            const bool stop = __shfl_sync(0xffffffffu, *(volatile int*)&sm.abort, 0) != 0;
+            if (stop || !mbar_wait_warp(&sm.ifull[b], iph)) { ok = false; break; }
+            const T3Item& it = sm.item[b];
+            const T3Const& cc = sm.cst[b];
+            if (it.end) break;
+            const int nkc = it.nkc;
+            for (int kc = 0; kc < nkc && ok; ++kc) {
+                // the chunk's accumulators added to the running sums in order
 #pragma unroll
-                for (int o = 2; o > 0; o >>= 1) {
-                    const bool up = (lane & o) != 0;
+                for (int a = 0; a < T3_NACC; ++a) {
+                    if (!mbar_wait_warp(&sm.accfull[a], aph)) { ok = false; break; }
+                    tc_fence_after();
+                    Frag V;
+                    tmem_ld_frag(tbase + (uint32_t)a * T + ((uint32_t)(32 * g) << 16) + (uint32_t)c0, V);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sm.accempty[a]);
+                    if (kc == 0 && a == 0) {
+                        G = V;
+                    } else {
 #pragma unroll
-                    for (int k = 0; k < o; ++k) {
-                        const float xs = __shfl_xor_sync(0xffffffffu, up ? fs[k] : fs[k + o], o);
-                        const float xc = __shfl_xor_sync(0xffffffffu, up ? fc[k] : fc[k + o], o);
-                        if (up) { fs[k] = fs[k + o]; fc[k] = fc[k + o]; }
-                        add_pair(fs[k], fc[k], xs, xc);
+                        for (int k = 0; k < 4; ++k)
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) G.v[k][j] = __fadd2_rn(G.v[k][j], V.v[k][j]);
                     }
                 }
-                su.row[0][cg][32 * g + 8 * lq + lr] = fs[0];
-                su.row[1][cg][32 * g + 8 * lq + lr] = fc[0];
-                if (more) settle(buf ^ 1, wn.x);
-                epi_bar();
-                if (*(volatile int*)&sm.abort) break;
-                if (etid < T) {
-                    double v = 0.0;
-                    for (int c = 0; c < 4; ++c) v += (double)su.row[0][c][etid] + (double)su.row[1][c][etid];
-                    dec.part[L * T + etid] = (float)v;
-                }
-                buf ^= 1;
+                aph ^= 1u;
             }
             if (!ok) break;
+            T3Sums& su = sm.sums[sb];
+            if (MODE == T3_FORM && norms_only) {
+                // diagonal tile: x_i . x_i is the Gram value at (r, r), of the
+                // lanes whose columns 2 lq, 2 lq + 1 contain row lr
+                const int4 w = it.w;
+                if (cg == g && (lr >> 1) == lq) {
+                    for (int k = w.x; k >= 0; k = tab[k].form_next - 1)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int x = w.y * T + r0 + 8 * u;
+                            if (x < tab[k].n) tab[k].sq3[x] = lr & 1 ? G.v[u][u].y : G.v[u][u].x;
+                        }
+                }
+            } else if (MODE == T3_DECIDE) {
+                const Rbf rb = rbf_of(it.gamma, it.lam2);
+                float2 f[4] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f)};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 sj = ld2(&cc.sq[0][cq + 8 * j]), wj = ld2(&cc.mu[0][cq + 8 * j]);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) f[k] = __ffma2_rn(wj, rbf2(rb, G.v[k][j], cc.sq[1][r0 + 8 * k], sj), f[k]);
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) add_pair(fs[k], fc[k], f[k].x + f[k].y, 0.f);
+                if (it.last) {
+                    // a row's four lanes: lane lq has rows 8 lq + lr
+#pragma unroll
+                    for (int o = 2; o > 0; o >>= 1) {
+                        const bool up = (lane & o) != 0;
+#pragma unroll
+                        for (int k = 0; k < o; ++k) {
+                            const float xs = __shfl_xor_sync(0xffffffffu, up ? fs[k] : fs[k + o], o);
+                            const float xc = __shfl_xor_sync(0xffffffffu, up ? fc[k] : fc[k + o], o);
+                            if (up) { fs[k] = fs[k + o]; fc[k] = fc[k + o]; }
+                            add_pair(fs[k], fc[k], xs, xc);
+                        }
+                    }
+                    su.row[0][cg][32 * g + 8 * lq + lr] = fs[0];
+                    su.row[1][cg][32 * g + 8 * lq + lr] = fc[0];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) fs[k] = fc[k] = 0.f;
+                    if (!meet()) { ok = false; break; }
+                    if (etid < T) {
+                        double v = 0.0;
+                        for (int c = 0; c < 4; ++c) v += (double)su.row[0][c][etid] + (double)su.row[1][c][etid];
+                        it.dst[0][etid] = (float)v;
+                    }
+                    sb ^= 1;
+                }
+            } else {
+                const Rbf rb = rbf_of(it.gamma, it.lam2);
+                const int rows = it.rows, cols = it.cols;
+                const bool diag = it.diag != 0, full = !diag && rows >= T && cols >= T;   // every pair valid
+                constexpr int NSUM = MODE == T3_FINAL ? 2 : 1;
+                // FORM: |Q|; FINAL: q mu and q alpha, the row's over the columns and the columns' over the rows
+                float2 rsum[NSUM][4], csum[NSUM][4];
+#pragma unroll
+                for (int s = 0; s < NSUM; ++s)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) rsum[s][k] = csum[s][k] = f2(0.f);
+                float tmx = 0.f;
+                float* const store = MODE == T3_FORM && it.store ? it.store + (size_t)r0 * T + cq : nullptr;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int c = cq + 8 * j;
+                    const float2 sj = ld2(&cc.sq[0][c]), yj = ld2(&cc.y[0][c]);
+                    const uint32_t sx = __float_as_uint(yj.x), sy = __float_as_uint(yj.y);
+                    float2 muj, alj;
+                    if (MODE == T3_FINAL) {
+                        muj = ld2(&cc.mu[0][c]);
+                        alj = ld2(&cc.al[0][c]);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int rk = r0 + 8 * k;
+                        float2 e = rbf2(rb, G.v[k][j], cc.sq[1][rk], sj);
+                        if (!full) {
+                            const int least = diag ? rk : -1;
+                            if (!(rk < rows && c < cols && c > least)) e.x = 0.f;
+                            if (!(rk < rows && c + 1 < cols && c + 1 > least)) e.y = 0.f;
+                        }
+                        const uint32_t si = __float_as_uint(cc.y[1][rk]);
+                        const float2 q = flip(e, si ^ sx, si ^ sy);
+                        if (MODE == T3_FORM) {
+                            rsum[0][k] = __fadd2_rn(rsum[0][k], e);
+                            csum[0][j] = __fadd2_rn(csum[0][j], e);
+                            tmx = fmaxf(tmx, fmaxf(e.x, e.y));
+                            if (store) *reinterpret_cast<float2*>(store + (8 * k) * T + 8 * j) = q;
+                        } else {
+                            rsum[0][k] = __ffma2_rn(q, muj, rsum[0][k]);
+                            rsum[NSUM - 1][k] = __ffma2_rn(q, alj, rsum[NSUM - 1][k]);
+                            csum[0][j] = __ffma2_rn(q, f2(cc.mu[1][rk]), csum[0][j]);
+                            csum[NSUM - 1][j] = __ffma2_rn(q, f2(cc.al[1][rk]), csum[NSUM - 1][j]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int s = 0; s < NSUM; ++s) {
+                    su.row[s][cg][32 * g + 8 * lq + lr] = row_sums4(rsum[s], lane);
+                    su.col[s][g][c0 + 8 * (lr >> 1) + 2 * lq + (lr & 1)] = col_sums8(csum[s], lane);
+                }
+                float* const tilemax = MODE == T3_FORM ? it.tilemax : nullptr;
+                if (MODE == T3_FORM && tilemax) {
+                    tmx = warp_max_f(tmx);
+                    if (lane == 0) su.tmx[ew] = tmx;
+                }
+                if (!meet()) { ok = false; break; }
+                // per-node slot partials (fixed order): row sums of the tile's rows,
+                // column sums of its columns; both roles on a diagonal tile.  Where
+                // fix is set they are added to the nodes' fixed-point sums instead.
+                if (etid < 2 * T) {
+                    const int off = etid & (T - 1), role = etid / T;
+                    if (off < (role ? cols : rows) && !(diag && role)) {
+#pragma unroll
+                        for (int s = 0; s < NSUM; ++s) {
+                            const float (*rw)[T] = su.row[s];
+                            const float (*cl)[T] = su.col[s];
+                            const float vr = (rw[0][off] + rw[1][off]) + (rw[2][off] + rw[3][off]);
+                            const float vc = ((cl[0][off] + cl[1][off]) + cl[2][off]) + cl[3][off];
+                            const float v = diag ? vr + vc : role ? vc : vr;
+                            if (MODE == T3_FORM && it.fix[0]) atomicAdd(it.fix[role] + off, (unsigned long long)rsum_fix(v, it.scale));
+                            else it.dst[role][s * it.plen + off] = v;
+                        }
+                    }
+                }
+                if (MODE == T3_FORM && etid == 0 && tilemax) {
+                    float m2 = 0.f;
+                    for (int e = 0; e < T3_EPI_WARPS; ++e) m2 = fmaxf(m2, su.tmx[e]);
+                    *tilemax = m2;
+                }
+                sb ^= 1;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.iempty[b]);
+            if ((b ^= 1) == 0) iph ^= 1u;
+        }
+        if (!ok && lane == 0) {
+            sm.abort = 1;
+            record_error(tab[work[blockIdx.x].x].ctrl, ST_ETIMEOUT, blockIdx.x);
         }
     }
     tc_fence_before();
