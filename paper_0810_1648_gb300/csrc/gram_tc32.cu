@@ -37,11 +37,11 @@
 //               (instances that recompute Q);
 //   decision    entries of test rows against training rows, times the weights,
 //               summed over a range of training tiles in registers.
-// Bound by the epilogue's latencies (the FMA pipe is 21 % busy, the stores'
-// path 60 %): with eight epilogue warps (64 columns each, all four accumulators
+// Bound by the epilogue's latencies (the FMA pipe is 28 % busy, the LSU
+// 14 %): with eight epilogue warps (64 columns each, all four accumulators
 // handed over at once) two warps a scheduler left it waiting; with the epilogue
 // looking up lists, tables and slots itself, formation took 522 us (n = 20000, m =
-// 128) and 162 us (n = 12000, m = 64), now 424 and 129.
+// 128) and 162 us (n = 12000, m = 64), now 350 and 104.
 #include "common.cuh"
 #include "ptx.cuh"
 #include "qtile_epi.cuh"
@@ -103,8 +103,8 @@ __device__ __forceinline__ size_t core_off16(int rr, int kg)
 //
 // What bounds it: 4 bytes read and 6 to 10 written per feature.  A thread takes 8
 // features of a row (32 bytes of FP32, one 16-byte unit of each plane); 8
-// consecutive threads take 8 rows of the same group, so that they write whole
-// 128-byte core matrices, and a warp reads 128 consecutive bytes of each row.
+// consecutive threads take the 8 rows of a core matrix (row_position), so that
+// they write its 128 bytes, and a warp reads 128 consecutive bytes of each row.
 // With one thread a row for the checks and norms and a second pass for the
 // planes: 107 + 14 us at n = 6238, m = 617; 40 + 10 us at n = 20000, m = 128;
 // now 22 and 10 us.
@@ -127,6 +127,16 @@ __device__ __forceinline__ void load8(const XT* __restrict__ x, float (&v)[8])
 __device__ __forceinline__ bool rows_aligned(const void* X, size_t row_bytes)
 {
     return ((reinterpret_cast<uintptr_t>(X) | row_bytes) & 15) == 0;
+}
+
+// Operand position of a row within its block: the rows 8 q + 2 j + b of each 32 (q,
+// j < 4, b < 2) lie at 8 j + 2 q + b, so that the lane of the epilogue that holds
+// positions 8 j + 2 q + {0, 1}, j = 0..3, of a tile row has eight consecutive
+// columns, which it stores as 32 bytes.  Its own inverse is the same with q and j
+// exchanged.
+__host__ __device__ __forceinline__ int row_position(int r)
+{
+    return (r & ~31) | (r >> 1 & 3) << 3 | (r >> 3 & 3) << 1 | (r & 1);
 }
 
 // Row r (of Nt*T, zero beyond n) and 8-feature group gk -> Xf where it is kept
@@ -165,7 +175,7 @@ __device__ __forceinline__ bool stage_group(const XT* __restrict__ X, bool vec, 
 #pragma unroll
     for (int pl = 0; pl < NPLANE; ++pl) {
         const size_t blk = ((size_t)I * nkc + kc) * NPLANE + pl;
-        Xp3[blk * (BLK_BYTES / 16) + core_off16(rr, kg)] = *reinterpret_cast<const uint4*>(v[pl]);
+        Xp3[blk * (BLK_BYTES / 16) + core_off16(row_position(rr), kg)] = *reinterpret_cast<const uint4*>(v[pl]);
     }
     return ok;
 }
@@ -184,12 +194,13 @@ __device__ __forceinline__ bool stage_label(float* __restrict__ y, float* __rest
     return task ? isfinite(yi) : yi == 1.f || yi == -1.f;
 }
 
-// Row (of 8 consecutive ones) and group of thread e of a pass over whole rows.
+// Row (of 8 in consecutive operand positions) and group of thread e of a pass
+// over whole rows.
 __device__ __forceinline__ void stage_item(long long e, int groups, int& r, int& gk)
 {
     const long long q = e >> 3;
     gk = (int)(q % groups);
-    r = (int)(q / groups) * 8 + (int)(e & 7);
+    r = row_position((int)(q / groups) * 8 + (int)(e & 7));
 }
 
 // A caller's rows (FP32, FP64 or BF16).  Xf: where the FP32 rows are kept (null:
@@ -294,10 +305,13 @@ struct T3Smem {
 // ---- epilogue
 // A warp has 32 rows (its lane quarter of TMEM) x 32 columns of the tile, in
 // the layout of 16 x 256-bit loads: lane (lr = lane / 4, lq = lane % 4) holds
-// rows 8 k + lr, k = 0..3, and columns 8 j + 2 lq and the next, j = 0..3, as
-// pairs.  Four rows and eight columns a lane leave little to reduce across lanes
-// (ten shuffles for the tile's row and column sums, where one row of 32 columns
-// a lane took 31), and the pairs go through two-wide arithmetic.
+// positions 8 k + lr, k = 0..3, of the rows and 8 j + 2 lq and the next, j = 0..3,
+// as pairs, of the columns: rows 8 (lr / 2) + 2 k + lr % 2 and columns 8 lq + 2 j and
+// the next (row_position).  Four rows and eight columns a lane leave little to
+// reduce across lanes (ten shuffles for the tile's row and column sums, where
+// one row of 32 columns a lane took 31), the pairs go through two-wide arithmetic,
+// and a row's eight entries are stored at once (in pairs, 8 bytes a lane, the
+// stores took 11 passes each: 424 us against 350 at n = 20000, m = 128).
 struct Frag {
     float2 v[4][4];   // [k][j]
 };
@@ -339,7 +353,7 @@ __device__ __forceinline__ float2 flip(float2 v, uint32_t sx, uint32_t sy)
 }
 __device__ __forceinline__ float2 ld2(const float* x) { return *reinterpret_cast<const float2*>(x); }
 
-// Sums over the four lanes of a row group: lane lq has that of value lq (rows 8 lq + lr).
+// Sums over the four lanes of a row: lane lq has that of value lq.
 __device__ __forceinline__ float row_sums4(const float2 (&x)[4], int lane)
 {
     float v[4];
@@ -353,7 +367,7 @@ __device__ __forceinline__ float row_sums4(const float2 (&x)[4], int lane)
     return (b1 ? y[1] : y[0]) + __shfl_xor_sync(0xffffffffu, b1 ? y[0] : y[1], 1);
 }
 // Sums over the eight lanes that share columns: lane lr has that of value lr of
-// {x[0].x, x[0].y, x[1].x, ...}, column 8 (lr / 2) + 2 lq + lr % 2.
+// {x[0].x, x[0].y, x[1].x, ...}, column 8 lq + lr.
 __device__ __forceinline__ float col_sums8(const float2 (&x)[4], int lane)
 {
     const bool b16 = (lane & 16) != 0, b8 = (lane & 8) != 0, b4 = (lane & 4) != 0;
@@ -592,7 +606,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
         // warp w reads TMEM lanes 32 (w % 4) ..: rows 32 g ..., columns [32 cg, 32 cg + 32)
         const int ew = warp - T3_CTL_WARPS, g = warp & 3, cg = ew >> 2;
         const int lr = lane >> 2, lq = lane & 3, c0 = 32 * cg;
-        const int r0 = 32 * g + lr, cq = c0 + 2 * lq;   // the lane's first row and column
+        const int r0 = 32 * g + 8 * (lr >> 1) + (lr & 1), cq = c0 + 8 * lq;   // the lane's first row and column
         const int etid = tid - T3_CTL_WARPS * 32;
         uint32_t aph = 0, iph = 0, sph = 0;
         int b = 0, sb = 0;
@@ -641,14 +655,14 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
             if (!ok) break;
             T3Sums& su = sm.sums[sb];
             if (MODE == T3_FORM && norms_only) {
-                // diagonal tile: x_i . x_i is the Gram value at (r, r), of the
-                // lanes whose columns 2 lq, 2 lq + 1 contain row lr
+                // diagonal tile: x_i . x_i is the Gram value at equal positions, of
+                // the lanes with lr = 2 lq or 2 lq + 1
                 const int4 w = it.w;
                 if (cg == g && (lr >> 1) == lq) {
                     for (int k = w.x; k >= 0; k = tab[k].form_next - 1)
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            const int x = w.y * T + r0 + 8 * u;
+                            const int x = w.y * T + r0 + 2 * u;
                             if (x < tab[k].n) tab[k].sq3[x] = lr & 1 ? G.v[u][u].y : G.v[u][u].x;
                         }
                 }
@@ -657,14 +671,14 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                 float2 f[4] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f)};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float2 sj = ld2(&cc.sq[0][cq + 8 * j]), wj = ld2(&cc.mu[0][cq + 8 * j]);
+                    const float2 sj = ld2(&cc.sq[0][cq + 2 * j]), wj = ld2(&cc.mu[0][cq + 2 * j]);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) f[k] = __ffma2_rn(wj, rbf2(rb, G.v[k][j], cc.sq[1][r0 + 8 * k], sj), f[k]);
+                    for (int k = 0; k < 4; ++k) f[k] = __ffma2_rn(wj, rbf2(rb, G.v[k][j], cc.sq[1][r0 + 2 * k], sj), f[k]);
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) add_pair(fs[k], fc[k], f[k].x + f[k].y, 0.f);
                 if (it.last) {
-                    // a row's four lanes: lane lq has rows 8 lq + lr
+                    // a row's four lanes: lane lq has row r0 + 2 lq
 #pragma unroll
                     for (int o = 2; o > 0; o >>= 1) {
                         const bool up = (lane & o) != 0;
@@ -676,8 +690,8 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                             add_pair(fs[k], fc[k], xs, xc);
                         }
                     }
-                    su.row[0][cg][32 * g + 8 * lq + lr] = fs[0];
-                    su.row[1][cg][32 * g + 8 * lq + lr] = fc[0];
+                    su.row[0][cg][r0 + 2 * lq] = fs[0];
+                    su.row[1][cg][r0 + 2 * lq] = fc[0];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) fs[k] = fc[k] = 0.f;
                     if (!meet()) { ok = false; break; }
@@ -701,33 +715,51 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                     for (int k = 0; k < 4; ++k) rsum[s][k] = csum[s][k] = f2(0.f);
                 float tmx = 0.f;
                 float* const store = MODE == T3_FORM && it.store ? it.store + (size_t)r0 * T + cq : nullptr;
+                const auto entry = [&](int k, float2 g2, float2 sj, int c) {
+                    const int rk = r0 + 2 * k;
+                    float2 e = rbf2(rb, g2, cc.sq[1][rk], sj);
+                    if (!full) {
+                        const int least = diag ? rk : -1;
+                        if (!(rk < rows && c < cols && c > least)) e.x = 0.f;
+                        if (!(rk < rows && c + 1 < cols && c + 1 > least)) e.y = 0.f;
+                    }
+                    return e;
+                };
+                if constexpr (MODE == T3_FORM) {
+                    float2 sj[4], yj[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int c = cq + 8 * j;
-                    const float2 sj = ld2(&cc.sq[0][c]), yj = ld2(&cc.y[0][c]);
-                    const uint32_t sx = __float_as_uint(yj.x), sy = __float_as_uint(yj.y);
-                    float2 muj, alj;
-                    if (MODE == T3_FINAL) {
-                        muj = ld2(&cc.mu[0][c]);
-                        alj = ld2(&cc.al[0][c]);
+                    for (int j = 0; j < 4; ++j) {
+                        sj[j] = ld2(&cc.sq[0][cq + 2 * j]);
+                        yj[j] = ld2(&cc.y[0][cq + 2 * j]);
                     }
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const int rk = r0 + 8 * k;
-                        float2 e = rbf2(rb, G.v[k][j], cc.sq[1][rk], sj);
-                        if (!full) {
-                            const int least = diag ? rk : -1;
-                            if (!(rk < rows && c < cols && c > least)) e.x = 0.f;
-                            if (!(rk < rows && c + 1 < cols && c + 1 > least)) e.y = 0.f;
-                        }
-                        const uint32_t si = __float_as_uint(cc.y[1][rk]);
-                        const float2 q = flip(e, si ^ sx, si ^ sy);
-                        if (MODE == T3_FORM) {
+                        const uint32_t si = __float_as_uint(cc.y[1][r0 + 2 * k]);
+                        float2 q[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const float2 e = entry(k, G.v[k][j], sj[j], cq + 2 * j);
                             rsum[0][k] = __fadd2_rn(rsum[0][k], e);
                             csum[0][j] = __fadd2_rn(csum[0][j], e);
                             tmx = fmaxf(tmx, fmaxf(e.x, e.y));
-                            if (store) *reinterpret_cast<float2*>(store + (8 * k) * T + 8 * j) = q;
-                        } else {
+                            q[j] = flip(e, si ^ __float_as_uint(yj[j].x), si ^ __float_as_uint(yj[j].y));
+                        }
+                        if (store)
+                            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(store + 2 * k * T),
+                                         "f"(q[0].x), "f"(q[0].y), "f"(q[1].x), "f"(q[1].y), "f"(q[2].x), "f"(q[2].y),
+                                         "f"(q[3].x), "f"(q[3].y)
+                                         : "memory");
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int c = cq + 2 * j;
+                        const float2 sj = ld2(&cc.sq[0][c]), yj = ld2(&cc.y[0][c]), muj = ld2(&cc.mu[0][c]), alj = ld2(&cc.al[0][c]);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int rk = r0 + 2 * k;
+                            const uint32_t si = __float_as_uint(cc.y[1][rk]);
+                            const float2 q = flip(entry(k, G.v[k][j], sj, c), si ^ __float_as_uint(yj.x), si ^ __float_as_uint(yj.y));
                             rsum[0][k] = __ffma2_rn(q, muj, rsum[0][k]);
                             rsum[NSUM - 1][k] = __ffma2_rn(q, alj, rsum[NSUM - 1][k]);
                             csum[0][j] = __ffma2_rn(q, f2(cc.mu[1][rk]), csum[0][j]);
@@ -737,8 +769,8 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                 }
 #pragma unroll
                 for (int s = 0; s < NSUM; ++s) {
-                    su.row[s][cg][32 * g + 8 * lq + lr] = row_sums4(rsum[s], lane);
-                    su.col[s][g][c0 + 8 * (lr >> 1) + 2 * lq + (lr & 1)] = col_sums8(csum[s], lane);
+                    su.row[s][cg][r0 + 2 * lq] = row_sums4(rsum[s], lane);
+                    su.col[s][g][cq + lr] = col_sums8(csum[s], lane);
                 }
                 float* const tilemax = MODE == T3_FORM ? it.tilemax : nullptr;
                 if (MODE == T3_FORM && tilemax) {
