@@ -1034,7 +1034,7 @@ gabp_status gabp_svm_decision(gabp_svm_t h, const void* Xtest, int64_t t, float*
     // their planes packed and checked in one pass over the caller's rows.
     const int64_t slab = std::min<int64_t>(t, (int64_t)1 << 17);
     const int Ntt = (int)((slab + T - 1) / T);
-    const int per = decision_splits(1, INT_MAX) + Ntt;   // entries of a slab: at most 2 * SMs + its tiles
+    const int per = decision_entries(Ntt);   // entries of a slab, at most
     const size_t bxp = align_up(pack3_bytes(Ntt, (int)m), 1024), bsq = align_up((size_t)Ntt * T * 4, 256);
     const size_t bin = dev ? 0 : align_up((size_t)slab * m * x_elem_bytes(xd), 256);
     const size_t bpart = align_up((size_t)per * T * sizeof(float), 256), bw = align_up((size_t)per * sizeof(int4), 256);

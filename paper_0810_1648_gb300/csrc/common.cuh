@@ -403,10 +403,9 @@ void launch_final_tiles_q(const Inst* tab, const StopOp* ops, const int4* tiles,
 cudaError_t launch_final_tiles_gram(const Inst* tab, const StopOp* ops, const int4* tiles, long long ntiles, cudaStream_t s);
 // Decision values of t test rows using alpha: tab = {the test rows as an
 // instance (n = t, Xp3 packed, sq3 to fill), the training instance}, diag = {0,
-// I, I, I} for its tiles; every test tile is summed in decision_splits(Ntt, Nt)
-// ranges of the training tiles, work and part hold so many entries (x T) per
-// test tile.  out is written unless check->status is set.
-int decision_splits(int Ntt, int Nt);
+// I, I, I} for its tiles; work and part hold decision_entries(Ntt) entries (x T).
+// out is written unless check->status is set.
+int decision_entries(int Ntt);
 cudaError_t launch_decision_tc(const Inst* tab, const int4* diag, int4* work, int t, int Nt, const float* alpha, float* part,
                                const Ctrl* check, float* out, cudaStream_t s);
 // Gather helpers for inspection.
