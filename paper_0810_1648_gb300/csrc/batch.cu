@@ -151,6 +151,18 @@ __global__ void k_fetch(const W* __restrict__ src, W* __restrict__ dst, size_t c
         dst[i] = src[i];
 }
 
+// Results to the caller's device buffers: job blockIdx.x.
+struct CopyJob {
+    const float* src;
+    float* dst;
+    int n;
+};
+__global__ void k_copy_results(const CopyJob* __restrict__ jobs)
+{
+    const CopyJob c = jobs[blockIdx.x];
+    for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < c.n; i += gridDim.y * blockDim.x) c.dst[i] = c.src[i];
+}
+
 // The round lists of the live instances (live[k] != 0), built on the device
 // so that a membership change costs one small copy and one launch instead of
 // host loops over every tile: tiles grouped by stage and, within a stage, by
@@ -347,6 +359,8 @@ class Engine {
     int chunk = 16;
     std::map<int, cudaGraphExec_t> graphs;
     std::vector<int> pending;     // added, Q not formed yet
+    std::vector<CopyJob> copies;  // results to copy to device buffers
+    CopyJob* d_copies = nullptr;
     DevBlock lists;               // the instance table, control blocks and lists
     size_t pinned_bytes = 0;      // their pinned mirrors (from h_ctrl on)
     char* arena = nullptr;        // one allocation for a known set of instances (gabp_batch_solve)
@@ -434,8 +448,9 @@ class Engine {
         const size_t b_bt = aup((size_t)cap_members * sizeof(double), 256);
         const size_t b_sched = aup((size_t)2 * kMaxStages * sizeof(Sched), 256);
         const size_t b_live = aup((size_t)cap_members * sizeof(int), 256);
+        const size_t b_copies = aup((size_t)2 * cap_members * sizeof(CopyJob), 256);
         EK(scratch_alloc(&lists, b_tab + b_ctrl + 2 * b_work + 2 * b_nbl + b_ops + b_f3 + b_mem + 2 * b_bl + 2 * b_bt +
-                                     b_sched + b_live, stream));
+                                     b_sched + b_live + b_copies, stream));
         char* base = static_cast<char*>(lists.p);
         size_t off = 0;
         auto carve = [&](size_t bytes) { char* r = base + off; off += bytes; return r; };
@@ -454,6 +469,7 @@ class Engine {
         d_restart_tol = (double*)carve(b_bt);
         d_sched = (Sched*)carve(b_sched);   // one per message path and stage
         d_live = (int*)carve(b_live);
+        d_copies = (CopyJob*)carve(b_copies);
         EK(cudaMemsetAsync(d_ctrl, 0, b_ctrl, stream));
         EK(cudaMemsetAsync(d_sched, 0, b_sched, stream));
         // the pinned mirrors in one block
@@ -564,6 +580,7 @@ class Engine {
     {
         for (auto& m : mem) m = Member{};
         pending.clear();
+        copies.clear();
         sb.stopped.clear();
         rejoin.clear();
         rejoin_event = false;
@@ -944,17 +961,35 @@ class Engine {
         return GABP_OK;
     }
 
+    // The queued results to their device buffers, in one launch (one copy per
+    // array: 1024 calls, 2 ms of the host's time, for 512 instances).
+    gabp_status copy_results(cudaStream_t ss)
+    {
+        if (copies.empty()) return GABP_OK;
+        int most = 0;
+        for (const CopyJob& c : copies) most = std::max(most, c.n);
+        EK(cudaMemcpyAsync(d_copies, copies.data(), copies.size() * sizeof(CopyJob), cudaMemcpyHostToDevice, ss));
+        k_copy_results<<<dim3((unsigned)copies.size(), (unsigned)std::min(64, (most + 1023) / 1024)), 256, 0, ss>>>(d_copies);
+        EK(cudaGetLastError());
+        ++launches;
+        copies.clear();
+        return GABP_OK;
+    }
+
     // Records the results of a stopped instance from its final residual /
     // objective / #SV (in h_f3) and queues the copy of alpha to the caller.
     gabp_status finish(int slot, const Ctrl& c, cudaStream_t ss)
     {
         Member& M = mem[(size_t)slot];
         const double* f3 = h_f3 + 3 * (size_t)slot;
-        const cudaMemcpyKind kind = M.out_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-        if (M.out_alpha) EK(cudaMemcpyAsync(M.out_alpha, M.alpha, (size_t)M.inst.n * 4, kind, ss));
-        // the means the final pass used (the refined accumulator or the round k* aggregates)
-        if (M.out_mu && h_ops[(size_t)slot].mu)
-            EK(cudaMemcpyAsync(M.out_mu, h_ops[(size_t)slot].mu, (size_t)M.inst.n * 4, kind, ss));
+        // alpha, and the means the final pass used (the refined accumulator or the round k* aggregates)
+        const float* src[2] = {M.alpha, h_ops[(size_t)slot].mu};
+        float* dst[2] = {M.out_alpha, M.out_mu};
+        for (int a = 0; a < 2; ++a) {
+            if (!dst[a] || !src[a]) continue;
+            if (M.out_dev) copies.push_back(CopyJob{src[a], dst[a], M.inst.n});   // (copy_results)
+            else EK(cudaMemcpyAsync(dst[a], src[a], (size_t)M.inst.n * 4, cudaMemcpyDeviceToHost, ss));
+        }
         M.res.residual_inf = f3[0];
         M.res.dual_objective = f3[1];
         M.res.n_support = (int64_t)std::llround(f3[2]);
@@ -1103,6 +1138,7 @@ class Engine {
             if (gabp_status st = finish(k, sb.snap[u], ss)) return st;
             if (finished) finished->push_back(k);
         }
+        if (gabp_status st = copy_results(ss)) return st;
         if (!blist.empty()) {
             if (!rnb.empty())
                 EK(cudaMemcpyAsync(d_stop_nbl, rnb.data(), rnb.size() * sizeof(int2), cudaMemcpyHostToDevice, ss));
