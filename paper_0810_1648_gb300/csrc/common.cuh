@@ -44,15 +44,19 @@ enum Status : int {
 // Device-resident control block of one solver instance.  Kernels of a sweep
 // read `t` and `done` from here, so a captured chunk of sweeps can be
 // replayed from any starting round.
-struct Ctrl {
+struct alignas(32) Ctrl {
+    // read at once by every block of a finalize (round_state): 32 bytes
     int t;                    // message updates applied since create/refit
     int done;                 // set once the solve must stop
-    int limit;                // stop when t reaches this
+    int p_frozen;             // P messages at their fixed point: sweeps no longer write them
+    int path;                 // PATH_HIST or PATH_STORED, set when a solve is armed (choose_path)
+    int terms;                // odd terms of E in the next round
+    int even;                 // whether the even orders beyond q^2 count
     int kstar;                // round whose aggregates are the answer
+    int zero_h;               // next sweep treats the H messages as 0 (restart of the b-dependent part)
+    int limit;                // stop when t reaches this
     int converged;            // 1 if the residual test stopped the solve
     int status;               // first error (Status), 0 if none
-    int zero_h;               // next sweep treats the H messages as 0 (restart of the b-dependent part)
-    int p_frozen;             // P messages at their fixed point: sweeps no longer write them
     int p_changed;            // some P message changed in the current round
     int t_frozen;             // first round run with frozen P (valid when p_frozen)
     long long bad_index;      // offending node (or pair row) of the first error
@@ -64,7 +68,6 @@ struct Ctrl {
                                          // ||b - Q mu||_inf * it
     double tol;
     double rinf;              // ||r(kstar)||_inf as seen by the convergence test
-    int path;                 // PATH_HIST or PATH_STORED, set when a solve is armed (choose_path)
     unsigned int rq_bits;         // formation: the largest 1 / Q_ii (float bits)
     unsigned int zpair_bits[2];   // formation, instances that it leaves open: the largest z and |q| / d over
                                   // the pairs at Step 1 (float bits, k_pair_z)
@@ -73,8 +76,6 @@ struct Ctrl {
     float z, u;
     unsigned int dmax_bits, mumax_bits;
     float change;             // the changes of the last rounds as E weighs them, relative to the largest mean
-    int even;                 // whether the even orders beyond q^2 count
-    int terms;                // odd terms of E in the next round
 };
 
 // How the rounds of an instance hold the messages.

@@ -97,7 +97,7 @@ __device__ __forceinline__ int even_orders(float z, float u)
 }
 // Whether the tiles of a round after the first write E (live rounds with even
 // orders always do).
-__device__ __forceinline__ bool round_has_e(const Ctrl* c, bool frozen) { return c->terms > 0 || (!frozen && c->even); }
+__device__ __forceinline__ bool round_has_e(int terms, int even, bool frozen) { return terms > 0 || (!frozen && even); }
 // The change of the round just done is `now`; u = |q| / d damps what earlier
 // ones leave, and a round that happens to change little counts for at least
 // half the one before.
