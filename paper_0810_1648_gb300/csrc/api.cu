@@ -830,6 +830,8 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
     for (int I = 0; I < h->Nt; ++I)
         wd[(size_t)I] = make_int4(0, I, I, (int)((long long)I * h->Nt - (long long)I * (I - 1) / 2));
     h->grid = round_grid(h->ntiles, nblk, o.q_mode, 0, o.msg_bf16);
+    h->grid.ctrls = h->inst.ctrl;
+    h->grid.one = h->Nt <= kWarpFinNt ? -nblk : nblk;
     h->nlive = h->ntiles;
     e = cudaMemcpyAsync(h->work_all, wl.data(), wl.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->nbl, nb.data(), nb.size() * sizeof(int2), cudaMemcpyHostToDevice, h->stream);

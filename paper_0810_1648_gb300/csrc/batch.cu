@@ -494,6 +494,7 @@ class Engine {
     {
         ctas_per_sm = cps;
         grid = round_grid(cap_tiles, cap_nblk, q_mode, cps, msg_bf16);
+        grid.ctrls = d_ctrl;
     }
 
     void release(Member& m)

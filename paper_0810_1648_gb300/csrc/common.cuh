@@ -267,6 +267,8 @@ struct StopOp {
 struct RoundGrid {
     int sweep = 1;
     int finalize = 1;
+    Ctrl* ctrls = nullptr;   // the instances' control blocks, by table index
+    int one = 0;             // a single instance (tab[0]): its node blocks, negative if it has at most kWarpFinNt tile rows
 };
 
 // Gram operands: rows [0, n) of an n x m FP32 matrix with row norms sq.
@@ -368,7 +370,7 @@ void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sche
                   const RoundGrid& g, int q_mode, int msg_bf16, int paths, Chain chain, cudaStream_t s,
                   cudaEvent_t* ev = nullptr);
 // One pair sweep of PATH_HIST instances over a stage's tile list (sweep_hist.cu).
-void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, int stage_no, int grid, int q_mode,
+void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, int stage_no, const RoundGrid& g, int q_mode,
                        bool chained, cudaStream_t s);
 cudaError_t prepare_sweep_hist();
 // Formation, after launch_init over the same instances: Ctrl::zpair_bits over

@@ -3,6 +3,8 @@
 #pragma once
 
 #include "common.cuh"
+
+#include <cstddef>
 #include "ptx.cuh"
 
 namespace gabp {
@@ -72,6 +74,24 @@ __device__ __forceinline__ void hist_pad(const Inst& p, int x)
     for (int k = 0; k < 3 * p.nstages; ++k) p.hnow[(size_t)k * p.npad + x] = 0.f;
     for (int k = 0; k < p.nstages * kHist; ++k) p.hring[(size_t)k * 4 * p.npad + x] = 1.f;
     hist_clear(p, x);
+}
+
+// What the kernels of a round read of an instance's control block, in two
+// 16-byte loads.
+struct CtrlHead {
+    int t, done, p_frozen, path, terms, even;
+};
+__device__ __forceinline__ CtrlHead ctrl_head(const Ctrl* c)
+{
+    static_assert(offsetof(Ctrl, t) == 0 && offsetof(Ctrl, done) == 4 && offsetof(Ctrl, p_frozen) == 8 &&
+                      offsetof(Ctrl, path) == 12 && offsetof(Ctrl, terms) == 16 && offsetof(Ctrl, even) == 20, "");
+    CtrlHead h;
+    int k, z;
+    asm volatile("ld.volatile.global.v4.s32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(h.t), "=r"(h.done), "=r"(h.p_frozen), "=r"(h.path) : "l"(c) : "memory");
+    asm volatile("ld.volatile.global.v4.s32 {%0, %1, %2, %3}, [%4 + 16];"
+                 : "=r"(h.terms), "=r"(h.even), "=r"(k), "=r"(z) : "l"(c) : "memory");
+    return h;
 }
 
 // What a round leaves out (sweep_hist.cu) moves a mean by at most this

@@ -1144,30 +1144,27 @@ struct RoundState {
     // needs anyway; the H slots hold E when there are terms of it
     bool from_r, with_e;
 };
-__device__ __forceinline__ RoundState round_state(const Inst& p, const Ctrl* ctrl, bool& done)
+__device__ __forceinline__ RoundState round_state(int nstages, const Ctrl* ctrl, bool& done)
 {
-    static_assert(offsetof(Ctrl, t) == 0 && offsetof(Ctrl, path) == 12 && offsetof(Ctrl, terms) == 16 && offsetof(Ctrl, even) == 20, "");
-    int t, fin, frozen, path, terms, even, k, z;
-    asm volatile("ld.volatile.global.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(t), "=r"(fin), "=r"(frozen), "=r"(path) : "l"(ctrl) : "memory");
-    asm volatile("ld.volatile.global.v4.s32 {%0, %1, %2, %3}, [%4 + 16];" : "=r"(terms), "=r"(even), "=r"(k), "=r"(z) : "l"(ctrl) : "memory");
+    const CtrlHead h = ctrl_head(ctrl);
     RoundState s;
-    done = fin != 0;
-    s.t = t;
-    s.frozen = frozen != 0;
-    s.hist = path == PATH_HIST;
-    s.from_r = s.hist && p.nstages == 1;
-    s.with_e = t > 0 && round_has_e(terms, even, s.frozen);
+    done = h.done != 0;
+    s.t = h.t;
+    s.frozen = h.p_frozen != 0;
+    s.hist = h.path == PATH_HIST;
+    s.from_r = s.hist && nstages == 1;
+    s.with_e = h.t > 0 && round_has_e(h.terms, h.even, s.frozen);
     return s;
 }
 // The same for a whole CTA, read by one thread: with every warp of 625 CTAs
 // asking for the same line, its values took 6 us to arrive at n = 20000 (of a
 // finalize of 16), and 2.4 us at n = 6238 (of 10).
-__device__ __forceinline__ RoundState round_state_cta(const Inst& p, const Ctrl* ctrl, bool& done)
+__device__ __forceinline__ RoundState round_state_cta(int nstages, const Ctrl* ctrl, bool& done)
 {
     __shared__ RoundState s_state;
     __shared__ bool s_done;
     __syncthreads();   // the last node block's values are read
-    if (threadIdx.x == 0) s_state = round_state(p, ctrl, s_done);
+    if (threadIdx.x == 0) s_state = round_state(nstages, ctrl, s_done);
     __syncthreads();
     done = s_done;
     return s_state;
@@ -1354,36 +1351,48 @@ __device__ __forceinline__ void slot_sums(const Inst& p, int x, int k0, int step
 // (eight warps over the slots, then one reduction).  An instance's blocks all
 // take the same mode, so its arithmetic does not depend on the other
 // instances of the list.
-__device__ __forceinline__ int fin_units(const Sched* sc, int& usmall)
-{
-    usmall = (sc->nsmall + 7) / 8;
-    return usmall + (sc->nblocks - sc->nsmall);
-}
+//
+// A handle's rounds (one != 0: its node blocks, negative where they take a warp
+// each) need neither the schedule nor the lists: every load that another one
+// waits for is 0.4 us of a kernel of 7 to 10.
+struct FinList {
+    int nsmall, usmall, units;
+    const int2* nbl;   // null for a handle
+    __device__ __forceinline__ FinList(const int2* list, const Sched* sc, int one)
+    {
+        const int blocks = one ? abs(one) : sc->nblocks;
+        nsmall = one ? (one < 0 ? blocks : 0) : sc->nsmall;
+        usmall = (nsmall + 7) / 8;
+        units = usmall + (blocks - nsmall);
+        nbl = one ? nullptr : list;
+    }
+    __device__ __forceinline__ int2 block(int k) const { return nbl ? nbl[k] : make_int2(0, k); }
+};
 
 // Per node x: compensated sums of its slots, next aggregates, residual
 // r_x(t) in FP64, max |r| -> ctrl; the last node block of an instance to
 // finish decides.  Five CTAs per SM (48 registers a thread), so that one
 // CTA per 32-node block of n = 20000 (625) runs in a single wave.
 __global__ void __launch_bounds__(256, 5)
-    k_finalize(const Inst* __restrict__ tab, const int2* __restrict__ nbl, const Sched* __restrict__ sched)
+    k_finalize(const Inst* __restrict__ tab, const int2* __restrict__ nbl, const Sched* __restrict__ sched,
+               Ctrl* ctrls, int nstages, int one)
 {
-    int usmall;
-    const int units = fin_units(sched, usmall), nsmall = sched->nsmall;
     __shared__ float red[6][8][32];
     __shared__ int s_last;
     chain_next();
     chain_wait();
+    const FinList fl(nbl, sched, one);
     const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
-    for (int u = blockIdx.x; u < units; u += gridDim.x) {
-        if (u < usmall) {
+    for (int u = blockIdx.x; u < fl.units; u += gridDim.x) {
+        if (u < fl.usmall) {
             // ---- one warp per node block
             const int bi = 8 * u + g;
-            if (bi >= nsmall) continue;
-            const int2 nb = nbl[bi];
+            if (bi >= fl.nsmall) continue;
+            const int2 nb = fl.block(bi);
             const Inst& p = tab[nb.x];
-            Ctrl* ctrl = p.ctrl;
+            Ctrl* ctrl = ctrls + nb.x;
             bool done;
-            const RoundState rs = round_state(p, ctrl, done);
+            const RoundState rs = round_state(nstages, ctrl, done);
             if (done) continue;
             const int x = nb.y * 32 + lane, n = p.n;
             NodeOut o{0.0, 0.f, 0.f};
@@ -1404,11 +1413,11 @@ __global__ void __launch_bounds__(256, 5)
             continue;
         }
         // ---- one CTA per node block: warp g sums slots g, g + 8, ...
-        const int2 nb = nbl[nsmall + (u - usmall)];
+        const int2 nb = fl.block(fl.nsmall + (u - fl.usmall));
         const Inst& p = tab[nb.x];
-        Ctrl* ctrl = p.ctrl;
+        Ctrl* ctrl = ctrls + nb.x;
         bool done;
-        const RoundState rs = round_state_cta(p, ctrl, done);
+        const RoundState rs = round_state_cta(nstages, ctrl, done);
         if (done) continue;
         const int x = nb.y * 32 + lane, n = p.n;
         NodeIn v{};
@@ -1518,22 +1527,23 @@ __device__ __forceinline__ NodeOut stage_node(const Inst& p, int st, int x, cons
 }
 
 __global__ void __launch_bounds__(256)
-    k_finalize_stage(const Inst* __restrict__ tab, const int2* __restrict__ nbl, const Sched* __restrict__ sched, int st)
+    k_finalize_stage(const Inst* __restrict__ tab, const int2* __restrict__ nbl, const Sched* __restrict__ sched,
+                     Ctrl* ctrls, int nstages, int one, int st)
 {
-    int usmall;
-    const int units = fin_units(sched, usmall), nsmall = sched->nsmall;
     __shared__ float red[4][8][32];
     chain_next();
     chain_wait();
+    const FinList fl(nbl, sched, one);
     const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
-    for (int u = blockIdx.x; u < units; u += gridDim.x) {
-        if (u < usmall) {
+    for (int u = blockIdx.x; u < fl.units; u += gridDim.x) {
+        if (u < fl.usmall) {
             const int bi = 8 * u + g;
-            if (bi >= nsmall) continue;
-            const int2 nb = nbl[bi];
+            if (bi >= fl.nsmall) continue;
+            const int2 nb = fl.block(bi);
             const Inst& p = tab[nb.x];
+            Ctrl* ctrl = ctrls + nb.x;
             bool done;
-            const RoundState rs = round_state(p, p.ctrl, done);
+            const RoundState rs = round_state(nstages, ctrl, done);
             if (done) continue;
             const int x = nb.y * 32 + lane;
             NodeOut o{0.0, 0.f, 0.f};
@@ -1542,14 +1552,14 @@ __global__ void __launch_bounds__(256)
                 slot_sums<2>(p, x, 0, 1, rs, sv, cv);
                 o = stage_node(p, st, x, rs, (double)sv[0] + (double)cv[0], (double)sv[1] + (double)cv[1]);
             }
-            note_block(p.ctrl, rs, o, lane);
+            note_block(ctrl, rs, o, lane);
             continue;
         }
-        const int2 nb = nbl[nsmall + (u - usmall)];
+        const int2 nb = fl.block(fl.nsmall + (u - fl.usmall));
         const Inst& p = tab[nb.x];
-        Ctrl* ctrl = p.ctrl;
+        Ctrl* ctrl = ctrls + nb.x;
         bool done;
-        const RoundState rs = round_state_cta(p, ctrl, done);
+        const RoundState rs = round_state_cta(nstages, ctrl, done);
         if (done) continue;
         const int x = nb.y * 32 + lane, n = p.n;
         float sv[2] = {0.f, 0.f}, cv[2] = {0.f, 0.f};
@@ -1956,7 +1966,7 @@ void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sche
         const Sched* sc = sched + kMaxStages + st;
         if (ev && st == 0) cudaEventRecordWithFlags(ev[0], s, cudaEventRecordExternal);
         if (paths & (1 << PATH_HIST)) {
-            launch_sweep_hist(tab, work, sched + st, st, g.sweep, q_mode, chain, s);
+            launch_sweep_hist(tab, work, sched + st, st, g, q_mode, chain, s);
             chain = mode != CHAIN_NONE;
         }
         if (paths & (1 << PATH_STORED)) {
@@ -1977,9 +1987,9 @@ void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sche
         }
         if (ev && st == nstages - 1) cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal);
         if (st < nstages - 1)
-            launch_chained(chain, k_finalize_stage, g.finalize, 256, 0, s, tab, nbl, sched, st + 1);
+            launch_chained(chain, k_finalize_stage, g.finalize, 256, 0, s, tab, nbl, sched, g.ctrls, nstages, g.one, st + 1);
         else
-            launch_chained(chain, k_finalize, g.finalize, 256, 0, s, tab, nbl, sched);
+            launch_chained(chain, k_finalize, g.finalize, 256, 0, s, tab, nbl, sched, g.ctrls, nstages, g.one);
     }
 }
 

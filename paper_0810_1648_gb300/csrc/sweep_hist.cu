@@ -77,7 +77,7 @@ struct HInfo {
 struct HTail {
     unsigned long long full[H_STAGES], empty[H_STAGES];
     unsigned long long tfull[2], tempty[2];
-    int cabort;
+    int cabort, go;
     HInfo info[2];
     alignas(16) float node[2][2][N_COUNT][T];   // [slot][row, column block]
     alignas(16) float cs[S_COUNT][HCW][T];      // column sums of each warp
@@ -100,7 +100,8 @@ __host__ __device__ constexpr int q_rows<void>() { return T; }
 template <typename QT, bool FINAL = false>
 __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, const int4* __restrict__ work,
                                               long long ntiles, HTail& sm, unsigned char* ring, volatile int* abort_flag,
-                                              int lane, int st, const StopOp* __restrict__ ops = nullptr)
+                                              int lane, int st, const StopOp* __restrict__ ops, const Ctrl* ctrls, bool one,
+                                              CtrlHead head)
 {
     constexpr bool STREAM = q_rows<QT>() < T;
     const uint64_t pol = l2_evict_first_policy(), pol_keep = l2_evict_last_policy();
@@ -131,10 +132,11 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
             use = 1u << N_MU0;
         } else if (w.x != inst) {
             inst = w.x;
-            done = *(volatile const int*)&ctrl->done != 0;
-            t = *(volatile const int*)&ctrl->t;
-            const int frozen = *(volatile const int*)&ctrl->p_frozen, terms = ctrl->terms;
-            even = ctrl->even;
+            if (!one) head = ctrl_head(ctrls + inst);
+            done = head.done != 0;
+            t = head.t;
+            const int frozen = head.p_frozen, terms = head.terms;
+            even = head.even;
             staged = p.nstages > 1;
             kind = frozen && t > 0                    ? (terms == 0 ? K_SUM : terms == 1 ? K_ONE : K_TWO)
                    : t == 0 || (!even && terms == 0)  ? K_LIVE0
@@ -766,21 +768,23 @@ __device__ __forceinline__ void init_htail(HTail& sm)
     sm.cabort = 0;
 }
 
-// A single instance that has stopped: the rest of a captured chunk of rounds
-// (skipping its tiles one by one took 640 us a round at n = 100000).
-__device__ __forceinline__ bool nothing_to_do(const Inst* tab, const Sched* sched)
+// Read by the producer warp at the start of a sweep, beside the schedule: a
+// handle's control block.  False where there is nothing to do: no tiles, or the
+// instance has stopped (the rest of a captured chunk of rounds, which would
+// otherwise pass through every tile: 640 us a round at n = 100000).
+__device__ __forceinline__ bool sweep_head(const Sched* sched, const Ctrl* ctrls, bool one, CtrlHead& head)
 {
-    return sched->ntiles == 0 || (sched->ninst == 1 && *(volatile const int*)&tab[0].ctrl->done != 0);
+    if (one) head = ctrl_head(ctrls);
+    return sched->ntiles > 0 && !(one && head.done);
 }
 
 // Q stored (FP32 or BF16) and streamed.
 template <typename QT>
 __global__ void __launch_bounds__(H_THREADS, 2)
-    k_sweep_hist(const Inst* __restrict__ tab, const int4* __restrict__ work, const Sched* __restrict__ sched, int stage_no)
+    k_sweep_hist(const Inst* __restrict__ tab, const int4* __restrict__ work, const Sched* __restrict__ sched, int stage_no,
+                 const Ctrl* ctrls, int one)
 {
     chain_next();
-    const long long ntiles = sched->ntiles;
-    work += sched->off;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* ring = align_smem(smem_raw, 128);
     HTail& sm = *reinterpret_cast<HTail*>(ring + H_STAGES * H_CHUNK);
@@ -789,11 +793,19 @@ __global__ void __launch_bounds__(H_THREADS, 2)
         init_htail(sm);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    __syncthreads();
     chain_wait();
-    if (nothing_to_do(tab, sched)) return;
-    if (tid >= HCW * 32) {
-        hist_producer<QT>(tab, work, ntiles, sm, ring, nullptr, tid & 31, stage_no);
+    const bool producer = tid >= HCW * 32;
+    CtrlHead head{};
+    if (producer) {
+        const bool go = sweep_head(sched, ctrls, one != 0, head);
+        if ((tid & 31) == 0) sm.go = go;
+    }
+    __syncthreads();
+    if (!sm.go) return;
+    const long long ntiles = sched->ntiles;
+    work += sched->off;
+    if (producer) {
+        hist_producer<QT>(tab, work, ntiles, sm, ring, nullptr, tid & 31, stage_no, nullptr, ctrls, one != 0, head);
         return;
     }
     StreamedQ<QT> src{ring, 0, 0u, false};
@@ -868,13 +880,10 @@ struct TileQ {
 
 __global__ void __launch_bounds__(HR_THREADS, 1)
     k_sweep_hist_rc(const Inst* __restrict__ tab, const int4* __restrict__ work, const Sched* __restrict__ sched,
-                    int stage_no)
+                    int stage_no, const Ctrl* ctrls, int one)
 {
     chain_next();
-    const long long ntiles = sched->ntiles;
     chain_wait();
-    if (nothing_to_do(tab, sched)) return;
-    work += sched->off;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* xops = align_smem(smem_raw, 1024);
     unsigned char* qtile = xops + HR_XSTAGES * 2 * BLK_BYTES;
@@ -894,6 +903,15 @@ __global__ void __launch_bounds__(HR_THREADS, 1)
         ex.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    CtrlHead head{};
+    if (warp == 8) {
+        const bool go = sweep_head(sched, ctrls, one != 0, head);
+        if (lane == 0) sm.go = go;
+    }
+    __syncthreads();
+    if (!sm.go) return;
+    const long long ntiles = sched->ntiles;
+    work += sched->off;
     if (warp == 10) tmem_alloc(&ex.tmem_base, HR_TMEM_COLS);
     tc_fence_before();
     __syncthreads();
@@ -905,7 +923,7 @@ __global__ void __launch_bounds__(HR_THREADS, 1)
         TileQ src{qtile, &ex, 0, false};
         hist_consumers(src, sm, tab, work, ntiles, tid);
     } else if (warp == 8) {
-        hist_producer<void>(tab, work, ntiles, sm, nullptr, abort_flag, lane, stage_no);
+        hist_producer<void>(tab, work, ntiles, sm, nullptr, abort_flag, lane, stage_no, nullptr, ctrls, one != 0, head);
     } else if (warp == 9) {
         if (lane == 0) {
             const uint64_t pol = l2_evict_last_policy();   // the features are read again by many tiles
@@ -1049,7 +1067,7 @@ __global__ void __launch_bounds__(H_THREADS, 2)
     }
     __syncthreads();
     if (tid >= HCW * 32) {
-        hist_producer<float, true>(tab, work, ntiles, sm, ring, nullptr, tid & 31, 0, ops);
+        hist_producer<float, true>(tab, work, ntiles, sm, ring, nullptr, tid & 31, 0, ops, nullptr, false, CtrlHead{});
         return;
     }
     StreamedQ<float> src{ring, 0, 0u, false};
@@ -1121,16 +1139,18 @@ cudaError_t prepare_sweep_hist()
     return e;
 }
 
-void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, int stage_no, int grid, int q_mode,
+void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, int stage_no, const RoundGrid& g, int q_mode,
                        bool chained, cudaStream_t s)
 {
     if (q_mode == 2)
-        launch_chained(chained, k_sweep_hist_rc, grid, HR_THREADS, hist_rc_smem_bytes(), s, tab, work, sched, stage_no);
+        launch_chained(chained, k_sweep_hist_rc, g.sweep, HR_THREADS, hist_rc_smem_bytes(), s, tab, work, sched, stage_no,
+                       g.ctrls, g.one);
     else if (q_mode == 1)
-        launch_chained(chained, k_sweep_hist<__nv_bfloat16>, grid, H_THREADS, hist_smem_bytes(), s, tab, work, sched,
-                       stage_no);
+        launch_chained(chained, k_sweep_hist<__nv_bfloat16>, g.sweep, H_THREADS, hist_smem_bytes(), s, tab, work, sched,
+                       stage_no, g.ctrls, g.one);
     else
-        launch_chained(chained, k_sweep_hist<float>, grid, H_THREADS, hist_smem_bytes(), s, tab, work, sched, stage_no);
+        launch_chained(chained, k_sweep_hist<float>, g.sweep, H_THREADS, hist_smem_bytes(), s, tab, work, sched, stage_no,
+                       g.ctrls, g.one);
 }
 
 void launch_final_tiles_q(const Inst* tab, const StopOp* ops, const int4* tiles, long long ntiles, cudaStream_t s)
