@@ -390,6 +390,8 @@ class Engine {
         if (side) cudaStreamDestroy(side);
         if (sstream) cudaStreamDestroy(sstream);
         if (rejoin_ev) cudaEventDestroy(rejoin_ev);
+        for (auto e : fork_ev)
+            if (e) cudaEventDestroy(e);
         if (own_stream && stream) cudaStreamDestroy(stream);
     }
 
@@ -426,6 +428,7 @@ class Engine {
         }
         EK(cudaStreamCreateWithFlags(&sstream, cudaStreamNonBlocking));
         EK(cudaEventCreateWithFlags(&rejoin_ev, cudaEventDisableTiming));
+        for (auto& e : fork_ev) EK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         {
             // keep freed instance memory in the stream-ordered pool for reuse
             int dev = 0;
@@ -925,9 +928,11 @@ class Engine {
         auto it = graphs.find(key);
         if (it != graphs.end()) { *out = it->second; return GABP_OK; }
         cudaGraph_t g = nullptr;
+        // (the side stream takes part in the capture only; its own work goes on)
+        const Fork fork{sstream, fork_ev[0], fork_ev[1]};
         EK(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
         for (int k = 0; k < rounds; ++k)
-            launch_round(d_tab, d_work, d_nbl, d_sched, nstages, grid, q_mode, msg_bf16, mask, CHAIN_NONE, stream);
+            launch_round(d_tab, d_work, d_nbl, d_sched, nstages, grid, q_mode, msg_bf16, mask, CHAIN_NONE, stream, nullptr, &fork);
         EK(cudaStreamEndCapture(stream, &g));
         cudaGraphExec_t ex = nullptr;
         cudaError_t e = cudaGraphInstantiate(&ex, g, 0);
@@ -1037,6 +1042,7 @@ class Engine {
     std::vector<int> rejoin;      // restarted, join the lists at the next launch
     bool rejoin_event = false;    // rejoin_ev orders their restart before that launch
     cudaEvent_t rejoin_ev = nullptr;
+    cudaEvent_t fork_ev[2] = {nullptr, nullptr};   // of a round's second sweep (graph_for)
 
     gabp_status stop_begin(cudaStream_t ss, int* running)
     {

@@ -342,6 +342,14 @@ cudaError_t prepare_sweep_rc();
 // round's path: n = 1000, 19.4 -> 16.4 us a round; n = 6238, 29.7 -> 27.1.  The
 // kernels of a captured graph are not chained: they start as early (15.2 and
 // 26.2 us), and chained ones later (staged, n = 12960: 133 -> 146 us).
+// Where the sweeps of the second message path run beside those of the first
+// (while a round is captured): most rounds of a batch that has both have little
+// on the second.  A batch of 512 problems: 38.6 ms one after the other, 37.1 side
+// by side.
+struct Fork {
+    cudaStream_t stream;
+    cudaEvent_t start, end;
+};
 enum Chain { CHAIN_NONE, CHAIN_AFTER_FIRST, CHAIN_ALL };   // which kernels of a round
 template <class... P, class... A>
 void launch_chained(bool chained, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args)
@@ -368,7 +376,7 @@ void launch_chained(bool chained, void (*kernel)(P...), int grid, int block, siz
 // stage st, sched[st] the PATH_HIST one.
 void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sched* sched, int nstages,
                   const RoundGrid& g, int q_mode, int msg_bf16, int paths, Chain chain, cudaStream_t s,
-                  cudaEvent_t* ev = nullptr);
+                  cudaEvent_t* ev = nullptr, const Fork* fork = nullptr);
 // One pair sweep of PATH_HIST instances over a stage's tile list (sweep_hist.cu).
 void launch_sweep_hist(const Inst* tab, const int4* work, const Sched* sched, int stage_no, const RoundGrid& g, int q_mode,
                        bool chained, cudaStream_t s);

@@ -1959,17 +1959,25 @@ cudaError_t prepare_sweep()
 }
 
 void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sched* sched, int nstages,
-                  const RoundGrid& g, int q_mode, int msg_bf16, int paths, Chain mode, cudaStream_t s, cudaEvent_t* ev)
+                  const RoundGrid& g, int q_mode, int msg_bf16, int paths, Chain mode, cudaStream_t s, cudaEvent_t* ev,
+                  const Fork* fork)
 {
+    const bool both = fork && (paths & (1 << PATH_HIST)) && (paths & (1 << PATH_STORED));
     bool chain = mode == CHAIN_ALL;
     for (int st = 0; st < nstages; ++st) {
         const Sched* sc = sched + kMaxStages + st;
         if (ev && st == 0) cudaEventRecordWithFlags(ev[0], s, cudaEventRecordExternal);
+        if (both) {
+            cudaEventRecord(fork->start, s);
+            cudaStreamWaitEvent(fork->stream, fork->start, 0);
+        }
         if (paths & (1 << PATH_HIST)) {
             launch_sweep_hist(tab, work, sched + st, st, g, q_mode, chain, s);
             chain = mode != CHAIN_NONE;
         }
         if (paths & (1 << PATH_STORED)) {
+            const cudaStream_t main = s;
+            const cudaStream_t s = both ? fork->stream : main;
             if (q_mode == 2 && msg_bf16)
                 launch_chained(chain, k_sweep_rc<MsgBF16>, g.sweep, RC_THREADS, rc_smem_bytes<MsgBF16>(), s, tab, work, sc, st);
             else if (q_mode == 2)
@@ -1984,6 +1992,10 @@ void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sche
                 launch_chained(chain, k_sweep<float, MsgF32>, g.sweep, SWEEP_THREADS, sweep_smem_bytes<float, MsgF32>(), s,
                                tab, work, sc, st);
             chain = mode != CHAIN_NONE;
+            if (both) {
+                cudaEventRecord(fork->end, s);
+                cudaStreamWaitEvent(main, fork->end, 0);
+            }
         }
         if (ev && st == nstages - 1) cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal);
         if (st < nstages - 1)
