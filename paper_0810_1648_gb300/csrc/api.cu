@@ -118,6 +118,7 @@ struct gabp_svm_s {
     Ctrl* hctrl = nullptr;          // pinned mirror of the control block, as of the last wait for the stream
     Ctrl* hdec = nullptr;           // and of a decision's
     double* hfinal = nullptr;       // pinned {rinf, objective, nsv}
+    int* hnote = nullptr;           // pinned, written by the device (Inst::note)
     struct Graph {
         cudaGraphExec_t exec = nullptr;
         std::vector<cudaEvent_t> ev;   // 2 per bracketed round when captured with profiling on
@@ -152,8 +153,8 @@ gabp_status check_formed(gabp_svm_t h)
     return GABP_OK;
 }
 
-// The pinned mirrors: two control blocks and {rinf, objective, nsv}.
-constexpr size_t kMirrorBytes = 2 * sizeof(Ctrl) + 4 * sizeof(double);
+// The pinned mirrors: two control blocks, {rinf, objective, nsv} and Inst::note.
+constexpr size_t kMirrorBytes = 2 * sizeof(Ctrl) + 4 * sizeof(double) + sizeof(int);
 
 // Device memory plan of one handle (bytes, 256-aligned sub-buffers).
 struct Plan {
@@ -383,13 +384,13 @@ gabp_status stage_and_form(gabp_svm_t h, const void* X, const float* y)
         static const float kNaN = NAN;
         CK(cudaMemcpyAsync((void*)(p.y + n / 2), &kNaN, sizeof(float), cudaMemcpyHostToDevice, s));
     }
-    void* tmp = nullptr;
+    DevBlock tmp;
     const void* src = X;
     if (!dev) {
         if (xd != 0) {   // FP64 / BF16 rows: widened to FP32 by the staging kernel
-            CK(pool_alloc(&tmp, (size_t)n * m * x_elem_bytes(xd), s));
-            CK(cudaMemcpyAsync(tmp, X, (size_t)n * m * x_elem_bytes(xd), cudaMemcpyHostToDevice, s));
-            src = tmp;
+            CK(scratch_alloc(&tmp, (size_t)n * m * x_elem_bytes(xd), s));
+            CK(cudaMemcpyAsync(tmp.p, X, (size_t)n * m * x_elem_bytes(xd), cudaMemcpyHostToDevice, s));
+            src = tmp.p;
         } else {
             CK(cudaMemcpyAsync((void*)p.X, X, (size_t)n * m * sizeof(float), cudaMemcpyHostToDevice, s));
             src = p.X;
@@ -399,9 +400,9 @@ gabp_status stage_and_form(gabp_svm_t h, const void* X, const float* y)
     CK(launch_stage(src, xd, (int)n, (int)m, h->Nt, (float*)p.X, const_cast<float*>(p.y), (float*)p.b,
                     const_cast<float*>(p.b0), p.task, (void*)p.Xp3, 0, p.ctrl, nullptr, s));
     h->prof.kernel_launches += 1;
-    if (tmp) CK(cudaFreeAsync(tmp, s));
     CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    scratch_free(&tmp, s);
     if (h->hctrl->status != 0)
         return fail(GABP_EINVAL, h->opts.task == GABP_TASK_KRR ? "row %lld: non-finite feature or target"
                                                                 : "row %lld: non-finite feature or label not +-1",
@@ -509,22 +510,45 @@ void destroy_all(gabp_svm_t h)
 // (every `stride`-th round: k = stride - 1, 2 stride - 1, ...), and its pair.
 static bool bracketed(int stride, int k) { return stride > 0 && k % stride == stride - 1; }
 
-// `rounds` synchronous rounds on the handle's stream.
-static void launch_rounds(gabp_svm_t h, int rounds, int path, gabp_svm_s::Graph* G)
+// Up to `iters` rounds, launched one after another (chained) until the device
+// notes that the solve has stopped, never more than kRoundsAhead beyond the last
+// one noted: the device always has the next rounds queued, and no more than
+// these run for nothing.  (In chunks of 16 with a wait after each, half a chunk
+// ran for nothing: n = 1000 from FP64 host arrays, create to destroy, 0.90 ms
+// against 0.77 with the input's buffer from the scratch pool too.)
+constexpr int kRoundsAhead = 3;
+gabp_status run_direct(gabp_svm_t h, int iters, int path)
 {
-    const int stride = G ? h->profiling : 0;
-    for (int k = 0; k < rounds; ++k)
-        launch_round(h->d_tab, h->work, h->nbl, h->sched, h->nstages, h->grid, h->opts.q_mode, h->opts.msg_bf16,
-                     1 << path, G ? CHAIN_NONE : k == 0 ? CHAIN_AFTER_FIRST : CHAIN_ALL, h->stream, bracketed(stride, k) ? &G->ev[(size_t)2 * (k / stride)] : nullptr);
+    cudaStream_t s = h->stream;
+    volatile int* note = h->hnote;
+    const int t0 = h->hctrl->t;
+    *note = t0;
+    for (int k = 0; k < iters; ++k) {
+        int seen = *note;
+        for (long spins = 1; !(seen & kNoteStopped) && k - (seen - t0) >= kRoundsAhead; seen = *note)
+            if ((++spins & 0xffff) == 0) {   // a note that does not come: the stream has ended, well or not
+                const cudaError_t e = cudaStreamQuery(s);
+                if (e == cudaSuccess) break;
+                if (e != cudaErrorNotReady) return fail(GABP_ECUDA, "rounds failed: %s", cudaGetErrorString(e));
+            }
+        if (seen & kNoteStopped) break;
+        launch_round(h->d_tab, h->work, h->nbl, h->sched, h->nstages, h->grid, h->opts.q_mode, h->opts.msg_bf16, 1 << path,
+                     k == 0 ? CHAIN_AFTER_FIRST : CHAIN_ALL, s);
+        h->prof.kernel_launches += 2;
+    }
+    CK(cudaGetLastError());
+    return GABP_OK;
 }
 
-// A handle's chunk becomes a graph at its kGraphAfter-th use: capturing and
-// instantiating 16 rounds costs the host 95 us, while launching them one by
-// one (70 us) goes on beside the device, one round of two kernels 1 us slower
-// than in the graph (a staged round of eight, n = 12960: 15 us, so those are
-// captured at once).  What a chunk launches depends only
-// on what is fixed at create, so its graph serves later refits too; the few
-// kept ones are dropped when calls with ever new round counts come.
+// A handle's rounds go by captured chunks from its kGraphAfter-th call on:
+// capturing and instantiating 16 rounds costs the host 95 us, while launching them
+// one by one goes on beside the device, each round 1 to 2 us slower than in the
+// graph (100 rounds at n = 20000: 14.00 against 13.86 ms), but without rounds run
+// for nothing after the last and without waits between chunks.  A staged round of
+// eight kernels loses 15 us (n = 12960), so those are captured at once.  What a chunk
+// launches depends only on what is fixed at create, so its graph serves later
+// refits too; the few kept ones are dropped when calls with ever new round counts
+// come.
 constexpr int kGraphAfter = 4;
 constexpr size_t kGraphsKept = 8;
 
@@ -546,7 +570,9 @@ gabp_status get_graph(gabp_svm_t h, int rounds, int path, gabp_svm_s::Graph** ou
     }
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    launch_rounds(h, rounds, path, &G);
+    for (int k = 0; k < rounds; ++k)
+        launch_round(h->d_tab, h->work, h->nbl, h->sched, h->nstages, h->grid, h->opts.q_mode, h->opts.msg_bf16, 1 << path,
+                     CHAIN_NONE, h->stream, bracketed(stride, k) ? &G.ev[(size_t)2 * (k / stride)] : nullptr);
     cudaError_t e = cudaStreamEndCapture(h->stream, &g);
     if (e != cudaSuccess) return fail(GABP_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
     e = cudaGraphInstantiate(&G.exec, g, 0);
@@ -576,18 +602,18 @@ gabp_status run_rounds(gabp_svm_t h, int iters, double tol, Ctrl* out)
         const int len = tol > 0 ? std::min<int>(h->opts.chunk, iters) : iters;
         const int path = h->hctrl->path;
         const int max_chunks = (iters + len - 1) / len + 1;
-        int t_before = h->hctrl->t;
+        const int t0 = h->hctrl->t;
+        int t_before = t0;
         for (int c = 0; c < max_chunks; ++c) {
             gabp_svm_s::Graph* g = nullptr;
             if (gabp_status st = get_graph(h, len, path, &g)) return st;
             ++g->uses;
             if (g->exec) {
                 CK(cudaGraphLaunch(g->exec, s));
-            } else {
-                launch_rounds(h, len, path, nullptr);
-                CK(cudaGetLastError());
+                h->prof.kernel_launches += 2 * len;
+            } else if (gabp_status st = run_direct(h, iters - (t_before - t0), path)) {
+                return st;
             }
-            h->prof.kernel_launches += 2 * len;
             CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
             const int ran = h->hctrl->t - t_before;
@@ -741,6 +767,7 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
     h->hctrl = static_cast<Ctrl*>(mirror);
     h->hdec = h->hctrl + 1;
     h->hfinal = reinterpret_cast<double*>(h->hctrl + 2);
+    h->hnote = reinterpret_cast<int*>(h->hfinal + 4);
     char* base = static_cast<char*>(h->pool.p);
     size_t off = 0;
     auto take = [&](size_t bytes) { void* r = base + off; off += bytes; return r; };
@@ -795,6 +822,7 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
     }
     h->nbl = (int2*)take(pl.nbl);
     p.ctrl = (Ctrl*)take(pl.ctrl);
+    p.note = h->hnote;
     p.rhist = (double*)take(pl.rhist);
     p.rhist_cap = kRhistCap;
     h->final3 = (double*)take(pl.final3);

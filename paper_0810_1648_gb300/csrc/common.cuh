@@ -44,6 +44,8 @@ enum Status : int {
 // Device-resident control block of one solver instance.  Kernels of a sweep
 // read `t` and `done` from here, so a captured chunk of sweeps can be
 // replayed from any starting round.
+constexpr int kNoteStopped = (int)0x80000000u;
+
 struct alignas(32) Ctrl {
     // read at once by every block of a finalize (round_state): 32 bytes
     int t;                    // message updates applied since create/refit
@@ -130,6 +132,7 @@ struct Inst {
     unsigned long long* rfix;  // formation: where set, the |Q| row-sum partials are added to these
                                // per-node fixed-point sums (rsum_fix) instead of written to slots
     Ctrl* ctrl;
+    int* note;        // pinned host word: the rounds done, with kNoteStopped once the solve has stopped; null: not told
     double* rhist;    // ||r(t)||_inf per round (rhist_cap entries)
     int rhist_cap;
     float gamma;      // RBF width

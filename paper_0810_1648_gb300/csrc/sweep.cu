@@ -1309,6 +1309,7 @@ __device__ __forceinline__ void finalize_decide(const Inst& p, Ctrl* ctrl, const
     ctrl->zero_h = 0;
     ctrl->rmax_bits = 0ull;
     ctrl->blocks_done = 0u;
+    if (p.note) *(volatile int*)p.note = (t + 1) | (status != 0 || rmax < tol || t + 1 >= limit ? kNoteStopped : 0);
 }
 
 // Compensated sums of node x's slots k = k0, k0 + step, ... (of the
