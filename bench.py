@@ -49,7 +49,7 @@ PRECISION_WORKLOAD = {
     "workload": "precision form, n=100000, m=64 FP32 3-component mixture (seed 2), RBF gamma=0.5/64, C=1, "
                 "100 synchronous sweeps per solve, Q as selected by q_mode",
     "n": 100000, "m": 64, "sweeps_per_step": ROUNDS,
-    "l2": "no flush: every sweep streams 80 GB of messages, far above the 129 MB L2",
+    "l2": "no flush: every sweep streams 10 GB (BF16) or 20 GB (FP32) of Q, far above the 129 MB L2",
 }
 # Stored bytes of one Q entry per unordered pair, by Q mode.
 Q_BYTES = {"f32": 4, "bf16": 2, "recompute": 0}
@@ -142,9 +142,9 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-# The sources the pair sweep is compiled from: sweep.cu and the headers it
+# The sources the pair sweep is compiled from: sweep_hist.cu and the headers it
 # includes.  The profile summaries record the SHA-256 of their concatenation.
-SWEEP_SOURCES = ("sweep.cu", "common.cuh", "ptx.cuh", "qtile_epi.cuh")
+SWEEP_SOURCES = ("sweep_hist.cu", "common.cuh", "hist.cuh", "ptx.cuh", "qtile_epi.cuh")
 
 
 def sweep_source_sha() -> str:
@@ -158,7 +158,7 @@ def sweep_source_sha() -> str:
 def _traffic_from_profile():
     """DRAM bytes per launch of the pair sweep from the committed ncu summary,
     or None when the kernel sources changed since the counters were taken."""
-    path = os.path.join(ROOT, "profiles", "k_sweep_plain_large.txt")
+    path = os.path.join(ROOT, "profiles", "k_sweep_hist_plain_large.txt")
     try:
         txt = open(path).read()
     except OSError:
@@ -341,23 +341,19 @@ def run_batch(args):
             last = res
         conv = sum(r["converged"] for r in last)
         ph = gabp.batch_last_phases()
-        # algorithmic bytes of all the rounds run, per pair and round: Q once,
-        # the message state read once and written once while P changes, only
-        # H written after the exact P-freeze (a few rounds in): the two give a
-        # range, since the freeze round of each instance is not reported
+        # algorithmic bytes of all the rounds run, per pair and round: Q once
+        # (the few instances that store their messages, at 14 to 36 B, are
+        # counted alike)
         qb = 2 if kw.get("q_mode", 0) == 1 else 4
-        ms = 4 if kw.get("msg_bf16") else 8
-        b_live, b_frozen = qb + 4 * ms, qb + 3 * ms
         pair_rounds = sum(r["iters_done"] * p.n * (p.n - 1) / 2 for p, r in zip(probs, last))
         rs = ph["rounds_ms"] / 1e3
         out[mode] = {"solves_per_s": len(probs) / float(np.median(times)), "ms_per_batch": 1e3 * float(np.median(times)),
                      "phases_ms": ph,
                      "converged": conv, "max_residual": max(r["residual_inf"] for r in last),
                      "mean_rounds": float(np.mean([r["iters_done"] for r in last])),
-                     "rounds_hbm": {"pair_rounds": pair_rounds, "bytes_per_pair_round": [b_frozen, b_live],
-                                    "GBps_over_rounds_phase": [pair_rounds * b / rs / 1e9 for b in (b_frozen, b_live)],
-                                    "frac_of_measured_peak": [pair_rounds * b / rs / 1e9 / _peak_gbs()
-                                                              for b in (b_frozen, b_live)]}}
+                     "rounds_hbm": {"pair_rounds": pair_rounds, "bytes_per_pair_round": qb,
+                                    "GBps_over_rounds_phase": pair_rounds * qb / rs / 1e9,
+                                    "frac_of_measured_peak": pair_rounds * qb / rs / 1e9 / _peak_gbs()}}
     # end to end: host (numpy) inputs, their copies inside the timed solves
     e2e_t = []
     kw_e2e = dict(q_mode=1, refine=8, msg_bf16=1)
@@ -455,7 +451,7 @@ def run_sparse(args):
         kept, total = int(stt["tiles_kept"]), int(stt["tiles_total"])
         nt = (p.n + T_TILE - 1) // T_TILE
         pairs = (kept - nt) * T_TILE * T_TILE + nt * T_TILE * (T_TILE - 1) // 2   # full-tile count, diagonal halves
-        bytes_frozen = 28 * pairs
+        bytes_round = 4 * pairs   # Q once
         sweep_ms = prof["sweep_ms"] / max(prof["sweep_launches"], 1)
         dev_bytes = int(stt["device_bytes"])
         gabp.svm_destroy(h)
@@ -473,7 +469,7 @@ def run_sparse(args):
         answers[name] = alpha.cpu().numpy().copy()
         out[name] = {"sweeps_per_s": args.steps * ROUNDS / (ms / 1e3), "tiles_kept": kept, "tiles_total": total,
                      "device_bytes": dev_bytes, "dense_message_state_bytes": 8 * p.n * p.n,
-                     "avg_sweep_ms": sweep_ms, "hbm_frac_frozen_bytes": bytes_frozen / (sweep_ms / 1e3) / 1e9 / _peak_gbs(),
+                     "avg_sweep_ms": sweep_ms, "hbm_frac": bytes_round / (sweep_ms / 1e3) / 1e9 / _peak_gbs(),
                      "to_tolerance": {"ms": float(e0.elapsed_time(e1)), "rounds": int(k), "residual_inf": float(rinf),
                                       "converged": int(st2["converged"]), "err_bound_over_C": st2["err_bound"] / p.C,
                                       "margin": st2["margin"]}}
@@ -716,13 +712,13 @@ def _extra_precision(gabp, torch, peak):
         ms = float(e0.elapsed_time(e1))
         prof = gabp.svm_get_profile(h)
         gabp.svm_destroy(h)
-        nz, nf, nl = prof["sweep_launches_zero_state"], prof["sweep_launches_p_frozen"], prof["sweep_launches"]
-        alg = pairs * ((4 * mb + qb) * (nl - nz - nf) + (3 * mb + qb) * nf + (2 * mb + qb) * nz)
-        achieved = alg / (prof["sweep_ms"] / 1e3) / 1e9 if prof["sweep_ms"] > 0 else None
+        nl = prof["sweep_launches"]
+        alg = pairs * qb * nl   # a round reads Q alone (recomputed Q: nothing per pair)
+        achieved = alg / (prof["sweep_ms"] / 1e3) / 1e9 if prof["sweep_ms"] > 0 and alg else None
         entry = {"sweeps_per_s": 2 * ROUNDS / (ms / 1e3),
                  "sweep_hbm": {"achieved_GBps": achieved, "frac_of_measured_peak": achieved / peak if achieved else None,
                                "avg_launch_ms": prof["sweep_ms"] / max(nl, 1), "launches_timed": nl,
-                               "bytes_per_pair": {"p_live": 4 * mb + qb, "p_frozen": 3 * mb + qb}}}
+                               "bytes_per_pair": qb}}
         # to tolerance: refinement removes the BF16 error (FP32-Gram residual, FP64 sums)
         opts = gabp.opts_default(stream=stream.cuda_stream, chunk=8, q_mode=qm, msg_bf16=mb16,
                                  refine=10 if qm else 0)
@@ -841,29 +837,28 @@ def run_ours(args):
 
     # roofline of the dominant kernel (the pair sweep), timed live by events
     pairs = n * (n - 1) // 2
-    nz = prof["sweep_launches_zero_state"]
     nf = prof["sweep_launches_p_frozen"]
     nl = prof["sweep_launches"]
-    # per pair: round 0 writes P and H (16 B); later rounds read and write
-    # both (32 B) until the P messages reach their fixed point, then read P and
-    # H and write H (24 B); every round reads the stored Q entry (qb B)
-    alg_bytes = pairs * ((4 * mb + qb) * (nl - nz - nf) + (3 * mb + qb) * nf + (2 * mb + qb) * nz)
+    # per pair a round reads the stored Q entry and nothing else: the messages
+    # are rebuilt from the nodes' last aggregates (with Q recomputed the round
+    # is bound by the Gram tiles' epilogue instead)
+    alg_bytes = pairs * qb * nl
     sweep_s = prof["sweep_ms"] / 1e3
-    achieved = alg_bytes / sweep_s / 1e9 if sweep_s > 0 else None
+    achieved = alg_bytes / sweep_s / 1e9 if sweep_s > 0 and alg_bytes else None
     peaks = _peaks()
     if peaks and "hbm_gbs" in peaks:
         peak, peak_src = float(peaks["hbm_gbs"]), "measured"
     else:
         peak, peak_src = 6800.0, "fallback"
     traffic = _traffic_from_profile()
-    roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+    roof = {"bound": "hbm" if qb else "epilogue ALU", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": (achieved / peak) if achieved else None,
             "traffic": traffic if (args.workload == "plain_large" and args.q_mode == "f32") else None,
             "traffic_note": "ncu dram read+write of one frozen-P launch of this workload "
-                            "(profiles/k_sweep_plain_large.txt); null if the kernel source changed since",
-            "kernel": {"f32": "k_sweep<float>", "bf16": "k_sweep<bf16>", "recompute": "k_sweep_rc"}[args.q_mode]
+                            "(profiles/k_sweep_hist_plain_large.txt); null if the kernel source changed since",
+            "kernel": {"f32": "k_sweep_hist<float>", "bf16": "k_sweep_hist<bf16>", "recompute": "k_sweep_hist_rc"}[args.q_mode]
                       + " (pair sweep)", "peak_source": peak_src,
-            "bytes_per_pair": {"round0": 2 * mb + qb, "p_live": 4 * mb + qb, "p_frozen": 3 * mb + qb},
+            "bytes_per_pair": qb,
             "launches_p_frozen": nf,
             "algorithmic_bytes_per_launch": alg_bytes / max(nl, 1),
             "avg_launch_ms": prof["sweep_ms"] / max(nl, 1), "launches_timed": nl,

@@ -221,8 +221,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const int r = 32 * g + lane;
         int acc = 0;
         uint32_t aph = 0;
+        // the next tile, and the constants of the next item (the next instance
+        // over this tile, or the first one of the next), loaded ahead
+        int4 wn = blockIdx.x < ntiles ? work[blockIdx.x] : make_int4(0, 0, 0, 0);
+        TileCols<2> ahead{};
+        if (blockIdx.x < ntiles) ahead = load_tile_cols<2>(tab[wn.x], wn.z, wn.y * T + r, lane, 2 * half);
         for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
-            const int4 w = work[L];
+            const int4 w = wn;
+            if (L + gridDim.x < ntiles) wn = work[L + gridDim.x];
             const bool stop = __shfl_sync(0xffffffffu, *(volatile int*)&sm.abort, 0) != 0;
             if (stop || !mbar_wait_warp(&sm.accfull[acc], aph)) {
                 if (lane == 0) {
@@ -233,18 +239,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             }
             tc_fence_after();
             const int I = w.y, J = w.z;
-            const int i = I * T + r;
             // the listed instance and every one chained behind it (same
             // features) take their BF16 Q tile from this accumulator
             ColTile& cs = sm.cols[warp - 2];
             for (int k = w.x; k >= 0;) {
                 const Inst& p = tab[k];
-                const int n = p.n;
-                const float* y = p.y;
-                const float* sqb = p.sqb;
+                const int n = p.n, next = p.form_next - 1;
                 const float gamma = p.gamma, lam2 = p.lam2;
-                const float yi = i < n ? y[i] : 0.f, si = i < n ? sqb[i] : 0.f;
-                stage_tile_cols(cs, y, sqb, n, J, gamma, lane, 2 * half, 2 * half + 2);
+                const float yi = ahead.yi, si = ahead.si;
+                put_tile_cols(cs, ahead, gamma, lane, 2 * half);
+                if (next >= 0) ahead = load_tile_cols<2>(tab[next], J, I * T + r, lane, 2 * half);
+                else if (L + gridDim.x < ntiles) ahead = load_tile_cols<2>(tab[wn.x], wn.z, wn.y * T + r, lane, 2 * half);
                 const float ai = -gamma * kLog2e * si, c2 = 2.f * gamma * kLog2e;
                 const uint32_t s1 = __float_as_uint(yi) & 0x80000000u, si2 = s1 | (s1 >> 16);
                 __nv_bfloat16* qrow = static_cast<__nv_bfloat16*>(p.qstore) + (size_t)w.w * TT + (size_t)r * T;
@@ -259,11 +264,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                                   v);
                         uint4 out[2];
                         q_half_bf16(v, 32 * cc + 16 * h, ai, si2, cs, c2, lam2, (valid >> (16 * h)) & 0xffffu, out);
-                        dst[2 * h] = out[0];
-                        dst[2 * h + 1] = out[1];
+                        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 2 * h), "r"(out[0].x),
+                                     "r"(out[0].y), "r"(out[0].z), "r"(out[0].w), "r"(out[1].x), "r"(out[1].y), "r"(out[1].z),
+                                     "r"(out[1].w)
+                                     : "memory");
                     }
                 }
-                k = p.form_next - 1;
+                k = next;
             }
             tc_fence_before();
             __syncwarp();

@@ -36,30 +36,42 @@ struct ColTile {
     alignas(16) uint32_t s2[T / 2];
 };
 
-// Lane l writes the constants of columns 32 cc + l for the chunks cc in
-// [cc0, cc1) from the labels y and the norms sqb of the column block J
-// (zeros beyond n: such columns are masked out).  The first __syncwarp keeps
-// the previous tile's constants until every lane has read them.
-__device__ __forceinline__ void stage_tile_cols(ColTile& ct, const float* __restrict__ y,
-                                                const float* __restrict__ sqb, int n, int J, float gamma,
-                                                int lane, int cc0, int cc1)
+// Lane l's labels y and norms sqb of the columns 32 (cc0 + u) + l, u < N, of column
+// block J (zeros beyond n: such columns are masked out), and the row's own: loaded
+// a tile ahead of their use.
+template <int N>
+struct TileCols {
+    float y[N], s[N], yi, si;
+};
+template <int N>
+__device__ __forceinline__ TileCols<N> load_tile_cols(const Inst& p, int J, int i, int lane, int cc0)
 {
-    float yl[4], sl[4];
+    TileCols<N> c;
+    const int n = p.n;
+    const float* __restrict__ y = p.y;
+    const float* __restrict__ sqb = p.sqb;
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc) {
-        const int j = J * T + 32 * cc + lane;
-        const bool in = cc >= cc0 && cc < cc1 && j < n;
-        yl[cc] = in ? y[j] : 0.f;
-        sl[cc] = in ? sqb[j] : 0.f;
+    for (int u = 0; u < N; ++u) {
+        const int j = J * T + 32 * (cc0 + u) + lane;
+        c.y[u] = j < n ? y[j] : 0.f;
+        c.s[u] = j < n ? sqb[j] : 0.f;
     }
+    c.yi = i < n ? y[i] : 0.f;
+    c.si = i < n ? sqb[i] : 0.f;
+    return c;
+}
+// Writes the columns' constants.  The first __syncwarp keeps the previous tile's
+// until every lane has read them.
+template <int N>
+__device__ __forceinline__ void put_tile_cols(ColTile& ct, const TileCols<N>& c, float gamma, int lane, int cc0)
+{
     __syncwarp();
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc) {
-        if (cc < cc0 || cc >= cc1) continue;
-        ct.b[32 * cc + lane] = -gamma * kLog2e * sl[cc];
-        const uint32_t sg = __float_as_uint(yl[cc]) & 0x80000000u;
+    for (int u = 0; u < N; ++u) {
+        ct.b[32 * (cc0 + u) + lane] = -gamma * kLog2e * c.s[u];
+        const uint32_t sg = __float_as_uint(c.y[u]) & 0x80000000u;
         const uint32_t other = __shfl_xor_sync(0xffffffffu, sg, 1);
-        if (!(lane & 1)) ct.s2[16 * cc + lane / 2] = (sg >> 16) | other;
+        if (!(lane & 1)) ct.s2[16 * (cc0 + u) + lane / 2] = (sg >> 16) | other;
     }
     __syncwarp();
 }

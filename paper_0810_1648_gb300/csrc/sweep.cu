@@ -1078,11 +1078,10 @@ __global__ void __launch_bounds__(RC_THREADS, 1)
             }
             tc_fence_after();
             const int I = w.y, J = w.z, i = I * T + r;
-            const float* y = p.y;
-            const float* sqb = p.sqb;
             const float gamma = p.gamma, lam2 = p.lam2;
-            const float yi = i < n ? y[i] : 0.f, si = i < n ? sqb[i] : 0.f;
-            stage_tile_cols(ex.cols[g], y, sqb, n, J, gamma, lane, 0, T / 32);
+            const TileCols<T / 32> cols = load_tile_cols<T / 32>(p, J, i, lane, 0);
+            const float yi = cols.yi, si = cols.si;
+            put_tile_cols(ex.cols[g], cols, gamma, lane, 0);
             const float ai = -gamma * kLog2e * si, c2 = 2.f * gamma * kLog2e;
             const uint32_t s1 = __float_as_uint(yi) & 0x80000000u, si2 = s1 | (s1 >> 16);
             uint4* qrow = reinterpret_cast<uint4*>(qtile + (size_t)acc * TT + (size_t)r * T);   // 16 chunks

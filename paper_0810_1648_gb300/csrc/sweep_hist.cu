@@ -878,6 +878,38 @@ struct TileQ {
     }
 };
 
+// A role's way through the CTA's tiles: list entries two tiles ahead of their
+// turn, and whether an instance has stopped read once per run of its tiles, so that
+// no role waits for either between two tiles.
+struct TileWalk {
+    const int4* work;
+    long long ntiles;
+    int4 w0, w1;      // the next tile and the one after
+    int inst = -1;
+    bool stopped = false;
+    __device__ __forceinline__ TileWalk(const int4* list, long long n) : work(list), ntiles(n)
+    {
+        const long long L = blockIdx.x;
+        w0 = L < ntiles ? work[L] : make_int4(0, 0, 0, 0);
+        w1 = L + gridDim.x < ntiles ? work[L + gridDim.x] : w0;
+    }
+    __device__ __forceinline__ int4 next(long long L)
+    {
+        const int4 w = w0;
+        w0 = w1;
+        if (L + 2LL * gridDim.x < ntiles) w1 = work[L + 2LL * gridDim.x];
+        return w;
+    }
+    __device__ __forceinline__ bool done(int k, const Ctrl* ctrls)
+    {
+        if (k != inst) {
+            inst = k;
+            stopped = *(volatile const int*)&ctrls[k].done != 0;
+        }
+        return stopped;
+    }
+};
+
 __global__ void __launch_bounds__(HR_THREADS, 1)
     k_sweep_hist_rc(const Inst* __restrict__ tab, const int4* __restrict__ work, const Sched* __restrict__ sched,
                     int stage_no, const Ctrl* ctrls, int one)
@@ -930,10 +962,11 @@ __global__ void __launch_bounds__(HR_THREADS, 1)
             int xs = 0;
             uint32_t ph = 0;
             bool run = true;
+            TileWalk walk(work, ntiles);
             for (long long L = blockIdx.x; L < ntiles && run; L += gridDim.x) {
-                const int4 w = work[L];
+                const int4 w = walk.next(L);
                 const Inst& p = tab[w.x];
-                if (*(volatile const int*)&p.ctrl->done) continue;
+                if (walk.done(w.x, ctrls)) continue;
                 const unsigned char* Xp = static_cast<const unsigned char*>(p.Xp);
                 const int nkc = p.nkc;
                 for (int kc = 0; kc < nkc; ++kc) {
@@ -956,9 +989,11 @@ __global__ void __launch_bounds__(HR_THREADS, 1)
             constexpr uint32_t IDESC = idesc_bf16_f32(T, T);
             int xs = 0, acc = 0;
             uint32_t ph = 0, aph = 0;
+            TileWalk walk(work, ntiles);
             for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
-                const Inst& p = tab[work[L].x];
-                if (*(volatile const int*)&p.ctrl->done) continue;
+                const int inst = walk.next(L).x;
+                const Inst& p = tab[inst];
+                if (walk.done(inst, ctrls)) continue;
                 const int nkc = p.nkc;
                 bool ok = !*abort_flag && mbar_wait(&ex.accempty[acc], aph ^ 1u);
                 tc_fence_after();
@@ -988,18 +1023,22 @@ __global__ void __launch_bounds__(HR_THREADS, 1)
     } else if (warp >= 12) {
         const int ew = warp - 12, g = warp & 3, half = ew >> 2, r = 32 * g + lane;
         int it = 0;
+        TileWalk walk(work, ntiles);
+        TileCols<2> ahead{};
+        if (blockIdx.x < ntiles) ahead = load_tile_cols<2>(tab[walk.w0.x], walk.w0.z, walk.w0.y * T + r, lane, 2 * half);
         for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
-            const int4 w = work[L];
+            const int4 w = walk.next(L);
+            const TileCols<2> cols = ahead;
+            if (L + gridDim.x < ntiles)
+                ahead = load_tile_cols<2>(tab[walk.w0.x], walk.w0.z, walk.w0.y * T + r, lane, 2 * half);
             const Inst& p = tab[w.x];
             Ctrl* ctrl = p.ctrl;
-            if (*(volatile const int*)&ctrl->done) continue;
-            const int n = p.n, I = w.y, J = w.z, i = I * T + r, acc = it & 1;
+            if (walk.done(w.x, ctrls)) continue;
+            const int n = p.n, I = w.y, J = w.z, acc = it & 1;
             const uint32_t par = (uint32_t)((it >> 1) & 1);
-            const float* y = p.y;
-            const float* sqb = p.sqb;
             const float gamma = p.gamma, lam2 = p.lam2;
-            const float yi = i < n ? y[i] : 0.f, si = i < n ? sqb[i] : 0.f;
-            stage_tile_cols(ex.cols[ew], y, sqb, n, J, gamma, lane, 2 * half, 2 * half + 2);
+            const float yi = cols.yi, si = cols.si;
+            put_tile_cols(ex.cols[ew], cols, gamma, lane, 2 * half);
             const bool stop = __shfl_sync(0xffffffffu, *abort_flag, 0) != 0;
             if (stop || !mbar_wait_warp(&ex.accfull[acc], par) || !mbar_wait_warp(&ex.qempty[acc], par ^ 1u)) {
                 if (lane == 0) {
