@@ -43,7 +43,7 @@ WORKLOAD = {
                 "(means N(0,1), sigma 0.7), RBF gamma=1/128, C=10, Q stored FP32 upper triangle, "
                 "100 synchronous sweeps per solve, seed 1",
     "n": 20000, "m": 128, "sweeps_per_step": ROUNDS, "q_mode": "f32",
-    "l2": "no flush: every sweep streams 3.3 GB of messages + 0.8 GB of Q, far above the 129 MB L2",
+    "l2": "no flush: every sweep streams 0.8 GB of Q, far above the 129 MB L2",
 }
 PRECISION_WORKLOAD = {
     "workload": "precision form, n=100000, m=64 FP32 3-component mixture (seed 2), RBF gamma=0.5/64, C=1, "
@@ -695,7 +695,6 @@ def _extra_precision(gabp, torch, peak):
     out = {}
     for name, qm, mb16 in modes:
         qb = Q_BYTES[name]
-        mb = 4 if mb16 else 8
         h = gabp.svm_create(Xd, yd, p.gamma, p.C, gabp.opts_default(stream=stream.cuda_stream, chunk=ROUNDS,
                                                                     q_mode=qm, msg_bf16=mb16))
         gabp.svm_set_profiling(h, PROFILE_STRIDE)
@@ -791,7 +790,6 @@ def run_ours(args):
         wl = dict(wl, task="krr", workload="kernel ridge regression (Section 1.2) on the same features: targets "
                   "sin(<w, x>) + 0.1 N(0, 1) (w ~ N(0, I/m), seed 11), ridge 1, dominant diagonal; " + wl["workload"])
     qb = Q_BYTES[args.q_mode]
-    mb = 4 if args.msg_bf16 else 8     # bytes of one stored message pair
     n = p.n
     stream = torch.cuda.Stream(device=dev)
     Xd = torch.from_numpy(p.X).to(dev)

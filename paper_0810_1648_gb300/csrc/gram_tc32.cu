@@ -283,7 +283,7 @@ struct T3Item {
     float* tilemax;          // where the largest |q| goes, or null
     float* dst[2];           // the row's and the column's slot sums (FINAL: of q mu; those of q alpha plen behind)
     unsigned long long* fix[2];   // where set, fixed-point sums instead of slots
-    double scale;
+    int shift;
     long long plen;
     int4 w;                  // norms_only: the work entry
     Ctrl* ctrl;
@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                             t.tilemax = MODE == T3_FORM && p.tilemax ? p.tilemax + w.w : nullptr;
                             t.fix[0] = MODE == T3_FORM && p.rfix ? p.rfix + (size_t)I * T : nullptr;
                             t.fix[1] = MODE == T3_FORM && p.rfix ? p.rfix + (size_t)J * T : nullptr;
-                            if (MODE == T3_FORM && p.rfix) t.scale = pow2i(rsum_shift(n, p.lam2));
+                            if (MODE == T3_FORM && p.rfix) t.shift = rsum_shift(n, p.lam2);
                         }
                     }
                     __syncwarp();
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                             const float vr = (rw[0][off] + rw[1][off]) + (rw[2][off] + rw[3][off]);
                             const float vc = ((cl[0][off] + cl[1][off]) + cl[2][off]) + cl[3][off];
                             const float v = diag ? vr + vc : role ? vc : vr;
-                            if (MODE == T3_FORM && it.fix[0]) atomicAdd(it.fix[role] + off, (unsigned long long)rsum_fix(v, it.scale));
+                            if (MODE == T3_FORM && it.fix[0]) atomicAdd(it.fix[role] + off, (unsigned long long)rsum_fix(v, it.shift));
                             else it.dst[role][s * it.plen + off] = v;
                         }
                     }

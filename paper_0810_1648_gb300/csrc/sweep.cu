@@ -1489,10 +1489,9 @@ __device__ __forceinline__ double offdiag_abs_sum(const Inst& p, int x, long lon
     long long a = 0;
     if (!p.rsum && x < p.n) {
         const int X = x / T, ns = slot_count(p, X);
-        const double scale = pow2i(sh);
         const float* s0 = p.part + (size_t)slot_begin(p, X) * T + (x - X * T);
 #pragma unroll 8
-        for (int k = g; k < ns; k += 8) a += rsum_fix(s0[(size_t)k * T], scale);
+        for (int k = g; k < ns; k += 8) a += rsum_fix(s0[(size_t)k * T], sh);
     }
     red[g][lane] = a;
     __syncthreads();
