@@ -12,7 +12,9 @@
 // i = I*T + r < j = J*T + c, where P_ij is the precision of the message
 // i -> j and H_ij = P_ij mu_ij.  They are separate so that, once the P
 // recursion (which does not depend on b) sits at its floating-point fixed
-// point, a round reads P and streams only H.
+// point, a round reads P and streams only H.  Most instances never write them:
+// PATH_HIST (hist.cuh, sweep_hist.cu) rebuilds what a round needs of the messages
+// from the nodes' last aggregates, which it keeps inside the same memory.
 //
 // Per-node partial sums: every kernel that reduces over pairs writes, for
 // node x and tile index k along the other axis, one value into
@@ -326,8 +328,7 @@ inline void launch_form_norms(const Inst* tab, const int4* diag_work, long long 
 {
     (void)launch_form_q_tc32(tab, diag_work, ntiles, 1, s);
 }
-// The three BF16 planes of FP32 rows (zero padding to whole tiles and chunks).
-// The planes of a caller's rows, checked, and their diagonal tile list (k_pack3_rows).
+// Bytes of the three BF16 planes of n x m FP32 rows (whole tiles and chunks).
 size_t pack3_bytes(int Nt, int m);
 // Precision form: BF16 operand packing + norms, and the tensor-core Q formation (BF16 store).
 cudaError_t launch_pack_bf16(const float* Xf, int n, int m, int nkc, int Nt, void* Xp, float* sqb, cudaStream_t s);

@@ -1,10 +1,10 @@
-// Input staging (FP64 -> FP32, label / finiteness checks), the final residual r
-// = 1 - Q mu and Q alpha for the dual objective from stored FP32 tiles, and SIMT
-// FP32 Gram tiles fused with the RBF kernel for the decision values of callers
-// without a handle (gabp_decision_noalloc).  (Q tiles, decisions of a handle and
-// final passes without stored tiles run on the tensor cores: gram_tc32.cu.)
+// The node sums of the final pass (residual r = 1 - Q mu and the dual objective
+// from Q alpha; the tiles' parts come from sweep_hist.cu and gram_tc32.cu), and SIMT
+// FP32 Gram tiles fused with the RBF kernel: decision values of callers without a
+// handle (gabp_decision_noalloc), and the pair pass of instances that do not store
+// Q.  (Staging, Q tiles and decisions of a handle: gram_tc32.cu.)
 //
-// One CTA computes one 128 x 128 Gram tile G = X_I X_J^T by SIMT FP32 FMAs
+// In gram_tile one CTA computes one 128 x 128 Gram tile G = X_I X_J^T by SIMT FP32 FMAs
 // (8 x 8 outputs per thread, K-chunks of 16 double-buffered in shared memory),
 // then runs an epilogue on the 64 values it holds: d^2 = max(0, s_i + s_j - 2 G),
 // K = expf(-gamma d^2), Q_ij = y_i y_j (K + lambda^2).  The distances use the

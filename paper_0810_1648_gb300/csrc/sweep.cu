@@ -1,6 +1,9 @@
 // The synchronous broadcast-GaBP round (Algorithm 2, Section 4) on the
 // device: a pair sweep over the stored upper triangle followed by a per-node
 // finalize that forms the next aggregates, the residual and the stop test.
+// The finalize serves both message paths; the sweep here is that of instances
+// that store their messages (PATH_STORED: pairs too strongly coupled for
+// sweep_hist.cu).
 //
 // Round t, information form (H = P mu):
 //   sweep    for every pair {i < j} with q = Q_ij, from the aggregates of t
