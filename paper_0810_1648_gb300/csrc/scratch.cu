@@ -119,7 +119,11 @@ cudaError_t scratch_alloc(DevBlock* b, size_t bytes, cudaStream_t s)
 
 void scratch_free(DevBlock* b, cudaStream_t s)
 {
-    if (b->p) b->pooled ? cudaFreeAsync(b->p, s) : cudaFree(b->p);
+    // (a pool block can be freed either way: cudaFree waits for the device)
+    if (b->p && (!b->pooled || cudaFreeAsync(b->p, s) != cudaSuccess)) {
+        if (b->pooled) cudaGetLastError();
+        cudaFree(b->p);
+    }
     *b = DevBlock{};
 }
 
