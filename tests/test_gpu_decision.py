@@ -65,3 +65,35 @@ def test_noalloc_decision(n, t, m):
     gabp.decision_noalloc(*(torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (X, y, alpha, Z)), p.gamma, 0.25, out)
     want, scale = _reference(X, y, alpha, p.gamma, 0.25, Z)
     assert np.max(np.abs(out.cpu().numpy() - want)) <= BAR * scale
+
+
+@pytest.mark.parametrize("m", [8, 64, 12])
+@pytest.mark.parametrize("dtype", ["float32", "bfloat16"])
+def test_rows_off_the_load_alignment(m, dtype):
+    """Device rows that begin one element past a 16-byte boundary (the wide
+    loads do not apply) give the bits of aligned ones: handle, decision and the
+    batched form, which reads FP32 rows in place."""
+    torch = pytest.importorskip("torch")
+    p = workloads.mixture(300, m, seed=m)
+    dt = getattr(torch, dtype)
+    Xa = torch.from_numpy(p.X).cuda().to(dt)
+    Za = torch.from_numpy(workloads.test_points(p, 140, seed=3)).cuda().to(dt)
+    y = torch.from_numpy(p.y).cuda()
+
+    def shifted(t):
+        buf = torch.zeros(t.numel() + 1, dtype=dt, device="cuda")
+        v = buf[1:].view(t.shape)
+        v.copy_(t)
+        assert v.data_ptr() % 16
+        return v
+
+    outs = []
+    for X, Z in ((Xa, Za), (shifted(Xa), shifted(Za))):
+        svm = gabp.GabpSVM(X, y, p.gamma, p.C)
+        alpha = svm.solve(20, 0.0)[0].clone()
+        dec = svm.decision(Z).clone()
+        svm.close()
+        both = gabp.batch_solve([workloads.Problem(X, y, p.gamma, c) for c in (p.C, 2.0)], 20, 0.0)[0]
+        outs.append((alpha, dec, both[0].clone(), both[1].clone()))
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
