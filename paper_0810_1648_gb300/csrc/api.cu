@@ -516,14 +516,15 @@ static bool bracketed(int stride, int k) { return stride > 0 && k % stride == st
 // these run for nothing.  (In chunks of 16 with a wait after each, half a chunk
 // ran for nothing: n = 1000 from FP64 host arrays, create to destroy, 0.90 ms
 // against 0.77 with the input's buffer from the scratch pool too.)
+// group: a captured group of `per` rounds to launch instead of single ones.
 constexpr int kRoundsAhead = 3;
-gabp_status run_direct(gabp_svm_t h, int iters, int path)
+gabp_status run_direct(gabp_svm_t h, int iters, int path, cudaGraphExec_t group, int per)
 {
     cudaStream_t s = h->stream;
     volatile int* note = h->hnote;
     const int t0 = h->hctrl->t;
     *note = t0;
-    for (int k = 0; k < iters; ++k) {
+    for (int k = 0; k < iters; k += per) {   // (rounds of a group beyond the limit do nothing)
         int seen = *note;
         for (long spins = 1; !(seen & kNoteStopped) && k - (seen - t0) >= kRoundsAhead; seen = *note)
             if ((++spins & 0xffff) == 0) {   // a note that does not come: the stream has ended, well or not
@@ -532,9 +533,12 @@ gabp_status run_direct(gabp_svm_t h, int iters, int path)
                 if (e != cudaErrorNotReady) return fail(GABP_ECUDA, "rounds failed: %s", cudaGetErrorString(e));
             }
         if (seen & kNoteStopped) break;
-        launch_round(h->d_tab, h->work, h->nbl, h->sched, h->nstages, h->grid, h->opts.q_mode, h->opts.msg_bf16, 1 << path,
-                     k == 0 ? CHAIN_AFTER_FIRST : CHAIN_ALL, s);
-        h->prof.kernel_launches += 2;
+        if (group)
+            CK(cudaGraphLaunch(group, s));
+        else
+            launch_round(h->d_tab, h->work, h->nbl, h->sched, h->nstages, h->grid, h->opts.q_mode, h->opts.msg_bf16, 1 << path,
+                         k == 0 ? CHAIN_AFTER_FIRST : CHAIN_ALL, s);
+        h->prof.kernel_launches += 2 * per;
     }
     CK(cudaGetLastError());
     return GABP_OK;
@@ -550,6 +554,10 @@ gabp_status run_direct(gabp_svm_t h, int iters, int path)
 // refits too; the few kept ones are dropped when calls with ever new round counts
 // come.
 constexpr int kGraphAfter = 4;
+// Rounds of a captured group of a staged solve to a tolerance: groups follow the
+// device's note as single rounds do (run_direct).  n = 12960, four stages, to
+// 1e-6: 2.42 ms, against 2.56 in chunks of 16 with a wait after each.
+constexpr int kGroupRounds = 2;
 constexpr size_t kGraphsKept = 8;
 
 // A chunk of `rounds` synchronous rounds, *out->exec null where it is launched
@@ -599,7 +607,8 @@ gabp_status run_rounds(gabp_svm_t h, int iters, double tol, Ctrl* out)
         CK(cudaMemcpyAsync(&p.ctrl->status, &kTimeout, sizeof(int), cudaMemcpyHostToDevice, s));
     }
     if (iters > 0) {
-        const int len = tol > 0 ? std::min<int>(h->opts.chunk, iters) : iters;
+        const bool grouped = tol > 0 && h->nstages > 1 && h->profiling == 0;
+        const int len = grouped ? kGroupRounds : tol > 0 ? std::min<int>(h->opts.chunk, iters) : iters;
         const int path = h->hctrl->path;
         const int max_chunks = (iters + len - 1) / len + 1;
         const int t0 = h->hctrl->t;
@@ -608,10 +617,10 @@ gabp_status run_rounds(gabp_svm_t h, int iters, double tol, Ctrl* out)
             gabp_svm_s::Graph* g = nullptr;
             if (gabp_status st = get_graph(h, len, path, &g)) return st;
             ++g->uses;
-            if (g->exec) {
+            if (g->exec && !grouped) {
                 CK(cudaGraphLaunch(g->exec, s));
                 h->prof.kernel_launches += 2 * len;
-            } else if (gabp_status st = run_direct(h, iters - (t_before - t0), path)) {
+            } else if (gabp_status st = run_direct(h, iters - (t_before - t0), path, g->exec, g->exec ? len : 1)) {
                 return st;
             }
             CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
