@@ -1119,25 +1119,29 @@ __global__ void __launch_bounds__(H_THREADS, 2)
 // decide alike.
 //
 // What bounds it: one read of the entries, 4 bytes a pair.  A warp has its 16
-// rows of a tile in flight at once and meets no barrier (whether an instance is
-// open is read by every thread, from lines that stay in L1).  With four rows in
+// rows of a tile in flight at once and meets no barrier.  With four rows in
 // flight and the check shared through a barrier: 38 us at n = 6238 (1225
 // tiles); now 27; a batch of 18 instances: 167 -> 73 us.
+//
+// Other warps raise the maxima meanwhile, so whether an instance is still open
+// is one lane's answer for its warp: all lanes take part in the shuffles below,
+// or none.
 __global__ void __launch_bounds__(256, 2) k_pair_z(const Inst* __restrict__ tab, const int4* __restrict__ work,
                                                   long long ntiles, bool single)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (single && !pair_z_open(tab[0])) return;
+    auto warp_agrees = [](bool mine) { return __shfl_sync(0xffffffffu, (int)mine, 0) != 0; };
+    if (single && !warp_agrees(pair_z_open(tab[0]))) return;
     for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
         const int4 w = work[L];
         for (int k = w.x; k >= 0; k = tab[k].form_next - 1) {
             const Inst& p = tab[k];
-            if (!pair_z_asks(p)) continue;
+            if (!pair_z_asks(p)) continue;   // (what it reads is fixed by now)
             const float* q = p.qref + (size_t)w.w * TT + warp * T + 4 * lane;
             float4 a[T / 8];
 #pragma unroll
             for (int r = 0; r < T / 8; ++r) a[r] = *reinterpret_cast<const float4*>(q + (size_t)r * 8 * T);
-            if (!orders_suffice(zu_pairs(p.ctrl))) continue;   // settled by other tiles
+            if (!warp_agrees(orders_suffice(zu_pairs(p.ctrl)))) continue;   // settled by other tiles
             float rj[4], ri = 0.f;
 #pragma unroll
             for (int e = 0; e < 4; ++e)
