@@ -535,15 +535,15 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                             }
                         }
                     }
-                    if (*(volatile int*)&sm.abort || !mbar_wait_warp(&sm.iempty[b], ph ^ 1u)) {
+                    const bool stop = __shfl_sync(0xffffffffu, *(volatile int*)&sm.abort, 0) != 0;
+                    if (stop || !mbar_wait_warp(&sm.iempty[b], ph ^ 1u)) {
                         if (lane == 0) {
                             sm.abort = 1;
                             record_error(p.ctrl, ST_ETIMEOUT, L);
                         }
                         run = false;
+                        break;
                     }
-                    run = __all_sync(0xffffffffu, run);
-                    if (!run) break;
                     if (consts) {
                         T3Const& c = sm.cst[b];
 #pragma unroll
