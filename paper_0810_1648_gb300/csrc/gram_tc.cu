@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     if (++stage == XSTAGES) { stage = 0; ph ^= 1u; }
                 }
             }
+            await_copies<XSTAGES>(sm.xfull, stage, ph);
         }
     } else if (warp == 1) {
         // ------------------------------------------------------ MMA issuer

@@ -459,6 +459,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                         if (++stage == T3_STAGES) { stage = 0; ph ^= 1u; }
                     }
             }
+            await_copies<T3_STAGES>(sm.xfull, stage, ph);
         }
     } else if (warp == 1) {
         // ------------------------------------------------------ MMA issuer

@@ -124,6 +124,23 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
         : "memory");
 }
 
+// Parity of the last fill of stage s of a ring, `stage` being the one to fill next
+// and `phase` the parity of this pass over the ring; of a stage that was never
+// filled, the parity that a fresh mbarrier counts as done.
+__host__ __device__ constexpr uint32_t last_fill_parity(int s, int stage, uint32_t phase)
+{
+    return s < stage ? phase : phase ^ 1u;
+}
+// A producer's last step: every copy that it has issued into its N stages has
+// landed (bounded, as every wait), so that none is under way when the CTA's shared
+// memory passes on, even where a role has given up and nobody reads them.
+template <int N>
+__device__ __forceinline__ void await_copies(unsigned long long* full, int stage, uint32_t phase)
+{
+#pragma unroll
+    for (int s = 0; s < N; ++s) mbar_wait(&full[s], last_fill_parity(s, stage, phase));
+}
+
 // 1/d for the cavity precisions: the hardware approximate reciprocal
 // refined by one Newton-Raphson step r <- r (2 - d r) (error within about one
 // unit in the last place for normal positive d; checked against IEEE division

@@ -278,6 +278,10 @@ __device__ __forceinline__ void sweep_producer(const Inst* __restrict__ tab, con
     int stage = 0, slot = 0;
     uint32_t phase = 0, tph = 0;
     auto stopped = [&]() { return __shfl_sync(0xffffffffu, abort_flag ? *abort_flag : 0, 0) != 0; };
+    auto landed = [&]() {
+        await_copies<stages<MSG>()>(sm.full, stage, phase);
+        await_copies<2>(sm.tfull, slot, tph);
+    };
     for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
         const int4 w = work[L];
         const Inst& p = tab[w.x];
@@ -297,6 +301,7 @@ __device__ __forceinline__ void sweep_producer(const Inst* __restrict__ tab, con
                 record_error(ctrl, ST_ETIMEOUT, L);
                 if (abort_flag) *abort_flag = 1;
             }
+            landed();
             return;
         }
         if (lane == 0) {
@@ -339,6 +344,7 @@ __device__ __forceinline__ void sweep_producer(const Inst* __restrict__ tab, con
                     record_error(ctrl, ST_ETIMEOUT, L);
                     if (abort_flag) *abort_flag = 1;
                 }
+                landed();
                 return;
             }
             unsigned char* S = ring + (size_t)stage * SB;
@@ -378,6 +384,7 @@ __device__ __forceinline__ void sweep_producer(const Inst* __restrict__ tab, con
         }
     }
     // end of this CTA's tiles
+    landed();
     if (!stopped() && mbar_wait_warp(&sm.tempty[slot], tph ^ 1u) && lane == 0) {
         sm.info[slot].end = 1;
         mbar_arrive(&sm.tfull[slot]);
@@ -1014,6 +1021,7 @@ __global__ void __launch_bounds__(RC_THREADS, 1)
                     if (++xs == RC_XSTAGES) { xs = 0; ph ^= 1u; }
                 }
             }
+            await_copies<RC_XSTAGES>(ex.xfull, xs, ph);
         }
     } else if (warp == 2) {
         // MMA issuer

@@ -108,11 +108,16 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
     int stage = 0, slot = 0;
     uint32_t phase = 0, tph = 0;
     auto stopped = [&]() { return abort_flag && __shfl_sync(0xffffffffu, *abort_flag, 0) != 0; };
+    auto landed = [&]() {
+        if constexpr (STREAM) await_copies<H_STAGES>(sm.full, stage, phase);
+        await_copies<2>(sm.tfull, slot, tph);
+    };
     auto give_up = [&](Ctrl* ctrl, long long L) {
         if (lane == 0) {
             record_error(ctrl, ST_ETIMEOUT, L);
             if (abort_flag) *abort_flag = 1;
         }
+        landed();
     };
     // The round's settings of an instance do not change during a sweep: they
     // are read once per run of tiles of the same instance, and the next tile's
@@ -208,6 +213,7 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
             }
         }
     }
+    landed();
     if (!stopped() && mbar_wait_warp(&sm.tempty[slot], tph ^ 1u) && lane == 0) {
         sm.info[slot].end = 1;
         mbar_arrive(&sm.tfull[slot]);
@@ -983,6 +989,7 @@ __global__ void __launch_bounds__(HR_THREADS, 1)
                     if (++xs == HR_XSTAGES) { xs = 0; ph ^= 1u; }
                 }
             }
+            await_copies<HR_XSTAGES>(ex.xfull, xs, ph);
         }
     } else if (warp == 10) {
         if (lane == 0) {
