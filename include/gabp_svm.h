@@ -225,7 +225,7 @@ GABP_API gabp_status gabp_svm_get_mean(gabp_svm_t h, float* mu);
  * rows Xtest (t x m, same dtype and pointer mode as X) with the alpha of the
  * last solve; the predicted label is sign(f).  KRR: the prediction
  * f(x) = sum_i c_i K(x_i, x) (+ lambda^2 sum_i c_i with the bias on).
- * out: t floats. */
+ * out: t floats (as they were when a row is refused). */
 GABP_API gabp_status gabp_svm_decision(gabp_svm_t h, const void* Xtest, int64_t t, float* out);
 
 /* Indices i with alpha_i > sv_threshold (KRR: |c_i| > sv_threshold),

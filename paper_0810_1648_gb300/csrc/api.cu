@@ -1070,14 +1070,16 @@ gabp_status gabp_svm_decision(gabp_svm_t h, const void* Xtest, int64_t t, float*
     const int xd = h->opts.x_dtype;
     const int64_t m = h->m;
     // The test rows go through in slabs (so that the workspace stays bounded),
-    // their planes packed and checked in one pass over the caller's rows.
+    // their planes packed and checked in one pass over the caller's rows.  A refused
+    // row leaves `out` as it is: the values stay in the workspace until every row has
+    // been checked (of one slab on the device, the last kernel itself looks).
     const int64_t slab = std::min<int64_t>(t, (int64_t)1 << 17);
     const int Ntt = (int)((slab + T - 1) / T);
     const int per = decision_entries(Ntt);   // entries of a slab, at most
     const size_t bxp = align_up(pack3_bytes(Ntt, (int)m), 1024), bsq = align_up((size_t)Ntt * T * 4, 256);
     const size_t bin = dev ? 0 : align_up((size_t)slab * m * x_elem_bytes(xd), 256);
     const size_t bpart = align_up((size_t)per * T * sizeof(float), 256), bw = align_up((size_t)per * sizeof(int4), 256);
-    const size_t bdiag = align_up((size_t)Ntt * sizeof(int4), 256), bout = dev ? 0 : align_up((size_t)slab * 4, 256);
+    const size_t bdiag = align_up((size_t)Ntt * sizeof(int4), 256), bout = dev && t <= slab ? 0 : align_up((size_t)t * 4, 256);
     const size_t btab = align_up(2 * sizeof(Inst), 256), bctrl = align_up(sizeof(Ctrl), 256);
     const size_t need = bxp + bsq + bin + bpart + bw + bdiag + bout + btab + bctrl;
     void* big = nullptr;
@@ -1104,7 +1106,7 @@ gabp_status gabp_svm_decision(gabp_svm_t h, const void* Xtest, int64_t t, float*
     float* part = (float*)take(bpart);
     int4* w = (int4*)take(bw);
     int4* diag = (int4*)take(bdiag);
-    float* dout = (float*)take(bout);
+    float* dout = bout ? (float*)take(bout) : out;
     Inst* tab = (Inst*)take(btab);
     te.ctrl = (Ctrl*)take(bctrl);
     auto run = [&]() -> gabp_status {
@@ -1121,15 +1123,18 @@ gabp_status gabp_svm_decision(gabp_svm_t h, const void* Xtest, int64_t t, float*
             }
             CK(launch_stage(src, xd, tc, (int)m, te.Nt, nullptr, nullptr, nullptr, nullptr, 0, (void*)te.Xp3, r0,
                             te.ctrl, diag, s));
-            CK(launch_decision_tc(tab, diag, w, tc, h->Nt, h->alpha, part, te.ctrl, dev ? out + r0 : dout, s));
+            CK(launch_decision_tc(tab, diag, w, tc, h->Nt, h->alpha, part, te.ctrl, dout + r0, s));
             h->prof.kernel_launches += 5;
-            if (!dev) CK(cudaMemcpyAsync(out + r0, dout, (size_t)tc * sizeof(float), cudaMemcpyDeviceToHost, s));
         }
         CK(cudaMemcpyAsync(h->hdec, te.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         if (h->hdec->status == ST_EINVAL)
             return fail(GABP_EINVAL, "test row %lld: non-finite feature", h->hdec->bad_index);
         if (h->hdec->status != 0) return fail(GABP_ETIMEOUT, "a bounded device wait ran out in the decision");
+        if (dout != out) {
+            CK(cudaMemcpyAsync(out, dout, (size_t)t * sizeof(float), dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+        }
         return GABP_OK;
     };
     gabp_status st = run();

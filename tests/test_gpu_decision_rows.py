@@ -1,0 +1,85 @@
+"""Decisions of many rows (several slabs of 2^17, workspaces that are kept, grow or
+are too large to keep) against FP64, and of rows that are refused: the caller's
+output is then as it was.
+
+Bar: as in test_gpu_decision.py, 1e-5 of sum_j |alpha_j y_j| (an FP32 kernel entry
+is off by a few units of 2^-24 (1 + gamma (|x|^2 + |z|^2)), gamma |x|^2 < 12 here).
+"""
+import numpy as np
+import pytest
+
+from paper_0810_1648_gb300 import gabp, workloads
+
+pytestmark = pytest.mark.gpu
+
+BAR = 1e-5
+SLAB = 1 << 17
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_0810_1648_gb300 import build as gbuild
+    gbuild.build()
+
+
+def _reference(X, y, alpha, gamma, lam, Z):
+    X, w = X.astype(np.float64), alpha.astype(np.float64) * y
+    out = np.empty(len(Z))
+    for a in range(0, len(Z), 8192):
+        z = Z[a:a + 8192].astype(np.float64)
+        d2 = np.maximum((z * z).sum(1)[:, None] + (X * X).sum(1)[None] - 2.0 * z @ X.T, 0.0)
+        out[a:a + 8192] = (np.exp(-gamma * d2) + lam * lam) @ w
+    return out, np.abs(w).sum()
+
+
+def _fit(p, dev):
+    torch = pytest.importorskip("torch")
+    svm = (gabp.GabpSVM(torch.from_numpy(p.X).cuda(), torch.from_numpy(p.y).cuda(), p.gamma, p.C) if dev
+           else gabp.GabpSVM(p.X, p.y, p.gamma, p.C))
+    alpha = svm.solve(30, 0.0)[0]
+    return svm, (alpha.cpu().numpy() if dev else np.array(alpha)), svm.stats()["lambda_"]
+
+
+def _rows(Z, t):
+    return np.ascontiguousarray(Z[np.arange(t) % len(Z)])
+
+
+@pytest.mark.parametrize("dev", [False, True])
+@pytest.mark.parametrize("m,ts", [(3, (SLAB, SLAB + 129)), (130, (100, 20001, 70001, 100, 2 * SLAB + 1))])
+def test_many_rows(m, ts, dev):
+    torch = pytest.importorskip("torch")
+    p = workloads.mixture(300, m, seed=m)
+    svm, alpha, lam = _fit(p, dev)
+    base = workloads.test_points(p, 997, seed=5)
+    want, scale = _reference(p.X, p.y, alpha, p.gamma, lam, base)
+    for t in ts:
+        Z = _rows(base, t)
+        got = svm.decision(torch.from_numpy(Z).cuda() if dev else Z)
+        got = got.cpu().numpy() if dev else np.asarray(got)
+        assert got.shape == (t,)
+        assert np.max(np.abs(got - want[np.arange(t) % len(base)])) <= BAR * scale, t
+    svm.close()
+
+
+@pytest.mark.parametrize("dev", [False, True])
+@pytest.mark.parametrize("t,bad", [(1, 0), (300, 7), (300, 299), (SLAB + 200, 5), (SLAB + 200, SLAB + 150)])
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_refused_row_leaves_the_output(t, bad, value, dev):
+    torch = pytest.importorskip("torch")
+    p = workloads.mixture(300, 4, seed=2)
+    svm, _, _ = _fit(p, dev)
+    good = _rows(workloads.test_points(p, 500, seed=6), t)
+    Z = good.copy()
+    Z[bad, 2] = value
+    if dev:
+        Z, out = torch.from_numpy(Z).cuda(), torch.full((t,), 123.0, device="cuda")
+    else:
+        out = np.full(t, 123.0, dtype=np.float32)
+    want = svm.decision(torch.from_numpy(good).cuda() if dev else good)   # (leaves its values in the workspace)
+    with pytest.raises(gabp.GabpError, match=f"test row {bad}:") as e:
+        gabp.svm_decision(svm.h, Z, out)
+    assert e.value.status == gabp.EINVAL
+    assert bool((out == 123.0).all())
+    again = svm.decision(torch.from_numpy(good).cuda() if dev else good)
+    assert bool((again == want).all())
+    svm.close()
