@@ -241,7 +241,10 @@ GABP_API gabp_status gabp_svm_get_stats(gabp_svm_t h, gabp_svm_stats* stats);
  *              available in recompute mode (GABP_ESTATE).
  *   get_pairs: for cnt index pairs (i[k] < j[k]) the current messages
  *              {P_ij, P_ji, H_ij, H_ji} with H = P mu (information form);
- *              out: 4*cnt floats.
+ *              out: 4*cnt floats.  Instances whose rounds store no messages
+ *              (all but strongly coupled ones): rebuilt in FP32, to its
+ *              rounding, from the nodes' last eight rounds and the pair's
+ *              entry of Q; msg_bf16 does not round them then.
  *   get_aggregates: Ptilde, htilde = Ptilde*mutilde and mutilde of the
  *              current message state (n floats each; any may be NULL).
  */

@@ -116,7 +116,7 @@ struct gabp_svm_s {
     DevBlock dws;                   // workspace of decisions, kept up to kDecisionKeep bytes
     size_t dws_bytes = 0;
     Ctrl* hctrl = nullptr;          // pinned mirror of the control block, as of the last wait for the stream
-    Ctrl* hdec = nullptr;           // and of a decision's
+    Ctrl* hdec = nullptr;           // and of a decision's or an inspection's
     double* hfinal = nullptr;       // pinned {rinf, objective, nsv}
     int* hnote = nullptr;           // pinned, written by the device (Inst::note)
     struct Graph {
@@ -1207,6 +1207,71 @@ gabp_status gabp_svm_get_q(gabp_svm_t h, float* Q)
     return GABP_OK;
 }
 
+// The pairs of a handle that recomputes Q: the tiles they lie in are formed by the
+// BF16 store's kernel (the sweep's values bit for bit), up to kPairTiles at a time.
+static gabp_status get_pairs_recomputed(gabp_svm_t h, const std::vector<long long>& ij, float* out)
+{
+    constexpr size_t kPairTiles = 2048;   // 64 MB
+    const size_t cnt = ij.size() / 2;
+    cudaStream_t s = h->stream;
+    std::map<std::pair<int, int>, std::vector<size_t>> by_tile;
+    for (size_t k = 0; k < cnt; ++k) by_tile[{(int)(ij[2 * k] / T), (int)(ij[2 * k + 1] / T)}].push_back(k);
+    const size_t most = std::min(kPairTiles, by_tile.size());
+    const size_t bq = most * TT * sizeof(__nv_bfloat16), bw = align_up(most * sizeof(int4), 256), btab = align_up(sizeof(Inst), 256),
+                 bctrl = align_up(sizeof(Ctrl), 256), bij = align_up(2 * cnt * sizeof(long long), 256),
+                 bslot = align_up(cnt * sizeof(int), 256);
+    char* mem = nullptr;
+    CK(pool_alloc((void**)&mem, bq + bw + btab + bctrl + bij + bslot + cnt * sizeof(float4), s));
+    char* b = mem;
+    auto take = [&](size_t bytes) { char* r = b; b += bytes; return r; };
+    Inst p = h->inst, former = h->inst;
+    p.qstore = former.qstore = take(bq);
+    int4* dw = (int4*)take(bw);
+    Inst* tab = (Inst*)take(btab);
+    former.ctrl = (Ctrl*)take(bctrl);
+    long long* dij = (long long*)take(bij);
+    int* dslot = (int*)take(bslot);
+    float4* dout = (float4*)take(cnt * sizeof(float4));
+    auto run = [&]() -> gabp_status {
+        CK(cudaMemsetAsync(former.ctrl, 0, sizeof(Ctrl), s));
+        CK(cudaMemcpyAsync(tab, &former, sizeof(Inst), cudaMemcpyHostToDevice, s));
+        std::vector<float4> got(cnt);
+        std::vector<int4> work;
+        std::vector<long long> part;   // the pairs of these tiles
+        std::vector<int> slot;
+        std::vector<size_t> at;
+        for (auto it = by_tile.begin(); it != by_tile.end();) {
+            work.clear(); part.clear(); slot.clear(); at.clear();
+            for (; it != by_tile.end() && work.size() < most; ++it) {
+                for (const size_t k : it->second) {
+                    part.push_back(ij[2 * k]);
+                    part.push_back(ij[2 * k + 1]);
+                    slot.push_back((int)work.size());
+                    at.push_back(k);
+                }
+                work.push_back(make_int4(0, it->first.first, it->first.second, (int)work.size()));
+            }
+            CK(cudaMemcpyAsync(dw, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+            CK(cudaMemcpyAsync(dij, part.data(), part.size() * sizeof(long long), cudaMemcpyHostToDevice, s));
+            CK(cudaMemcpyAsync(dslot, slot.data(), slot.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+            CK(launch_form_q_tc(tab, dw, (long long)work.size(), s));
+            launch_get_pairs(p, dij, dslot, (long long)at.size(), dout, s);
+            CK(cudaGetLastError());
+            CK(cudaMemcpyAsync(got.data(), dout, at.size() * sizeof(float4), cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+            for (size_t e = 0; e < at.size(); ++e) std::memcpy(out + 4 * at[e], &got[e], sizeof(float4));
+        }
+        CK(cudaMemcpyAsync(h->hdec, former.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        if (h->hdec->status != 0) return fail(GABP_ETIMEOUT, "a bounded device wait ran out in the inspection");
+        return GABP_OK;
+    };
+    const gabp_status st = run();
+    cudaFreeAsync(mem, s);
+    cudaStreamSynchronize(s);
+    return st;
+}
+
 gabp_status gabp_svm_get_pairs(gabp_svm_t h, const int64_t* i, const int64_t* j, int64_t cnt, float* out)
 {
     g_err.clear();
@@ -1220,12 +1285,13 @@ gabp_status gabp_svm_get_pairs(gabp_svm_t h, const int64_t* i, const int64_t* j,
         ij[2 * k] = i[k];
         ij[2 * k + 1] = j[k];
     }
+    if (h->opts.q_mode == GABP_Q_RECOMPUTE) return get_pairs_recomputed(h, ij, out);
     long long* dij = nullptr;
     float4* dout = nullptr;
     CK(cudaMallocAsync((void**)&dij, ij.size() * sizeof(long long), h->stream));
     CK(cudaMallocAsync((void**)&dout, (size_t)cnt * sizeof(float4), h->stream));
     CK(cudaMemcpyAsync(dij, ij.data(), ij.size() * sizeof(long long), cudaMemcpyHostToDevice, h->stream));
-    launch_get_pairs(h->inst, dij, cnt, dout, h->stream);
+    launch_get_pairs(h->inst, dij, nullptr, cnt, dout, h->stream);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(out, dout, (size_t)cnt * sizeof(float4), cudaMemcpyDeviceToHost, h->stream));
     cudaFreeAsync(dij, h->stream);

@@ -439,7 +439,7 @@ cudaError_t launch_decision_tc(const Inst* tab, const int4* diag, int4* work, in
 // Gather helpers for inspection.
 void launch_get_q(const Inst& p, const int4* work, long long ntiles, int q_bf16, float* Qdense,
                   cudaStream_t s);
-void launch_get_pairs(const Inst& p, const long long* ij, long long cnt, float4* out,
+void launch_get_pairs(const Inst& p, const long long* ij, const int* slot, long long cnt, float4* out,
                       cudaStream_t s);
 
 // Reciprocal used by the pair sweep, evaluated on d[0..cnt) (device arrays).

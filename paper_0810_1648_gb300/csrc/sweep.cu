@@ -1801,18 +1801,6 @@ __global__ void k_begin(Inst* tab, int ninst, int iters, double tol)
     c->done = (c->status != 0 || iters <= 0) ? 1 : 0;
 }
 
-// Q_ij as the recomputing sweep forms it, from a plain sum over the features
-// (the tensor-core sum can round to the neighbouring BF16 value).
-__device__ float recomputed_q(const Inst& p, int i, int j)
-{
-    float g = 0.f;
-    for (int k = 0; k < p.m; ++k)
-        g = fmaf(__bfloat162float(__float2bfloat16_rn(p.X[(size_t)i * p.m + k])),
-                 __bfloat162float(__float2bfloat16_rn(p.X[(size_t)j * p.m + k])), g);
-    const float t = p.gamma * kLog2e * (2.f * g - p.sqb[i] - p.sqb[j]);
-    return p.y[i] * p.y[j] * __bfloat162float(__float2bfloat16_rn(ex2_approx(fminf(t, 0.f)) + p.lam2));
-}
-
 // The messages {P_ij, P_ji, H_ij, H_ji} of a PATH_HIST pair after t rounds
 // (t > 0), rebuilt from the history of the pair's stage as the sweep of round
 // t - 1 did, with the whole history as chain.
@@ -1850,7 +1838,10 @@ __device__ float4 hist_pair(const Inst& p, int t, float q, int i, int j)
     return make_float4(PA, PB, HA, HB);
 }
 
-__global__ void k_get_pairs(Inst p, const long long* __restrict__ ij, long long cnt, float4* __restrict__ out)
+// slot: for an instance that recomputes Q, each pair's tile among those formed
+// for it (p.qstore, BF16); null: p's own tiles.
+__global__ void k_get_pairs(Inst p, const long long* __restrict__ ij, const int* __restrict__ slot, long long cnt,
+                            float4* __restrict__ out)
 {
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (e >= cnt) return;
@@ -1862,10 +1853,9 @@ __global__ void k_get_pairs(Inst p, const long long* __restrict__ ij, long long 
     if (p.ctrl->t == 0 || L < 0) {
         out[e] = make_float4(0.f, 0.f, 0.f, 0.f);
     } else if (p.ctrl->path == PATH_HIST) {
-        const size_t o = (size_t)L * TT + r * T + c;
+        const size_t o = (size_t)(slot ? slot[e] : L) * TT + r * T + c;
         float q;
-        if (!p.qstore) q = recomputed_q(p, (int)i, (int)j);
-        else if (p.qstore != p.qref) q = __bfloat162float(static_cast<const __nv_bfloat16*>(p.qstore)[o]);
+        if (p.qstore != p.qref) q = __bfloat162float(static_cast<const __nv_bfloat16*>(p.qstore)[o]);
         else q = p.qref[o];
         out[e] = hist_pair(p, p.ctrl->t, q, (int)i, (int)j);
     } else {
@@ -2015,9 +2005,9 @@ void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sche
     }
 }
 
-void launch_get_pairs(const Inst& p, const long long* ij, long long cnt, float4* out, cudaStream_t s)
+void launch_get_pairs(const Inst& p, const long long* ij, const int* slot, long long cnt, float4* out, cudaStream_t s)
 {
-    if (cnt > 0) k_get_pairs<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(p, ij, cnt, out);
+    if (cnt > 0) k_get_pairs<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(p, ij, slot, cnt, out);
 }
 
 }  // namespace gabp
