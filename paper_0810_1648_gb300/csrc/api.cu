@@ -16,6 +16,7 @@
 #include <map>
 #include <new>
 #include <string>
+#include <thread>
 #include <tuple>
 #include <vector>
 
@@ -125,6 +126,7 @@ struct gabp_svm_s {
         int uses = 0;                  // chunks run with this key
     };
     std::map<std::tuple<int, int, int>, Graph> graphs;   // by (rounds, profiling stride, message path)
+    unsigned schedule = 0;   // cudaDeviceSchedule*: how the program wants its threads to wait for the device, read at create
     int profiling = 0;   // 0 off, k >= 1: the pair sweep of every k-th round is bracketed by events
     gabp_svm_profile prof{};
     bool solved = false;
@@ -517,8 +519,11 @@ static bool bracketed(int stride, int k) { return stride > 0 && k % stride == st
 // ran for nothing: n = 1000 from FP64 host arrays, create to destroy, 0.90 ms
 // against 0.77 with the input's buffer from the scratch pool too.)
 // group: a captured group of `per` rounds to launch instead of single ones.
+// The host looks at the note without a pause, as cudaStreamSynchronize does by
+// default; where the program has asked CUDA's waits to yield, so does this one, and
+// where it has asked them to block, run_rounds leaves this way out.
 constexpr int kRoundsAhead = 3;
-gabp_status run_direct(gabp_svm_t h, int iters, int path, cudaGraphExec_t group, int per)
+gabp_status run_direct(gabp_svm_t h, int iters, int path, cudaGraphExec_t group, int per, bool yields)
 {
     cudaStream_t s = h->stream;
     volatile int* note = h->hnote;
@@ -526,12 +531,14 @@ gabp_status run_direct(gabp_svm_t h, int iters, int path, cudaGraphExec_t group,
     *note = t0;
     for (int k = 0; k < iters; k += per) {   // (rounds of a group beyond the limit do nothing)
         int seen = *note;
-        for (long spins = 1; !(seen & kNoteStopped) && k - (seen - t0) >= kRoundsAhead; seen = *note)
+        for (long spins = 1; !(seen & kNoteStopped) && k - (seen - t0) >= kRoundsAhead; seen = *note) {
+            if (yields) std::this_thread::yield();
             if ((++spins & 0xffff) == 0) {   // a note that does not come: the stream has ended, well or not
                 const cudaError_t e = cudaStreamQuery(s);
                 if (e == cudaSuccess) break;
                 if (e != cudaErrorNotReady) return fail(GABP_ECUDA, "rounds failed: %s", cudaGetErrorString(e));
             }
+        }
         if (seen & kNoteStopped) break;
         if (group)
             CK(cudaGraphLaunch(group, s));
@@ -561,17 +568,17 @@ constexpr int kGroupRounds = 2;
 constexpr size_t kGraphsKept = 8;
 
 // A chunk of `rounds` synchronous rounds, *out->exec null where it is launched
-// directly; with profiling on it is always captured, and the
-// pair sweep of every profiling-th round in it is bracketed by two
+// directly; at_once: it is captured at its first use; with profiling on it always
+// is, and the pair sweep of every profiling-th round in it is bracketed by two
 // event-record nodes.
-gabp_status get_graph(gabp_svm_t h, int rounds, int path, gabp_svm_s::Graph** out)
+gabp_status get_graph(gabp_svm_t h, int rounds, int path, bool at_once, gabp_svm_s::Graph** out)
 {
     const int stride = h->profiling;
     const auto key = std::make_tuple(rounds, stride, path);
     if (h->graphs.size() >= kGraphsKept && h->graphs.find(key) == h->graphs.end()) clear_graphs(h);
     gabp_svm_s::Graph& G = h->graphs[key];
     *out = &G;
-    if (G.exec || (stride == 0 && h->nstages == 1 && G.uses < kGraphAfter)) return GABP_OK;
+    if (G.exec || (stride == 0 && !at_once && G.uses < kGraphAfter)) return GABP_OK;
     if (stride > 0) {
         G.ev.resize((size_t)2 * (rounds / stride));
         for (auto& e : G.ev) CK(cudaEventCreate(&e));
@@ -607,7 +614,8 @@ gabp_status run_rounds(gabp_svm_t h, int iters, double tol, Ctrl* out)
         CK(cudaMemcpyAsync(&p.ctrl->status, &kTimeout, sizeof(int), cudaMemcpyHostToDevice, s));
     }
     if (iters > 0) {
-        const bool grouped = tol > 0 && h->nstages > 1 && h->profiling == 0;
+        const bool blocks = h->schedule == cudaDeviceScheduleBlockingSync, yields = h->schedule == cudaDeviceScheduleYield;
+        const bool grouped = tol > 0 && h->nstages > 1 && h->profiling == 0 && !blocks;
         const int len = grouped ? kGroupRounds : tol > 0 ? std::min<int>(h->opts.chunk, iters) : iters;
         const int path = h->hctrl->path;
         const int max_chunks = (iters + len - 1) / len + 1;
@@ -615,12 +623,12 @@ gabp_status run_rounds(gabp_svm_t h, int iters, double tol, Ctrl* out)
         int t_before = t0;
         for (int c = 0; c < max_chunks; ++c) {
             gabp_svm_s::Graph* g = nullptr;
-            if (gabp_status st = get_graph(h, len, path, &g)) return st;
+            if (gabp_status st = get_graph(h, len, path, blocks || h->nstages > 1, &g)) return st;
             ++g->uses;
             if (g->exec && !grouped) {
                 CK(cudaGraphLaunch(g->exec, s));
                 h->prof.kernel_launches += 2 * len;
-            } else if (gabp_status st = run_direct(h, iters - (t_before - t0), path, g->exec, g->exec ? len : 1)) {
+            } else if (gabp_status st = run_direct(h, iters - (t_before - t0), path, g->exec, g->exec ? len : 1, yields)) {
                 return st;
             }
             CK(cudaMemcpyAsync(h->hctrl, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
@@ -773,6 +781,8 @@ gabp_status gabp_svm_create_ex(const void* X, const float* y, int64_t n, int64_t
         destroy_all(h);
         return fail(GABP_ENOMEM, "pinned host allocation failed");
     }
+    if (cudaGetDeviceFlags(&h->schedule) == cudaSuccess) h->schedule &= cudaDeviceScheduleMask;
+    else { cudaGetLastError(); h->schedule = 0; }
     h->hctrl = static_cast<Ctrl*>(mirror);
     h->hdec = h->hctrl + 1;
     h->hfinal = reinterpret_cast<double*>(h->hctrl + 2);
