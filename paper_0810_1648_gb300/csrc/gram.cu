@@ -267,7 +267,6 @@ __global__ void k_final_reduce(const Inst* __restrict__ tab, const StopOp* __res
     }
 }
 
-// ----------------------------------------------------------------- decision
 // ---------------------------------------------------------------- inspection
 __global__ void k_get_q(Inst p, const int4* __restrict__ work, int q_bf16, float* __restrict__ Qd)
 {
@@ -326,9 +325,8 @@ void launch_get_q(const Inst& p, const int4* work, long long ntiles, int q_bf16,
 // loops that cannot afford the implicit device-wide synchronisation of
 // cudaMalloc/cudaFree.  gabp_decision_noalloc serves them:
 // the caller passes every input and output as device memory, and the
-// temporaries (row norms and per-tile partial sums) live in the file-scope
-// array below, which every GPU that loads this library holds until the
-// process exits.
+// per-tile partial sums live in the file-scope array below, which every GPU that
+// loads this library holds until the process exits.
 namespace gabp {
 namespace {
 
@@ -500,9 +498,12 @@ extern "C" GABP_API gabp_status gabp_decision_noalloc(const float* X, const floa
         scratch = g_noalloc_dev_ptr[dev];
     }
     // Every scratch element read below is written earlier in the same call.  64 x
-    // 64 tiles have twice the partial sums, of fewer than 152 x 128 rows.
+    // 64 tiles (up to where 128 x 128 ones fill the chip, see
+    // k_decision_tiles_noalloc) take ceil(n / 64) t floats of it; the limit above,
+    // which counts n + t floats more than 128 x 128 tiles need, is what callers
+    // know.
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (Ntt * Nt < num_sms())
+    if (Ntt * Nt < num_sms() && (n + 63) / 64 * t <= kNoAllocScratchFloats)
         launch_decision_noalloc<4>(X, y, alpha, (int)n, (int)m, Xtest, (int)t, (float)gamma, (float)(lambda * lambda),
                                    scratch, out, s);
     else

@@ -83,3 +83,22 @@ def test_refused_row_leaves_the_output(t, bad, value, dev):
     again = svm.decision(torch.from_numpy(good).cuda() if dev else good)
     assert bool((again == want).all())
     svm.close()
+
+
+# the largest of the small tiles (one 128 x 128 tile fewer than SMs either way, and
+# one more) and of the scratch
+@pytest.mark.parametrize("n,t", [(151 * 128, 128), (128, 151 * 128), (152 * 128, 127), (127, 152 * 128 + 1), (1, 349525), (1_039_000, 1)])
+def test_noalloc_at_its_limits(n, t):
+    torch = pytest.importorskip("torch")
+    p = workloads.mixture(1000, 3, seed=n % 97)
+    X, y = p.X[np.arange(n) % p.n], p.y[np.arange(n) % p.n]
+    base = workloads.test_points(p, 61, seed=t % 89)
+    alpha = np.random.default_rng(7).random(n, dtype=np.float32) / n
+    out = torch.full((t,), float("nan"), device="cuda")
+    args = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (X, y, alpha, _rows(base, t))]
+    gabp.decision_noalloc(*args, p.gamma, 0.25, out)
+    w = np.zeros(p.n)
+    np.add.at(w, np.arange(n) % p.n, alpha.astype(np.float64) * y)
+    want, _ = _reference(p.X, np.ones(p.n), w, p.gamma, 0.25, base)
+    scale = np.abs(alpha.astype(np.float64) * y).sum()
+    assert np.max(np.abs(out.cpu().numpy() - want[np.arange(t) % len(base)])) <= BAR * scale
