@@ -18,13 +18,14 @@ __host__ __device__ __forceinline__ size_t hist_offset(int npad, int st, int t)
 __device__ __forceinline__ float* hist_slot(const Inst& p, int st, int t) { return p.hring + hist_offset(p.npad, st, t); }
 
 // Appends node x's aggregates of round t to stage st's history; mu2 and D2 are
-// its mean and D two rounds earlier.
+// its mean and D two rounds earlier.  D(0) counts as 0, and D(1) once in the
+// weight of q^5: no message precedes round 0 (sweep_hist.cu).
 __device__ __forceinline__ void hist_push(const Inst& p, int st, int t, int x, float P, float h, float mu, float mu2,
                                           float D2)
 {
     const size_t np = p.npad;
     float* s = hist_slot(p, st, t);
-    const float D = mu - mu2, ip = 1.f / P;
+    const float D = t > 0 ? mu - mu2 : 0.f, ip = 1.f / P;
     s[x] = P;
     s[np + x] = h;
     s[2 * np + x] = mu;
@@ -32,7 +33,7 @@ __device__ __forceinline__ void hist_push(const Inst& p, int st, int t, int x, f
     float* w = p.hnow + (size_t)3 * st * np;
     w[x] = ip;
     w[np + x] = D * ip;
-    w[2 * np + x] = (D2 - 2.f * D) * ip * ip;
+    w[2 * np + x] = (D2 - (t > 1 ? 2.f : 1.f) * D) * ip * ip;
 }
 
 // Node x's means and htilde before round t: 0 (Step 1, or a restart of the H

@@ -18,7 +18,10 @@
 //   sum q^3 r_i D_i                E, times r
 //   sum q^5 r_i^2 (D_i(t-2) - 2 D_i)   E, times r^2
 // with r = r_j(t-1); the terms of higher orders are below FP32 rounding on this
-// path (choose_path).  Once no Ptilde changes, the P sums are known (Ptilde -
+// path (choose_path).  Before round 0 there is no message: E(1) = 0 and P_ji(0) = 0,
+// the factor of D_i(0) (which so counts as 0), and what P_ji(t) of later rounds
+// adds to the expansions is missing from the first ones: round 1 has S2 - r S4 + r^2
+// S6 and -D_i in place of -2 D_i, round 2 has -2 D_j(t-1) in place of -3.  Once no Ptilde changes, the P sums are known (Ptilde -
 // Q_jj; S4 and S6 of the last live round), and E needs its sums only while it counts
 // (e_terms): most rounds are one symmetric product Q mu.  Under the staged
 // schedule mu in H is the mean of the stage and the P sums are the tile's own.
@@ -640,6 +643,7 @@ __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* 
         const int c = tid & (T - 1);
         const size_t o = (size_t)(tid < T ? ti.sR : ti.sC) * T + c;
         float* s46 = nullptr;
+        const float p6 = ti.t > 1 ? 2.f : 1.f, n6 = ti.t == 2 ? 2.f : 3.f;   // (of the first rounds: see above)
         float mu1 = 0.f, r1 = 0.f, D1 = 0.f, D3 = 0.f, S4 = 0.f, S6 = 0.f, P = 0.f;
         if (ti.t > 0 && (staged || kind != K_SUM)) {
             const size_t np = ti.npad;
@@ -696,7 +700,7 @@ __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* 
                 const float M = staged ? node_sum(sm, base + 1, tid, rows, diag) : 0.f;
                 const float S2 = live ? node_sum(sm, base + 1 + staged, tid, rows, diag) : 0.f;
                 const float W3 = (kind == K_ONE || kind == K_LIVE1) ? node_sum(sm, base + 2, tid, rows, diag) : 0.f;
-                const float E = r1 * (fmaf(S4, D1, W3) + r1 * S6 * (D3 - 3.f * D1));
+                const float E = r1 * (fmaf(S4, D1, W3) + r1 * S6 * (D3 - n6 * D1));
                 if (live) P = -S2;
                 if (mine) {
                     if (live) d[0] = P;
@@ -713,11 +717,11 @@ __device__ __forceinline__ void hist_consumers(SRC& src, HTail& sm, const Inst* 
                     S4 = node_sum(sm, S_4, tid, rows, diag);
                     S6 = kind == K_LIVE ? node_sum(sm, S_6, tid, rows, diag) : 0.f;
                 }
-                P = fmaf(r1, fmaf(-2.f * r1, S6, S4), -S2);
+                P = fmaf(r1, fmaf(-p6 * r1, S6, S4), -S2);
             }
             const float W3 = node_sum(sm, S_W3, tid, rows, diag);
             const float W5 = kind == K_LIVE || kind == K_TWO ? node_sum(sm, S_W5, tid, rows, diag) : 0.f;
-            const float E = r1 * (fmaf(S4, D1, W3) + r1 * fmaf(S6, D3 - 3.f * D1, W5));
+            const float E = r1 * (fmaf(S4, D1, W3) + r1 * fmaf(S6, D3 - n6 * D1, W5));
             if (mine) {
                 d[2 * plen] = R;
                 if (live) d[0] = P;
