@@ -1378,6 +1378,7 @@ gabp_status gabp_batch_solve(const gabp_problem* probs, int64_t count, const gab
     } else {
         E.chunk = o.chunk;
     }
+    E.chunk = std::min(E.chunk, std::max(1, (int)iters));   // no pass has more
     ph.tune_ms = ms_since(t0);
     // The end-of-solve work of the instances that stopped in one chunk runs
     // on its own stream while the others sweep the next chunk; restarted
@@ -1486,7 +1487,7 @@ gabp_status gabp_server_create(const gabp_server_cfg* cfg, gabp_server_t* out)
     const int cap_nblk = (int)std::min<long long>(cap_tiles * 4 + 1024, 1LL << 28);
     gabp_server_t s = new gabp_server_s();
     if (gabp_status st = s->E.init(c.max_members, cap_tiles, cap_nblk, c.opts)) { delete s; return st; }
-    s->E.chunk = c.opts.chunk > 0 ? c.opts.chunk : 8;
+    s->E.chunk = std::min(c.opts.chunk > 0 ? c.opts.chunk : 8, std::max(1, (int)c.iters));
     s->cfg = c;
     s->budget = budget;
     *out = s;
