@@ -1201,20 +1201,29 @@ class Engine {
 
     // Picks sweep CTAs per SM and the chunk length by timing candidate
     // schedules for a few rounds of the real set (then restarts it).
-    gabp_status autotune(int iters)
+    gabp_status autotune(int iters, bool refined)
     {
         NvtxRange nv("gabp.batch.autotune");
         long long tiles = 0;
         int members = 0;
         for (auto& M : mem)
             if (M.used && M.active) { tiles += M.ntiles; ++members; }
+        // What a chunk has left when its last instance stops runs for nothing, so
+        // its length is bounded where a solve is short: to a tolerance it takes 10
+        // to 60 rounds, in passes of a few each when it is refined, and a staged
+        // round, even one of stopped instances, is six launches and more.  (24
+        // problems of 100 to 1400 points, to 1e-5, ms in chunks of 16 / 32 / 64: FP32
+        // 2.52 / 2.46 / 2.53, staged 3.31 / 3.20 / 3.42; with strongly coupled pairs
+        // 1.58 / 1.66 / 1.82, staged 1.75 / 1.96 / 2.38; recomputed, refined and
+        // staged 5.57 / 6.61 / 7.16.)
+        const int longest = refined || nstages > 1 ? 16 : 32;
         TuneKey key{q_mode, msg_bf16, nstages, tiles >> 8, members >> 3};
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
             auto it = g_tune_cache.find(key);
             if (it != g_tune_cache.end()) {
                 set_grid(it->second.ctas_per_sm);
-                chunk = it->second.chunk;
+                chunk = std::min(it->second.chunk, longest);
                 return GABP_OK;
             }
         }
@@ -1250,9 +1259,9 @@ class Engine {
         // about 2% of the rounds it covers, within [4, 64]
         int ch = 4;
         while (ch < 64 && 0.05 / (ch * round_ms) > 0.02) ch *= 2;
-        chunk = ch;
+        chunk = std::min(ch, longest);
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune_cache[key] = TuneVal{best_c, chunk};
+        g_tune_cache[key] = TuneVal{best_c, ch};
         return GABP_OK;
     }
 };
@@ -1372,7 +1381,7 @@ gabp_status gabp_batch_solve(const gabp_problem* probs, int64_t count, const gab
     ph.form_ms = ms_since(t0);
     t0 = clk::now();
     if (o.chunk <= 0) {
-        if (gabp_status st = E.autotune(iters)) return st;
+        if (gabp_status st = E.autotune(iters, o.q_mode != 0 && o.refine > 0)) return st;
         const double t0 = (o.q_mode != 0 && o.refine > 0) ? std::max(tol, E.handover) : tol;
         for (int64_t k = 0; k < count; ++k) gabp::launch_begin(E.d_tab + k, 1, iters, t0, E.stream);
     } else {
