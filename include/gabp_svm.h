@@ -37,6 +37,13 @@
  *     gabp_svm_destroy().  A handle is not thread-safe: one thread at a time.
  *   - All work is issued on the handle's stream (opts.stream, or a stream the
  *     handle creates).  Every call returns after its work has completed.
+ *   - A round reads Q alone where every pair is weakly coupled: strictly dominant
+ *     rows, |Q_ij| at most Q_ii / 4 and Q_ij^2 / (Q_ii Q_jj) up to about 1.8e-3.  One
+ *     pair beyond that (near-duplicate rows with few other neighbours) or one row
+ *     that is not strictly dominant (possible under GABP_DIAG_SOFT2) makes the
+ *     instance store its messages: 28 to 36 bytes a pair and round in FP32 in
+ *     place of 4, a solve about six times as long at n = 20000.  Device memory
+ *     is reserved for either.
  *   - Non-convergence is not an error: gabp_svm_solve() returns GABP_OK with
  *     *iters_done == iters and the residual of the last round.
  */
@@ -107,7 +114,11 @@ typedef struct {
     int32_t refine;        /* precision form only: up to this many defect-correction passes with the
                               FP32-Gram residual (FP64 sums); 0 = plain BF16 solve */
     double  sv_threshold;  /* support vectors are the i with alpha_i > sv_threshold (default 0) */
-    int32_t chunk;         /* sweeps per captured CUDA graph replay between convergence checks; 0 = 16 */
+    int32_t chunk;         /* rounds per captured CUDA graph replay between convergence checks of the host;
+                              0 = 16.  No result depends on it.  A handle goes by it where it replays
+                              graphs: not in its first solves of a kind, which launch round by round and
+                              follow the device, and not in staged solves to a tolerance, which replay
+                              groups of two (unless the program has set its device to blocking waits) */
     int32_t msg_bf16;      /* precision forms only: store the messages in BF16 (arithmetic stays FP32);
                               use with refine > 0, which removes the rounding error */
     float   refine_handover; /* refinement only: the first solve hands over to the defect correction

@@ -551,11 +551,15 @@ gabp_status run_direct(gabp_svm_t h, int iters, int path, cudaGraphExec_t group,
     return GABP_OK;
 }
 
-// A handle's rounds go by captured chunks from its kGraphAfter-th call on:
-// capturing and instantiating 16 rounds costs the host 95 us, while launching them
-// one by one goes on beside the device, each round 1 to 2 us slower than in the
-// graph (100 rounds at n = 20000: 14.00 against 13.86 ms), but without rounds run
-// for nothing after the last and without waits between chunks.  A staged round of
+// A handle's rounds go by captured chunks once it has run kGraphAfter solves of
+// a kind (rounds of a chunk, message path): capturing and instantiating 16 rounds
+// costs the host 95 us, while launching them one by one goes on beside the device,
+// each round 1 to 2 us slower than in the graph (100 rounds at n = 20000: 14.00
+// against 13.86 ms), but without rounds run for nothing after the last and without
+// waits between chunks.  Solves to 1e-6, us directly / from the graphs: n = 1000
+// 578 / 614, n = 3000 950 / 650, n = 6238 1080 / 1018, n = 20000 4643 / 4667; so a
+// handle that is used once goes the way that needs no graph, one that is kept the
+// other.  A staged round of
 // eight kernels loses 15 us (n = 12960), so those are captured at once.  What a chunk
 // launches depends only on what is fixed at create, so its graph serves later
 // refits too; the few kept ones are dropped when calls with ever new round counts
@@ -1230,9 +1234,18 @@ static gabp_status get_pairs_recomputed(gabp_svm_t h, const std::vector<long lon
     const size_t bq = most * TT * sizeof(__nv_bfloat16), bw = align_up(most * sizeof(int4), 256), btab = align_up(sizeof(Inst), 256),
                  bctrl = align_up(sizeof(Ctrl), 256), bij = align_up(2 * cnt * sizeof(long long), 256),
                  bslot = align_up(cnt * sizeof(int), 256);
-    char* mem = nullptr;
-    CK(pool_alloc((void**)&mem, bq + bw + btab + bctrl + bij + bslot + cnt * sizeof(float4), s));
-    char* b = mem;
+    struct Block {   // given back on every way out
+        char* p = nullptr;
+        cudaStream_t s;
+        ~Block()
+        {
+            if (!p) return;
+            cudaFreeAsync(p, s);
+            cudaStreamSynchronize(s);
+        }
+    } mem{nullptr, s};
+    CK(pool_alloc((void**)&mem.p, bq + bw + btab + bctrl + bij + bslot + cnt * sizeof(float4), s));
+    char* b = mem.p;
     auto take = [&](size_t bytes) { char* r = b; b += bytes; return r; };
     Inst p = h->inst, former = h->inst;
     p.qstore = former.qstore = take(bq);
@@ -1242,48 +1255,42 @@ static gabp_status get_pairs_recomputed(gabp_svm_t h, const std::vector<long lon
     long long* dij = (long long*)take(bij);
     int* dslot = (int*)take(bslot);
     float4* dout = (float4*)take(cnt * sizeof(float4));
-    auto run = [&]() -> gabp_status {
-        CK(cudaMemsetAsync(former.ctrl, 0, sizeof(Ctrl), s));
-        CK(cudaMemcpyAsync(tab, &former, sizeof(Inst), cudaMemcpyHostToDevice, s));
-        std::vector<float4> got(cnt);
-        std::vector<int4> work;
-        std::vector<long long> part;   // the pairs of these tiles
-        std::vector<int> slot;
-        std::vector<size_t> at;
-        for (auto it = by_tile.begin(); it != by_tile.end();) {
-            work.clear(); part.clear(); slot.clear(); at.clear();
-            for (; it != by_tile.end() && work.size() < most; ++it) {
-                for (const size_t k : it->second) {
-                    part.push_back(ij[2 * k]);
-                    part.push_back(ij[2 * k + 1]);
-                    slot.push_back((int)work.size());
-                    at.push_back(k);
-                }
-                work.push_back(make_int4(0, it->first.first, it->first.second, (int)work.size()));
+    CK(cudaMemsetAsync(former.ctrl, 0, sizeof(Ctrl), s));
+    CK(cudaMemcpyAsync(tab, &former, sizeof(Inst), cudaMemcpyHostToDevice, s));
+    std::vector<float4> got(cnt);
+    std::vector<int4> work;
+    std::vector<long long> part;   // the pairs of these tiles
+    std::vector<int> slot;
+    std::vector<size_t> at;
+    for (auto it = by_tile.begin(); it != by_tile.end();) {
+        work.clear(); part.clear(); slot.clear(); at.clear();
+        for (; it != by_tile.end() && work.size() < most; ++it) {
+            for (const size_t k : it->second) {
+                part.push_back(ij[2 * k]);
+                part.push_back(ij[2 * k + 1]);
+                slot.push_back((int)work.size());
+                at.push_back(k);
             }
-            CK(cudaMemcpyAsync(dw, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
-            CK(cudaMemcpyAsync(dij, part.data(), part.size() * sizeof(long long), cudaMemcpyHostToDevice, s));
-            CK(cudaMemcpyAsync(dslot, slot.data(), slot.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-            CK(launch_form_q_tc(tab, dw, (long long)work.size(), s));
-            launch_get_pairs(p, dij, dslot, (long long)at.size(), dout, s);
-            CK(cudaGetLastError());
-            CK(cudaMemcpyAsync(got.data(), dout, at.size() * sizeof(float4), cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-            for (size_t e = 0; e < at.size(); ++e) std::memcpy(out + 4 * at[e], &got[e], sizeof(float4));
+            work.push_back(make_int4(0, it->first.first, it->first.second, (int)work.size()));
         }
-        CK(cudaMemcpyAsync(h->hdec, former.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(dw, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+        CK(cudaMemcpyAsync(dij, part.data(), part.size() * sizeof(long long), cudaMemcpyHostToDevice, s));
+        CK(cudaMemcpyAsync(dslot, slot.data(), slot.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+        CK(launch_form_q_tc(tab, dw, (long long)work.size(), s));
+        launch_get_pairs(p, dij, dslot, (long long)at.size(), dout, s);
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(got.data(), dout, at.size() * sizeof(float4), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        if (h->hdec->status != 0) return fail(GABP_ETIMEOUT, "a bounded device wait ran out in the inspection");
-        return GABP_OK;
-    };
-    const gabp_status st = run();
-    cudaFreeAsync(mem, s);
-    cudaStreamSynchronize(s);
-    return st;
+        for (size_t e = 0; e < at.size(); ++e) std::memcpy(out + 4 * at[e], &got[e], sizeof(float4));
+    }
+    CK(cudaMemcpyAsync(h->hdec, former.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    if (h->hdec->status != 0) return fail(GABP_ETIMEOUT, "a bounded device wait ran out in the inspection");
+    return GABP_OK;
 }
 
 gabp_status gabp_svm_get_pairs(gabp_svm_t h, const int64_t* i, const int64_t* j, int64_t cnt, float* out)
-{
+try {
     g_err.clear();
     if (gabp_status s = check_formed(h)) return s;
     if (cnt < 0 || (cnt > 0 && (!i || !j || !out))) return fail(GABP_EINVAL, "bad pair list");
@@ -1308,6 +1315,8 @@ gabp_status gabp_svm_get_pairs(gabp_svm_t h, const int64_t* i, const int64_t* j,
     cudaFreeAsync(dout, h->stream);
     CK(cudaStreamSynchronize(h->stream));
     return GABP_OK;
+} catch (const std::exception&) {   // (bad_alloc, length_error)
+    return fail(GABP_ENOMEM, "get_pairs: no host memory for the pair list");
 }
 
 gabp_status gabp_svm_set_profiling(gabp_svm_t h, int32_t on)

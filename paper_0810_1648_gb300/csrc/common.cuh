@@ -353,12 +353,6 @@ RoundGrid round_grid(long long max_tiles, int max_nblocks, int q_mode, int ctas_
 cudaError_t prepare_sweep();
 // Fused-recompute form: also raises the shared-memory limit of its sweep kernel.
 cudaError_t prepare_sweep_rc();
-// Launches a kernel of a round.  chained: it may start while the stream's last
-// kernel, of the same chain, still runs (it passes chain_wait() before it reads
-// what that one writes), which takes the launch and the kernel's start off a
-// round's path: n = 1000, 19.4 -> 16.4 us a round; n = 6238, 29.7 -> 27.1.  The
-// kernels of a captured graph are not chained: they start as early (15.2 and
-// 26.2 us), and chained ones later (staged, n = 12960: 133 -> 146 us).
 // Where the sweeps of the second message path run beside those of the first
 // (while a round is captured): most rounds of a batch that has both have little
 // on the second.  A batch of 512 problems: 38.6 ms one after the other, 37.1 side
@@ -367,6 +361,12 @@ struct Fork {
     cudaStream_t stream;
     cudaEvent_t start, end;
 };
+// Launches a kernel of a round.  chained: it may start while the stream's last
+// kernel, of the same chain, still runs (it passes chain_wait() before it reads
+// what that one writes), which takes the launch and the kernel's start off a
+// round's path: n = 1000, 19.4 -> 16.4 us a round; n = 6238, 29.7 -> 27.1.  The
+// kernels of a captured graph are not chained: they start as early (15.2 and
+// 26.2 us), and chained ones later (staged, n = 12960: 133 -> 146 us).
 enum Chain { CHAIN_NONE, CHAIN_AFTER_FIRST, CHAIN_ALL };   // which kernels of a round
 template <class... P, class... A>
 void launch_chained(bool chained, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args)

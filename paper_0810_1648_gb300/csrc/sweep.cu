@@ -1976,25 +1976,24 @@ void launch_round(const Inst* tab, const int4* work, const int2* nbl, const Sche
             chain = mode != CHAIN_NONE;
         }
         if (paths & (1 << PATH_STORED)) {
-            const cudaStream_t main = s;
-            const cudaStream_t s = both ? fork->stream : main;
+            const cudaStream_t q = both ? fork->stream : s;
             if (q_mode == 2 && msg_bf16)
-                launch_chained(chain, k_sweep_rc<MsgBF16>, g.sweep, RC_THREADS, rc_smem_bytes<MsgBF16>(), s, tab, work, sc, st);
+                launch_chained(chain, k_sweep_rc<MsgBF16>, g.sweep, RC_THREADS, rc_smem_bytes<MsgBF16>(), q, tab, work, sc, st);
             else if (q_mode == 2)
-                launch_chained(chain, k_sweep_rc<MsgF32>, g.sweep, RC_THREADS, rc_smem_bytes<MsgF32>(), s, tab, work, sc, st);
+                launch_chained(chain, k_sweep_rc<MsgF32>, g.sweep, RC_THREADS, rc_smem_bytes<MsgF32>(), q, tab, work, sc, st);
             else if (q_mode == 1 && msg_bf16)
                 launch_chained(chain, k_sweep<__nv_bfloat16, MsgBF16>, g.sweep, SWEEP_THREADS,
-                               sweep_smem_bytes<__nv_bfloat16, MsgBF16>(), s, tab, work, sc, st);
+                               sweep_smem_bytes<__nv_bfloat16, MsgBF16>(), q, tab, work, sc, st);
             else if (q_mode == 1)
                 launch_chained(chain, k_sweep<__nv_bfloat16, MsgF32>, g.sweep, SWEEP_THREADS,
-                               sweep_smem_bytes<__nv_bfloat16, MsgF32>(), s, tab, work, sc, st);
+                               sweep_smem_bytes<__nv_bfloat16, MsgF32>(), q, tab, work, sc, st);
             else
-                launch_chained(chain, k_sweep<float, MsgF32>, g.sweep, SWEEP_THREADS, sweep_smem_bytes<float, MsgF32>(), s,
+                launch_chained(chain, k_sweep<float, MsgF32>, g.sweep, SWEEP_THREADS, sweep_smem_bytes<float, MsgF32>(), q,
                                tab, work, sc, st);
             chain = mode != CHAIN_NONE;
             if (both) {
-                cudaEventRecord(fork->end, s);
-                cudaStreamWaitEvent(main, fork->end, 0);
+                cudaEventRecord(fork->end, q);
+                cudaStreamWaitEvent(s, fork->end, 0);
             }
         }
         if (ev && st == nstages - 1) cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal);
