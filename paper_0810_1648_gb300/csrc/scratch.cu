@@ -9,8 +9,12 @@
 // requests take a few us each (with the waits that went in the same step: 2.50
 // -> 1.62 ms and 1.75 -> 1.07 ms).
 //
-// What is kept is bounded: the pool holds at most kScratchKeep unused bytes
-// per device past a synchronisation, the list kPinnedKeep bytes a process.  The pool
+// What is kept is bounded: the pool has at most kScratchKeep bytes per device past a
+// synchronisation, used and unused (the driver counts both), the list kPinnedKeep
+// bytes a process.  So blocks come from the pool only while those in use stay
+// within it, and from cudaMalloc beyond: a pool that has to grow past its reserve
+// maps and unmaps the memory of every block (n = 6500, a second handle beside one
+// of 430 MB: create 540 us, now as with cudaMalloc alone, 280).  The pool
 // gives its unused memory back as soon as a larger request (device_available
 // with trim, or pool_alloc) needs it, and in gabp_batch_release.  Both are safe
 // with several threads; blocks are given back only after the work that used
@@ -67,14 +71,20 @@ cudaMemPool_t scratch_pool(bool make)
     return pool;
 }
 
-size_t unused_bytes(cudaMemPool_t pool)
+uint64_t pool_bytes(cudaMemPool_t pool, cudaMemPoolAttr what)
 {
-    uint64_t reserved = 0, used = 0;
-    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
-        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+    uint64_t v = 0;
+    if (cudaMemPoolGetAttribute(pool, what, &v) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
+    return v;
+}
+
+size_t unused_bytes(cudaMemPool_t pool)
+{
+    const uint64_t reserved = pool_bytes(pool, cudaMemPoolAttrReservedMemCurrent),
+                   used = pool_bytes(pool, cudaMemPoolAttrUsedMemCurrent);
     return reserved > used ? (size_t)(reserved - used) : 0;
 }
 
@@ -98,7 +108,8 @@ cudaError_t scratch_alloc(DevBlock* b, size_t bytes, cudaStream_t s)
 {
     *b = DevBlock{};
     if (scratch_fits(bytes)) {
-        if (cudaMemPool_t pool = scratch_pool(true)) {
+        const cudaMemPool_t pool = scratch_pool(true);
+        if (pool && pool_bytes(pool, cudaMemPoolAttrUsedMemCurrent) + bytes <= kScratchKeep) {
             if (cudaMallocFromPoolAsync(&b->p, bytes, pool, s) == cudaSuccess) {
                 b->pooled = true;
                 return cudaSuccess;
@@ -107,9 +118,13 @@ cudaError_t scratch_alloc(DevBlock* b, size_t bytes, cudaStream_t s)
             b->p = nullptr;
         }
     }
-    size_t avail = 0;
-    device_available(&avail, true);   // the pools' unused memory back first
-    const cudaError_t e = cudaMalloc(&b->p, bytes);
+    cudaError_t e = cudaMalloc(&b->p, bytes);
+    if (e == cudaErrorMemoryAllocation) {   // the pools' unused memory back first
+        cudaGetLastError();
+        size_t avail = 0;
+        device_available(&avail, true);
+        e = cudaMalloc(&b->p, bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         b->p = nullptr;
