@@ -289,13 +289,6 @@ struct RoundGrid {
     int one = 0;             // a single instance (tab[0]): its node blocks, negative if it has at most kWarpFinNt tile rows
 };
 
-// Gram operands: rows [0, n) of an n x m FP32 matrix with row norms sq.
-struct GramSide {
-    const float* X;
-    const float* sq;
-    int n;
-};
-
 // ---- launchers (defined in the .cu files) --------------------------------
 // Inputs: convert/validate X and y, right-hand sides, and the three BF16 planes
 // of the rows (gram_tc32.cu).  SVM (task 0): y must be +-1, b = b0 = 1.  KRR (task
@@ -404,7 +397,7 @@ cudaError_t prepare_sweep_hist();
 // FP32 Gram's when Q is recomputed).
 // single: tab holds one instance.
 void launch_pair_z(const Inst* tab, const int4* tiles, long long ntiles, int q_mode, bool single, cudaStream_t s);
-void launch_pair_z_gram(const Inst* tab, const int4* tiles, long long ntiles, int grid, bool single, cudaStream_t s);
+cudaError_t launch_pair_z_gram(const Inst* tab, const int4* tiles, long long ntiles, bool single, cudaStream_t s);
 
 // Final FP32-Gram residual r = 1 - Q mu (FP64 sums), dual objective and
 // alpha = clip(mu, 0, C) of the listed instances (their tiles, node blocks

@@ -1,18 +1,14 @@
 // The node sums of the final pass (residual r = 1 - Q mu and the dual objective
-// from Q alpha; the tiles' parts come from sweep_hist.cu and gram_tc32.cu), and SIMT
-// FP32 Gram tiles fused with the RBF kernel: decision values of callers without a
-// handle (gabp_decision_noalloc), and the pair pass of instances that do not store
-// Q.  (Staging, Q tiles and decisions of a handle: gram_tc32.cu.)
-//
-// In gram_tile one CTA computes one 128 x 128 Gram tile G = X_I X_J^T by SIMT FP32 FMAs
-// (8 x 8 outputs per thread, K-chunks of 16 double-buffered in shared memory),
-// then runs an epilogue on the 64 values it holds: d^2 = max(0, s_i + s_j - 2 G),
-// K = expf(-gamma d^2), Q_ij = y_i y_j (K + lambda^2).  The distances use the
-// norm expansion with norms of the same FP32 rows, so d^2_ii is 0 up to
-// rounding and is clamped at 0.
+// from Q alpha; the tiles' parts come from sweep_hist.cu and gram_tc32.cu), Q read
+// back, and decision values of callers without a handle (gabp_decision_noalloc):
+// SIMT FP32 Gram tiles by FMAs, K-chunks of 16 double-buffered in shared memory, with
+// an epilogue on the values that a thread holds: d^2 = max(0, s_i + s_j - 2 G), K =
+// expf(-gamma d^2) + lambda^2.  The distances use the norm expansion with norms of
+// the same FP32 rows, so d^2_ii is 0 up to rounding and is clamped at 0.  (Staging, Q
+// tiles and decisions of a handle: gram_tc32.cu.)
 #include "common.cuh"
 #include "gabp_svm.h"
-#include "hist.cuh"
+#include "ptx.cuh"
 
 #include <float.h>
 #include <mutex>
@@ -23,70 +19,6 @@ namespace gabp {
 namespace {
 
 constexpr int KC = 16;
-
-struct GramSmem {
-    float A[2][KC][T + 4];   // double-buffered K-chunks
-    float B[2][KC][T + 4];
-};
-
-// acc[a][b] = <x_{I*T + ty*8 + a}, x_{J*T + tx*8 + b}>.  K-chunks of KC
-// features go through two shared-memory buffers: the next chunk's global
-// loads are in flight (in registers) while the current chunk's FMAs run, and
-// one barrier per chunk separates the buffer swaps.  Every output sums its
-// products in ascending k, as a plain loop would.
-__device__ __forceinline__ void gram_tile(const GramSide& A, const GramSide& B, int m, int I, int J,
-                                          GramSmem& sm, float (&acc)[8][8])
-{
-    constexpr int LD = (T * KC) / NTHREADS;   // elements of each operand a thread stages per chunk
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
-    float ra[LD], rb[LD];
-    auto load = [&](int k0) {
-#pragma unroll
-        for (int u = 0; u < LD; ++u) {
-            const int e = tid + NTHREADS * u;
-            const int row = e / KC, kk = e % KC, k = k0 + kk;
-            const int ga = I * T + row, gb = J * T + row;
-            ra[u] = (ga < A.n && k < m) ? A.X[(size_t)ga * m + k] : 0.f;
-            rb[u] = (gb < B.n && k < m) ? B.X[(size_t)gb * m + k] : 0.f;
-        }
-    };
-    auto store = [&](int buf) {
-#pragma unroll
-        for (int u = 0; u < LD; ++u) {
-            const int e = tid + NTHREADS * u;
-            const int row = e / KC, kk = e % KC;
-            sm.A[buf][kk][row] = ra[u];
-            sm.B[buf][kk][row] = rb[u];
-        }
-    };
-    const int nch = (m + KC - 1) / KC;
-    load(0);
-    store(0);
-    __syncthreads();
-    for (int c = 0; c < nch; ++c) {
-        const int buf = c & 1;
-        if (c + 1 < nch) load((c + 1) * KC);
-#pragma unroll
-        for (int kk = 0; kk < KC; ++kk) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&sm.A[buf][kk][ty * 8]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&sm.A[buf][kk][ty * 8 + 4]);
-            const float4 b0 = *reinterpret_cast<const float4*>(&sm.B[buf][kk][tx * 8]);
-            const float4 b1 = *reinterpret_cast<const float4*>(&sm.B[buf][kk][tx * 8 + 4]);
-            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-            for (int a = 0; a < 8; ++a)
-#pragma unroll
-                for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(av[a], bv[b], acc[a][b]);
-        }
-        if (c + 1 < nch) store(buf ^ 1);
-        __syncthreads();
-    }
-}
 
 // RBF entry from a Gram value (norm expansion, clamped distance).
 __device__ __forceinline__ float rbf_from_gram(float g, float si, float sj, float gamma)
@@ -101,54 +33,6 @@ __device__ __forceinline__ float sum16(float v)
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-// k_pair_z (sweep_hist.cu) for instances that do not store Q (only those that
-// their margin leaves open get as far as the Gram tile).
-__global__ void __launch_bounds__(NTHREADS) k_pair_z_gram(const Inst* __restrict__ tab, const int4* __restrict__ work,
-                                                          long long ntiles, bool single)
-{
-    __shared__ __align__(16) GramSmem sm;
-    __shared__ int s_go;
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    if (single) {
-        if (tid == 0) s_go = pair_z_open(tab[0]);
-        __syncthreads();
-        if (!s_go) return;
-        __syncthreads();
-    }
-    for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
-        const int4 w = work[L];
-        for (int k = w.x; k >= 0; k = tab[k].form_next - 1) {
-            const Inst& p = tab[k];
-            if (tid == 0) s_go = pair_z_open(p);
-            __syncthreads();
-            const int go = s_go;
-            __syncthreads();   // s_go is read before the next instance writes it
-            if (!go) continue;
-            float acc[8][8];
-            const GramSide S{p.X, p.sq3, p.n};
-            gram_tile(S, S, p.m, w.y, w.z, sm, acc);
-            float best[2] = {0.f, FLT_MIN};   // the second never 0: the pass has run
-#pragma unroll
-            for (int a = 0; a < 8; ++a) {
-                const int i = w.y * T + ty * 8 + a, ii = min(i, p.n - 1);
-                const float si = p.sq3[ii], ri = 1.f / p.qdiag[ii];
-#pragma unroll
-                for (int b = 0; b < 8; ++b) {
-                    const int j = w.z * T + tx * 8 + b;
-                    if (i < j && j < p.n)
-                        note_pair_z(rbf_from_gram(acc[a][b], si, p.sq3[j], p.gamma) + p.lam2, ri, 1.f / p.qdiag[j], best);
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                best[q] = warp_max_f(best[q]);
-                if ((tid & 31) == 0) atomicMax(&p.ctrl->zpair_bits[q], __float_as_uint(best[q]));
-            }
-            __syncthreads();
-        }
-    }
 }
 
 // Sum of FP32 values to more than FP64's bits without the FP64 pipe, which on
@@ -289,12 +173,6 @@ __global__ void k_get_q(Inst p, const int4* __restrict__ work, int q_bf16, float
 }
 
 }  // namespace
-
-void launch_pair_z_gram(const Inst* tab, const int4* tiles, long long ntiles, int grid, bool single,
-                        cudaStream_t s)
-{
-    k_pair_z_gram<<<grid, NTHREADS, 0, s>>>(tab, tiles, ntiles, single);
-}
 
 void launch_final(const Inst* tab, const StopOp* ops, const int4* tiles, long long ntiles, const int2* nbl,
                   int nblocks, const int* members, int nmembers, double* f3_all, int q_stored, cudaStream_t s)

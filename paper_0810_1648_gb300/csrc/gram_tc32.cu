@@ -36,13 +36,20 @@
 //   final pass  the same entries, not stored, times the means and the weights
 //               (instances that recompute Q);
 //   decision    entries of test rows against training rows, times the weights,
-//               summed over a range of training tiles in registers.
+//               summed over a range of training tiles in registers;
+//   pair pass   the largest z and |q| / d over the pairs (k_pair_z of
+//               sweep_hist.cu) for instances that recompute Q.  The entries are
+//               those that the other forms store, bit for bit, so that all of them
+//               choose the same message path.  (From SIMT FP32 tiles, whose sums
+//               round otherwise, refits of such handles took 1064 us at n = 6000, m
+//               = 784 and 539 at n = 9000, m = 128.)
 // Bound by the epilogue's latencies (the FMA pipe is 28 % busy, the LSU
 // 14 %): with eight epilogue warps (64 columns each, all four accumulators
 // handed over at once) two warps a scheduler left it waiting; with the epilogue
 // looking up lists, tables and slots itself, formation took 522 us (n = 20000, m =
 // 128) and 162 us (n = 12000, m = 64), now 350 and 104.
 #include "common.cuh"
+#include "hist.cuh"
 #include "ptx.cuh"
 #include "qtile_epi.cuh"
 
@@ -250,6 +257,7 @@ __global__ void __launch_bounds__(256) k_stage_list(const Inst* __restrict__ tab
 enum T3Mode {
     T3_FORM,     // Q tiles, |Q| sums (and, norms_only, the squared norms)
     T3_FINAL,    // sums q mu and q alpha of a tile's pairs, Q not stored
+    T3_PAIRZ,    // the largest z and |q| / d of a tile's pairs, Q not stored (norms_only: one instance)
     T3_DECIDE    // decision values: rows = test rows, sums over the training columns
 };
 
@@ -276,7 +284,7 @@ struct T3Const {
 // instance tables and slots were a third of its time.
 struct T3Item {
     int nkc;                 // chunks of accumulators to take in first; 0: the Gram at hand
-    int end, diag, last;     // no item; a diagonal tile; decision: the entry's last tile
+    int end, diag, last;     // no item; a diagonal tile; decision: the entry's last tile, pair pass: to be looked at
     int rows, cols;          // rows and columns that there are (may exceed T)
     float gamma, lam2;
     float* store;            // where the entries go, or null
@@ -410,6 +418,17 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
     unsigned char* oper = align_smem(smem_raw, 1024);
     T3Smem& sm = *reinterpret_cast<T3Smem*>(oper + T3_STAGES * T3_STAGE_BYTES);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (what pair_z_asks reads is fixed by now: every role finds the same)
+    if (MODE == T3_PAIRZ && norms_only && !pair_z_asks(tab[0])) return;
+    auto skipped = [&](int4 w) {
+        if constexpr (MODE == T3_PAIRZ) {
+            bool none = !norms_only;
+            for (int k = none ? w.x : -1; k >= 0 && none; k = tab[k].form_next - 1) none = !pair_z_asks(tab[k]);
+            return none;
+        } else {
+            return false;
+        }
+    };
 
     if (tid == 0) {
         for (int s = 0; s < T3_STAGES; ++s) { mbar_init(&sm.xfull[s], 1); mbar_init(&sm.xempty[s], 1); }
@@ -438,6 +457,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
             bool run = true;
             for (long long L = blockIdx.x; L < ntiles && run; L += gridDim.x) {
                 const int4 w = work[L];
+                if (skipped(w)) continue;
                 const Inst& p = tab[w.x];
                 const unsigned char* A3 = static_cast<const unsigned char*>(p.Xp3);
                 const unsigned char* B3 = MODE == T3_DECIDE ? static_cast<const unsigned char*>(tab[1].Xp3) : A3;
@@ -469,6 +489,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
             bool run = true;
             for (long long L = blockIdx.x; L < ntiles && run; L += gridDim.x) {
                 const int4 w = work[L];
+                if (skipped(w)) continue;
                 const Inst& p = tab[w.x];
                 Ctrl* ctrl = p.ctrl;
                 const int chunks = p.nkc * (last_j(w) - first_j(w));
@@ -512,13 +533,14 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
         for (long long L = blockIdx.x; L < ntiles && run; L += gridDim.x) {
             const int4 w = wn;
             if (L + gridDim.x < ntiles) wn = work[L + gridDim.x];
+            if (skipped(w)) continue;
             const int I = w.y;
             for (int J = first_j(w); J < last_j(w) && run; ++J) {
                 for (int k = w.x; k >= 0 && run;) {
                     const Inst& p = tab[k];                              // rows
                     const Inst& cp = MODE == T3_DECIDE ? tab[1] : p;     // columns
                     const int n = p.n, rows = n - I * T, cols = cp.n - J * T;
-                    const int next = MODE == T3_FORM && consts ? p.form_next - 1 : -1;
+                    const int next = (MODE == T3_FORM && consts) || MODE == T3_PAIRZ ? p.form_next - 1 : -1;
                     // lane + 32 u of the tile's columns ([0]) and rows ([1])
                     float y[2][4], q[2][4], m[2][4];
                     if (consts) {
@@ -530,9 +552,10 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                             for (int u = 0; u < 4; ++u) {
                                 const int x = (r ? I : J) * T + lane + 32 * u;
                                 const bool in = x < o.n;
-                                y[r][u] = in && (MODE != T3_DECIDE || r == 0) ? o.y[x] : 0.f;
+                                y[r][u] = in && MODE != T3_PAIRZ && (MODE != T3_DECIDE || r == 0) ? o.y[x] : 0.f;
                                 q[r][u] = in ? o.sq3[x] : 0.f;
-                                m[r][u] = in && mu ? mu[x] : 0.f;
+                                if (MODE == T3_PAIRZ) m[r][u] = in ? __fdividef(1.f, o.qdiag[x]) : 0.f;
+                                else m[r][u] = in && mu ? mu[x] : 0.f;
                             }
                         }
                     }
@@ -557,6 +580,10 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                                     if (r == 0) c.mu[0][x] = m[0][u] * y[0][u];
                                     continue;
                                 }
+                                if (MODE == T3_PAIRZ) {
+                                    c.mu[r][x] = m[r][u];
+                                    continue;
+                                }
                                 c.y[r][x] = __uint_as_float(__float_as_uint(y[r][u]) & 0x80000000u);
                                 if (MODE == T3_FINAL) {
                                     c.mu[r][x] = m[r][u];
@@ -569,7 +596,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                         t.nkc = k == w.x ? p.nkc : 0;
                         t.end = 0;
                         t.diag = MODE != T3_DECIDE && I == J;
-                        t.last = J + 1 == last_j(w);
+                        t.last = MODE == T3_PAIRZ ? pair_z_asks(p) : J + 1 == last_j(w);
                         t.rows = rows;
                         t.cols = cols;
                         t.gamma = cp.gamma;
@@ -578,7 +605,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                         t.w = w;
                         if (MODE == T3_DECIDE) {
                             t.dst[0] = dec.part + L * T;
-                        } else if (consts) {
+                        } else if (consts && MODE != T3_PAIRZ) {
                             const int2 sl = p.rfix ? make_int2(0, 0) : tile_slots(p, w);
                             t.plen = (long long)part_len(p);
                             float* part = p.part + (MODE == T3_FINAL ? 2 * t.plen : 0);
@@ -702,6 +729,32 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                         it.dst[0][etid] = (float)v;
                     }
                     sb ^= 1;
+                }
+            } else if (MODE == T3_PAIRZ) {
+                if (it.last) {
+                    const Rbf rb = rbf_of(it.gamma, it.lam2);
+                    const int rows = it.rows, cols = it.cols;
+                    float best[2] = {0.f, FLT_MIN};   // the second never 0: the pass has run
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int c = cq + 2 * j;
+                        const float2 sj = ld2(&cc.sq[0][c]), rj = ld2(&cc.mu[0][c]);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int rk = r0 + 2 * k, least = it.diag ? rk : -1;
+                            const float ri = cc.mu[1][rk];
+                            const float2 e = rbf2(rb, G.v[k][j], cc.sq[1][rk], sj);
+                            if (rk < rows && c < cols && c > least) note_pair_z(e.x, ri, rj.x, best);
+                            if (rk < rows && c + 1 < cols && c + 1 > least) note_pair_z(e.y, ri, rj.y, best);
+                        }
+                    }
+                    unsigned* const to = it.ctrl->zpair_bits;
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        best[u] = warp_max_f(best[u]);
+                        if (lane == 0 && __float_as_uint(best[u]) > *(volatile unsigned*)&to[u])
+                            atomicMax(&to[u], __float_as_uint(best[u]));
+                    }
                 }
             } else {
                 const Rbf rb = rbf_of(it.gamma, it.lam2);
@@ -908,6 +961,11 @@ cudaError_t launch_stage_list(const Inst* tab, const int2* nbl, int nblocks, cud
 cudaError_t launch_form_q_tc32(const Inst* tab, const int4* work, long long ntiles, int norms_only, cudaStream_t s)
 {
     return launch_gram<T3_FORM>(tab, work, ntiles, norms_only, nullptr, DecideArgs{}, s);
+}
+
+cudaError_t launch_pair_z_gram(const Inst* tab, const int4* tiles, long long ntiles, bool single, cudaStream_t s)
+{
+    return launch_gram<T3_PAIRZ>(tab, tiles, ntiles, single, nullptr, DecideArgs{}, s);
 }
 
 cudaError_t launch_final_tiles_gram(const Inst* tab, const StopOp* ops, const int4* tiles, long long ntiles, cudaStream_t s)

@@ -1216,10 +1216,12 @@ void launch_final_tiles_q(const Inst* tab, const StopOp* ops, const int4* tiles,
 void launch_pair_z(const Inst* tab, const int4* tiles, long long ntiles, int q_mode, bool single, cudaStream_t s)
 {
     if (ntiles <= 0) return;
-    const long long most = (q_mode == 2 ? 4 : 2) * num_sms();
-    const int grid = (int)(ntiles < most ? ntiles : most);
-    if (q_mode == 2) launch_pair_z_gram(tab, tiles, ntiles, grid, single, s);
-    else k_pair_z<<<grid, 256, 0, s>>>(tab, tiles, ntiles, single);
+    if (q_mode == 2) {
+        (void)launch_pair_z_gram(tab, tiles, ntiles, single, s);   // errors surface at the caller's cudaGetLastError
+        return;
+    }
+    const long long most = 2 * num_sms();
+    k_pair_z<<<(int)(ntiles < most ? ntiles : most), 256, 0, s>>>(tab, tiles, ntiles, single);
 }
 
 }  // namespace gabp
