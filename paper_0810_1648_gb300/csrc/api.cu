@@ -50,6 +50,8 @@ constexpr int kRhistCap = 1 << 16;
 // A handle keeps its decision workspace for the next call up to this size
 // (allocating it on each call took longer than a small decision).
 constexpr size_t kDecisionKeep = (size_t)64 << 20;
+// Test rows of a decision that go through at a time.
+constexpr int64_t kSlabRows = (int64_t)1 << 17, kSlabLeast = 16 * T, kSlabPlanes = (int64_t)1 << 30;
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -1087,7 +1089,10 @@ gabp_status gabp_svm_decision(gabp_svm_t h, const void* Xtest, int64_t t, float*
     // their planes packed and checked in one pass over the caller's rows.  A refused
     // row leaves `out` as it is: the values stay in the workspace until every row has
     // been checked (of one slab on the device, the last kernel itself looks).
-    const int64_t slab = std::min<int64_t>(t, (int64_t)1 << 17);
+    // A slab's planes take kSlabPlanes bytes at most (with wide rows: fewer of them,
+    // down to kSlabLeast), so that a call needs no more memory than its rows do.
+    const int64_t row_planes = (int64_t)pack3_bytes(1, (int)m) / T;
+    const int64_t slab = std::min({t, kSlabRows, std::max(kSlabLeast, kSlabPlanes / row_planes / T * T)});
     const int Ntt = (int)((slab + T - 1) / T);
     const int per = decision_entries(Ntt);   // entries of a slab, at most
     const size_t bxp = align_up(pack3_bytes(Ntt, (int)m), 1024), bsq = align_up((size_t)Ntt * T * 4, 256);

@@ -102,3 +102,28 @@ def test_noalloc_at_its_limits(n, t):
     want, _ = _reference(p.X, np.ones(p.n), w, p.gamma, 0.25, base)
     scale = np.abs(alpha.astype(np.float64) * y).sum()
     assert np.max(np.abs(out.cpu().numpy() - want[np.arange(t) % len(base)])) <= BAR * scale
+
+
+def test_wide_rows_need_no_more_memory_than_they_take():
+    """2^17 rows of 8000 features (4.2 GB) with 5.5 GB left on the device: the three
+    planes of all of them at once would take 6.3."""
+    torch = pytest.importorskip("torch")
+    n, m, t = 300, 8000, SLAB
+    p = workloads.mixture(n, m, seed=9, gamma=0.2 / m)
+    svm, alpha, lam = _fit(p, True)
+    X = torch.from_numpy(p.X).cuda()
+    g = torch.Generator(device="cuda").manual_seed(3)
+    Z = X[torch.arange(t, device="cuda") % n]
+    Z[:, ::7] += 0.5 * torch.randn((t, len(range(0, m, 7))), device="cuda", generator=g)
+    torch.cuda.empty_cache()
+    gabp.batch_release()
+    filler = torch.empty(max(0, torch.cuda.mem_get_info()[0] - int(5.5e9)), dtype=torch.uint8, device="cuda")
+    try:
+        got = svm.decision(Z).cpu().numpy()
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    rows = np.unique(np.concatenate([np.arange(0, t, 4001), [t - 1]]))
+    want, scale = _reference(p.X, p.y, alpha, p.gamma, lam, Z[torch.from_numpy(rows).cuda()].cpu().numpy())
+    assert np.max(np.abs(got[rows] - want)) <= BAR * scale
+    svm.close()
