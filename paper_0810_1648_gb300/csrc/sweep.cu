@@ -278,11 +278,8 @@ __device__ __forceinline__ void sweep_producer(const Inst* __restrict__ tab, con
     int stage = 0, slot = 0;
     uint32_t phase = 0, tph = 0;
     auto stopped = [&]() { return __shfl_sync(0xffffffffu, abort_flag ? *abort_flag : 0, 0) != 0; };
-    auto landed = [&]() {
-        await_copies<stages<MSG>()>(sm.full, stage, phase);
-        await_copies<2>(sm.tfull, slot, tph);
-    };
-    for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
+    bool ok = true;
+    for (long long L = blockIdx.x; L < ntiles && ok; L += gridDim.x) {
         const int4 w = work[L];
         const Inst& p = tab[w.x];
         Ctrl* ctrl = p.ctrl;
@@ -301,8 +298,8 @@ __device__ __forceinline__ void sweep_producer(const Inst* __restrict__ tab, con
                 record_error(ctrl, ST_ETIMEOUT, L);
                 if (abort_flag) *abort_flag = 1;
             }
-            landed();
-            return;
+            ok = false;
+            break;
         }
         if (lane == 0) {
             TileInfo& ti = sm.info[slot];
@@ -344,8 +341,8 @@ __device__ __forceinline__ void sweep_producer(const Inst* __restrict__ tab, con
                     record_error(ctrl, ST_ETIMEOUT, L);
                     if (abort_flag) *abort_flag = 1;
                 }
-                landed();
-                return;
+                ok = false;
+                break;
             }
             unsigned char* S = ring + (size_t)stage * SB;
             unsigned long long* bar = &sm.full[stage];
@@ -384,8 +381,9 @@ __device__ __forceinline__ void sweep_producer(const Inst* __restrict__ tab, con
         }
     }
     // end of this CTA's tiles
-    landed();
-    if (!stopped() && mbar_wait_warp(&sm.tempty[slot], tph ^ 1u) && lane == 0) {
+    await_copies<stages<MSG>()>(sm.full, stage, phase);
+    await_copies<2>(sm.tfull, slot, tph);
+    if (ok && !stopped() && mbar_wait_warp(&sm.tempty[slot], tph ^ 1u) && lane == 0) {
         sm.info[slot].end = 1;
         mbar_arrive(&sm.tfull[slot]);
     }

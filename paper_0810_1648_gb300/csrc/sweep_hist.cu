@@ -111,16 +111,13 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
     int stage = 0, slot = 0;
     uint32_t phase = 0, tph = 0;
     auto stopped = [&]() { return abort_flag && __shfl_sync(0xffffffffu, *abort_flag, 0) != 0; };
-    auto landed = [&]() {
-        if constexpr (STREAM) await_copies<H_STAGES>(sm.full, stage, phase);
-        await_copies<2>(sm.tfull, slot, tph);
-    };
+    bool ok = true;
     auto give_up = [&](Ctrl* ctrl, long long L) {
         if (lane == 0) {
             record_error(ctrl, ST_ETIMEOUT, L);
             if (abort_flag) *abort_flag = 1;
         }
-        landed();
+        ok = false;
     };
     // The round's settings of an instance do not change during a sweep: they
     // are read once per run of tiles of the same instance, and the next tile's
@@ -130,7 +127,7 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
     bool done = true, staged = false;
     uint32_t use = 0;
     int4 wn = blockIdx.x < ntiles ? work[blockIdx.x] : make_int4(0, 0, 0, 0);
-    for (long long L = blockIdx.x; L < ntiles; L += gridDim.x) {
+    for (long long L = blockIdx.x; L < ntiles && ok; L += gridDim.x) {
         const int4 w = wn;
         if (L + gridDim.x < ntiles) wn = work[L + gridDim.x];
         const Inst& p = tab[w.x];
@@ -159,7 +156,7 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
         const int I = w.y, J = w.z, rows = min(T, p.n - I * T);
         if (stopped() || !mbar_wait_warp(&sm.tempty[slot], tph ^ 1u)) {
             give_up(ctrl, L);
-            return;
+            break;
         }
         if (lane == 0) {
             HInfo& ti = sm.info[slot];
@@ -205,7 +202,7 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
             for (int c = 0; c < nch; ++c) {
                 if (!mbar_wait_warp(&sm.empty[stage], phase ^ 1u)) {
                     give_up(ctrl, L);
-                    return;
+                    break;
                 }
                 if (lane == 0) {
                     mbar_arrive_expect_tx(&sm.full[stage], (uint32_t)H_CHUNK);
@@ -216,8 +213,9 @@ __device__ __forceinline__ void hist_producer(const Inst* __restrict__ tab, cons
             }
         }
     }
-    landed();
-    if (!stopped() && mbar_wait_warp(&sm.tempty[slot], tph ^ 1u) && lane == 0) {
+    if constexpr (STREAM) await_copies<H_STAGES>(sm.full, stage, phase);
+    await_copies<2>(sm.tfull, slot, tph);
+    if (ok && !stopped() && mbar_wait_warp(&sm.tempty[slot], tph ^ 1u) && lane == 0) {
         sm.info[slot].end = 1;
         mbar_arrive(&sm.tfull[slot]);
     }
